@@ -137,19 +137,6 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
         fence_proxy_async();
         prefetch_tmap(&tmKV); prefetch_tmap(&tmQ); prefetch_tmap(&tmDO); prefetch_tmap(&tmOut);
     }
-    grid_dep_launch();
-    grid_dep_wait();                                        // inputs come from the previous kernels
-    int early = 0;                                          // sub-tiles of the first item requested in the prologue
-    if (threadIdx.x == 0) {
-        KvItem it;
-        const int idx0 = draw();
-        item_slot[0] = idx0;
-        mbar_arrive(bar(L::kIF));
-        if (kv_item(p, idx0, it)) {
-            load_kv(it, 0);
-            for (; early < it.n_u && early < L::kStages; ++early) load_q(it, early, early);
-        }
-    }
     if (warp == 1) {
         tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
@@ -158,20 +145,21 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-
+    grid_dep_launch();                                      // (after the TMEM allocation: see grid_dep_launch)
+    grid_dep_wait();                                        // inputs come from the previous kernels
+    // the producer and the MMA role are each the loop of one elected thread (see the forward kernel)
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t m = 0;                                 // sub-tiles requested so far
             bool ok = true;
             KvItem it;
-            int idx = item_slot[0];
+            int idx = draw();
+            item_slot[0] = idx;
+            mbar_arrive(bar(L::kIF));
             for (int k = 0; ok && kv_item(p, idx, it); ++k) {
-                if (k > 0) {
-                    if (!mbar_wait(bar(2 + (k & 1)), ((k >> 1) & 1) ^ 1, abort_flag, p.status, 501)) break;
-                    load_kv(it, k & 1);
-                }
+                if (!mbar_wait(bar(2 + (k & 1)), ((k >> 1) & 1) ^ 1, abort_flag, p.status, 501)) break;
+                load_kv(it, k & 1);
                 for (int i = 0; i < it.n_u && ok; ++i, ++m) {
-                    if (k == 0 && i < early) continue;
                     const int s = m % L::kStages;
                     if (!mbar_wait(bar(L::kQE + s), ((m / L::kStages) & 1) ^ 1, abort_flag, p.status, 500)) { ok = false; break; }
                     load_q(it, i, s);
@@ -185,18 +173,18 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
             }
         }
     } else if (warp == 1) {
-        // converged warp, one elected lane issues (see the forward kernel)
+        if (elect_one()) {
         constexpr uint32_t idesc_st = make_idesc_bf16(128, 64, false, false);
         constexpr uint32_t idesc_acc = make_idesc_bf16(128, DH, false, true);
-        const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0);
-        const uint32_t sb = __shfl_sync(0xffffffffu, sbase, 0);
+        const uint32_t tb = tmem_base;
+        const uint32_t sb = sbase;
         auto issue_scores = [&](uint32_t g, int buf) {      // S^T and dP^T of stream position g into buffer g % kBufs
             const int s = g % L::kStages, hb = g % L::kBufs;
             const uint64_t desc_k = make_smem_desc_sw128(sb + L::kK + buf * 2 * L::kKV, 16, 1024);
             const uint64_t desc_v = desc_advance(desc_k, L::kKV);
             const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + s * 2 * L::kSub, 16, 1024), dg = desc_advance(dq, L::kSub);
             const uint32_t st = tb + hb * 64;
-            if (elect_one()) {
+            {
                 // the two products are independent accumulation chains: their steps alternate, so that a step
                 // never has to wait for the one before it to leave the pipe
 #pragma unroll
@@ -210,14 +198,13 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
                     }
                 umma_commit(bar(L::kSF + hb));
             }
-            __syncwarp();
         };
         auto issue_acc = [&](uint32_t g, bool first) {      // dV += P^T dO_u, dK += dS^T Q_u
             const int s = g % L::kStages, hb = g % L::kBufs;
             const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + s * 2 * L::kSub, 8192, 1024), dg = desc_advance(dq, L::kSub);
             const uint32_t pt = tb + hb * 64;
             const uint32_t acc0 = first ? 0u : 1u;
-            if (elect_one()) {
+            {
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks) {             // dV and dK alternate (independent accumulators)
                     umma_f16_ta(tb + L::kDV, pt + (ks >> 1) * 32 + (ks & 1) * 8, desc_advance(dg, ks * 2048), idesc_acc,
@@ -227,20 +214,17 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
                 }
                 umma_commit(bar(L::kQE + s));               // Q_u / dO_u stage free
             }
-            __syncwarp();
         };
         auto wait = [&](int b, uint32_t parity, int site) {
-            const bool w = mbar_wait(bar(b), parity, abort_flag, p.status, site);
-            return __all_sync(0xffffffffu, w);
+            return mbar_wait(bar(b), parity, abort_flag, p.status, site);
         };
         uint32_t g0 = 0;                                    // stream position of this item's first sub-tile
         bool ok = true;
         KvItem it;
         for (int k = 0; ok; ++k) {
             if (!wait(L::kIF + (k & 1), (k >> 1) & 1, 514)) break;
-            const int idx = __shfl_sync(0xffffffffu, item_slot[k & 1], 0);   // broadcast: everything derived from it is warp-uniform
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(L::kIE + (k & 1)));
+            const int idx = item_slot[k & 1];
+            mbar_arrive(bar(L::kIE + (k & 1)));
             if (!kv_item(p, idx, it)) break;
             const int buf = k & 1, n_u = it.n_u;
             // the scores run kBufs - 1 sub-tiles ahead of the accumulation products
@@ -269,9 +253,9 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
                 issue_acc(g, i == 0);
             }
             if (!ok) break;
-            if (elect_one()) umma_commit(bar(L::kAF));
-            __syncwarp();
+            umma_commit(bar(L::kAF));
             g0 += n_u;
+        }
         }
     } else {
         const int q = warp & 3, ch = (warp - 2) >> 2;       // lane quarter, column half (32 of the 64 queries)
@@ -487,21 +471,6 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
         fence_proxy_async();
         prefetch_tmap(&tmQ); prefetch_tmap(&tmDO); prefetch_tmap(&tmKV); prefetch_tmap(&tmOut);
     }
-    grid_dep_launch();
-    grid_dep_wait();                                        // inputs come from the previous kernels
-    if (threadIdx.x == 0) {
-        // the first item's first loads go out before the TMEM allocation and the CTA-wide barrier
-        DqItem it;
-        const int idx0 = draw();
-        item_slot[0] = idx0;
-        mbar_arrive(bar(17));
-        if (dq_item(p, idx0, it)) {
-            load_kv(it, 0, 0);
-            load_q(it, 0);
-            if (it.nB) load_q(it, 1);
-            load_kv(it, 1, 1);
-        }
-    }
     if (warp == 1) {
         tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
@@ -510,33 +479,32 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    grid_dep_launch();                                      // (after the TMEM allocation: see grid_dep_launch)
+    grid_dep_wait();                                        // inputs come from the previous kernels
     // TMEM columns of tile t: S at t*256, dP at t*256 + 64, dQ at t*256 + 128
-
+    // the producer and the MMA role are each the loop of one elected thread (see the forward kernel)
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t n = 0;                                 // key sub-tiles requested so far
             uint32_t qn[2] = {0, 0};                        // items each query tile took part in
             bool ok = true;
             DqItem it;
-            int idx = item_slot[0];
+            int idx = draw();
+            item_slot[0] = idx;
+            mbar_arrive(bar(17));
             for (int k = 0; ok && dq_item(p, idx, it); ++k) {
                 const int n_kv = it.nB ? it.nB : it.nA;
                 for (int v = 0; v < n_kv && ok; ++v, ++n) {
                     const int s = n & 1;
                     const uint32_t ph = (n >> 1) & 1;
-                    const bool early = k == 0 && v < 2;     // requested in the prologue
-                    if (!early) {
-                        if (!mbar_wait(bar(6 + s), ph ^ 1, abort_flag, p.status, 600)) { ok = false; break; }
-                        load_kv(it, v, s);
-                    }
+                    if (!mbar_wait(bar(6 + s), ph ^ 1, abort_flag, p.status, 600)) { ok = false; break; }
+                    load_kv(it, v, s);
                     if (v == 0) {
                         // Q_t / dO_t follow the first key sub-tile; their buffers are free once the
                         // previous item's last scores of tile t have been computed
                         for (int t = 0; t < (it.nB ? 2 : 1) && ok; ++t) {
-                            if (k > 0) {
-                                if (!mbar_wait(bar(2 + t), (qn[t] & 1) ^ 1, abort_flag, p.status, 601)) { ok = false; break; }
-                                load_q(it, t);
-                            }
+                            if (!mbar_wait(bar(2 + t), (qn[t] & 1) ^ 1, abort_flag, p.status, 601)) { ok = false; break; }
+                            load_q(it, t);
                             ++qn[t];
                         }
                     }
@@ -550,18 +518,18 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
             }
         }
     } else if (warp == 1) {
-        // converged warp, one elected lane issues (see the forward kernel)
+        if (elect_one()) {
         constexpr uint32_t idesc_sc = make_idesc_bf16(128, 64, false, false);
         constexpr uint32_t idesc_dq = make_idesc_bf16(128, DH, false, true);
-        const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0);
-        const uint32_t sb = __shfl_sync(0xffffffffu, sbase, 0);
+        const uint32_t tb = tmem_base;
+        const uint32_t sb = sbase;
         auto issue_scores = [&](int t, int s) {             // S_t = Q_t K_v^T, dP_t = dO_t V_v^T
             const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + t * L::kTile, 16, 1024);
             const uint64_t dg = desc_advance(dq, 2 * L::kTile);
             const uint64_t dk = make_smem_desc_sw128(sb + L::kKV + s * 2 * L::kSub, 16, 1024);
             const uint64_t dv = desc_advance(dk, L::kSub);
             const uint32_t dst = tb + t * 256;
-            if (elect_one()) {
+            {
 #pragma unroll
                 for (int kb = 0; kb < L::kBlocks; ++kb)
 #pragma unroll
@@ -576,27 +544,23 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
                                  idesc_sc, (kb | kk) ? 1u : 0u);
                 umma_commit(bar(8 + t));
             }
-            __syncwarp();
         };
         auto issue_dq = [&](int t, int s, bool acc) {       // dQ_t += dS_t K_v (dS packed in the S columns)
             const uint64_t dk = make_smem_desc_sw128(sb + L::kKV + s * 2 * L::kSub, 8192, 1024);
             const uint32_t dst = tb + t * 256 + 128, src = tb + t * 256;
-            if (elect_one()) {
+            {
                 // dS packed bf16: keys 0..31 in columns 0..15 of S_t, keys 32..63 in columns 32..47
                 umma_f16_ta(dst, src, dk, idesc_dq, acc ? 1u : 0u);
 #pragma unroll
                 for (int kq = 1; kq < 4; ++kq)
                     umma_f16_ta(dst, src + (kq >> 1) * 32 + (kq & 1) * 8, desc_advance(dk, kq * 2048), idesc_dq, 1u);
             }
-            __syncwarp();
         };
         auto commit = [&](int b) {
-            if (elect_one()) umma_commit(bar(b));
-            __syncwarp();
+            umma_commit(bar(b));
         };
         auto wait = [&](int b, uint32_t parity, int site) {
-            const bool w = mbar_wait(bar(b), parity, abort_flag, p.status, site);
-            return __all_sync(0xffffffffu, w);
+            return mbar_wait(bar(b), parity, abort_flag, p.status, site);
         };
         uint32_t n = 0;                                     // key sub-tiles consumed before this item
         uint32_t nd[2] = {0, 0};                            // dS tiles consumed per query tile
@@ -605,9 +569,8 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
         DqItem it;
         for (int k = 0; ok; ++k) {
             if (!wait(17 + (k & 1), (k >> 1) & 1, 616)) break;
-            const int idx = __shfl_sync(0xffffffffu, item_slot[k & 1], 0);   // broadcast: everything derived from it is warp-uniform
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(19 + (k & 1)));
+            const int idx = item_slot[k & 1];
+            mbar_arrive(bar(19 + (k & 1)));
             if (!dq_item(p, idx, it)) break;
             const int nA = it.nA, nB = it.nB, n_kv = nB ? nB : nA;
             {
@@ -663,6 +626,7 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
             n += n_kv;
             ++qn[0];
             if (nB) ++qn[1];
+        }
         }
     } else {
         // Element-wise: two threads per query row.  Warps 2..9 serve tile A, 10..17 tile B; the lane

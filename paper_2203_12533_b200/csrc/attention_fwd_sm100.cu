@@ -2,8 +2,8 @@
 //
 // One CTA owns two adjacent 128-query tiles (A, B) of one (sequence, head) and streams the
 // 128-key tiles up to the diagonal through a 2-stage K ring and a 2-stage V ring.  10 warps:
-//   warp 0      TMA producer (one lane): Q once, then K_j / V_j.
-//   warp 1      MMA issuer (one lane), owns the TMEM allocation (512 columns):
+//   warp 0      TMA producer: Q once, then K_j / V_j.
+//   warp 1      MMA issuer, owns the TMEM allocation (512 columns):
 //                 S_t = Q_t K_j^T   (128x128, fp32)  -> columns t*128
 //                 O_t += P_t V_j    (128xdh,  fp32)  -> columns 256 + t*128, P_t read from TMEM
 //               issued so that the tensor pipe works on one tile while the other is in softmax:
@@ -135,21 +135,6 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         prefetch_tmap(&tmQKV);
         prefetch_tmap(&tmO);
     }
-    grid_dep_launch();
-    grid_dep_wait();                                        // qkv comes from the previous kernel
-    if (threadIdx.x == 0) {
-        // the first item's first loads go out before the TMEM allocation and the CTA-wide barrier
-        FwdItem it;
-        const int idx0 = draw();
-        item_slot[0] = idx0;
-        mbar_arrive(bar(21));
-        if (fwd_item(p, idx0, it)) {
-            load_k(it, 0, 0);
-            load_q(it, 0);
-            if (it.nB) load_q(it, 1);
-            load_v(it, 0, 0);
-        }
-    }
     if (warp == 1) {
         tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
@@ -158,40 +143,40 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-
+    grid_dep_launch();                                      // (after the TMEM allocation: see grid_dep_launch)
+    grid_dep_wait();                                        // qkv comes from the previous kernel
+    // The producer and the MMA role are each the loop of ONE thread, picked by elect.sync for the whole role: a
+    // wait, eight products and a commit then cost what the products take.  As a converged warp that votes on every
+    // wait and elects a lane to issue, a wait alone cost the role about 130 cycles, and a copy out of a divergent
+    // `if (lane == 0)` about 300.
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t n = 0;                                 // key/value tiles requested so far
             uint32_t qn[2] = {0, 0};                        // items each query tile took part in
             bool ok = true;
             FwdItem it;
-            int idx = item_slot[0];
+            int idx = draw();
+            item_slot[0] = idx;
+            mbar_arrive(bar(21));
             for (int k = 0; ok && fwd_item(p, idx, it); ++k) {
                 const int n_kv = it.nB ? it.nB : it.nA;
                 for (int j = 0; j < n_kv && ok; ++j, ++n) {
                     const int s = n & 1;
                     const uint32_t ph = (n >> 1) & 1;
-                    const bool early = k == 0 && j == 0;    // requested in the prologue
-                    if (!early) {
-                        if (!mbar_wait(bar(6 + s), ph ^ 1, abort_flag, p.status, 400)) { ok = false; break; }
-                        load_k(it, j, s);
-                    }
+                    if (!mbar_wait(bar(6 + s), ph ^ 1, abort_flag, p.status, 400)) { ok = false; break; }
+                    load_k(it, j, s);
                     if (j == 0) {
                         // Q follows the first key tile; its buffer is free once the previous item's
                         // last S = Q K^T has been computed.
                         for (int t = 0; t < (it.nB ? 2 : 1) && ok; ++t) {
-                            if (!early) {
-                                if (!mbar_wait(bar(2 + t), (qn[t] & 1) ^ 1, abort_flag, p.status, 402)) { ok = false; break; }
-                                load_q(it, t);
-                            }
+                            if (!mbar_wait(bar(2 + t), (qn[t] & 1) ^ 1, abort_flag, p.status, 402)) { ok = false; break; }
+                            load_q(it, t);
                             ++qn[t];
                         }
                         if (!ok) break;
                     }
-                    if (!early) {
-                        if (!mbar_wait(bar(10 + s), ph ^ 1, abort_flag, p.status, 401)) { ok = false; break; }
-                        load_v(it, j, s);
-                    }
+                    if (!mbar_wait(bar(10 + s), ph ^ 1, abort_flag, p.status, 401)) { ok = false; break; }
+                    load_v(it, j, s);
                 }
                 if (!ok) break;
                 // next item: its number goes into slot (k+1)&1 once every role has read what was there
@@ -203,18 +188,17 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
             }
         }
     } else if (warp == 1) {
-        // The whole warp runs this role converged (waits and address arithmetic stay uniform);
-        // one elected lane issues the tcgen05 instructions.
+        if (elect_one()) {
         constexpr uint32_t idesc_s = make_idesc_bf16(128, 128, false, false);
         constexpr uint32_t idesc_pv = make_idesc_bf16(128, DH, false, true);
-        const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0);
-        const uint32_t sb = __shfl_sync(0xffffffffu, sbase, 0);
+        const uint32_t tb = tmem_base;
+        const uint32_t sb = sbase;
         // S_t = Q_t K^T from K stage s
         auto issue_s = [&](int t, int s) {
             const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + t * L::kTile, 16, 1024);
             const uint64_t dk = make_smem_desc_sw128(sb + L::kK + s * L::kTile, 16, 1024);
             const uint32_t dst = tb + t * 128;
-            if (elect_one()) {
+            {
 #pragma unroll
                 for (int kb = 0; kb < L::kBlocks; ++kb)
 #pragma unroll
@@ -223,28 +207,24 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
                                  idesc_s, (kb | kk) ? 1u : 0u);
                 umma_commit(bar(12 + t));
             }
-            __syncwarp();
         };
         // O_t (+)= P_t V from V stage s; P_t is bf16 packed over the S columns it came from: the 16
         // keys of step ks sit in 8 columns at (ks/4)*64 + ((ks%4)/2)*32 + (ks%2)*8 of S_t
         auto issue_pv = [&](int t, int s, bool acc) {
             const uint64_t dv = make_smem_desc_sw128(sb + L::kV + s * L::kTile, 16384, 1024);
             const uint32_t dst = tb + 256 + t * 128, src = tb + t * 128;
-            if (elect_one()) {
+            {
                 umma_f16_ta(dst, src, dv, idesc_pv, acc ? 1u : 0u);
 #pragma unroll
                 for (int ks = 1; ks < 8; ++ks)
                     umma_f16_ta(dst, src + (ks >> 2) * 64 + ((ks & 3) >> 1) * 32 + (ks & 1) * 8, desc_advance(dv, ks * 2048), idesc_pv, 1u);
             }
-            __syncwarp();
         };
         auto commit = [&](int b) {
-            if (elect_one()) umma_commit(bar(b));
-            __syncwarp();
+            umma_commit(bar(b));
         };
         auto wait = [&](int b, uint32_t parity, int site) {
-            bool w = mbar_wait(bar(b), parity, abort_flag, p.status, site);
-            return __all_sync(0xffffffffu, w);
+            return mbar_wait(bar(b), parity, abort_flag, p.status, site);
         };
         uint32_t n = 0;                                 // key/value tiles consumed before this item
         uint32_t np[2] = {0, 0};                        // P tiles consumed per query tile
@@ -253,9 +233,8 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         FwdItem it;
         for (int k = 0; ok; ++k) {
             if (!wait(21 + (k & 1), (k >> 1) & 1, 423)) break;
-            const int idx = __shfl_sync(0xffffffffu, item_slot[k & 1], 0);   // broadcast: everything derived from it is warp-uniform
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(23 + (k & 1)));
+            const int idx = item_slot[k & 1];
+            mbar_arrive(bar(23 + (k & 1)));
             if (!fwd_item(p, idx, it)) break;
             const int nA = it.nA, nB = it.nB, n_kv = nB ? nB : nA;
             {
@@ -316,6 +295,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
             n += n_kv;
             ++qn[0];
             if (nB) ++qn[1];
+        }
         }
     } else {
         // Softmax: two threads per query row.  Warps 2..9 serve tile A, 10..17 tile B; inside a tile

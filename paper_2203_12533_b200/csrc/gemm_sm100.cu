@@ -279,15 +279,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
         tmem_relinquish();
     }
-    grid_dep_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dep_launch();                                  // (after the TMEM allocation: see grid_dep_launch)
     const uint32_t tmem_base = *tmem_slot;
     grid_dep_wait();                                    // inputs of this GEMM come from the previous kernel
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t stage = 0, phase = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
@@ -316,7 +316,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc_full = make_idesc_bf16(BM, p.bn, A_MN, B_MN);
             const uint32_t idesc_half = make_idesc_bf16(BM, p.bn >> 1, A_MN, B_MN);
             uint32_t stage = 0, phase = 0, it = 0;
@@ -463,30 +463,28 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t tmem_base = *tmem_slot;
     grid_dep_wait();                                    // inputs of this GEMM come from the previous kernel
 
-    // Both roles run as a converged warp (waits and addresses stay warp-uniform) and one elected lane
-    // issues.  Inside a divergent `if (lane == 0)` a k block (two loads, or four products and a commit) takes
-    // 620 cycles whatever its size, more than the 512 that its products need at the full rate.  Measured, before ->
-    // after: 8192 x 6144 x 2048 139.2 -> 132.1 us, 2048 x 1024 x 4096 (dgrad) 23.4 -> 16.6 us, 1024 x 1024 x 4096
-    // 25.0 -> 18.6 us.
+    // Both roles are the loop of ONE thread, picked by elect.sync for the whole role.  Cycles per 64-wide k block
+    // (wait, four M = 128, N = 64 products, commit) in isolation: 242, which is what the products take; 300 without
+    // the wait as a divergent `if (lane == 0)`; 353 as a converged warp that votes on every wait and elects a lane to
+    // issue.  Measured on the GEMM, `lane == 0` -> elected: 1024 x 1024 x 4096 25.0 -> 17.9 us,
+    // 2048 x 1024 x 4096 (dgrad) 23.4 -> 16.1 us, 8192 x 6144 x 2048 139.2 -> 131.5 us.
     if (warp == 0) {
-        uint32_t stage = 0, phase = 0;
-        bool ok = true;
-        const uint32_t pair_tx = 2u * (A_TILE_BYTES + half_n * BK * 2);
-        const uint32_t ring0 = smem_u32(tiles), full_lead = mapa_shared(full0, 0);   // the leader's barriers
-        for (int unit = pair_id; unit < total_tiles && ok; unit += n_pairs) {
-            const PairUnit un = pair_unit(p, unit, num_k);
-            const int tile = un.tile;
-            const int mi = p.n_fastest ? tile / p.n_tiles : tile % p.m_tiles;
-            const int ni = p.n_fastest ? tile % p.n_tiles : tile / p.m_tiles;
-            const int m0 = mi * 256 + rank * 128;
-            const int n0 = ni * bn + rank * half_n;
-            for (int kb = un.kb0; kb < un.kb1; ++kb) {
-                ok = mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.status, 700);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                const uint32_t a_dst = ring0 + stage * P_STAGE_BYTES, b_dst = a_dst + A_TILE_BYTES;
-                const uint32_t fb = full_lead + 8 * stage;
-                if (elect_one()) {
+        if (elect_one()) {
+            uint32_t stage = 0, phase = 0;
+            bool ok = true;
+            const uint32_t pair_tx = 2u * (A_TILE_BYTES + half_n * BK * 2);
+            const uint32_t ring0 = smem_u32(tiles), full_lead = mapa_shared(full0, 0);   // the leader's barriers
+            for (int unit = pair_id; unit < total_tiles && ok; unit += n_pairs) {
+                const PairUnit un = pair_unit(p, unit, num_k);
+                const int tile = un.tile;
+                const int mi = p.n_fastest ? tile / p.n_tiles : tile % p.m_tiles;
+                const int ni = p.n_fastest ? tile % p.n_tiles : tile / p.m_tiles;
+                const int m0 = mi * 256 + rank * 128;
+                const int n0 = ni * bn + rank * half_n;
+                for (int kb = un.kb0; kb < un.kb1; ++kb) {
+                    if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.status, 700)) { ok = false; break; }
+                    const uint32_t a_dst = ring0 + stage * P_STAGE_BYTES, b_dst = a_dst + A_TILE_BYTES;
+                    const uint32_t fb = full_lead + 8 * stage;
                     if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * stage, pair_tx);
                     if constexpr (!A_MN) {
                         tma_load_2d_pair(a_dst, &tmA, kb * BK, m0, fb);
@@ -500,15 +498,13 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         tma_load_2d_pair(b_dst, &tmB, n0, kb * BK, fb);
                         if (half_n > 64) tma_load_2d_pair(b_dst + 8192, &tmB, n0 + 64, kb * BK, fb);
                     }
+                    if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
                 }
-                __syncwarp();
-                if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
             }
         }
     } else if (warp == 1) {
-        if (rank == 0) {
+        if (rank == 0 && elect_one()) {
             const uint32_t idesc = make_idesc_bf16(256, bn, A_MN, B_MN);
-            const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0);
             const uint64_t adesc0 = make_smem_desc_sw128(smem_u32(tiles), A_MN ? 8192 : 16, 1024);
             const uint64_t bdesc0 = make_smem_desc_sw128(smem_u32(tiles) + A_TILE_BYTES, B_MN ? 8192 : 16, 1024);
             uint32_t stage = 0, phase = 0, it = 0;
@@ -516,30 +512,22 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             for (int unit = pair_id; unit < total_tiles && ok; unit += n_pairs, ++it) {
                 const PairUnit un = pair_unit(p, unit, num_k);
                 const uint32_t buf = it & 1, acc_phase = (it >> 1) & 1;
-                ok = mbar_wait(acce0 + 8 * buf, acc_phase ^ 1, abort_flag, p.status, 710);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
+                if (!mbar_wait(acce0 + 8 * buf, acc_phase ^ 1, abort_flag, p.status, 710)) break;
                 tc_fence_after();
-                const uint32_t d_tmem = tb + buf * BN_MAX;
+                const uint32_t d_tmem = tmem_base + buf * BN_MAX;
                 for (int kb = un.kb0; kb < un.kb1; ++kb) {
-                    ok = mbar_wait(full0 + 8 * stage, phase, abort_flag, p.status, 711);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
+                    if (!mbar_wait(full0 + 8 * stage, phase, abort_flag, p.status, 711)) { ok = false; break; }
                     tc_fence_after();
                     const uint64_t ad = desc_advance(adesc0, stage * P_STAGE_BYTES), bd = desc_advance(bdesc0, stage * P_STAGE_BYTES);
-                    if (elect_one()) {
-                        // K-major: 16 k = 32 bytes along the swizzled 128-byte row; MN-major: two 8-k groups of 1024 B
+                    // K-major: 16 k = 32 bytes along the swizzled 128-byte row; MN-major: two 8-k groups of 1024 B
 #pragma unroll
-                        for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                            umma_f16_pair(d_tmem, desc_advance(ad, kk * (A_MN ? 2048 : 32)), desc_advance(bd, kk * (B_MN ? 2048 : 32)), idesc,
-                                          (kb != un.kb0 || kk != 0) ? 1u : 0u);
-                        umma_commit_pair(empty0 + 8 * stage, 3);     // frees the stage in both CTAs
-                    }
-                    __syncwarp();
+                    for (int kk = 0; kk < BK / UMMA_K; ++kk)
+                        umma_f16_pair(d_tmem, desc_advance(ad, kk * (A_MN ? 2048 : 32)), desc_advance(bd, kk * (B_MN ? 2048 : 32)), idesc,
+                                      (kb != un.kb0 || kk != 0) ? 1u : 0u);
+                    umma_commit_pair(empty0 + 8 * stage, 3);     // frees the stage in both CTAs
                     if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
                 }
-                if (ok && elect_one()) umma_commit_pair(accf0 + 8 * buf, 3);     // both CTAs' accumulators complete
-                __syncwarp();
+                if (ok) umma_commit_pair(accf0 + 8 * buf, 3);     // both CTAs' accumulators complete
             }
         }
     } else {

@@ -97,6 +97,9 @@ __device__ __forceinline__ float gelu_grad_f(float u, int act)
 // early as possible; grid_dep_wait() blocks until the previous kernel has completed and its
 // memory is visible - every kernel calls it before its first global-memory access, so only the
 // launch latency and the on-chip set-up overlap.  Both are no-ops for a plain launch.
+// A kernel that uses TMEM allocates it (and passes a CTA-wide barrier) BEFORE grid_dep_launch(): the next
+// kernel's CTAs may then share an SM with it, and one that got its TMEM first would wait for a predecessor
+// that waits for its TMEM.
 // Consequence for every kernel here: no input pointer is `const __restrict__` and nothing is read
 // with __ldg - the compiler treats such loads as invariant over the kernel's lifetime and may hoist
 // them above the wait, where the producer has not written the data yet.
