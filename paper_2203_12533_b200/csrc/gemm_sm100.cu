@@ -103,10 +103,6 @@ __device__ __forceinline__ void epilogue_group(const uint32_t* v, int row, int c
     }
 }
 
-// Epilogue of one accumulator tile for one warp: TMEM -> registers -> swizzled shared slab -> TMA
-// store (rows >= M and columns >= N are clipped by the tensor map).  `taddr` addresses this warp's
-// lane quarter of the accumulator, row0 is the first of its 32 rows, pi selects which of the two
-// warps of the quarter it is (they take alternate column chunks).
 // Partial sums of one 32 x 32 accumulator chunk as the K halves of a cut tile exchange them: eight
 // 512-byte rows of [lane][4 floats], so that every access of a warp is one contiguous 512 bytes.
 __device__ __forceinline__ void add_partner_chunk(uint32_t (&v)[32], const float* partner_chunk, int lane)
@@ -121,8 +117,34 @@ __device__ __forceinline__ void add_partner_chunk(uint32_t (&v)[32], const float
     }
 }
 
+// First of the 32-column chunks that warp pi of the pstride warps of a lane quarter handles, and the step to the
+// next: alternate chunks - except with the row-dot epilogue, where each takes a run of neighbouring chunks, so that all
+// columns of a head meet in one thread.
+template <int EPI>
+__device__ __forceinline__ int first_chunk(int bn, int pi, int pstride) { return EPI == kEpiRowDot ? pi * (bn / 32 / pstride) : pi; }
+
+// Residual / saved pre-activation / second dot operand: 8 columns of a row, or 32 (zeros outside).
+__device__ __forceinline__ uint4 load_aux8(const GemmParams& p, int row, int col)
+{
+    return row < p.M && col < p.N ? *reinterpret_cast<const uint4*>(p.aux_in + static_cast<size_t>(row) * p.ld_aux + col) : make_uint4(0, 0, 0, 0);
+}
+__device__ __forceinline__ void load_aux(uint4 (&aux)[4], const GemmParams& p, int row, int col0)
+{
+#pragma unroll
+    for (int g = 0; g < 4; ++g) aux[g] = load_aux8(p, row, col0 + g * 8);
+}
+
+// Epilogue of one accumulator tile for one warp: TMEM -> registers -> swizzled shared slab -> TMA
+// store (rows >= M and columns >= N are clipped by the tensor map).  `taddr` addresses this warp's
+// lane quarter of the accumulator, row0 is the first of its 32 rows, pi selects which of the pstride
+// warps of the quarter it is.
+// `aux`: the first chunk's pieces, requested by the caller before it waited for the accumulator; a further
+// chunk's are requested as soon as their registers are free, ahead of that chunk's TMEM load, so the reads
+// (row-strided, L2 or DRAM latency) overlap the work.  Measured, requested at the start of their own chunk -> so:
+// 16384 x 4096 x 1024 x GeLU' 126 -> 122 us, 1024 x 4096 x 1024 x GeLU' 14.8 -> 14.1 us, 1024 x 1024 x 4096 + residual
+// 17.9 -> 16.8 us.
 template <int EPI, bool SINGLE_SLAB = false, bool SPLIT = false>
-__device__ __forceinline__ void epilogue_tile(uint32_t taddr, int row0, int n0, int bn, int pi, int pstride, int lane,
+__device__ __forceinline__ void epilogue_tile(uint4 (&aux)[4], uint32_t taddr, int row0, int n0, int bn, int pi, int pstride, int lane,
                                               uint8_t* slab, uint32_t slab_u32, uint32_t& nout, const CUtensorMap* tmC,
                                               const CUtensorMap* tmAux, const GemmParams& p,
                                               const float* partner = nullptr /* SPLIT: the other K half's partial sums, [chunk][1024] */)
@@ -158,9 +180,8 @@ __device__ __forceinline__ void epilogue_tile(uint32_t taddr, int row0, int n0, 
         // swizzle) used alternately, so one store is always in flight behind the math.
         const int nchunks = bn / 32;
         const uint32_t sw = (lane >> 1) & 3;
-        // The warps of a lane quarter take alternate chunks - except with the row-dot epilogue, where each
-        // takes a run of neighbouring chunks, so that all columns of a head meet in one thread.
-        const int ch_first = EPI == kEpiRowDot ? pi * (nchunks / pstride) : pi;
+        constexpr bool kHasAux = EPI == kEpiBiasResid || EPI == kEpiDGelu || EPI == kEpiRowDot;
+        const int ch_first = first_chunk<EPI>(bn, pi, pstride);
         const int ch_step = EPI == kEpiRowDot ? 1 : pstride;
         const int ch_end = EPI == kEpiRowDot ? ch_first + nchunks / pstride : nchunks;
         float dot = 0.f;
@@ -168,17 +189,6 @@ __device__ __forceinline__ void epilogue_tile(uint32_t taddr, int row0, int n0, 
         for (int ch = ch_first; ch < ch_end; ch += ch_step) {
             const int col0 = n0 + ch * 32;
             if (col0 >= p.N) break;
-            // residual / saved pre-activation of this chunk: requested before the TMEM load so that the
-            // (row-strided, L2-latency) reads overlap it
-            uint4 aux[4] = {};
-            if constexpr (EPI == kEpiBiasResid || EPI == kEpiDGelu || EPI == kEpiRowDot) {
-                if (row < p.M) {
-#pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        if (col0 + g * 8 < p.N)
-                            aux[g] = *reinterpret_cast<const uint4*>(p.aux_in + static_cast<size_t>(row) * p.ld_aux + col0 + g * 8);
-                }
-            }
             uint32_t v[32];
             tmem_ld32(taddr + ch * 32, v);
             tc_wait_ld();
@@ -195,6 +205,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t taddr, int row0, int n0, 
 #pragma unroll
                     for (int j = 0; j < 8; ++j) dot = fmaf(f[j], r[j], dot);
                 }
+                if (kHasAux && ch + ch_step < ch_end) aux[g] = load_aux8(p, row, col0 + 32 * ch_step + g * 8);
                 if constexpr (EPI == kEpiBiasGelu) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) v[8 * g + j] = __float_as_uint(f[j]);   // fp32 pre-activation, kept for GeLU
@@ -359,12 +370,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             int m0, n0, bn;
             tile_info(p, tile, m0, n0, bn);
             const uint32_t buf = it & 1, acc_phase = (it >> 1) & 1;
+            uint4 aux[4];
+            if (EPI == kEpiBiasResid || EPI == kEpiDGelu || EPI == kEpiRowDot)
+                load_aux(aux, p, m0 + q * 32 + lane, n0 + 32 * first_chunk<EPI>(bn, pi, 2));
             bool ok = mbar_wait(accf0 + 8 * buf, acc_phase, abort_flag, p.status, 300);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * BN_MAX;
-            epilogue_tile<EPI>(taddr, m0 + q * 32, n0, bn, pi, 2, lane, slab, slab_u32, nout, &tmC, &tmAux, p);
+            epilogue_tile<EPI>(aux, taddr, m0 + q * 32, n0, bn, pi, 2, lane, slab, slab_u32, nout, &tmC, &tmAux, p);
             tc_fence_before();
             mbar_arrive(acce0 + 8 * buf);
         }
@@ -542,13 +556,16 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const int ni = p.n_fastest ? tile % p.n_tiles : tile / p.m_tiles;
             const int m0 = mi * 256 + rank * 128, n0 = ni * bn;
             const uint32_t buf = it & 1, acc_phase = (it >> 1) & 1;
+            uint4 aux[4];
+            if (EPI == kEpiBiasResid || EPI == kEpiDGelu || EPI == kEpiRowDot)
+                load_aux(aux, p, m0 + q * 32 + lane, n0 + 32 * first_chunk<EPI>(bn, pi, NEPI / 4));
             bool ok = mbar_wait(accf0 + 8 * buf, acc_phase, abort_flag, p.status, 720);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * BN_MAX;
             if (EPI == kEpiF32 || un.slot < 0) {                 // (the fp32-output GEMMs are never cut)
-                epilogue_tile<EPI, NEPI == 16>(taddr, m0 + q * 32, n0, bn, pi, NEPI / 4, lane, slab, slab_u32, nout, &tmC, &tmAux, p);
+                epilogue_tile<EPI, NEPI == 16>(aux, taddr, m0 + q * 32, n0, bn, pi, NEPI / 4, lane, slab, slab_u32, nout, &tmC, &tmAux, p);
             } else {
                 // Half of a cut tile's K range.  Every epilogue warp leaves its part of the partial sums in
                 // the scratch, then draws a ticket shared with the same warp of the CTA that has the
@@ -580,7 +597,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if (before != 0) {
                     if (lane == 0) *ticket = 0;                                  // both halves have drawn: ready for the next launch
                     __threadfence();
-                    epilogue_tile<EPI, NEPI == 16, true>(taddr, m0 + q * 32, n0, bn, pi, NEPI / 4, lane, slab, slab_u32, nout, &tmC, &tmAux, p, other);
+                    epilogue_tile<EPI, NEPI == 16, true>(aux, taddr, m0 + q * 32, n0, bn, pi, NEPI / 4, lane, slab, slab_u32, nout, &tmC, &tmAux, p, other);
                 }
             }
             tc_fence_before();
