@@ -1,0 +1,366 @@
+// bf16 GEMM for sm_100a whose tiles are cut along K inside a thread-block cluster.
+//
+// Made for products with fewer output tiles than the persistent CTA-pair kernel (gemm_sm100.cu) needs to
+// fill the chip: a cluster computes ONE tile, every slice of it (a CTA, or a CTA pair working as
+// cta_group::2) over its share of the K range.  Nothing is persistent; the tile's latency is all that counts:
+//   warp 0      TMA producer: a ring as deep as the launch has shared memory for
+//   warp 1      MMA issuer (in the leader CTA), owns the TMEM allocation (bn columns, one accumulator)
+//   warps 2..9  epilogue.  The K slices of a tile finish 128 / slices of its rows each: every CTA writes its
+//               partial sums from TMEM straight into the shared memory of the CTA that finishes those rows
+//               (distributed shared memory, over the ring, which is idle by then), the cluster meets at a
+//               barrier, and each CTA adds the slices up in slice order (fp32, the same bits every time) and
+//               runs bias / residual / GeLU / GeLU' / row dots on row-contiguous 8-column groups with
+//               16-byte global accesses.
+// Ownership by rows (not columns) keeps whole heads in one CTA, which the row-dot epilogue needs.
+//
+// The accumulator-full barrier of every CTA gets one arrival from each slice's tcgen05.commit (multicast
+// over the cluster): when it completes, all CTAs' products are done, so every ring may be overwritten.
+// Every mbarrier wait is bounded (see mbar_wait); a CTA that gave up still meets the cluster barriers.
+#include "gemm_epilogue.cuh"
+
+namespace pw {
+namespace {
+
+constexpr int kThreads = 320;
+constexpr int kEpiThreads = 256;
+constexpr int kATile = 128 * 64 * 2;                     // a CTA's 128 x 64 part of the A operand
+constexpr int kBatch = 4;                                // 8-column groups a thread works on at once
+
+struct ClusterParams {
+    GemmEpilogue e;
+    int K, bn, slices, stages, tmem_cols, log_groups;    // log_groups: log2 of the 8-column groups per tile row
+    int m_tiles;
+    DeviceStatus* status;
+};
+
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+// One CTA's commit, signalled to the same barrier offset in every CTA of `mask` (a barrier signal, not a data copy).
+__device__ __forceinline__ void umma_commit_mask(uint32_t bar, uint16_t mask)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(bar), "h"(mask) : "memory");
+}
+
+template <bool PAIR, bool A_MN, bool B_MN, int EPI>
+__global__ void __launch_bounds__(kThreads, 2)
+gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const ClusterParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ uint64_t bars[2 * 8 + 1];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_word;
+    volatile int* abort_flag = &abort_word;
+    const int stages = p.stages;
+    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + 8), accf = smem_u32(bars + 16);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int csize = PAIR ? 2 * p.slices : p.slices;
+    const int rank = blockIdx.x % csize;                 // = %cluster_ctarank of a one-dimensional cluster
+    const int parity = PAIR ? rank & 1 : 0, slice = PAIR ? rank >> 1 : rank;
+    const int tile = blockIdx.x / csize;
+    const int b_rows = PAIR ? p.bn >> 1 : p.bn;
+    const int stage_bytes = kATile + b_rows * 128;
+    const int m0 = (tile % p.m_tiles) * (PAIR ? 256 : 128) + parity * 128;
+    const int n0 = (tile / p.m_tiles) * p.bn;
+    const int num_k = (p.K + 63) / 64;
+    const int kb0 = num_k * slice / p.slices, kb1 = num_k * (slice + 1) / p.slices;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < stages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
+        mbar_init(accf, p.slices);
+        *abort_flag = 0;
+        fence_barrier_init();
+        fence_proxy_async();
+        prefetch_tmap(&tmA);
+        prefetch_tmap(&tmB);
+    }
+    if (warp == 1) {
+        if constexpr (PAIR) { tmem_alloc_pair(smem_u32(&tmem_slot), p.tmem_cols); tmem_relinquish_pair(); }
+        else { tmem_alloc(smem_u32(&tmem_slot), p.tmem_cols); tmem_relinquish(); }
+    }
+    tc_fence_before();
+    if (csize > 1) cluster_sync_all(); else __syncthreads();     // everyone's barriers exist before anyone signals them
+    tc_fence_after();
+    grid_dep_launch();                                   // (after the TMEM allocation: see grid_dep_launch)
+    const uint32_t tmem_base = tmem_slot;
+    grid_dep_wait();                                     // inputs of this GEMM come from the previous kernel
+
+    // Epilogue thread i handles 8-column groups i, i + 256, ... of the rows this CTA finishes: always the same column.
+    const int owner_rows = 128 / p.slices;               // rows this CTA finishes: owner_rows * slice ...
+    const int pitch = p.bn + 4;                          // floats per staged row: 16-byte accesses of neighbouring rows hit different banks
+    const int et = static_cast<int>(threadIdx.x) - 64;
+    const int cg = et & ((1 << p.log_groups) - 1);
+    const int col = n0 + 8 * cg;
+    const int row_step = kEpiThreads >> p.log_groups;
+    int lr = et >> p.log_groups;                         // row inside the owned ones
+    const int row0 = m0 + slice * owner_rows;
+    const bool col_ok = et >= 0 && col < p.e.N;
+    constexpr bool kHasBias = EPI == kEpiBias || EPI == kEpiBiasResid || EPI == kEpiBiasGelu;
+    constexpr bool kHasAux = EPI == kEpiBiasResid || EPI == kEpiDGelu || EPI == kEpiRowDot;
+    uint4 bias_raw = make_uint4(0, 0, 0, 0), aux[kBatch];
+    auto fetch_aux = [&](int r) {
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+            const int rr = r + i * row_step;
+            aux[i] = col_ok && rr < owner_rows && row0 + rr < p.e.M
+                ? *reinterpret_cast<const uint4*>(p.e.aux_in + static_cast<size_t>(row0 + rr) * p.e.ld_aux + col) : make_uint4(0, 0, 0, 0);
+        }
+    };
+
+    // Each single-issuer role is the loop of one elected thread (see gemm_pair_kernel).
+    if (warp == 0) {
+        if (elect_one()) {
+            const uint32_t tx = (PAIR ? 2u : 1u) * stage_bytes;
+            const int b0 = n0 + parity * b_rows;
+            const uint32_t ring0 = smem_u32(ring);
+            const uint32_t full_lead = PAIR ? mapa_shared(full0, rank & ~1) : full0;       // the leader's barriers
+            uint32_t stage = 0, phase = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.status, 730)) break;
+                const uint32_t a_dst = ring0 + stage * stage_bytes, b_dst = a_dst + kATile, fb = full_lead + 8 * stage;
+                if (parity == 0) mbar_arrive_expect_tx(full0 + 8 * stage, tx);
+                auto load = [&](uint32_t dst, const CUtensorMap* map, int x, int y) {
+                    if constexpr (PAIR) tma_load_2d_pair(dst, map, x, y, fb); else tma_load_2d(dst, map, x, y, fb);
+                };
+                if constexpr (!A_MN) load(a_dst, &tmA, kb * 64, m0);
+                else { load(a_dst, &tmA, m0, kb * 64); load(a_dst + 8192, &tmA, m0 + 64, kb * 64); }
+                if constexpr (!B_MN) load(b_dst, &tmB, kb * 64, b0);
+                else for (int j = 0; j < b_rows / 64; ++j) load(b_dst + j * 8192, &tmB, b0 + 64 * j, kb * 64);
+                if (++stage == static_cast<uint32_t>(stages)) { stage = 0; phase ^= 1; }
+            }
+        }
+    } else if (warp == 1) {
+        if (parity == 0 && elect_one()) {
+            const uint32_t idesc = make_idesc_bf16(PAIR ? 256 : 128, p.bn, A_MN, B_MN);
+            const uint64_t adesc0 = make_smem_desc_sw128(smem_u32(ring), A_MN ? 8192 : 16, 1024);
+            const uint64_t bdesc0 = make_smem_desc_sw128(smem_u32(ring) + kATile, B_MN ? 8192 : 16, 1024);
+            uint32_t stage = 0, phase = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait(full0 + 8 * stage, phase, abort_flag, p.status, 731)) break;
+                tc_fence_after();
+                const uint64_t ad = desc_advance(adesc0, stage * stage_bytes), bd = desc_advance(bdesc0, stage * stage_bytes);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const uint64_t adesc = desc_advance(ad, kk * (A_MN ? 2048 : 32)), bdesc = desc_advance(bd, kk * (B_MN ? 2048 : 32));
+                    if constexpr (PAIR) umma_f16_pair(tmem_base, adesc, bdesc, idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
+                    else umma_f16(tmem_base, adesc, bdesc, idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
+                }
+                if constexpr (PAIR) umma_commit_pair(empty0 + 8 * stage, static_cast<uint16_t>(3u << rank));
+                else umma_commit(empty0 + 8 * stage);
+                if (++stage == static_cast<uint32_t>(stages)) { stage = 0; phase ^= 1; }
+            }
+            // (after a wait that gave up this signals early: the other CTAs then finish with wrong sums, and the
+            // status word says why)
+            const uint16_t all = static_cast<uint16_t>((1u << csize) - 1u);
+            if constexpr (PAIR) umma_commit_pair(accf, all);
+            else if (csize > 1) umma_commit_mask(accf, all);
+            else umma_commit(accf);
+        }
+    } else {
+        // bias and the first residual / pre-activation pieces are on their way while the products run
+        if (kHasBias && col_ok) bias_raw = *reinterpret_cast<const uint4*>(p.e.bias + col);
+        if (kHasAux) fetch_aux(lr);
+        const int q = warp & 3, pi = (warp - 2) >> 2;
+        bool ok = mbar_wait(accf, 0, abort_flag, p.status, 732);
+        ok = __all_sync(0xffffffffu, ok);
+        tc_fence_after();
+        if (ok) {
+            const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
+            const int row = q * 32 + lane, owner = row / owner_rows;
+            uint32_t dst = smem_u32(ring) + ((slice * owner_rows + row - owner * owner_rows) * pitch) * 4;
+            if (csize > 1) dst = mapa_shared(dst, PAIR ? 2 * owner + parity : owner);
+            else dst = mapa_shared(dst, 0);
+#pragma unroll 1
+            for (int c = pi * 32; c < p.bn; c += 64) {
+                uint32_t v[32];
+                tmem_ld32(taddr + c, v);
+                tc_wait_ld();
+#pragma unroll
+                for (int g = 0; g < 8; ++g) st_cluster_v4(dst + (c + 4 * g) * 4, v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+            }
+        }
+        tc_fence_before();
+    }
+
+    __syncwarp();
+    if (*abort_flag) {                                   // give copies and MMAs still in flight time to land
+        const long long t0 = clock64();
+        while (clock64() - t0 < (1ll << 22)) {}
+    }
+    __syncwarp();
+    if (csize > 1) cluster_sync_all(); else __syncthreads();     // partial sums are where they belong; TMEM has been read
+    if (warp == 1) {
+        tc_fence_after();
+        if constexpr (PAIR) tmem_dealloc_pair(tmem_base, p.tmem_cols); else tmem_dealloc(tmem_base, p.tmem_cols);
+    }
+    if (et < 0 || *abort_flag) return;
+
+    const float* staged = reinterpret_cast<const float*>(ring);
+    const int swap = (cg >> 2) & 1;                      // order of a group's two 16-byte reads: 8 neighbouring lanes then hit 8 bank groups
+#pragma unroll 1
+    for (; lr < owner_rows; lr += kBatch * row_step) {
+        float f[kBatch][8];
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+            float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+            const int r = lr + i * row_step;
+            if (r < owner_rows) {
+#pragma unroll 1
+                for (int j = 0; j < p.slices; ++j) {
+                    const float* src = staged + (j * owner_rows + r) * pitch + cg * 8;
+                    const float4 a = *reinterpret_cast<const float4*>(src + 4 * swap), b = *reinterpret_cast<const float4*>(src + 4 * (swap ^ 1));
+                    lo.x += a.x; lo.y += a.y; lo.z += a.z; lo.w += a.w;
+                    hi.x += b.x; hi.y += b.y; hi.z += b.z; hi.w += b.w;
+                }
+            }
+            f[i][0] = swap ? hi.x : lo.x; f[i][1] = swap ? hi.y : lo.y; f[i][2] = swap ? hi.z : lo.z; f[i][3] = swap ? hi.w : lo.w;
+            f[i][4] = swap ? lo.x : hi.x; f[i][5] = swap ? lo.y : hi.y; f[i][6] = swap ? lo.z : hi.z; f[i][7] = swap ? lo.w : hi.w;
+        }
+        if constexpr (EPI == kEpiF32) {
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i) {
+                const int r = lr + i * row_step;
+                if (!(col_ok && r < owner_rows && row0 + r < p.e.M)) continue;
+                float* out = static_cast<float*>(p.e.C) + static_cast<size_t>(row0 + r) * p.e.ldc + col;
+                if (p.e.accumulate) {
+                    const float4 c0 = *reinterpret_cast<const float4*>(out), c1 = *reinterpret_cast<const float4*>(out + 4);
+                    f[i][0] += c0.x; f[i][1] += c0.y; f[i][2] += c0.z; f[i][3] += c0.w;
+                    f[i][4] += c1.x; f[i][5] += c1.y; f[i][6] += c1.z; f[i][7] += c1.w;
+                }
+                *reinterpret_cast<float4*>(out) = make_float4(f[i][0], f[i][1], f[i][2], f[i][3]);
+                *reinterpret_cast<float4*>(out + 4) = make_float4(f[i][4], f[i][5], f[i][6], f[i][7]);
+            }
+        } else {
+            if constexpr (kHasBias) {
+                float bias[8];
+                unpack8(bias_raw, bias);
+#pragma unroll
+                for (int i = 0; i < kBatch; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) f[i][j] += bias[j];
+            }
+            if constexpr (kHasAux) {
+                uint4 now[kBatch];
+#pragma unroll
+                for (int i = 0; i < kBatch; ++i) now[i] = aux[i];
+                if (lr + kBatch * row_step < owner_rows) fetch_aux(lr + kBatch * row_step);
+#pragma unroll
+                for (int i = 0; i < kBatch; ++i) {
+                    float r[8];
+                    unpack8(now[i], r);
+                    if constexpr (EPI == kEpiBiasResid) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) f[i][j] += r[j];
+                    } else if constexpr (EPI == kEpiDGelu) {
+                        gelu_grad_mul8(f[i], r, p.e.act);
+                    } else {
+                        float dot = 0.f;                     // zeros beyond M and N
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) dot = fmaf(f[i][j], r[j], dot);
+                        // the head_dim / 8 lanes of a (row, head) are neighbours
+                        for (int o = p.e.head_dim >> 4; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+                        const int row = row0 + lr + i * row_step;
+                        if (col_ok && lr + i * row_step < owner_rows && row < p.e.M && (col % p.e.head_dim) == 0) {
+                            const int b = row / p.e.seq_len, sq = row - b * p.e.seq_len, h = col / p.e.head_dim;
+                            p.e.row_dot[(static_cast<size_t>(b) * (p.e.N / p.e.head_dim) + h) * p.e.seq_len + sq] = dot;
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i) {
+                const int r = lr + i * row_step;
+                if (!(col_ok && r < owner_rows && row0 + r < p.e.M)) continue;
+                const size_t off = static_cast<size_t>(row0 + r) * p.e.ldc + col;
+                *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.e.C) + off) = pack8(f[i]);
+                if constexpr (EPI == kEpiBiasGelu) {
+                    gelu8(f[i], p.e.act);
+                    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.e.aux_out) + off) = pack8(f[i]);
+                }
+            }
+        }
+    }
+}
+
+template <bool PAIR, bool A_MN, bool B_MN, int EPI>
+const char* launch_inst(const CUtensorMap& tmA, const CUtensorMap& tmB, const ClusterParams& p, int grid, size_t smem, cudaStream_t stream)
+{
+    auto kern = gemm_cluster_kernel<PAIR, A_MN, B_MN, EPI>;
+    return launch_cluster_k(kern, dim3(grid), dim3(kThreads), smem, PAIR ? 2 * p.slices : p.slices, stream, tmA, tmB, p) == cudaSuccess
+               ? nullptr : "gemm (K slices in a cluster) launch failed";
+}
+
+template <bool PAIR>
+const char* launch_key(int key, const CUtensorMap& tmA, const CUtensorMap& tmB, const ClusterParams& p, int grid, size_t smem, cudaStream_t stream)
+{
+    switch (key) {
+        case kTN * 16 + kEpiNone: return launch_inst<PAIR, false, false, kEpiNone>(tmA, tmB, p, grid, smem, stream);
+        case kTN * 16 + kEpiBias: return launch_inst<PAIR, false, false, kEpiBias>(tmA, tmB, p, grid, smem, stream);
+        case kTN * 16 + kEpiBiasResid: return launch_inst<PAIR, false, false, kEpiBiasResid>(tmA, tmB, p, grid, smem, stream);
+        case kTN * 16 + kEpiBiasGelu: return launch_inst<PAIR, false, false, kEpiBiasGelu>(tmA, tmB, p, grid, smem, stream);
+        case kNN * 16 + kEpiNone: return launch_inst<PAIR, false, true, kEpiNone>(tmA, tmB, p, grid, smem, stream);
+        case kNN * 16 + kEpiDGelu: return launch_inst<PAIR, false, true, kEpiDGelu>(tmA, tmB, p, grid, smem, stream);
+        case kNN * 16 + kEpiRowDot: return launch_inst<PAIR, false, true, kEpiRowDot>(tmA, tmB, p, grid, smem, stream);
+        case kNT * 16 + kEpiF32: return launch_inst<PAIR, true, true, kEpiF32>(tmA, tmB, p, grid, smem, stream);
+        default: return "gemm: unsupported layout/epilogue combination";
+    }
+}
+
+constexpr size_t kMaxSmem = 226 * 1024;                  // dynamic part (the barriers are static shared memory)
+
+template <bool PAIR, bool A_MN, bool B_MN, int EPI>
+bool set_attr()
+{
+    return cudaFuncSetAttribute(gemm_cluster_kernel<PAIR, A_MN, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(kMaxSmem)) == cudaSuccess;
+}
+template <bool PAIR>
+bool set_attrs()
+{
+    return set_attr<PAIR, false, false, kEpiNone>() && set_attr<PAIR, false, false, kEpiBias>() &&
+           set_attr<PAIR, false, false, kEpiBiasResid>() && set_attr<PAIR, false, false, kEpiBiasGelu>() &&
+           set_attr<PAIR, false, true, kEpiNone>() && set_attr<PAIR, false, true, kEpiDGelu>() &&
+           set_attr<PAIR, false, true, kEpiRowDot>() && set_attr<PAIR, true, true, kEpiF32>();
+}
+
+}  // namespace
+
+const char* configure_gemm_cluster() { return set_attrs<false>() && set_attrs<true>() ? nullptr : "cudaFuncSetAttribute(gemm cluster) failed"; }
+
+const char* launch_gemm_cluster(Runtime* rt, const GemmArgs& a, const GemmClusterPlan& plan, DeviceStatus* status, cudaStream_t stream)
+{
+    const bool a_mn = a.layout == kNT, b_mn = a.layout == kNN || a.layout == kNT;
+    const int tile_m = plan.pair ? 256 : 128, b_rows = plan.pair ? plan.bn / 2 : plan.bn;
+    CUtensorMap tmA, tmB;
+    const char* e;
+    // K-major operand [rows, K]: box 64 k x rows.  MN-major operand stored [K, rows]: box 64 rows x 64 k.
+    e = a_mn ? encode_2d(rt, &tmA, a.A, a.M, a.K, a.lda, 64, 64) : encode_2d(rt, &tmA, a.A, a.K, a.M, a.lda, 64, 128);
+    if (e) return e;
+    e = b_mn ? encode_2d(rt, &tmB, a.B, a.N, a.K, a.ldb, 64, 64) : encode_2d(rt, &tmB, a.B, a.K, a.N, a.ldb, 64, b_rows);
+    if (e) return e;
+    ClusterParams p;
+    p.e.M = a.M; p.e.N = a.N; p.e.C = a.C; p.e.ldc = a.ldc;
+    p.e.bias = static_cast<const __nv_bfloat16*>(a.bias);
+    p.e.aux_in = static_cast<const __nv_bfloat16*>(a.aux_in); p.e.ld_aux = a.ld_aux;
+    p.e.aux_out = a.aux_out; p.e.accumulate = a.accumulate; p.e.act = a.act;
+    p.e.row_dot = static_cast<float*>(a.row_dot); p.e.head_dim = a.head_dim; p.e.seq_len = a.seq_len;
+    p.K = a.K; p.bn = plan.bn; p.slices = plan.slices; p.stages = plan.stages;
+    p.tmem_cols = plan.bn;                               // 64, 128 or 256: what an allocation may be
+    p.log_groups = plan.bn == 256 ? 5 : plan.bn == 128 ? 4 : 3;
+    p.m_tiles = (a.M + tile_m - 1) / tile_m;
+    p.status = status;
+    const int n_tiles = (a.N + plan.bn - 1) / plan.bn;
+    const size_t ring = static_cast<size_t>(plan.stages) * (kATile + b_rows * 128), staged = 128ull * (plan.bn + 4) * 4;
+    size_t smem = (ring > staged ? ring : staged) + 1024;
+    if (smem < kGemmClusterMinSmem) smem = kGemmClusterMinSmem;
+    if (smem > kMaxSmem) return "gemm: cluster plan does not fit shared memory";
+    const int grid = p.m_tiles * n_tiles * plan.slices * (plan.pair ? 2 : 1);
+    const int key = a.layout * 16 + a.epilogue;
+    return plan.pair ? launch_key<true>(key, tmA, tmB, p, grid, smem, stream) : launch_key<false>(key, tmA, tmB, p, grid, smem, stream);
+}
+
+}  // namespace pw

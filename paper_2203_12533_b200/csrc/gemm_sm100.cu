@@ -14,7 +14,7 @@
 // all roles leave their loops, the TMEM allocation is released and the kernel returns.
 #include <cstdlib>
 
-#include "pw_kernels.h"
+#include "gemm_epilogue.cuh"
 
 namespace pw {
 namespace {
@@ -91,13 +91,7 @@ __device__ __forceinline__ void epilogue_group(const uint32_t* v, int row, int c
             if (row < p.M) {
                 float u[8];
                 unpack8(aux, u);
-                if (p.act == 0) {                           // one uniform branch per group, not per pair
-#pragma unroll
-                    for (int j = 0; j < 8; j += 2) gelu_grad_mul2_erf(f[j], f[j + 1], u[j], u[j + 1]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 8; j += 2) gelu_grad_mul2(f[j], f[j + 1], u[j], u[j + 1], p.act);
-                }
+                gelu_grad_mul8(f, u, p.act);
             }
         }
     }
@@ -242,13 +236,7 @@ __device__ __forceinline__ void epilogue_tile(uint4 (&aux)[4], uint32_t taddr, i
                     float f[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) f[j] = __uint_as_float(v[8 * g + j]);
-                    if (p.act == 0) {                       // one uniform branch per group, not per pair
-#pragma unroll
-                        for (int j = 0; j < 8; j += 2) gelu2_erf(f[j], f[j + 1]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 8; j += 2) gelu2(f[j], f[j + 1], p.act);
-                    }
+                    gelu8(f, p.act);
                     o[g] = pack8(f);
                 }
                 store_chunk(o, tmAux);
@@ -621,26 +609,6 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// 2-D tensor map (bf16, or fp32 when f32 is set): `inner` contiguous elements per row, `outer`
-// rows, row pitch ld elements; 128-byte swizzle, so box_inner * element size must be 128 bytes.
-const char* encode_2d(Runtime* rt, CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer, uint64_t ld,
-                      uint32_t box_inner, uint32_t box_outer, bool f32 = false, bool swizzle64 = false)
-{
-    cuuint64_t dims[2] = {inner, outer};
-    cuuint64_t strides[1] = {ld * (f32 ? 4 : 2)};
-    cuuint32_t box[2] = {box_inner, box_outer};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = reinterpret_cast<EncodeTiledFn>(rt->encode_tiled)(
-        map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-        CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? nullptr : "cuTensorMapEncodeTiled failed";
-}
-
 template <bool A_MN, bool B_MN, int EPI>
 const char* launch_inst(Runtime* rt, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmBh,
                         const CUtensorMap& tmC, const CUtensorMap& tmAux, const GemmParams& p, cudaStream_t stream)
@@ -699,7 +667,8 @@ static const char* launch_gemm_pair(Runtime* rt, const GemmArgs& a, DeviceStatus
         auto cost = [&](int w) {
             const long long tiles = static_cast<long long>(m_tiles) * ((a.N + w - 1) / w);
             const long long rounds = (tiles + pairs - 1) / pairs;
-            return static_cast<double>(rounds) * w * (w == 128 ? 1.6 : 1.0);   // 128-wide pair tiles measured ~1.6x slower per FLOP
+            // a 128-wide pair tile takes 1.14x as long per FLOP (2048 x 2048 x 8192: 58.1 us in two rounds against 50.9 in one)
+            return static_cast<double>(rounds) * w * (w == 128 ? 1.15 : 1.0);
         };
         if (cost(128) < cost(256)) bn = 128;
         if (forced == 128 || forced == 256) bn = forced;
@@ -755,6 +724,39 @@ static const char* launch_gemm_pair(Runtime* rt, const GemmArgs& a, DeviceStatus
     }
 }
 
+// Products with few output tiles go to the kernel that gives every tile a cluster of its own
+// (gemm_cluster_sm100.cu).  t64 / t128: output tiles of 128 x 64 / 128 x 128.  Measured at 148 SMs, us per
+// launch back to back, pair kernel -> cluster kernel:
+//   one 128 x 64 tile per SM      256 x 256 x 256 + residual 5.6 -> 3.5, 1024 x 1024 x 1024 + residual 7.8 -> 6.0,
+//                                 1024 x 512 x 512 row dots 8.8 -> 6.1
+//   K cut while SMs are idle      256 x 256 x 1024 + residual 7.3 -> 4.7 (4 slices), 1024 x 512 x 2048 + residual 11.6 -> 7.0 (2),
+//                                 512 x 512 x 1024 weight gradient 6.7 -> 5.7 (2)
+//   256 x 128 tiles cut in two    1024 x 1024 x 4096 + residual 16.8 -> 12.1, dgrad 15.0 -> 12.6
+//   one 128 x 128 tile per SM     2048 x 1024 x 1024 + residual 9.7 -> 8.3, row dots 12.8 -> 11.3; 2048 x 1024 x 4096 + residual 18.1 -> 16.6
+//   two 256 x 128 tiles per pair  1920 x 1280 x 1280 + residual 13.5 -> 12.5, 2048 x 2048 x 2048 + residual 18.4 -> 16.7
+// Where the pair kernel stays the faster one: weight gradients with more than 74 tiles (1024 x 1024 x 1024 7.3 against
+// 7.6: MN-major operands need twice the copies and the fp32 tile leaves through registers), plain dgrads with
+// t64 > 148 (2048 x 1024 x 4096 15.4 against 17.4), and everything whose tiles fill the chip more than once.
+static bool plan_cluster(const GemmArgs& a, int sms, GemmClusterPlan* plan)
+{
+    const int kb = (a.K + 63) / 64;
+    const long long m_tiles = (a.M + 127) / 128, t64 = m_tiles * ((a.N + 63) / 64), t128 = m_tiles * ((a.N + 127) / 128);
+    const bool wgrad = a.layout == kNT, plain_dgrad = a.layout == kNN && a.epilogue == kEpiNone;
+    const bool head128 = a.epilogue == kEpiRowDot && a.head_dim == 128;      // a tile must hold whole heads
+    const bool may_cut = tuning().gemm_split != 0;
+    if (t64 <= sms && !head128) {
+        int slices = 1;
+        if (may_cut && kb >= 12 && 2 * t64 <= sms) slices = 2;
+        if (may_cut && ((kb >= 12 && 8 * t64 <= sms) || (kb >= 24 && 4 * t64 <= sms))) slices = 4;
+        if (slices > 1 || (kb <= 16 && (!wgrad || 2 * t64 <= sms))) { *plan = {0, 64, slices, 8}; return true; }
+    }
+    if (may_cut && a.M > 128 && 2 * t128 <= sms && kb > (wgrad ? 32 : 16)) { *plan = {1, 128, 2, 8}; return true; }
+    if (wgrad || plain_dgrad) return false;
+    if (t128 <= sms) { *plan = kb > 16 && a.M > 128 ? GemmClusterPlan{1, 128, 1, 8} : GemmClusterPlan{0, 128, 1, 6}; return true; }
+    if (t128 <= 2 * sms && a.epilogue == kEpiBiasResid && kb <= 64 && a.M > 128) { *plan = {1, 128, 1, 4}; return true; }
+    return false;
+}
+
 // Scratch for the K halves of cut tiles: (cut tile, half, CTA of the pair) x 128 rows x 256 columns, fp32.
 size_t gemm_split_ws_bytes() { return static_cast<size_t>(kSplitMaxTiles) * 2 * 2 * 128 * BN_MAX * sizeof(float); }
 
@@ -777,6 +779,11 @@ const char* launch_gemm(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cu
     const bool a_mn = a.layout == kNT, b_mn = a.layout == kNN || a.layout == kNT;
     const bool f32_out = a.epilogue == kEpiF32;
     const int pair_mode = tuning().gemm_pair;
+    GemmClusterPlan plan;
+    if (pair_mode && tuning().gemm_bn == 0 && plan_cluster(a, rt->sm_count, &plan)) {
+        if (f32_out && (a.ldc % 4)) return "gemm: fp32 ldc must be a multiple of 4";
+        return launch_gemm_cluster(rt, a, plan, status, stream);
+    }
     if (pair_mode && a.M >= 256) return launch_gemm_pair(rt, a, status, stream);
     if (f32_out && (a.ldc % 4)) return "gemm: fp32 ldc must be a multiple of 4";
     // Tile width: the one that needs the least (rounds x width) on this many SMs; ties go to the

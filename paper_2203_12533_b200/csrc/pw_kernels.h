@@ -46,19 +46,34 @@ struct Tuning {
 Tuning& tuning();
 
 // Launch with the programmatic-serialization attribute (see grid_dep_wait in pw_common.cuh).
+// cluster_size: CTAs per cluster along x (1: none given at launch).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
+inline cudaError_t launch_cluster_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, int cluster_size, cudaStream_t st, Args&&... args)
 {
     Tuning& tn = tuning();
     if (tn.fail_launch_countdown > 0 && --tn.fail_launch_countdown == 0) return cudaErrorLaunchFailure;   // injected by a test
     const bool pdl = tn.pdl != 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;
+    cudaLaunchAttribute at[2];
+    unsigned n = 0;
+    if (pdl) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster_size > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = static_cast<unsigned>(cluster_size);
+        at[n].val.clusterDim.y = 1;
+        at[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = at; cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
+{
+    return launch_cluster_k(kern, grid, block, smem, 1, st, static_cast<Args&&>(args)...);
 }
 
 enum GemmLayout { kTN = 0, kNN = 1, kNT = 2 };
@@ -84,6 +99,19 @@ struct GemmArgs {
     void* row_dot = nullptr; int head_dim = 0, seq_len = 0;
 };
 size_t gemm_split_ws_bytes();
+// One cluster per output tile, the K range cut into slices (gemm_cluster_sm100.cu).
+struct GemmClusterPlan {
+    int pair;                   // 1: 256-row tiles on CTA pairs, 0: 128-row tiles on single CTAs
+    int bn;                     // tile width: 64 (single CTAs only), 128 or 256
+    int slices;                 // K slices: 1, 2, 4 or 8; at most eight CTAs in a cluster
+    int stages;                 // ring depth, at most 8
+};
+// At least a third of an SM's shared memory per CTA: never more than two of them on an SM, whose TMEM two
+// allocations of up to 256 columns always fit, so no CTA of a cluster can block on another cluster's TMEM.
+constexpr size_t kGemmClusterMinSmem = 80 * 1024;
+const char* configure_gemm_cluster();
+const char* launch_gemm_cluster(Runtime* rt, const GemmArgs& a, const GemmClusterPlan& plan, DeviceStatus* status, cudaStream_t stream);
+
 // Encodes the two tensor maps and launches.  Returns nullptr on success, else a static message.
 const char* launch_gemm(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cudaStream_t stream);
 
