@@ -55,7 +55,9 @@ struct KvSmem {
     static constexpr int kK = 0;                             // item buffer i: K_j at i*2*kKV, V_j right after (two buffers)
     static constexpr int kQ = 4 * kKV;                       // ring: stage s holds Q_u at kQ + s*2*kSub, dO_u right after
     static constexpr int kBars = kQ + kStages * 2 * kSub;
-    static constexpr int kBytes = kBars + 256 + 1024;
+    static constexpr int kRow = kBars + 256;                 // per ring stage: lse and delta of the 64 queries (2 x 256 bytes)
+    static constexpr int kBytes = kRow + kStages * 512 + 1024;
+    static_assert(kBytes <= 232448, "shared memory of one CTA");
 };
 
 // Work items of the dK/dV kernel: one per (sequence, head, 128-key tile), heaviest first (key tile
@@ -115,8 +117,11 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
             tma_load_2d(vs + kb * 16384, &tmKV, 2 * d + it.h * DH + kb * 64, it.b * p.S + it.j * 128, bar(0 + buf));
         }
     };
-    auto load_q = [&](const KvItem& it, int i, int s) {     // Q_u and dO_u, u = 2j + i
-        mbar_arrive_expect_tx(bar(L::kQF + s), 2 * L::kSub);
+    auto load_q = [&](const KvItem& it, int i, int s) {     // Q_u and dO_u, u = 2j + i, and their rows' lse and delta
+        mbar_arrive_expect_tx(bar(L::kQF + s), 2 * L::kSub + 512);
+        const size_t row = (static_cast<size_t>(it.b) * p.H + it.h) * p.S + (2 * it.j + i) * 64;
+        bulk_load(sbase + L::kRow + s * 512, p.lse + row, 256, bar(L::kQF + s));
+        bulk_load(sbase + L::kRow + s * 512 + 256, p.delta + row, 256, bar(L::kQF + s));
         const uint32_t qs = sbase + L::kQ + s * 2 * L::kSub, gs = qs + L::kSub;
         const int qrow = it.b * p.S + (2 * it.j + i) * 64;
         for (int kb = 0; kb < L::kBlocks; ++kb) {
@@ -145,8 +150,12 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    // No grid_dep_wait() here: the kernel in front of this one is the dQ kernel, which reads the same inputs and lets
+    // this one start only once they are there, and nothing that it writes is read here.  So the two run side by side: on the
+    // SMs that a small problem leaves idle, and through the dQ kernel's last items on a large one.  The wait at the end makes
+    // the end of this kernel the end of both.  Backward, one after the other -> side by side: 2 x 512 x 16 heads x 64
+    // 29.5 -> 20.7 us, 1 x 2048 x 16 x 128 91.3 -> 72.0 us, 16 x 1024 x 16 x 64 230 -> 217 us.
     grid_dep_launch();                                      // (after the TMEM allocation: see grid_dep_launch)
-    grid_dep_wait();                                        // inputs come from the previous kernels
     // the producer and the MMA role are each the loop of one elected thread (see the forward kernel)
     if (warp == 0) {
         if (elect_one()) {
@@ -274,19 +283,8 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
             if (lane == 0) mbar_arrive(bar(L::kIE + (k & 1)));
             if (!kv_item(p, idx, it)) break;
             const int kv0 = it.j * 128, u0 = 2 * it.j;
-            const float* lse_row = p.lse + (static_cast<size_t>(it.b) * p.H + it.h) * p.S;
-            const float* dl_row = p.delta + (static_cast<size_t>(it.b) * p.H + it.h) * p.S;
             for (int i = 0; i < it.n_u; ++i, ++g) {
                 const int hb = g % L::kBufs, qc0 = (u0 + i) * 64 + ch * 32;   // first query column of this thread's slice
-                // -lse*log2e and -delta of this slice's 32 queries, as two-wide operands
-                uint64_t nl2[16], ndl[16];
-#pragma unroll
-                for (int gg = 0; gg < 8; ++gg) {
-                    const float4 a = *(reinterpret_cast<const float4*>(lse_row + qc0) + gg);
-                    const float4 c = *(reinterpret_cast<const float4*>(dl_row + qc0) + gg);
-                    nl2[2 * gg] = pack_f32x2(-a.x * kLog2e, -a.y * kLog2e); nl2[2 * gg + 1] = pack_f32x2(-a.z * kLog2e, -a.w * kLog2e);
-                    ndl[2 * gg] = pack_f32x2(-c.x, -c.y); ndl[2 * gg + 1] = pack_f32x2(-c.z, -c.w);
-                }
                 ok = mbar_wait(bar(L::kSF + hb), (g / L::kBufs) & 1, abort_flag, p.status, 520);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -296,21 +294,32 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
                 tmem_ld32(tmem_base + lane_addr + L::kDP + hb * 64 + ch * 32, dv);
                 tc_wait_ld();
                 const bool diag = qc0 < kv0 + 128;           // some (key, query) pairs of this slice are masked
+                // lse and delta of this slice's 32 queries: they came with Q_u, whose products are complete, and the
+                // stage is not released before dV / dK have used it (every lane reads the same address: one broadcast)
+                const float4* lse4 = reinterpret_cast<const float4*>(sm + L::kRow + (g % L::kStages) * 512 + ch * 128);
+                const uint64_t nlog2e = pack_f32x2(-kLog2e, -kLog2e), neg1 = pack_f32x2(-1.0f, -1.0f);
                 uint32_t pp[16], dd[16];
                 const uint64_t sl2x2 = pack_f32x2(sl2, sl2);
 #pragma unroll
-                for (int c = 0; c < 32; c += 2) {
-                    float a0, a1, d0, d1;
-                    unpack_f32x2(ffma2(pack_f32x2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1])), sl2x2, nl2[c >> 1]), a0, a1);
-                    float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
-                    if (diag) {
-                        if (qc0 + c < kv0 + r) p0 = 0.f;
-                        if (qc0 + c + 1 < kv0 + r) p1 = 0.f;
+                for (int c4 = 0; c4 < 32; c4 += 4) {
+                    const float4 l4 = lse4[c4 >> 2], d4 = lse4[16 + (c4 >> 2)];
+#pragma unroll
+                    for (int h2 = 0; h2 < 2; ++h2) {
+                        const int c = c4 + 2 * h2;
+                        const uint64_t nl2 = fmul2(h2 ? pack_f32x2(l4.z, l4.w) : pack_f32x2(l4.x, l4.y), nlog2e);
+                        const uint64_t dl = h2 ? pack_f32x2(d4.z, d4.w) : pack_f32x2(d4.x, d4.y);
+                        float a0, a1, d0, d1;
+                        unpack_f32x2(ffma2(pack_f32x2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1])), sl2x2, nl2), a0, a1);
+                        float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
+                        if (diag) {
+                            if (qc0 + c < kv0 + r) p0 = 0.f;
+                            if (qc0 + c + 1 < kv0 + r) p1 = 0.f;
+                        }
+                        const uint64_t pv = pack_f32x2(p0, p1);
+                        unpack_f32x2(fmul2(pv, ffma2(dl, neg1, pack_f32x2(__uint_as_float(dv[c]), __uint_as_float(dv[c + 1])))), d0, d1);
+                        pp[c >> 1] = pack_bf16(p0, p1);
+                        dd[c >> 1] = pack_bf16(d0, d1);
                     }
-                    const uint64_t pv = pack_f32x2(p0, p1);
-                    unpack_f32x2(fmul2(pv, fadd2(pack_f32x2(__uint_as_float(dv[c]), __uint_as_float(dv[c + 1])), ndl[c >> 1])), d0, d1);
-                    pp[c >> 1] = pack_bf16(p0, p1);
-                    dd[c >> 1] = pack_bf16(d0, d1);
                 }
                 // packed operands go back into this warp's own columns: P^T over S^T, dS^T over dP^T
                 tmem_st16(tmem_base + lane_addr + hb * 64 + ch * 32, pp);
@@ -378,6 +387,7 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
     }
+    grid_dep_wait();                                        // the dQ kernel has ended too
 }
 
 // ------------------------------------------------------------------------------------------- dQ
@@ -479,8 +489,8 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    grid_dep_launch();                                      // (after the TMEM allocation: see grid_dep_launch)
     grid_dep_wait();                                        // inputs come from the previous kernels
+    grid_dep_launch();                                      // in this order: the dK/dV kernel starts without a wait of its own
     // TMEM columns of tile t: S at t*256, dP at t*256 + 64, dQ at t*256 + 128
     // the producer and the MMA role are each the loop of one elected thread (see the forward kernel)
     if (warp == 0) {
