@@ -230,6 +230,9 @@ enum {
     PW_SCHEDULE_PER_MICROBATCH = 1 /* forward and backward of micro-batch m before m+1              */
 };
 
+/* Outside OPBYOP the micro-batches of a chain take turns on up to four streams of the stage (forked from and joined to
+ * the caller's), where the workspace that this takes is at most 1 GB beyond one stream's and no two micro-batches' buffers
+ * overlap.  Same bits as on one stream; pw_stage_set_side_stream(stage, 0) keeps everything on the calling stream. */
 pw_status_t pw_stage_create(const pw_layer_config_t* cfg, int n_layers, pw_stage_t** out);
 void pw_stage_destroy(pw_stage_t* stage);
 

@@ -8,10 +8,12 @@
 #include <cstring>
 #include <cstddef>
 #include <cmath>
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -127,7 +129,10 @@ struct pw_layer {
     pw::LayerPlan plan;
     pw::Runtime* rt;
     pw::DeviceStatus* status;
-    unsigned* whole_sync = nullptr; // grid-barrier and split-K words of the whole-layer kernels (zero between launches)
+    // Grid-barrier and split-K words of the whole-layer kernels, one set for launches on all SMs and one for launches
+    // that share them with the other lanes of a stage (a set is tied to one grid size).
+    unsigned* whole_sync = nullptr;
+    int whole_share = 1;            // lanes that share the SMs in the call being enqueued
     cudaStream_t aux = nullptr;     // side stream: weight gradients and bias column sums run beside the dgrad chain
     cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     uint64_t launches = 0;          // kernels launched (or replayed) through this handle
@@ -146,11 +151,32 @@ struct pw_layer {
 struct pw_stage {
     pw_layer_t* layer;
     int n_layers;
+    // Lanes: the micro-batches of a chain take turns on several streams when one layer call is too small to fill the
+    // GPU (see stage_lanes).  Lane 0 is the caller's stream with `layer`; every further one has a handle (status word,
+    // side stream, events), a stream and, in the workspace, a scratch of its own.
+    struct Lane { pw_layer_t* layer; cudaStream_t stream; cudaEvent_t done; };
+    std::vector<Lane> lanes;                // lanes 1, 2, ... (made by the first chain that uses them)
+    std::vector<cudaEvent_t> lane_events;   // [l]: layer l's gradients hold every micro-batch enqueued so far; last: fork
     struct Cached { cudaGraphExec_t exec; uint64_t nodes; };
     std::map<std::vector<uint64_t>, Cached> graphs;
 };
 
 namespace pw {
+
+constexpr int kMaxLanes = 4;
+constexpr size_t kMaxLaneExtra = size_t(1) << 30;       // workspace that the lanes beyond the first may take
+
+static void destroy_lanes(std::vector<pw_stage::Lane>& lanes, std::vector<cudaEvent_t>& events)
+{
+    for (auto& lane : lanes) {
+        if (lane.stream) cudaStreamDestroy(lane.stream);
+        if (lane.done) cudaEventDestroy(lane.done);
+        pw_layer_destroy(lane.layer);
+    }
+    for (auto ev : events) cudaEventDestroy(ev);
+    lanes.clear();
+    events.clear();
+}
 
 static pw_status_t validate_cfg(const pw_layer_config_t* c)
 {
@@ -368,12 +394,12 @@ static pw_status_t do_whole_layer(pw_layer_t* L, const pw_layer_params_t* P, con
         a.g_w_fc2 = G->w_fc2; a.g_b_fc2 = G->b_fc2;
     }
     a.splitk = at(scratch, p.off_whole_splitk);
-    a.sync = L->whole_sync;
+    a.sync = L->whole_sync + (L->whole_share > 1 ? kWholeLayerSyncWords : 0);
     a.status = L->status;
     const double T = p.T, d = p.d, F = p.F;
     const double fwd_flops = 2.0 * T * d * (4.0 * d + 2.0 * F) + 2.0 * T * (p.S + 1.0) * d;
     LaunchScope sc(L, PW_K_WHOLE_LAYER, 1, backward ? 2.0 * fwd_flops + T * (p.S + 1.0) * d : fwd_flops, 0.0, st);
-    const char* e = launch_whole_layer(L->rt, a, backward, st);
+    const char* e = launch_whole_layer(L->rt, a, backward, L->whole_share, st);
     if (e) sc.cancel(1);
     return e ? fail(PW_ERR_CUDA, e) : PW_OK;
 }
@@ -595,7 +621,7 @@ pw_status_t pw_layer_create(const pw_layer_config_t* cfg, pw_layer_t** out)
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&L->status), sizeof(DeviceStatus));
     if (e == cudaSuccess) e = cudaMemset(L->status, 0, sizeof(DeviceStatus));
     if (e == cudaSuccess && L->plan.whole) {
-        const size_t bytes = (2 + kWholeLayerMaxTiles) * sizeof(unsigned);
+        const size_t bytes = 2 * kWholeLayerSyncWords * sizeof(unsigned);
         e = cudaMalloc(reinterpret_cast<void**>(&L->whole_sync), bytes);
         if (e == cudaSuccess) e = cudaMemset(L->whole_sync, 0, bytes);
     }
@@ -713,6 +739,54 @@ pw_status_t pw_layer_launch_count(const pw_layer_t* layer, uint64_t* count)
 
 // ---------------------------------------------------------------------------------------- stage
 
+// Streams over which the micro-batches of a chain take turns.  A layer call is a chain of dependent kernels, so
+// on one stream the SMs idle at every hand-over and, on small shapes, through most of every kernel.  Measured on 4 layers x
+// 8 micro-batches, us per chain on 1 / 2 / 4 / 8 lanes: 256 tokens x 256 wide 3052 / 1805 / 1159 / 1085, 1024 x 512
+// 5209 / 3620 / 3339 / 3283, 1024 x 1024 7511 / 6126 / 5878 / 5860; 4 micro-batches of 2048 x 1024 (saved) 4544 / 3824 / 3814,
+// of 8192 x 2048 47224 / 44959.  Whole-layer kernels share the SMs by lanes, so they stop gaining earlier: 256 x 256
+// 3252 / 2031 / 1782 / 2514, 1024 x 256 4791 / 3706 / 3748.
+static int stage_lanes(const pw_stage_t* stage)
+{
+    const LayerPlan& p = stage->layer->plan;
+    if (stage->n_layers < 2 || stage->n_layers > 64) return 1;
+    const long long tiles = static_cast<long long>((p.T + 127) / 128) * (p.d / 128);     // 128 x 128 tiles of a [T,d] activation
+    return tiles <= (p.whole ? 8 : 64) ? kMaxLanes : 2;
+}
+
+// Creates the handles, streams and events of the lanes, once per stage.  False: the call goes on on one stream (no memory
+// for them, or the stream is being captured, when nothing can be allocated).
+static bool ensure_lanes(pw_stage_t* stage, cudaStream_t st)
+{
+    const int n = stage_lanes(stage);
+    if (n <= 1 || stage->lanes.size() + 1 == static_cast<size_t>(n)) return n > 1;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+    if (cs != cudaStreamCaptureStatusNone) return false;
+    std::vector<pw_stage::Lane> lanes;
+    std::vector<cudaEvent_t> events;
+    cudaError_t e = cudaSuccess;
+    for (int i = 1; i < n && e == cudaSuccess; ++i) {
+        pw_stage::Lane lane = {nullptr, nullptr, nullptr};
+        if (pw_layer_create(&stage->layer->plan.cfg, &lane.layer) != PW_OK) { e = cudaErrorMemoryAllocation; break; }
+        e = cudaStreamCreateWithFlags(&lane.stream, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&lane.done, cudaEventDisableTiming);
+        lanes.push_back(lane);
+    }
+    for (int l = 0; l <= stage->n_layers && e == cudaSuccess; ++l) {
+        cudaEvent_t ev = nullptr;
+        e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e == cudaSuccess) events.push_back(ev);
+    }
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        destroy_lanes(lanes, events);
+        return false;
+    }
+    stage->lanes = lanes;
+    stage->lane_events = events;
+    return true;
+}
+
 pw_status_t pw_stage_create(const pw_layer_config_t* cfg, int n_layers, pw_stage_t** out)
 {
     if (!out) return fail(PW_ERR_INVALID_ARG, "out is NULL");
@@ -733,6 +807,7 @@ void pw_stage_destroy(pw_stage_t* stage)
 {
     if (!stage) return;
     for (auto& kv : stage->graphs) cudaGraphExecDestroy(kv.second.exec);
+    destroy_lanes(stage->lanes, stage->lane_events);
     pw_layer_destroy(stage->layer);
     delete stage;
 }
@@ -742,6 +817,8 @@ struct StageLayout {
     size_t act_bytes, n_act;      // hand-off buffers [T,d] bf16 between layers
     size_t ctx_bytes, n_ctx;      // saved contexts (recompute == 0)
     size_t off_act, off_ctx, off_g0, off_g1, off_scratch, total;
+    int lanes;                    // streams in use; each has its own gradient buffers and scratch
+    size_t lane_bytes;            // pitch of those
 };
 pw_status_t stage_layout(const pw_stage_t* stage, int M, int schedule, int recompute, StageLayout* lay)
 {
@@ -749,18 +826,26 @@ pw_status_t stage_layout(const pw_stage_t* stage, int M, int schedule, int recom
     if (schedule != PW_SCHEDULE_GPIPE && schedule != PW_SCHEDULE_PER_MICROBATCH) return fail(PW_ERR_INVALID_ARG, "unknown schedule");
     if (recompute != 0 && recompute != 1) return fail(PW_ERR_INVALID_ARG, "recompute must be 0 or 1");
     const LayerPlan& p = stage->layer->plan;
-    const size_t L = stage->n_layers, live = (schedule == PW_SCHEDULE_GPIPE) ? M : 1;
+    const size_t L = stage->n_layers;
     lay->act_bytes = align256(static_cast<size_t>(p.T) * p.d * 2);
-    lay->n_act = (L - 1) * live;
     lay->ctx_bytes = p.ctx_bytes;
+    const size_t lane_bytes = 2 * lay->act_bytes + align256(p.scratch_bytes);
+    // what a lane takes beside its gradient buffers and scratch: with one micro-batch alive at a time, that one's activations
+    const size_t lane_live = schedule == PW_SCHEDULE_GPIPE ? 0 : (L - 1) * lay->act_bytes + (recompute ? 0 : L * lay->ctx_bytes);
+    lay->lanes = stage_lanes(stage);
+    if (lay->lanes > M) lay->lanes = M;
+    while (lay->lanes > 1 && (lay->lanes - 1) * (lane_bytes + lane_live) > kMaxLaneExtra) --lay->lanes;
+    const size_t live = (schedule == PW_SCHEDULE_GPIPE) ? M : lay->lanes;
+    lay->n_act = (L - 1) * live;
     lay->n_ctx = recompute ? 0 : L * live;
     size_t s = 0;
     lay->off_act = s; s += lay->act_bytes * lay->n_act;
     lay->off_ctx = s; s += lay->ctx_bytes * lay->n_ctx;
-    lay->off_g0 = s; s += lay->act_bytes;
-    lay->off_g1 = s; s += lay->act_bytes;
-    lay->off_scratch = s; s += p.scratch_bytes;
-    lay->total = s;
+    lay->off_g0 = s;
+    lay->off_g1 = lay->off_g0 + lay->act_bytes;
+    lay->off_scratch = lay->off_g1 + lay->act_bytes;
+    lay->lane_bytes = lane_bytes;
+    lay->total = s + lay->lanes * lane_bytes;
     return PW_OK;
 }
 }  // namespace
@@ -777,25 +862,53 @@ pw_status_t pw_stage_workspace_bytes(const pw_stage_t* stage, int n_microbatches
 }
 
 namespace {
+// Do buffers of different micro-batches overlap (a caller that does not need every y may pass one for all)?  Then their
+// order matters and the chain keeps to one stream.
+bool microbatches_overlap(const void* const* x, const void* const* dy, void* const* y, void* const* dx, int M, size_t bytes)
+{
+    std::vector<std::pair<uintptr_t, int>> b;
+    b.reserve(4 * static_cast<size_t>(M));
+    for (int m = 0; m < M; ++m)
+        for (const void* q : {x[m], dy[m], static_cast<const void*>(y[m]), static_cast<const void*>(dx[m])})
+            b.emplace_back(reinterpret_cast<uintptr_t>(q), m);
+    std::sort(b.begin(), b.end());
+    uintptr_t end = 0, other_end = 0;            // furthest end so far, and the furthest of another micro-batch than that one's
+    int owner = -1;
+    for (const auto& [start, m] : b) {
+        if (start < (m == owner ? other_end : end)) return true;
+        if (m != owner) { other_end = end; owner = m; }
+        end = start + bytes;                     // starts ascend and all lengths are equal
+    }
+    return false;
+}
+
 // Enqueues the whole chain on `st`.  sync_each = OPBYOP.
+// With lanes, micro-batch m runs on lane m % lanes.  A lane keeps its own micro-batches in order; across lanes
+// the only ties are the parameter gradients: layer l of micro-batch m adds to what layer l of micro-batch m - 1 left, so its
+// backward starts after that one's.  (Letting only the weight gradients wait measured the same.)  The sums have the same order, and every result the same bits, as on one stream.
 pw_status_t enqueue_chain(pw_stage_t* stage, const pw_layer_params_t* params, const pw_layer_grads_t* grads,
                           const void* const* x_mb, const void* const* dy_mb, void* const* y_mb, void* const* dx_mb,
                           int M, int schedule, int recompute, void* ws, const StageLayout& lay, bool sync_each,
                           cudaStream_t st)
 {
-    pw_layer_t* Lh = stage->layer;
     const int L = stage->n_layers;
     const bool gpipe = schedule == PW_SCHEDULE_GPIPE;
+    const int lanes = sync_each || stage->layer->profiling || stage->layer->single_stream || stage->lanes.empty() ||
+                      (lay.lanes > 1 && microbatches_overlap(x_mb, dy_mb, y_mb, dx_mb, M, static_cast<size_t>(stage->layer->plan.T) * stage->layer->plan.d * 2))
+                          ? 1 : lay.lanes;
+    auto lane_of = [&](int m) { return m % lanes; };
+    auto handle = [&](int m) { return lane_of(m) == 0 ? stage->layer : stage->lanes[lane_of(m) - 1].layer; };
+    auto stream = [&](int m) { return lane_of(m) == 0 ? st : stage->lanes[lane_of(m) - 1].stream; };
     auto act = [&](int m, int l) -> void* {   // input of layer l (l >= 1) for micro-batch m
-        const size_t slot = (gpipe ? static_cast<size_t>(m) * (L - 1) : 0) + (l - 1);
+        const size_t slot = static_cast<size_t>(gpipe ? m : lane_of(m)) * (L - 1) + (l - 1);
         return at(ws, lay.off_act + slot * lay.act_bytes);
     };
     auto ctxp = [&](int m, int l) -> void* {
         if (recompute) return nullptr;
-        const size_t slot = (gpipe ? static_cast<size_t>(m) * L : 0) + l;
+        const size_t slot = static_cast<size_t>(gpipe ? m : lane_of(m)) * L + l;
         return at(ws, lay.off_ctx + slot * lay.ctx_bytes);
     };
-    void* scratch = at(ws, lay.off_scratch);
+    auto lane_at = [&](int m, size_t off) -> void* { return at(ws, off + lane_of(m) * lay.lane_bytes); };
     auto sync = [&]() -> pw_status_t {
         if (!sync_each) return PW_OK;
         cudaError_t e = cudaStreamSynchronize(st);
@@ -805,10 +918,10 @@ pw_status_t enqueue_chain(pw_stage_t* stage, const pw_layer_params_t* params, co
         for (int l = 0; l < L; ++l) {
             const void* in = l == 0 ? x_mb[m] : act(m, l);
             void* out = l == L - 1 ? y_mb[m] : act(m, l + 1);
+            void* scratch = lane_at(m, lay.off_scratch);
             void* c = ctxp(m, l);
-            pw_status_t s = enqueue_fwd(Lh, &params[l], in, out, c ? c : scratch, scratch, true, st);
-            if (s != PW_OK) return s;
-            if ((s = sync()) != PW_OK) return s;
+            PW_DO(enqueue_fwd(handle(m), &params[l], in, out, c ? c : scratch, scratch, true, stream(m)));
+            PW_DO(sync());
         }
         return PW_OK;
     };
@@ -816,25 +929,57 @@ pw_status_t enqueue_chain(pw_stage_t* stage, const pw_layer_params_t* params, co
         const void* g = dy_mb[m];
         for (int l = L - 1; l >= 0; --l) {
             const void* in = l == 0 ? x_mb[m] : act(m, l);
-            void* out = l == 0 ? dx_mb[m] : at(ws, (l & 1) ? lay.off_g1 : lay.off_g0);
-            pw_status_t s = enqueue_bwd(Lh, &params[l], in, g, out, &grads[l], m > 0 ? 1 : 0, ctxp(m, l), scratch, st);
-            if (s != PW_OK) return s;
-            if ((s = sync()) != PW_OK) return s;
+            void* out = l == 0 ? dx_mb[m] : lane_at(m, (l & 1) ? lay.off_g1 : lay.off_g0);
+            if (lanes > 1 && m > 0) {
+                cudaError_t e = cudaStreamWaitEvent(stream(m), stage->lane_events[l], 0);
+                if (e != cudaSuccess) return fail_cuda("stage lane ordering", e);
+            }
+            PW_DO(enqueue_bwd(handle(m), &params[l], in, g, out, &grads[l], m > 0 ? 1 : 0, ctxp(m, l), lane_at(m, lay.off_scratch), stream(m)));
+            if (lanes > 1 && m + 1 < M) {
+                cudaError_t e = cudaEventRecord(stage->lane_events[l], stream(m));
+                if (e != cudaSuccess) return fail_cuda("stage lane ordering", e);
+            }
+            PW_DO(sync());
             g = out;
         }
         return PW_OK;
     };
-    pw_status_t s;
-    if (gpipe) {
-        for (int m = 0; m < M; ++m) if ((s = fwd_mb(m)) != PW_OK) return s;
-        for (int m = 0; m < M; ++m) if ((s = bwd_mb(m)) != PW_OK) return s;
-    } else {
-        for (int m = 0; m < M; ++m) {
-            if ((s = fwd_mb(m)) != PW_OK) return s;
-            if ((s = bwd_mb(m)) != PW_OK) return s;
+    auto fork = [&]() -> pw_status_t {
+        if (lanes == 1) return PW_OK;
+        cudaError_t e = cudaEventRecord(stage->lane_events[L], st);
+        for (int i = 1; i < lanes && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(stage->lanes[i - 1].stream, stage->lane_events[L], 0);
+        return e == cudaSuccess ? PW_OK : fail_cuda("stage lane fork", e);
+    };
+    auto join = [&]() -> pw_status_t {
+        cudaError_t e = cudaSuccess;
+        for (int i = 1; i < lanes && e == cudaSuccess; ++i) {
+            e = cudaEventRecord(stage->lanes[i - 1].done, stage->lanes[i - 1].stream);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, stage->lanes[i - 1].done, 0);
         }
-    }
-    return PW_OK;
+        return e == cudaSuccess ? PW_OK : fail_cuda("stage lane join", e);
+    };
+    auto run = [&]() -> pw_status_t {
+        if (gpipe) {
+            for (int m = 0; m < M; ++m) PW_DO(fwd_mb(m));
+            for (int m = 0; m < M; ++m) PW_DO(bwd_mb(m));
+        } else {
+            for (int m = 0; m < M; ++m) {
+                PW_DO(fwd_mb(m));
+                PW_DO(bwd_mb(m));
+            }
+        }
+        return PW_OK;
+    };
+    auto share = [&](int n) {
+        stage->layer->whole_share = n;
+        for (auto& lane : stage->lanes) lane.layer->whole_share = n;
+    };
+    PW_DO(fork());
+    if (lanes > 1) share(static_cast<int>(stage->lanes.size()) + 1);
+    const pw_status_t s = run();
+    share(1);
+    const pw_status_t j = join();                // also after a failure: a stream capture must find its forks joined
+    return s != PW_OK ? s : j;
 }
 }  // namespace
 
@@ -864,6 +1009,7 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
         if (x_mb[m] == y_mb[m] || x_mb[m] == dx_mb[m]) return fail(PW_ERR_INVALID_ARG, "y and dx must not alias x");
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (dispatch_mode != PW_DISPATCH_OPBYOP && lay.lanes > 1) ensure_lanes(stage, st);
 
     if (dispatch_mode != PW_DISPATCH_GRAPH)
         return enqueue_chain(stage, params, grads, x_mb, dy_mb, y_mb, dx_mb, M, schedule, recompute, workspace, lay,
@@ -890,10 +1036,17 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
         if (st == nullptr) return fail(PW_ERR_INVALID_ARG, "GRAPH mode needs a non-default stream (the legacy stream cannot be captured)");
         cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return fail_cuda("cudaStreamBeginCapture", e);
-        stage->layer->capturing = true;
+        auto set_capturing = [&](bool on) {
+            stage->layer->capturing = on;
+            for (auto& lane : stage->lanes) lane.layer->capturing = on;
+        };
+        set_capturing(true);
         stage->layer->graph_nodes = 0;
+        for (auto& lane : stage->lanes) lane.layer->graph_nodes = 0;
         s = enqueue_chain(stage, params, grads, x_mb, dy_mb, y_mb, dx_mb, M, schedule, recompute, workspace, lay, false, st);
-        stage->layer->capturing = false;
+        set_capturing(false);
+        uint64_t nodes = stage->layer->graph_nodes;
+        for (auto& lane : stage->lanes) nodes += lane.layer->graph_nodes;
         cudaGraph_t graph = nullptr;
         e = cudaStreamEndCapture(st, &graph);
         if (s != PW_OK) { if (graph) cudaGraphDestroy(graph); return s; }
@@ -906,7 +1059,7 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
             for (auto& kv : stage->graphs) cudaGraphExecDestroy(kv.second.exec);
             stage->graphs.clear();
         }
-        it = stage->graphs.emplace(key, pw_stage::Cached{exec, stage->layer->graph_nodes}).first;
+        it = stage->graphs.emplace(key, pw_stage::Cached{exec, nodes}).first;
     }
     cudaError_t e = cudaGraphLaunch(it->second.exec, st);
     if (e != cudaSuccess) return fail_cuda("cudaGraphLaunch", e);
@@ -917,7 +1070,12 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
 pw_status_t pw_stage_status(pw_stage_t* stage, int* device_status, int* site)
 {
     if (!stage) return fail(PW_ERR_INVALID_ARG, "stage is NULL");
-    return read_status(stage->layer->status, device_status, site);
+    int code = 0, where = 0;
+    PW_DO(read_status(stage->layer->status, &code, &where));
+    for (size_t i = 0; i < stage->lanes.size() && code == 0; ++i) PW_DO(read_status(stage->lanes[i].layer->status, &code, &where));
+    if (device_status) *device_status = code;
+    if (site) *site = where;
+    return PW_OK;
 }
 pw_status_t pw_stage_profile_begin(pw_stage_t* stage)
 {
@@ -931,8 +1089,10 @@ pw_status_t pw_stage_profile_end(pw_stage_t* stage, pw_profile_t* out)
 }
 pw_status_t pw_stage_launch_count(const pw_stage_t* stage, uint64_t* count)
 {
-    if (!stage) return fail(PW_ERR_INVALID_ARG, "stage is NULL");
-    return pw_layer_launch_count(stage->layer, count);
+    if (!stage || !count) return fail(PW_ERR_INVALID_ARG, "stage or count is NULL");
+    *count = stage->layer->launches;
+    for (const auto& lane : stage->lanes) *count += lane.layer->launches;
+    return PW_OK;
 }
 
 pw_status_t pw_layer_set_side_stream(pw_layer_t* layer, int enabled)

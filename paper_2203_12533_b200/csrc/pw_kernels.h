@@ -193,6 +193,7 @@ const char* launch_attention_bwd(Runtime* rt, const void* qkv, const void* o, co
 // Tensor names are those of the layer plan: ctx tensors (h1 ... r2), backward temporaries (big =
 // du, later dqkv; td0 = dh2, dout, dh1; dx1), the 12 parameters and their fp32 gradients.
 constexpr int kWholeLayerMaxTiles = 1024;           // (tokens / 64) * (d_model / 64): one split-K ticket each
+constexpr int kWholeLayerSyncWords = 2 + kWholeLayerMaxTiles;
 struct WholeLayerArgs {
     int T, d, H, F, B, S, act, accumulate, with_fc2;
     int split_o, split_fc2, split_dh2, split_dh1;   // K slices of the GEMMs with [T, d] outputs (set by the launcher)
@@ -204,12 +205,13 @@ struct WholeLayerArgs {
     void *big, *td0, *dx1;
     void *g_ln1_g, *g_ln1_b, *g_w_qkv, *g_b_qkv, *g_w_o, *g_b_o, *g_ln2_g, *g_ln2_b, *g_w_fc1, *g_b_fc1, *g_w_fc2, *g_b_fc2;
     void* splitk;                                   // whole_layer_splitk_bytes() of fp32 partial tiles
-    unsigned* sync;                                 // 2 + kWholeLayerMaxTiles words, zero when the handle is created
+    unsigned* sync;                                 // kWholeLayerSyncWords words, zero when the handle is created
     DeviceStatus* status;
 };
 const char* configure_whole_layer();
 const char* whole_layer_unsupported(int T, int d, int H, int dh, int F, int S);   // nullptr if the shape is served
 size_t whole_layer_splitk_bytes(int T, int d);
-const char* launch_whole_layer(Runtime* rt, WholeLayerArgs a, bool backward, cudaStream_t stream);
+// share: how many such launches may run side by side (each then takes that part of the SMs).  `sync` belongs to one value of it.
+const char* launch_whole_layer(Runtime* rt, WholeLayerArgs a, bool backward, int share, cudaStream_t stream);
 
 }  // namespace pw

@@ -1157,15 +1157,16 @@ static int pick_slices(int tiles, int K, int room)
 
 size_t whole_layer_splitk_bytes(int T, int d) { return static_cast<size_t>(T >> 6) * (d >> 6) * 8 * 4096 * sizeof(float); }
 
-const char* launch_whole_layer(Runtime* rt, WholeLayerArgs a, bool backward, cudaStream_t stream)
+const char* launch_whole_layer(Runtime* rt, WholeLayerArgs a, bool backward, int share, cudaStream_t stream)
 {
+    // The K slices are those of a launch that has all SMs, so the sums do not depend on how many launches share them.
     const int grid = rt->sm_count;
     const int tiles = (a.T >> 6) * (a.d >> 6);
     a.split_o = pick_slices(tiles, a.d, grid - (a.d >> 6) * (a.d >> 6));
     a.split_fc2 = pick_slices(tiles, a.F, grid);
     a.split_dh2 = pick_slices(tiles, a.F, grid - (a.F >> 6) * (a.d >> 6));
     a.split_dh1 = pick_slices(tiles, 3 * a.d, grid - (3 * a.d >> 6) * (a.d >> 6));
-    const cudaError_t e = launch_coop(backward ? whole_layer_bwd_kernel : whole_layer_fwd_kernel, grid, stream, a);
+    const cudaError_t e = launch_coop(backward ? whole_layer_bwd_kernel : whole_layer_fwd_kernel, grid / share, stream, a);
     return e == cudaSuccess ? nullptr : cudaGetErrorString(e);
 }
 

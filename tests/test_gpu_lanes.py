@@ -1,0 +1,75 @@
+"""A chain whose micro-batches take turns on several streams gives the bits of the chain on one stream.
+
+OPBYOP runs on the calling stream alone; ASYNC and GRAPH use the lanes.  Micro-batch counts below, at and beyond the lane
+count, and not a multiple of it."""
+import pytest
+import torch
+
+from paper_2203_12533_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pw():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2203_12533_b200 import binding
+    binding.lib()
+    return binding
+
+
+@pytest.mark.parametrize("width,heads,seq,batch,layers,M,flags", [
+    (256, 4, 128, 2, 3, 1, 0), (256, 4, 128, 2, 3, 2, 0), (256, 4, 128, 1, 2, 5, 0), (256, 4, 128, 2, 3, 9, 0),     # four lanes
+    (256, 4, 128, 2, 2, 6, "lean"), (256, 4, 128, 2, 3, 6, "whole"), (512, 8, 256, 2, 2, 3, "whole"),
+    (1024, 8, 1024, 2, 2, 3, 0), (1024, 16, 1152, 1, 2, 2, 0)])                                                  # two lanes
+@pytest.mark.parametrize("gpipe,recompute", [(True, True), (True, False), (False, True), (False, False)])
+def test_lanes_change_no_bit(pw, width, heads, seq, batch, layers, M, flags, gpipe, recompute):
+    w = inputs.Workload("lanes", width, heads, width // heads, 2 * width, seq, batch)
+    flags = {"lean": pw.FLAG_LEAN_CTX, "whole": pw.FLAG_WHOLE_LAYER, 0: 0}[flags]
+    schedule = pw.SCHEDULE_GPIPE if gpipe else pw.SCHEDULE_PER_MICROBATCH
+    params = [[p.cuda() for p in inputs.layer_params(w, 0, l, random_ln=True)] for l in range(layers)]
+    xs, dys = zip(*[[t.cuda().view(w.tokens, -1) for t in inputs.microbatch(w, 0, m)] for m in range(M)])
+    stage = pw.Stage(layers, w.d_model, w.n_heads, w.head_dim, w.d_ff, w.seq_len, w.batch, flags=flags)
+    ws = torch.empty(stage.workspace_bytes(M, schedule, recompute), dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.Stream()
+
+    def chain(dispatch):
+        ws.fill_(255)                                        # stale activations would not go unseen (bf16 NaN)
+        ys, dxs = [torch.full_like(x, 7.0) for x in xs], [torch.full_like(x, 7.0) for x in xs]
+        grads = [[torch.full(p.shape, 7.0, device="cuda") for p in ps] for ps in params]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, schedule, recompute, stream=stream)
+        torch.cuda.synchronize()
+        assert stage.status() == (0, 0)
+        return ys + dxs + [g for gs in grads for g in gs]
+
+    ref = chain(pw.DISPATCH_OPBYOP)
+    assert all(torch.isfinite(t).all() for t in ref)
+    n0 = stage.launch_count()
+    for dispatch in (pw.DISPATCH_ASYNC, pw.DISPATCH_GRAPH, pw.DISPATCH_ASYNC):
+        for a, b in zip(ref, chain(dispatch)):
+            assert torch.equal(a, b)
+    assert stage.launch_count() == 4 * n0                    # every lane's launches are counted, a graph's too
+
+
+def test_one_buffer_for_every_output_keeps_the_last_micro_batch(pw):
+    """Overlapping buffers keep the chain on one stream: the last micro-batch's y is what stays."""
+    w = inputs.Workload("lanes", 256, 4, 64, 512, 128, 2)
+    M, L = 5, 2
+    params = [[p.cuda() for p in inputs.layer_params(w, 0, l)] for l in range(L)]
+    grads = [[torch.zeros(p.shape, device="cuda") for p in ps] for ps in params]
+    xs, dys = zip(*[[t.cuda().view(w.tokens, -1) for t in inputs.microbatch(w, 0, m)] for m in range(M)])
+    stage = pw.Stage(L, w.d_model, w.n_heads, w.head_dim, w.d_ff, w.seq_len, w.batch)
+    ws = torch.empty(stage.workspace_bytes(M, pw.SCHEDULE_GPIPE, True), dtype=torch.uint8, device="cuda")
+    ys, dxs = [torch.empty_like(x) for x in xs], [torch.empty_like(x) for x in xs]
+    stage.run_chain(params, grads, xs, dys, ys, dxs, ws, pw.DISPATCH_ASYNC)
+    y = torch.empty_like(xs[0])
+    buf = torch.empty((w.tokens + 8, 256), dtype=torch.bfloat16, device="cuda")
+    stage.run_chain(params, grads, xs, dys, [y] * M, dxs, ws, pw.DISPATCH_ASYNC)
+    part = [buf[:w.tokens]] + ys[1:-1] + [buf[8:]]           # the first and the last overlap by all but eight rows
+    want = ys[-1].clone()
+    stage.run_chain(params, grads, xs, dys, part, dxs, ws, pw.DISPATCH_ASYNC)
+    torch.cuda.synchronize()
+    assert torch.equal(y, want) and torch.equal(buf[8:], want)
