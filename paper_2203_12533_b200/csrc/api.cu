@@ -113,7 +113,7 @@ struct LayerPlan {
     float eps;
     size_t ctx_off[PW_CTX_COUNT], ctx_size[PW_CTX_COUNT], ctx_bytes;
     // scratch = [ctx-shaped region used when the caller passes ctx == NULL] [backward temporaries]
-    size_t off_big, off_td0, off_td1, off_delta, off_partials, off_partials2, off_partials3, off_partials4, scratch_bytes;
+    size_t off_big, off_dqkv, off_td0, off_td1, off_delta, off_partials, off_partials2, off_partials3, off_partials4, scratch_bytes;
     // lean ctx: h1, h2, a (and the statistics the re-derivation writes again) live in scratch
     bool lean;
     size_t off_lean_h1, off_lean_h2, off_lean_a, off_lean_stats;
@@ -133,8 +133,8 @@ struct pw_layer {
     // that share them with the other lanes of a stage (a set is tied to one grid size).
     unsigned* whole_sync = nullptr;
     int whole_share = 1;            // lanes that share the SMs in the call being enqueued
-    cudaStream_t aux = nullptr;     // side stream: weight gradients and bias column sums run beside the dgrad chain
-    cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    cudaStream_t aux = nullptr;     // side stream: what a lean save set makes again runs beside the dgrad chain
+    cudaEvent_t ev[2] = {nullptr, nullptr};
     uint64_t launches = 0;          // kernels launched (or replayed) through this handle
     bool single_stream = false;     // pw_layer_set_side_stream(layer, 0): everything on the calling stream
     bool capturing = false;         // inside a stream capture: count launches into graph_nodes instead
@@ -219,7 +219,11 @@ static void build_plan(const pw_layer_config_t& c, Runtime* rt, LayerPlan* p)
     for (int i = 0; i < PW_CTX_COUNT; ++i) { p->ctx_off[i] = off; p->ctx_size[i] = sz[i]; off += align256(sz[i]); }
     p->ctx_bytes = off;
     size_t s = p->ctx_bytes;
-    p->off_big = s; s += align256((F > 3 * d ? T * F : T * 3 * d) * 2);
+    const bool whole = (c.flags & PW_FLAG_WHOLE_LAYER) != 0;
+    // du and dqkv have a buffer each, so that attention's backward need not wait for the weight gradient and the column
+    // sum of du on the side stream; the whole-layer kernels, which have no side stream, share one.
+    p->off_big = s; s += align256((whole ? std::max(T * F, T * 3 * d) : T * F) * 2);
+    p->off_dqkv = s; s += whole ? 0 : align256(T * 3 * d * 2);
     p->off_td0 = s; s += align256(T * d * 2);
     p->off_td1 = s; s += align256(T * d * 2);
     p->off_delta = s; s += align256(static_cast<size_t>(p->B) * p->H * p->S * 4);
@@ -241,7 +245,7 @@ static void build_plan(const pw_layer_config_t& c, Runtime* rt, LayerPlan* p)
         p->off_lean_a = s; s += align256(T * F * 2);
         p->off_lean_stats = s; s += 2 * align256(T * 4);
     }
-    p->whole = (c.flags & PW_FLAG_WHOLE_LAYER) != 0;
+    p->whole = whole;
     p->off_whole_splitk = 0;
     if (p->whole) { p->off_whole_splitk = s; s += align256(whole_layer_splitk_bytes(p->T, p->d)); }
     p->scratch_bytes = s;
@@ -309,6 +313,15 @@ static pw_status_t do_gemm(pw_layer_t* L, const GemmArgs& g, cudaStream_t st)
     if (e) sc.cancel(1);
     return e ? fail(PW_ERR_CUDA, e) : PW_OK;
 }
+static pw_status_t do_wgrad(pw_layer_t* L, const WgradJob* jobs, int n, int accumulate, bool late, cudaStream_t st)
+{
+    double flops = 0.0;
+    for (int j = 0; j < n; ++j) flops += 2.0 * jobs[j].M * jobs[j].N * L->plan.T;
+    LaunchScope sc(L, PW_K_GEMM_NT, 1, flops, 0.0, st);
+    const char* e = launch_wgrad(L->rt, jobs, n, L->plan.T, accumulate, late, L->status, st);
+    if (e) sc.cancel(1);
+    return e ? fail(PW_ERR_CUDA, e) : PW_OK;
+}
 static pw_status_t do_ln_fwd(pw_layer_t* L, const void* x, const void* gamma, const void* beta, void* h, void* mu,
                              void* rstd, cudaStream_t st)
 {
@@ -337,7 +350,7 @@ static pw_status_t do_colsum(pw_layer_t* L, const void* in, int N, void* out, in
 {
     const LayerPlan& p = L->plan;
     LaunchScope sc(L, PW_K_COLSUM, defer ? 1 : 2, 0.0, 2.0 * p.T * N, st);
-    const char* e = defer ? launch_colsum_partial(L->rt, in, p.T, N, N, out, partials, defer, st)
+    const char* e = defer ? launch_colsum_partial(L->rt, in, p.T, N, N, out, partials, defer, true, st)
                           : launch_colsum(L->rt, in, p.T, N, N, out, accumulate, partials, st);
     return e ? fail(PW_ERR_CUDA, e) : PW_OK;
 }
@@ -460,7 +473,8 @@ static pw_status_t enqueue_bwd(pw_layer_t* L, const pw_layer_params_t* P, const 
     const void* u = at(ctx, p.ctx_off[PW_CTX_U]);     const void* lse = at(ctx, p.ctx_off[PW_CTX_LSE]);
     const void* mu1 = at(ctx, p.ctx_off[PW_CTX_MU1]); const void* r1 = at(ctx, p.ctx_off[PW_CTX_R1]);
     const void* mu2 = at(ctx, p.ctx_off[PW_CTX_MU2]); const void* r2 = at(ctx, p.ctx_off[PW_CTX_R2]);
-    void* big = at(scratch, p.off_big);        // du [T,F], later dqkv [T,3d]
+    void* du = at(scratch, p.off_big);
+    void* dqkv = at(scratch, p.off_dqkv);
     void* td0 = at(scratch, p.off_td0);        // dh2, then dout, then dh1
     void* dx1 = at(scratch, p.off_td1);
     void* delta = at(scratch, p.off_delta);
@@ -471,11 +485,10 @@ static pw_status_t enqueue_bwd(pw_layer_t* L, const pw_layer_params_t* P, const 
     void* part4 = at(scratch, p.off_partials4);
     ReduceJob jobs[4];                                   // LN2, db1, LN1, dbqkv: summed by one launch at the end
 
-    // The weight gradients and the bias column sums hang off the dgrad chain, so they run on a
-    // side stream: their CTAs fill the SMs that the last, partly filled round of a dgrad GEMM
-    // leaves idle (and the HBM-bound kernels share SMs with GEMM CTAs).  Events order the two
-    // streams; the side stream always rejoins before this call returns, so a captured graph sees
-    // a plain fork/join.  While per-kernel profiling is on everything stays on one stream.
+    // The four weight gradients hang off the data-gradient chain and nothing waits for them: they run as one pool of tiles
+    // at the end of the call.  (On a side stream, each behind the kernel that makes its operand, they finished about as
+    // early on large shapes, ended in four partly filled rounds instead of one, held up the chain wherever one of
+    // their tiles got an SM first, and cost the host a dozen event calls.)
     cudaStream_t ax = (L->profiling || L->single_stream) ? st : L->aux;
     auto order = [&](cudaEvent_t ev, cudaStream_t from, cudaStream_t to) -> pw_status_t {
         if (from == to) return PW_OK;
@@ -483,66 +496,61 @@ static pw_status_t enqueue_bwd(pw_layer_t* L, const pw_layer_params_t* P, const 
         if (e == cudaSuccess) e = cudaStreamWaitEvent(to, ev, 0);
         return e == cudaSuccess ? PW_OK : fail_cuda("stream ordering", e);
     };
-    PW_DO(order(L->ev[0], st, ax));                      // side stream starts after everything already enqueued
-    // Lean ctx: the three operands of the weight-gradient GEMMs that were not kept are made again on
-    // the side stream, each just before the GEMM that reads it.  The statistics the LayerNorm kernel
-    // writes once more go to scratch (the ctx is read-only here).
-    void* lean_st1 = p.lean ? at(scratch, p.off_lean_stats) : nullptr;
-    void* lean_st2 = p.lean ? at(scratch, p.off_lean_stats + align256(static_cast<size_t>(T) * 4)) : nullptr;
+    // Lean ctx: the three operands of the weight-gradient GEMMs that were not kept are made again on the side
+    // stream, beside the data-gradient chain.  The statistics the LayerNorm kernel writes once more go to scratch (the ctx is
+    // read-only here).
     if (rederive) {
-        LaunchScope sc(L, PW_K_GELU, 1, 0.0, 4.0 * T * F, ax);
-        const char* e = launch_gelu_fwd(L->rt, u, const_cast<void*>(a), static_cast<long long>(T) * F, act, ax);
-        if (e) return fail(PW_ERR_CUDA, e);
+        void* lean_st1 = at(scratch, p.off_lean_stats);
+        void* lean_st2 = at(scratch, p.off_lean_stats + align256(static_cast<size_t>(T) * 4));
+        PW_DO(order(L->ev[0], st, ax));
+        {
+            LaunchScope sc(L, PW_K_GELU, 1, 0.0, 4.0 * T * F, ax);
+            const char* e = launch_gelu_fwd(L->rt, u, const_cast<void*>(a), static_cast<long long>(T) * F, act, ax);
+            if (e) return fail(PW_ERR_CUDA, e);
+        }
+        PW_DO(do_ln_fwd(L, x1, P->ln2_gamma, P->ln2_beta, const_cast<void*>(h2), lean_st1, lean_st2, ax));
+        PW_DO(do_ln_fwd(L, x, P->ln1_gamma, P->ln1_beta, const_cast<void*>(h1), lean_st1, lean_st2, ax));
+    }
+    void* sk = at(scratch, p.off_splitk);                // GEMMs run one after the other on the calling stream
+    const WgradJob wj[4] = {{F, d, du, F, h2, d, G->w_fc1, d}, {3 * d, d, dqkv, 3 * d, h1, d, G->w_qkv, d},
+                            {d, d, dx1, d, o, d, G->w_o, d}, {d, F, dy, d, a, F, G->w_fc2, F}};
+    // A caller may have dx written over dy: then dW2, which reads dy, cannot wait for the end.
+    const uintptr_t dy_at = reinterpret_cast<uintptr_t>(dy), dx_at = reinterpret_cast<uintptr_t>(dx), act_bytes = static_cast<uintptr_t>(T) * d * 2;
+    const bool dx_over_dy = dy_at < dx_at + act_bytes && dx_at < dy_at + act_bytes;
+    if (dx_over_dy) {
+        if (rederive) PW_DO(order(L->ev[1], ax, st));
+        PW_DO(do_wgrad(L, wj + 3, 1, accumulate, false, st));
     }
     // y = x1 + a W2^T + b2  ->  du = (dy W2) * gelu'(u),  dW2 = dy^T a
-    PW_DO(do_gemm(L, gemm_args(kNT, kEpiF32, act, d, F, T, dy, d, a, F, G->w_fc2, F, nullptr, nullptr, 0,
-                                     nullptr, accumulate), ax));
-    void* sk = at(scratch, p.off_splitk);                // dgrad GEMMs run one after the other on the calling stream
-    PW_DO(do_gemm(L, gemm_args(kNN, kEpiDGelu, act, T, F, d, dy, d, P->w_fc2, F, big, F, nullptr, u, F,
+    PW_DO(do_gemm(L, gemm_args(kNN, kEpiDGelu, act, T, F, d, dy, d, P->w_fc2, F, du, F, nullptr, u, F,
                                      nullptr, 0, sk), st));
-    PW_DO(order(L->ev[1], st, ax));                      // du ready
     // u = h2 W1^T + b1  ->  dh2 = du W1,  dW1 = du^T h2,  db1 = colsum(du)
-    if (rederive) PW_DO(do_ln_fwd(L, x1, P->ln2_gamma, P->ln2_beta, const_cast<void*>(h2), lean_st1, lean_st2, ax));
-    PW_DO(do_gemm(L, gemm_args(kNT, kEpiF32, act, F, d, T, big, F, h2, d, G->w_fc1, d, nullptr, nullptr, 0,
-                                     nullptr, accumulate), ax));
-    PW_DO(do_colsum(L, big, F, G->b_fc1, accumulate, part2, ax, &jobs[1]));
-    if (ax != st) {                                      // remembered: du may be overwritten only after these two
-        cudaError_t e = cudaEventRecord(L->ev[2], ax);
-        if (e != cudaSuccess) return fail_cuda("stream ordering", e);
-    }
-    PW_DO(do_gemm(L, gemm_args(kNN, kEpiNone, act, T, d, F, big, F, P->w_fc1, d, td0, d, nullptr, nullptr, 0,
+    PW_DO(do_gemm(L, gemm_args(kNN, kEpiNone, act, T, d, F, du, F, P->w_fc1, d, td0, d, nullptr, nullptr, 0,
                                      nullptr, 0, sk), st));
     // LN2 backward + residual: dx1 = dy + LNbwd(dh2); also db2 = colsum(dy), dbo = colsum(dx1)
     PW_DO(do_ln_bwd(L, td0, x1, mu2, r2, P->ln2_gamma, dy, dx1, G->ln2_gamma, G->ln2_beta,
                                 G->b_fc2, G->b_o, accumulate, part, st, &jobs[0]));
-    PW_DO(order(L->ev[3], st, ax));                      // dx1 ready
     // x1 = x + o Wo^T + bo  ->  dout = dx1 Wo,  dWo = dx1^T o
-    PW_DO(do_gemm(L, gemm_args(kNT, kEpiF32, act, d, d, T, dx1, d, o, d, G->w_o, d, nullptr, nullptr, 0,
-                                     nullptr, accumulate), ax));
     // (the epilogue also takes delta = rowsum(dout * o) per token and head, which attention backward starts from)
     {
         GemmArgs g = gemm_args(kNN, kEpiRowDot, act, T, d, d, dx1, d, P->w_o, d, td0, d, nullptr, o, d, nullptr, 0, sk);
         g.row_dot = delta; g.head_dim = p.dh; g.seq_len = p.S;
         PW_DO(do_gemm(L, g, st));
     }
-    // attention backward -> dqkv (reuses the du buffer)
-    if (ax != st) {
-        cudaError_t e = cudaStreamWaitEvent(st, L->ev[2], 0);
-        if (e != cudaSuccess) return fail_cuda("stream ordering", e);
-    }
-    PW_DO(do_attn_bwd(L, qkv, nullptr, td0, lse, big, delta, st));
-    PW_DO(order(L->ev[4], st, ax));                      // dqkv ready
+    // attention backward -> dqkv
+    PW_DO(do_attn_bwd(L, qkv, nullptr, td0, lse, dqkv, delta, st));
     // qkv = h1 Wqkv^T + bqkv  ->  dh1 = dqkv Wqkv,  dWqkv = dqkv^T h1,  dbqkv = colsum(dqkv)
-    if (rederive) PW_DO(do_ln_fwd(L, x, P->ln1_gamma, P->ln1_beta, const_cast<void*>(h1), lean_st1, lean_st2, ax));
-    PW_DO(do_gemm(L, gemm_args(kNT, kEpiF32, act, 3 * d, d, T, big, 3 * d, h1, d, G->w_qkv, d, nullptr, nullptr,
-                                     0, nullptr, accumulate), ax));
-    PW_DO(do_colsum(L, big, 3 * d, G->b_qkv, accumulate, part4, ax, &jobs[3]));
-    PW_DO(do_gemm(L, gemm_args(kNN, kEpiNone, act, T, d, 3 * d, big, 3 * d, P->w_qkv, d, td0, d, nullptr,
+    PW_DO(do_gemm(L, gemm_args(kNN, kEpiNone, act, T, d, 3 * d, dqkv, 3 * d, P->w_qkv, d, td0, d, nullptr,
                                      nullptr, 0, nullptr, 0, sk), st));
     // LN1 backward + residual: dx = dx1 + LNbwd(dh1)
     PW_DO(do_ln_bwd(L, td0, x, mu1, r1, P->ln1_gamma, dx1, dx, G->ln1_gamma, G->ln1_beta, nullptr,
                                 nullptr, accumulate, part3, st, &jobs[2]));
-    PW_DO(order(L->ev[5], ax, st));                      // join
+    // From here on nothing reads what LN1 backward writes until the reduce launch: the column sums and the weight gradients
+    // start beside it and beside one another.
+    PW_DO(do_colsum(L, du, F, G->b_fc1, accumulate, part2, st, &jobs[1]));
+    PW_DO(do_colsum(L, dqkv, 3 * d, G->b_qkv, accumulate, part4, st, &jobs[3]));
+    if (rederive && !dx_over_dy) PW_DO(order(L->ev[1], ax, st));
+    PW_DO(do_wgrad(L, wj, dx_over_dy ? 3 : 4, accumulate, true, st));
     // dgamma1/2, dbeta1/2, db2, dbo, db1, dbqkv: eight vectors, one fixed-order launch
     PW_DO(do_reduce(L, jobs, 4, accumulate, st));
     return PW_OK;
@@ -626,7 +634,7 @@ pw_status_t pw_layer_create(const pw_layer_config_t* cfg, pw_layer_t** out)
         if (e == cudaSuccess) e = cudaMemset(L->whole_sync, 0, bytes);
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&L->aux, cudaStreamNonBlocking);
-    for (int i = 0; i < 6 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&L->ev[i], cudaEventDisableTiming);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&L->ev[i], cudaEventDisableTiming);
     if (e != cudaSuccess) { pw_layer_destroy(L); return fail_cuda("handle resources (status word, side stream, events)", e); }
     if (log_enabled(PW_LOG_INFO)) {
         const LayerPlan& p = L->plan;

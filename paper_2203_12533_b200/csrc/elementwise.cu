@@ -207,8 +207,8 @@ ln_bwd_kernel(const __nv_bfloat16* dh, const __nv_bfloat16* x,
     __shared__ float red[2][2][kMaxWarps];
     const int row_in_cta = threadIdx.x / tpr, tr = threadIdx.x % tpr;
     const int wpr = tpr >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    grid_dep_launch();
     grid_dep_wait();
+    grid_dep_launch();                                  // in this order: kernels that start late may follow (see launch_wgrad)
     uint64_t gm[CHUNKS][4];
     uint64_t acc_g[CHUNKS][4], acc_b[CHUNKS][4], acc_r[CHUNKS][4], acc_x[CHUNKS][4];
 #pragma unroll
@@ -393,12 +393,12 @@ reduce_partials_kernel(const __grid_constant__ ReduceTable tab, int accumulate)
 // eight rows are in flight per thread.
 constexpr int kColsumCols = 2048;
 __global__ void __launch_bounds__(256)
-colsum_kernel(const __nv_bfloat16* in, int T, int N, int ld, float* partials)
+colsum_kernel(const __nv_bfloat16* in, int T, int N, int ld, float* partials, int late)
 {
     const int col = blockIdx.x * kColsumCols + threadIdx.x * 8;
     grid_dep_launch();
-    grid_dep_wait();
-    if (col >= N) return;
+    if (!late) grid_dep_wait();
+    if (col >= N) { if (late) grid_dep_wait(); return; }
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const int R = gridDim.y;
     int t = blockIdx.y;
@@ -423,6 +423,7 @@ colsum_kernel(const __nv_bfloat16* in, int T, int N, int ld, float* partials)
     float* p = partials + static_cast<size_t>(blockIdx.y) * N + col;
     *reinterpret_cast<float4*>(p) = make_float4(acc[0], acc[1], acc[2], acc[3]);
     *reinterpret_cast<float4*>(p + 4) = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    if (late) grid_dep_wait();                          // (see launch_colsum_partial)
 }
 
 int colsum_splits(Runtime* rt, int T, int N)
@@ -581,12 +582,12 @@ size_t colsum_scratch_bytes(Runtime* rt, int T, int N)
 }
 
 const char* launch_colsum_partial(Runtime* rt, const void* in, int T, int N, int ld, void* out, void* partials,
-                                  ReduceJob* job, cudaStream_t stream)
+                                  ReduceJob* job, bool late, cudaStream_t stream)
 {
     if (T <= 0 || N <= 0 || (N % 8) || (ld % 8)) return "colsum: N and ld must be multiples of 8";
     const int R = colsum_splits(rt, T, N);
     dim3 grid((N + kColsumCols - 1) / kColsumCols, R);
-    if (launch_k(colsum_kernel, grid, dim3(256), 0, stream, static_cast<const __nv_bfloat16*>(in), T, N, ld, static_cast<float*>(partials)) != cudaSuccess)
+    if (launch_k(colsum_kernel, grid, dim3(256), 0, stream, static_cast<const __nv_bfloat16*>(in), T, N, ld, static_cast<float*>(partials), late ? 1 : 0) != cudaSuccess)
         return "colsum launch failed";
     job->partials = static_cast<const float*>(partials); job->nrows = R; job->nq = 1; job->n = N;
     job->out[0] = static_cast<float*>(out); job->out[1] = job->out[2] = job->out[3] = nullptr;
@@ -597,7 +598,7 @@ const char* launch_colsum(Runtime* rt, const void* in, int T, int N, int ld, voi
                           void* partials, cudaStream_t stream)
 {
     ReduceJob job;
-    const char* e = launch_colsum_partial(rt, in, T, N, ld, out, partials, &job, stream);
+    const char* e = launch_colsum_partial(rt, in, T, N, ld, out, partials, &job, false, stream);
     return e ? e : launch_reduce_jobs(&job, 1, accumulate, stream);
 }
 
@@ -662,7 +663,7 @@ const char* launch_colsum_noalloc(const void* in, int T, int N, int ld, void* ou
     if (R > T) R = T;
     if (R < 1) R = 1;
     dim3 grid(col_blocks, static_cast<unsigned>(R));
-    colsum_kernel<<<grid, 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(in), T, N, ld, sc.ptr);
+    colsum_kernel<<<grid, 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(in), T, N, ld, sc.ptr, 0);
     if (cudaGetLastError() != cudaSuccess) return "colsum launch failed";
     ReduceTable tab = {};
     tab.e[0].src = sc.ptr; tab.e[0].out = static_cast<float*>(out);

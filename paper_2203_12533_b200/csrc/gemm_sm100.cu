@@ -128,6 +128,35 @@ __device__ __forceinline__ void load_aux(uint4 (&aux)[4], const GemmParams& p, i
     for (int g = 0; g < 4; ++g) aux[g] = load_aux8(p, row, col0 + g * 8);
 }
 
+// fp32 outputs: TMEM -> registers -> swizzled shared slab -> TMA store or reduce-add.
+__device__ __forceinline__ void epilogue_f32(uint32_t taddr, int row0, int n0, int bn, int N, int pi, int pstride, int lane, uint8_t* slab,
+                                             uint32_t slab_u32, const CUtensorMap* tmC, int accumulate)
+{
+    uint8_t* my_row = slab + lane * 128;
+    const int nsteps = bn / 32;
+#pragma unroll 1
+    for (int s = pi; s < nsteps; s += pstride) {
+        const int col0 = n0 + s * 32;
+        if (col0 >= N) break;
+        uint32_t v[32];
+        tmem_ld32(taddr + s * 32, v);
+        tc_wait_ld();
+        if (lane == 0) bulk_wait_read0();
+        __syncwarp();
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+            *reinterpret_cast<uint4*>(my_row + ((g ^ (lane & 7)) << 4)) =
+                make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+            if (accumulate) tma_reduce_add_2d(tmC, slab_u32, col0, row0);
+            else tma_store_2d(tmC, slab_u32, col0, row0);
+            bulk_commit();
+        }
+    }
+}
+
 // Epilogue of one accumulator tile for one warp: TMEM -> registers -> swizzled shared slab -> TMA
 // store (rows >= M and columns >= N are clipped by the tensor map).  `taddr` addresses this warp's
 // lane quarter of the accumulator, row0 is the first of its 32 rows, pi selects which of the pstride
@@ -144,31 +173,8 @@ __device__ __forceinline__ void epilogue_tile(uint4 (&aux)[4], uint32_t taddr, i
                                               const float* partner = nullptr /* SPLIT: the other K half's partial sums, [chunk][1024] */)
 {
     const int row = row0 + lane;
-    uint8_t* my_row = slab + lane * 128;
     if constexpr (EPI == kEpiF32) {
-        const int nsteps = bn / 32;
-#pragma unroll 1
-        for (int s = pi; s < nsteps; s += pstride) {
-            const int col0 = n0 + s * 32;
-            if (col0 >= p.N) break;
-            uint32_t v[32];
-            tmem_ld32(taddr + s * 32, v);
-            tc_wait_ld();
-            if constexpr (SPLIT) add_partner_chunk(v, partner + s * 1024, lane);
-            if (lane == 0) bulk_wait_read0();
-            __syncwarp();
-#pragma unroll
-            for (int g = 0; g < 8; ++g)
-                *reinterpret_cast<uint4*>(my_row + ((g ^ (lane & 7)) << 4)) =
-                    make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
-            fence_proxy_async();
-            __syncwarp();
-            if (lane == 0) {
-                if (p.accumulate) tma_reduce_add_2d(tmC, slab_u32, col0, row0);
-                else tma_store_2d(tmC, slab_u32, col0, row0);
-                bulk_commit();
-            }
-        }
+        epilogue_f32(taddr, row0, n0, bn, p.N, pi, pstride, lane, slab, slab_u32, tmC, p.accumulate);
     } else {
         // 32 columns per chunk; the slab is two 2 KB halves (32 rows x 64 bytes, 64-byte
         // swizzle) used alternately, so one store is always in flight behind the math.
@@ -552,7 +558,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (!ok) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * BN_MAX;
-            if (EPI == kEpiF32 || un.slot < 0) {                 // (the fp32-output GEMMs are never cut)
+            if (un.slot < 0) {
                 epilogue_tile<EPI, NEPI == 16>(aux, taddr, m0 + q * 32, n0, bn, pi, NEPI / 4, lane, slab, slab_u32, nout, &tmC, &tmAux, p);
             } else {
                 // Half of a cut tile's K range.  Every epilogue warp leaves its part of the partial sums in
@@ -609,6 +615,159 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
 }
 
+// ------------------------------------------------------------------------------------------------
+// Weight gradients, C[M,N] (+)= A^T B with A [K,M], B [K,N] bf16 and C fp32: up to four products of the same K (the
+// tokens) in one launch of the CTA-pair kernel.  A layer's four weight gradients hang off the data-gradient chain and
+// nothing waits for them, so they make one pool of 256 x bn tiles that ends in one partly filled round instead of four: 1024
+// tokens, 1024 wide (192 tiles of 256 x 256) 42 us in four launches -> 24 us in one.  Dealing the last rounds out by k blocks, so
+// that all pairs end together (a tile then cut between two of them, the sums exchanged through L2), was slower at every size:
+// 24 -> 33 us here, 129 -> 161 us with 8192 tokens.
+struct WgradParams {
+    struct Job { int M, N, m_tiles, n_tiles, n_fastest, first; } job[kWgradMaxJobs];   // first: number of its first tile
+    int n_jobs, K, bn, accumulate, late;
+    int total;                   // tiles of all jobs
+    DeviceStatus* status;
+};
+// Tile number t of the pool -> job and the tile's place in it.
+__device__ __forceinline__ int wgrad_tile(const WgradParams& p, int t, int& mi, int& ni)
+{
+    int j = 0;
+#pragma unroll
+    for (int i = 1; i < kWgradMaxJobs; ++i) if (i < p.n_jobs && t >= p.job[i].first) j = i;
+    const WgradParams::Job& jb = p.job[j];
+    t -= jb.first;
+    mi = jb.n_fastest ? t / jb.n_tiles : t % jb.m_tiles;
+    ni = jb.n_fastest ? t % jb.n_tiles : t / jb.m_tiles;
+    return j;
+}
+struct WgradMaps { CUtensorMap a[kWgradMaxJobs], b[kWgradMaxJobs], c[kWgradMaxJobs]; };
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<kEpiF32>::kThreads, 1)
+wgrad_group_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant__ WgradParams p)
+{
+    constexpr int P_STAGES = PairCfg<kEpiF32>::kStages, NEPI = PairCfg<kEpiF32>::kEpiWarps;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* slabs = tiles + P_STAGES * P_STAGE_BYTES;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(slabs + NEPI * PairCfg<kEpiF32>::kSlab);
+    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + P_STAGES);
+    const uint32_t accf0 = smem_u32(bars + 2 * P_STAGES), acce0 = smem_u32(bars + 2 * P_STAGES + 2);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * P_STAGES + 4);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();            // 0 = leader
+    const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+    const int num_k = (p.K + BK - 1) / BK;
+    const int bn = p.bn, half_n = bn >> 1;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < P_STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 2 * NEPI); }
+        *abort_flag = 0;
+        fence_barrier_init();
+        fence_proxy_async();
+        for (int j = 0; j < p.n_jobs; ++j) { prefetch_tmap(&maps.a[j]); prefetch_tmap(&maps.b[j]); prefetch_tmap(&maps.c[j]); }
+    }
+    if (warp == 1) {
+        tmem_alloc_pair(smem_u32(tmem_slot), TMEM_COLS);
+        tmem_relinquish_pair();
+    }
+    tc_fence_before();
+    __syncthreads();
+    grid_dep_launch();
+    cluster_sync_all();                                 // both CTAs' barriers exist before anyone signals them
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    if (!p.late) grid_dep_wait();
+
+    // (the producer and the MMA role are each the loop of one elected thread: see gemm_pair_kernel)
+    if (warp == 0) {
+        if (elect_one()) {
+            uint32_t stage = 0, phase = 0;
+            bool ok = true;
+            const uint32_t pair_tx = 2u * (A_TILE_BYTES + half_n * BK * 2);
+            const uint32_t ring0 = smem_u32(tiles), full_lead = mapa_shared(full0, 0);   // the leader's barriers
+            for (int t = pair_id; t < p.total && ok; t += n_pairs) {
+                int mi, ni;
+                const int job = wgrad_tile(p, t, mi, ni);
+                const int m0 = mi * 256 + rank * 128, n0 = ni * bn + rank * half_n;
+                const CUtensorMap* tmA = &maps.a[job];
+                const CUtensorMap* tmB = &maps.b[job];
+                for (int kb = 0; kb < num_k; ++kb) {
+                    if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.status, 740)) { ok = false; break; }
+                    const uint32_t a_dst = ring0 + stage * P_STAGE_BYTES, b_dst = a_dst + A_TILE_BYTES;
+                    const uint32_t fb = full_lead + 8 * stage;
+                    if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * stage, pair_tx);
+                    tma_load_2d_pair(a_dst, tmA, m0, kb * BK, fb);
+                    tma_load_2d_pair(a_dst + 8192, tmA, m0 + 64, kb * BK, fb);
+                    tma_load_2d_pair(b_dst, tmB, n0, kb * BK, fb);
+                    if (half_n > 64) tma_load_2d_pair(b_dst + 8192, tmB, n0 + 64, kb * BK, fb);
+                    if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (rank == 0 && elect_one()) {
+            const uint32_t idesc = make_idesc_bf16(256, bn, true, true);
+            const uint64_t adesc0 = make_smem_desc_sw128(smem_u32(tiles), 8192, 1024), bdesc0 = desc_advance(adesc0, A_TILE_BYTES);
+            uint32_t stage = 0, phase = 0, it = 0;
+            bool ok = true;
+            for (int t = pair_id; t < p.total && ok; t += n_pairs, ++it) {
+                const uint32_t buf = it & 1, acc_phase = (it >> 1) & 1;
+                if (!mbar_wait(acce0 + 8 * buf, acc_phase ^ 1, abort_flag, p.status, 750)) break;
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + buf * BN_MAX;
+                for (int kb = 0; kb < num_k; ++kb) {
+                    if (!mbar_wait(full0 + 8 * stage, phase, abort_flag, p.status, 751)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint64_t ad = desc_advance(adesc0, stage * P_STAGE_BYTES), bd = desc_advance(bdesc0, stage * P_STAGE_BYTES);
+#pragma unroll
+                    for (int kk = 0; kk < BK / UMMA_K; ++kk)
+                        umma_f16_pair(d_tmem, desc_advance(ad, kk * 2048), desc_advance(bd, kk * 2048), idesc, (kb | kk) != 0 ? 1u : 0u);
+                    umma_commit_pair(empty0 + 8 * stage, 3);     // frees the stage in both CTAs
+                    if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+                }
+                if (ok) umma_commit_pair(accf0 + 8 * buf, 3);     // both CTAs' accumulators complete
+            }
+        }
+    } else {
+        const int q = warp & 3, pi = (warp - 2) >> 2;
+        uint8_t* slab = slabs + (warp - 2) * PairCfg<kEpiF32>::kSlab;
+        const uint32_t slab_u32 = smem_u32(slab);
+        uint32_t it = 0;
+        for (int t = pair_id; t < p.total; t += n_pairs, ++it) {
+            int mi, ni;
+            const int job = wgrad_tile(p, t, mi, ni);
+            const uint32_t buf = it & 1, acc_phase = (it >> 1) & 1;
+            bool ok = mbar_wait(accf0 + 8 * buf, acc_phase, abort_flag, p.status, 760);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * BN_MAX;
+            epilogue_f32(taddr, mi * 256 + rank * 128 + q * 32, ni * bn, bn, p.job[job].N, pi, NEPI / 4, lane, slab, slab_u32, &maps.c[job], p.accumulate);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(mapa_shared(acce0 + 8 * buf, 0));
+        }
+        if (lane == 0) bulk_wait0();
+    }
+
+    __syncwarp();
+    if (*abort_flag) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < (1ll << 22)) {}
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                                 // neither CTA releases TMEM or exits while its peer may still touch it
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, TMEM_COLS);
+    }
+    if (p.late) grid_dep_wait();
+}
+
 template <bool A_MN, bool B_MN, int EPI>
 const char* launch_inst(Runtime* rt, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmBh,
                         const CUtensorMap& tmC, const CUtensorMap& tmAux, const GemmParams& p, cudaStream_t stream)
@@ -635,10 +794,11 @@ const char* launch_pair(Runtime* rt, const CUtensorMap& tmA, const CUtensorMap& 
 template <bool A_MN, bool B_MN, int EPI>
 bool set_attr()
 {
-    return cudaFuncSetAttribute(gemm_kernel<A_MN, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                SMEM_BYTES) == cudaSuccess &&
-           cudaFuncSetAttribute(gemm_pair_kernel<A_MN, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                PairCfg<EPI>::kSmem) == cudaSuccess;
+    if (cudaFuncSetAttribute(gemm_kernel<A_MN, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess) return false;
+    if constexpr (EPI == kEpiF32)
+        return cudaFuncSetAttribute(wgrad_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<EPI>::kSmem) == cudaSuccess;
+    else
+        return cudaFuncSetAttribute(gemm_pair_kernel<A_MN, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<EPI>::kSmem) == cudaSuccess;
 }
 
 }  // namespace
@@ -656,8 +816,8 @@ const char* configure_gemm()
 
 static const char* launch_gemm_pair(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cudaStream_t stream)
 {
-    const bool a_mn = a.layout == kNT, b_mn = a.layout == kNN || a.layout == kNT;
-    const bool f32_out = a.epilogue == kEpiF32;
+    const bool a_mn = false, b_mn = a.layout == kNN;             // (weight gradients: launch_wgrad)
+    const bool f32_out = false;
     const int m_tiles = (a.M + 255) / 256, pairs = rt->sm_count / 2;
     // Tile width: 256 unless the rounds it needs waste more than a 128-wide tiling does (a
     // 128-wide pair tile moves as many operand bytes per FLOP as the one-CTA 256-wide tile).
@@ -719,7 +879,6 @@ static const char* launch_gemm_pair(Runtime* rt, const GemmArgs& a, DeviceStatus
         case kNN * 16 + kEpiNone: return launch_pair<false, true, kEpiNone>(rt, tmA, tmB, tmC, tmAux, p, stream);
         case kNN * 16 + kEpiDGelu: return launch_pair<false, true, kEpiDGelu>(rt, tmA, tmB, tmC, tmAux, p, stream);
         case kNN * 16 + kEpiRowDot: return launch_pair<false, true, kEpiRowDot>(rt, tmA, tmB, tmC, tmAux, p, stream);
-        case kNT * 16 + kEpiF32: return launch_pair<true, true, kEpiF32>(rt, tmA, tmB, tmC, tmAux, p, stream);
         default: return "gemm: unsupported layout/epilogue combination";
     }
 }
@@ -760,6 +919,47 @@ static bool plan_cluster(const GemmArgs& a, int sms, GemmClusterPlan* plan)
 // Scratch for the K halves of cut tiles: (cut tile, half, CTA of the pair) x 128 rows x 256 columns, fp32.
 size_t gemm_split_ws_bytes() { return static_cast<size_t>(kSplitMaxTiles) * 2 * 2 * 128 * BN_MAX * sizeof(float); }
 
+const char* launch_wgrad(Runtime* rt, const WgradJob* jobs, int n_jobs, int K, int accumulate, bool late, DeviceStatus* status,
+                         cudaStream_t stream)
+{
+    if (n_jobs < 1 || n_jobs > kWgradMaxJobs || K <= 0 || (K % 8)) return "weight gradients: bad job count or K";
+    auto misaligned = [](const void* q) { return q == nullptr || (reinterpret_cast<uintptr_t>(q) & 15) != 0; };
+    for (int j = 0; j < n_jobs; ++j) {
+        const WgradJob& w = jobs[j];
+        if (w.M <= 0 || w.N <= 0 || (w.M % 8) || (w.N % 8) || (w.lda % 8) || (w.ldb % 8) || (w.ldc % 4)) return "weight gradients: bad dimension";
+        if (misaligned(w.A) || misaligned(w.B) || misaligned(w.C)) return "weight gradients: null or misaligned operand";
+    }
+    const int pairs = rt->sm_count / 2;
+    auto rounds = [&](int bn) {
+        long long t = 0;
+        for (int j = 0; j < n_jobs; ++j) t += static_cast<long long>((jobs[j].M + 255) / 256) * ((jobs[j].N + bn - 1) / bn);
+        return static_cast<double>((t + pairs - 1) / pairs);
+    };
+    int bn = rounds(128) * 0.575 < rounds(256) ? 128 : 256;      // (see launch_gemm_pair for the width's price)
+    const int forced = tuning().gemm_bn;
+    if (forced == 128 || forced == 256) bn = forced;
+    WgradMaps maps;
+    WgradParams p;
+    p.n_jobs = n_jobs; p.K = K; p.bn = bn; p.accumulate = accumulate; p.late = late ? 1 : 0;
+    p.status = status;
+    const char* e;
+    int first = 0;
+    for (int j = 0; j < n_jobs; ++j) {
+        const WgradJob& w = jobs[j];
+        if ((e = encode_2d(rt, &maps.a[j], w.A, w.M, K, w.lda, 64, BK))) return e;
+        if ((e = encode_2d(rt, &maps.b[j], w.B, w.N, K, w.ldb, 64, BK))) return e;
+        if ((e = encode_2d(rt, &maps.c[j], w.C, w.N, w.M, w.ldc, 32, 32, true))) return e;
+        const int mt = (w.M + 255) / 256, nt = (w.N + bn - 1) / bn;
+        p.job[j] = {w.M, w.N, mt, nt, nt < mt ? 1 : 0, first};
+        first += mt * nt;
+    }
+    for (int j = n_jobs; j < kWgradMaxJobs; ++j) { p.job[j] = p.job[0]; maps.a[j] = maps.a[0]; maps.b[j] = maps.b[0]; maps.c[j] = maps.c[0]; }
+    p.total = first;
+    const int used = first < pairs ? first : pairs;
+    return launch_k(wgrad_group_kernel, dim3(2 * used), dim3(PairCfg<kEpiF32>::kThreads), PairCfg<kEpiF32>::kSmem, stream, maps, p) == cudaSuccess
+               ? nullptr : "weight-gradient launch failed";
+}
+
 const char* launch_gemm(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cudaStream_t stream)
 {
     if (a.M <= 0 || a.N <= 0 || a.K <= 0) return "gemm: non-positive dimension";
@@ -784,7 +984,11 @@ const char* launch_gemm(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cu
         if (f32_out && (a.ldc % 4)) return "gemm: fp32 ldc must be a multiple of 4";
         return launch_gemm_cluster(rt, a, plan, status, stream);
     }
-    if (pair_mode && a.M >= 256) return launch_gemm_pair(rt, a, status, stream);
+    if (pair_mode && a.M >= 256) {
+        if (!f32_out) return launch_gemm_pair(rt, a, status, stream);
+        const WgradJob w = {a.M, a.N, a.A, a.lda, a.B, a.ldb, a.C, a.ldc};
+        return launch_wgrad(rt, &w, 1, a.K, a.accumulate, false, status, stream);
+    }
     if (f32_out && (a.ldc % 4)) return "gemm: fp32 ldc must be a multiple of 4";
     // Tile width: the one that needs the least (rounds x width) on this many SMs; ties go to the
     // wider tile (less operand traffic per FLOP).

@@ -112,6 +112,13 @@ constexpr size_t kGemmClusterMinSmem = 80 * 1024;
 const char* configure_gemm_cluster();
 const char* launch_gemm_cluster(Runtime* rt, const GemmArgs& a, const GemmClusterPlan& plan, DeviceStatus* status, cudaStream_t stream);
 
+// C[M,N] (+)= A^T B, fp32, A [K,M], B [K,N] bf16: up to kWgradMaxJobs products of one K in one launch.  late: the kernel
+// starts without waiting for the one in front of it, which must have let it start only after its own wait (its end
+// still comes after that one's).
+constexpr int kWgradMaxJobs = 4;
+struct WgradJob { int M, N; const void* A; int lda; const void* B; int ldb; void* C; int ldc; };
+const char* launch_wgrad(Runtime* rt, const WgradJob* jobs, int n_jobs, int K, int accumulate, bool late, DeviceStatus* status, cudaStream_t stream);
+
 // Encodes the two tensor maps and launches.  Returns nullptr on success, else a static message.
 const char* launch_gemm(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cudaStream_t stream);
 
@@ -140,8 +147,9 @@ const char* launch_layernorm_bwd_partial(Runtime* rt, const void* dh, const void
                                          const void* gamma, const void* resid, int T, int d, void* dx, void* dgamma,
                                          void* dbeta, void* db_resid, void* db_dx, void* partials, ReduceJob* job,
                                          cudaStream_t stream);
+// late: as for launch_wgrad.
 const char* launch_colsum_partial(Runtime* rt, const void* in, int T, int N, int ld, void* out, void* partials,
-                                  ReduceJob* job, cudaStream_t stream);
+                                  ReduceJob* job, bool late, cudaStream_t stream);
 const char* launch_reduce_jobs(const ReduceJob* jobs, int njobs, int accumulate, cudaStream_t stream);
 
 // Column sums with the partial sums in a fixed device array inside the library (no allocation, no Runtime).
