@@ -176,8 +176,8 @@ bool plan_warp_rows(int d, int* W, int* CH)
 }
 
 // LayerNorm backward.  Persistent over rows; every thread keeps the column sums of its own
-// columns in registers and writes them once at the end as one partial row per (CTA, row slot):
-// partials[(cta*rows_per_cta + row_in_cta)][4][d] = {dgamma, dbeta, sum resid, sum dx}.
+// columns in registers; they leave at the end as one partial row per CTA:
+// partials[cta][4][d] = {dgamma, dbeta, sum resid, sum dx} (its row slots' sums added in slot order).
 // The next row's three inputs are fetched before the current row's reduction, and the two row
 // sums share one barrier.
 // rows in the prefetch ring (six were measured slower than four at every width)
@@ -323,7 +323,32 @@ ln_bwd_kernel(const __nv_bfloat16* dh, const __nv_bfloat16* x,
         }
     }
     constexpr int NQ = BIAS_SUMS ? 4 : 2;
-    float* prow = partials + static_cast<size_t>(blockIdx.x * rows_per_cta + row_in_cta) * NQ * d;
+    float* prow = partials + static_cast<size_t>(blockIdx.x) * NQ * d;
+    if (rows_per_cta > 1) {                             // narrow rows (one piece per thread): the CTA's row slots add up first
+        float* sums = reinterpret_cast<float*>(ln_bwd_ring);             // [slot][NQ][d], at most 8 K floats; the ring is idle
+        cp_async_wait<0>();
+        __syncthreads();
+        float* mine = sums + (row_in_cta * NQ) * d + 8 * tr;
+#pragma unroll
+        for (int k = 0; k < 4; k += 2) {
+            *reinterpret_cast<ulonglong2*>(mine + 2 * k) = make_ulonglong2(acc_g[0][k], acc_g[0][k + 1]);
+            *reinterpret_cast<ulonglong2*>(mine + d + 2 * k) = make_ulonglong2(acc_b[0][k], acc_b[0][k + 1]);
+            if (BIAS_SUMS) {
+                *reinterpret_cast<ulonglong2*>(mine + 2 * d + 2 * k) = make_ulonglong2(acc_r[0][k], acc_r[0][k + 1]);
+                *reinterpret_cast<ulonglong2*>(mine + 3 * d + 2 * k) = make_ulonglong2(acc_x[0][k], acc_x[0][k + 1]);
+            }
+        }
+        __syncthreads();
+        for (int c = 4 * threadIdx.x; c < NQ * d; c += 4 * blockDim.x) {
+            float4 s = *reinterpret_cast<const float4*>(sums + c);
+            for (int r = 1; r < rows_per_cta; ++r) {
+                const float4 v = *reinterpret_cast<const float4*>(sums + r * NQ * d + c);
+                s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+            }
+            *reinterpret_cast<float4*>(prow + c) = s;
+        }
+        return;
+    }
 #pragma unroll
     for (int j = 0; j < CHUNKS; ++j) {
         const int col = 8 * (tr + j * tpr);
@@ -389,57 +414,75 @@ reduce_partials_kernel(const __grid_constant__ ReduceTable tab, int accumulate)
     }
 }
 
-// Column sums of a bf16 [T, N] matrix: CTA (x, y) owns columns 2048*x .. +2047 and rows y, y+R, ...;
-// eight rows are in flight per thread.
-constexpr int kColsumCols = 2048;
+// Column sums of a bf16 [T, N] matrix: CTA (x, y) owns columns 256 x .. +255 and, eight rows at a time (one per warp), rows
+// 8 y + w, 8 (y + R) + w, ...; four rows are in flight per thread.  The eight warps' sums meet in shared memory in warp
+// order, so a CTA leaves one partial row whatever its share of the rows.
+constexpr int kColsumCols = 256;
 __global__ void __launch_bounds__(256)
 colsum_kernel(const __nv_bfloat16* in, int T, int N, int ld, float* partials, int late)
 {
-    const int col = blockIdx.x * kColsumCols + threadIdx.x * 8;
+    __shared__ float4 sm[kMaxWarps][2][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int col = blockIdx.x * kColsumCols + lane * 8;
     grid_dep_launch();
     if (!late) grid_dep_wait();
-    if (col >= N) { if (late) grid_dep_wait(); return; }
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    const int R = gridDim.y;
-    int t = blockIdx.y;
-    for (; t + 7 * R < T; t += 8 * R) {
-        uint4 v[8];
+    if (col < N) {
+        const int step = 8 * gridDim.y;
+        int t = 8 * blockIdx.y + warp;
+        for (; t + 3 * step < T; t += 4 * step) {
+            uint4 v[4];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = *reinterpret_cast<const uint4*>(in + static_cast<size_t>(t + u * R) * ld + col);
+            for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(in + static_cast<size_t>(t + u * step) * ld + col);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < 4; ++u) {
+                float f[8];
+                unpack8(v[u], f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) acc[k] += f[k];
+            }
+        }
+        for (; t < T; t += step) {
             float f[8];
-            unpack8(v[u], f);
+            unpack8(*reinterpret_cast<const uint4*>(in + static_cast<size_t>(t) * ld + col), f);
 #pragma unroll
             for (int k = 0; k < 8; ++k) acc[k] += f[k];
         }
     }
-    for (; t < T; t += R) {
-        float f[8];
-        unpack8(*reinterpret_cast<const uint4*>(in + static_cast<size_t>(t) * ld + col), f);
+    sm[warp][0][lane] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    sm[warp][1][lane] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    __syncthreads();
+    if (warp < 2 && col < N) {
+        float4 s = sm[0][warp][lane];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] += f[k];
+        for (int w = 1; w < kMaxWarps; ++w) {
+            const float4 v = sm[w][warp][lane];
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        *reinterpret_cast<float4*>(partials + static_cast<size_t>(blockIdx.y) * N + col + 4 * warp) = s;
     }
-    float* p = partials + static_cast<size_t>(blockIdx.y) * N + col;
-    *reinterpret_cast<float4*>(p) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    *reinterpret_cast<float4*>(p + 4) = make_float4(acc[4], acc[5], acc[6], acc[7]);
     if (late) grid_dep_wait();                          // (see launch_colsum_partial)
 }
 
-int colsum_splits(Runtime* rt, int T, int N)
+// Partial rows: about four CTAs per SM, but at least 32 rows of the matrix for each, so that on few tokens the
+// partial rows stay a small part of what they summarise: 1024 x 2048 8.1 -> 3.7 us with the reduce launch, 1024 x 4096
+// 6.6 -> 3.8, 8192 x 4096 15.6 -> 14.5 (against one warp-wide row per thread column and up to T partial rows).
+int colsum_splits(int sm_count, int T, int N)
 {
     const int col_blocks = (N + kColsumCols - 1) / kColsumCols;
-    int r = (4 * rt->sm_count + col_blocks - 1) / col_blocks;
-    if (r > T) r = T;
-    if (r < 1) r = 1;
+    int r = (4 * sm_count + col_blocks - 1) / col_blocks;
+    if (r > (T + 31) / 32) r = (T + 31) / 32;
     return r;
 }
 
+// A row slot takes at least four rows: on few tokens the partial rows, one per CTA, then stay a small part of the input.
+// (With one partial row per slot and a CTA for every group of rows, 1024 tokens x 512 left as many partial rows as there are
+// tokens: 11.8 us with the reduce launch, 5.5 now; 1024 x 1024 10.9 -> 7.5, 16384 x 1024 35.3 -> 32.1.)
 int ln_bwd_grid(Runtime* rt, int T, const RowPlan& rp)
 {
     const int row_groups = (T + rp.rows_per_cta - 1) / rp.rows_per_cta;
-    const int cap = (rp.chunks == 1 ? 2 : 1) * rt->sm_count;
-    return row_groups < cap ? row_groups : cap;
+    const int cap = (rp.chunks == 1 ? 2 : 1) * rt->sm_count, want = (row_groups + 3) / 4;
+    return want < cap ? want : cap;
 }
 
 }  // namespace
@@ -481,7 +524,7 @@ size_t layernorm_bwd_scratch_bytes(Runtime* rt, int T, int d)
 {
     RowPlan rp;
     if (T <= 0 || !plan_rows(d, &rp)) return 0;
-    return static_cast<size_t>(ln_bwd_grid(rt, T, rp)) * rp.rows_per_cta * 4 * d * sizeof(float);
+    return static_cast<size_t>(ln_bwd_grid(rt, T, rp)) * 4 * d * sizeof(float);
 }
 
 // Main kernel only: the partial rows stay in `partials` and `job` says how to reduce them.
@@ -512,7 +555,7 @@ const char* launch_layernorm_bwd_partial(Runtime* rt, const void* dh, const void
     }
 #undef PW_LN_BWD
     if (le != cudaSuccess) return "layernorm bwd launch failed";
-    job->partials = P; job->nrows = grid * rp.rows_per_cta; job->nq = sums ? 4 : 2; job->n = d;
+    job->partials = P; job->nrows = grid; job->nq = sums ? 4 : 2; job->n = d;
     job->out[0] = static_cast<float*>(dgamma); job->out[1] = static_cast<float*>(dbeta);
     job->out[2] = static_cast<float*>(db_resid); job->out[3] = static_cast<float*>(db_dx);
     return nullptr;
@@ -578,14 +621,14 @@ const char* launch_gelu_fwd(Runtime* rt, const void* u, void* a, long long n, in
 size_t colsum_scratch_bytes(Runtime* rt, int T, int N)
 {
     if (T <= 0 || N <= 0) return 0;
-    return static_cast<size_t>(colsum_splits(rt, T, N)) * N * sizeof(float);
+    return static_cast<size_t>(colsum_splits(rt->sm_count, T, N)) * N * sizeof(float);
 }
 
 const char* launch_colsum_partial(Runtime* rt, const void* in, int T, int N, int ld, void* out, void* partials,
                                   ReduceJob* job, bool late, cudaStream_t stream)
 {
     if (T <= 0 || N <= 0 || (N % 8) || (ld % 8)) return "colsum: N and ld must be multiples of 8";
-    const int R = colsum_splits(rt, T, N);
+    const int R = colsum_splits(rt->sm_count, T, N);
     dim3 grid((N + kColsumCols - 1) / kColsumCols, R);
     if (launch_k(colsum_kernel, grid, dim3(256), 0, stream, static_cast<const __nv_bfloat16*>(in), T, N, ld, static_cast<float*>(partials), late ? 1 : 0) != cudaSuccess)
         return "colsum launch failed";
@@ -657,11 +700,9 @@ const char* launch_colsum_noalloc(const void* in, int T, int N, int ld, void* ou
     *err_kind = kErrCuda;
     // as many row groups as the fixed scratch can hold, at most what the allocating variant uses
     const int col_blocks = (N + kColsumCols - 1) / kColsumCols;
-    long long R = (4ll * sc.sm_count + col_blocks - 1) / col_blocks;
+    long long R = colsum_splits(sc.sm_count, T, N);
     const long long fit = static_cast<long long>(kStaticScratchFloats / static_cast<size_t>(N));
     if (R > fit) R = fit;
-    if (R > T) R = T;
-    if (R < 1) R = 1;
     dim3 grid(col_blocks, static_cast<unsigned>(R));
     colsum_kernel<<<grid, 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(in), T, N, ld, sc.ptr, 0);
     if (cudaGetLastError() != cudaSuccess) return "colsum launch failed";
