@@ -480,7 +480,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (elect_one()) {
             uint32_t stage = 0, phase = 0;
             bool ok = true;
-            const uint32_t pair_tx = 2u * (A_TILE_BYTES + half_n * BK * 2);
+            const uint32_t pair_tx = 2u * (A_TILE_BYTES + (B_MN ? (half_n + 63) / 64 * 8192 : half_n * BK * 2));   // MN-major: whole 64-column boxes
             const uint32_t ring0 = smem_u32(tiles), full_lead = mapa_shared(full0, 0);   // the leader's barriers
             for (int unit = pair_id; unit < total_tiles && ok; unit += n_pairs) {
                 const PairUnit un = pair_unit(p, unit, num_k);
@@ -686,7 +686,7 @@ wgrad_group_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant
         if (elect_one()) {
             uint32_t stage = 0, phase = 0;
             bool ok = true;
-            const uint32_t pair_tx = 2u * (A_TILE_BYTES + half_n * BK * 2);
+            const uint32_t pair_tx = 2u * (A_TILE_BYTES + (half_n + 63) / 64 * 8192);
             const uint32_t ring0 = smem_u32(tiles), full_lead = mapa_shared(full0, 0);   // the leader's barriers
             for (int t = pair_id; t < p.total && ok; t += n_pairs) {
                 int mi, ni;
@@ -814,24 +814,36 @@ const char* configure_gemm()
     return ok ? nullptr : "cudaFuncSetAttribute(gemm) failed";
 }
 
+// Tile width of the pair kernels: the one whose rounds are cheapest.  Narrower tiles move more operand bytes per FLOP: a
+// 128-wide one takes 1.15x, a 192-wide one 1.08x as long (2048 x 2048 x 8192: 58.1 us in two rounds of 128, 50.9 in one of
+// 256; 8192 x 6144 x 2048 142 us in 14 rounds of 192, 134 in 11 of 256), but fill the last round better: 1024 x 3072 x 1024
+// 10.0 us with 192 against 10.7 / 11.6 with 128 / 256, 1920 x 1280 x 3456 (dgrad) 17.0 against 21.6 / 21.6,
+// 1920 x 3456 x 1280 + GeLU 18.2 against 20.0 / 20.6.
+static double pair_cost(long long tiles, int width, int pairs)
+{
+    return static_cast<double>((tiles + pairs - 1) / pairs) * width * (width == 128 ? 1.15 : width == 192 ? 1.08 : 1.0);
+}
+static int pair_tile_width(int m_tiles, int N, int pairs)
+{
+    int best = 256;
+    double cost = pair_cost(static_cast<long long>(m_tiles) * ((N + 255) / 256), 256, pairs);
+    for (int w : {192, 128}) {
+        const double c = pair_cost(static_cast<long long>(m_tiles) * ((N + w - 1) / w), w, pairs);
+        if (c < cost) { cost = c; best = w; }
+    }
+    return best;
+}
+
 static const char* launch_gemm_pair(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cudaStream_t stream)
 {
     const bool a_mn = false, b_mn = a.layout == kNN;             // (weight gradients: launch_wgrad)
     const bool f32_out = false;
     const int m_tiles = (a.M + 255) / 256, pairs = rt->sm_count / 2;
-    // Tile width: 256 unless the rounds it needs waste more than a 128-wide tiling does (a
-    // 128-wide pair tile moves as many operand bytes per FLOP as the one-CTA 256-wide tile).
-    int bn = 256;
+    int bn;
     {
         const int forced = tuning().gemm_bn;
-        auto cost = [&](int w) {
-            const long long tiles = static_cast<long long>(m_tiles) * ((a.N + w - 1) / w);
-            const long long rounds = (tiles + pairs - 1) / pairs;
-            // a 128-wide pair tile takes 1.14x as long per FLOP (2048 x 2048 x 8192: 58.1 us in two rounds against 50.9 in one)
-            return static_cast<double>(rounds) * w * (w == 128 ? 1.15 : 1.0);
-        };
-        if (cost(128) < cost(256)) bn = 128;
-        if (forced == 128 || forced == 256) bn = forced;
+        bn = pair_tile_width(m_tiles, a.N, pairs);
+        if (forced == 128 || forced == 192 || forced == 256) bn = forced;
         if (a.epilogue == kEpiRowDot) bn = 256;              // an epilogue warp must own whole heads (128 columns)
     }
     CUtensorMap tmA, tmB, tmC, tmAux;
@@ -892,7 +904,7 @@ static const char* launch_gemm_pair(Runtime* rt, const GemmArgs& a, DeviceStatus
 //                                 512 x 512 x 1024 weight gradient 6.7 -> 5.7 (2)
 //   256 x 128 tiles cut in two    1024 x 1024 x 4096 + residual 16.8 -> 12.1, dgrad 15.0 -> 12.6
 //   one 128 x 128 tile per SM     2048 x 1024 x 1024 + residual 9.7 -> 8.3, row dots 12.8 -> 11.3; 2048 x 1024 x 4096 + residual 18.1 -> 16.6
-//   two 256 x 128 tiles per pair  1920 x 1280 x 1280 + residual 13.5 -> 12.5, 2048 x 2048 x 2048 + residual 18.4 -> 16.7
+//   two 256 x 128 tiles per pair  2048 x 2048 x 2048 + residual 18.4 -> 16.7
 // Where the pair kernel stays the faster one: weight gradients with more than 74 tiles (1024 x 1024 x 1024 7.3 against
 // 7.6: MN-major operands need twice the copies and the fp32 tile leaves through registers), plain dgrads with
 // t64 > 148 (2048 x 1024 x 4096 15.4 against 17.4), and everything whose tiles fill the chip more than once.
@@ -912,7 +924,8 @@ static bool plan_cluster(const GemmArgs& a, int sms, GemmClusterPlan* plan)
     if (may_cut && a.M > 128 && 2 * t128 <= sms && kb > (wgrad ? 32 : 16)) { *plan = {1, 128, 2, 8}; return true; }
     if (wgrad || plain_dgrad) return false;
     if (t128 <= sms) { *plan = kb > 16 && a.M > 128 ? GemmClusterPlan{1, 128, 1, 8} : GemmClusterPlan{0, 128, 1, 6}; return true; }
-    if (t128 <= 2 * sms && a.epilogue == kEpiBiasResid && kb <= 64 && a.M > 128) { *plan = {1, 128, 1, 4}; return true; }
+    const bool one_round = static_cast<long long>((a.M + 255) / 256) * ((a.N + 191) / 192) <= sms / 2;     // of the pair kernel, 192 wide
+    if (t128 <= 2 * sms && !one_round && a.epilogue == kEpiBiasResid && kb <= 64 && a.M > 128) { *plan = {1, 128, 1, 4}; return true; }
     return false;
 }
 
@@ -930,14 +943,15 @@ const char* launch_wgrad(Runtime* rt, const WgradJob* jobs, int n_jobs, int K, i
         if (misaligned(w.A) || misaligned(w.B) || misaligned(w.C)) return "weight gradients: null or misaligned operand";
     }
     const int pairs = rt->sm_count / 2;
-    auto rounds = [&](int bn) {
+    auto cost = [&](int bn) {
         long long t = 0;
         for (int j = 0; j < n_jobs; ++j) t += static_cast<long long>((jobs[j].M + 255) / 256) * ((jobs[j].N + bn - 1) / bn);
-        return static_cast<double>((t + pairs - 1) / pairs);
+        return pair_cost(t, bn, pairs);
     };
-    int bn = rounds(128) * 0.575 < rounds(256) ? 128 : 256;      // (see launch_gemm_pair for the width's price)
+    int bn = 256;
+    for (int w : {192, 128}) if (cost(w) < cost(bn)) bn = w;
     const int forced = tuning().gemm_bn;
-    if (forced == 128 || forced == 256) bn = forced;
+    if (forced == 128 || forced == 192 || forced == 256) bn = forced;
     WgradMaps maps;
     WgradParams p;
     p.n_jobs = n_jobs; p.K = K; p.bn = bn; p.accumulate = accumulate; p.late = late ? 1 : 0;

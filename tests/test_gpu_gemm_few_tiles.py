@@ -25,7 +25,8 @@ SIZES = [(8, 8, 8), (128, 64, 64), (264, 256, 768), (200, 328, 1544), (1024, 512
          (1024, 1152, 2056),     # 72 tiles of 128 x 128, cut in two
          (512, 4736, 520),       # 148 tiles of 128 x 128
          (1016, 4728, 1096),     # two per SM, ragged edges
-         (1024, 4864, 512)]      # more than two per SM: the persistent kernel
+         (1024, 4864, 512),      # more than two per SM: the persistent kernel
+         (1016, 3072, 1096), (1920, 3464, 1288)]     # its 192-wide tiles: one round, a ragged second one
 
 
 @pytest.mark.parametrize("M,N,K", SIZES)
