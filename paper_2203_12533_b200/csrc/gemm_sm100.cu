@@ -1,9 +1,5 @@
-// bf16 GEMM for sm_100a: TMA -> 4-stage shared-memory ring -> tcgen05.mma (fp32 accumulators in
-// TMEM, double buffered) -> epilogue warps (tcgen05.ld -> bias / GeLU / residual -> global).
-//
-// One persistent CTA per SM, 6 warps: warp 0 = TMA producer (one lane), warp 1 = MMA issuer (one
-// lane; the warp also owns the TMEM allocation), warps 2..5 = epilogue (warp w reads TMEM lanes
-// 32*(w%4) .. +31, i.e. 32 rows of the 128-row tile each).  Output tile 128 x 256, K step 64.
+// bf16 GEMM for sm_100a on CTA pairs: TMA -> shared-memory ring -> tcgen05.mma (fp32 accumulators in TMEM, double
+// buffered) -> epilogue warps (tcgen05.ld -> bias / GeLU / residual -> swizzled shared slab -> TMA store).
 //
 // Operand layouts are handled without physical transposes: an operand whose contraction index
 // is contiguous in memory ("K-major") is loaded as [rows][64 k] boxes, one whose row index is
@@ -12,90 +8,39 @@
 //
 // Every wait on an mbarrier is bounded (see mbar_wait); on expiry the CTA raises an abort flag,
 // all roles leave their loops, the TMEM allocation is released and the kernel returns.
-#include <cstdlib>
-
 #include "gemm_epilogue.cuh"
 
 namespace pw {
 namespace {
 
-constexpr int BM = 128, BN_MAX = 256, BK = 64, STAGES = 4, UMMA_K = 16;
+constexpr int BM = 128, BN_MAX = 256, BK = 64, UMMA_K = 16;
 constexpr int A_TILE_BYTES = BM * BK * 2;       // 16 KB
-constexpr int B_TILE_BYTES = BN_MAX * BK * 2;   // 32 KB (a narrower tile uses the front of it)
-constexpr int STAGE_BYTES = A_TILE_BYTES + B_TILE_BYTES;
-constexpr int EPI_WARPS = 8;
-constexpr int GEMM_THREADS = 64 + 32 * EPI_WARPS;   // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
 constexpr int TMEM_COLS = 2 * BN_MAX;           // two accumulators: the whole 512-column TMEM
-constexpr int SLAB_BYTES = 4096;                // per epilogue warp: 32 rows x 128 bytes, swizzled
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_WARPS * SLAB_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
 
 struct GemmParams {
     int M, N, K;
     int bn;                      // tile width actually used: 128, 192 or 256
     const __nv_bfloat16* bias;
-    const __nv_bfloat16* aux_in; int ld_aux;
-    int accumulate, act;
+    int act;
     int m_tiles, n_tiles;
     int n_fastest;               // tile numbering: 1 = consecutive tiles share the A row panel, 0 = the B panel
-    int split_begin;             // tiles >= split_begin are issued as two units (tail balancing): half-width
-                                 // tiles in the one-CTA kernel, halves of the K range in the CTA-pair kernel
+    int split_begin;             // tiles >= split_begin are issued as two halves of the K range (tail balancing)
     int total_virtual;           // split_begin + 2 * (m_tiles*n_tiles - split_begin)
-    float* split_ws;             // CTA-pair kernel: where the K halves leave their partial sums
+    float* split_ws;             // where the K halves leave their partial sums
     float* row_dot; int head_dim, seq_len;   // kEpiRowDot: per (row, head) dot products with aux_in, [B, H, S]
     DeviceStatus* status;
 };
 
-// Virtual tile v -> (m0, n0, width).  Tiles that run at the same time should touch as few distinct
-// operand panels as possible (they have to sit in L2 together), so the numbering runs fastest along
-// the dimension with fewer tiles.  The tiles of the last,
-// partly filled round are cut in two half-width tiles so that every SM gets one.
-__device__ __forceinline__ void tile_info(const GemmParams& p, int v, int& m0, int& n0, int& bn)
-{
-    int t = v, half = 0;
-    bn = p.bn;
-    if (v >= p.split_begin) {
-        const int hv = v - p.split_begin;
-        t = p.split_begin + (hv >> 1);
-        half = hv & 1;
-        bn = p.bn >> 1;
-    }
-    const int mi = p.n_fastest ? t / p.n_tiles : t % p.m_tiles;
-    const int ni = p.n_fastest ? t % p.n_tiles : t / p.m_tiles;
-    m0 = mi * BM;
-    n0 = ni * p.bn + half * (p.bn >> 1);
-}
-
-// One 8-column group of the bf16 epilogues: f = acc (+bias) (+residual | x GeLU'(u)).  `aux` holds the
-// group's 8 residual / pre-activation values, fetched by the caller ahead of the TMEM load.
-template <int EPI>
-__device__ __forceinline__ void epilogue_group(const uint32_t* v, int row, int c, const GemmParams& p, const uint4& aux, float* f)
-{
-#pragma unroll
-    for (int j = 0; j < 8; ++j) f[j] = __uint_as_float(v[j]);
-    if (c < p.N) {
-        if constexpr (EPI == kEpiBias || EPI == kEpiBiasResid || EPI == kEpiBiasGelu) {
-            float b[8];
-            unpack8(*(reinterpret_cast<const uint4*>(p.bias + c)), b);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) f[j] += b[j];
-        }
-        if constexpr (EPI == kEpiBiasResid) {
-            if (row < p.M) {
-                float r[8];
-                unpack8(aux, r);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) f[j] += r[j];
-            }
-        }
-        if constexpr (EPI == kEpiDGelu) {
-            if (row < p.M) {
-                float u[8];
-                unpack8(aux, u);
-                gelu_grad_mul8(f, u, p.act);
-            }
-        }
-    }
-}
+// ------------------------------------------------------------------------------------------------
+// CTA pairs (cta_group::2): a cluster of two CTAs computes one 256 x bn tile.  CTA r of the
+// pair loads its own 128 rows of A and its own half (bn/2 rows) of B - with plain per-CTA TMA loads
+// whose bytes are credited to the leader's "full" barrier - and the leader CTA issues one M = 256
+// MMA that reads both CTAs' shared memory and writes each CTA's 128 x bn accumulator into that
+// CTA's own TMEM.  Per FLOP this moves a third less data into shared memory than a one-CTA tile
+// and makes 128-wide tiles affordable, which removes most of the wave-quantisation loss on the
+// N = d_model GEMMs.  Barriers: full[s] (leader, 1 arrival + both CTAs' bytes), empty[s] and
+// acc_full[b] (one in each CTA, signalled by the leader's tcgen05.commit to both), acc_empty[b]
+// (leader, one arrival per epilogue warp of both CTAs).
 
 // Partial sums of one 32 x 32 accumulator chunk as the K halves of a cut tile exchange them: eight
 // 512-byte rows of [lane][4 floats], so that every access of a warp is one contiguous 512 bytes.
@@ -109,23 +54,6 @@ __device__ __forceinline__ void add_partner_chunk(uint32_t (&v)[32], const float
         v[4 * i + 2] = __float_as_uint(__uint_as_float(v[4 * i + 2]) + t.z);
         v[4 * i + 3] = __float_as_uint(__uint_as_float(v[4 * i + 3]) + t.w);
     }
-}
-
-// First of the 32-column chunks that warp pi of the pstride warps of a lane quarter handles, and the step to the
-// next: alternate chunks - except with the row-dot epilogue, where each takes a run of neighbouring chunks, so that all
-// columns of a head meet in one thread.
-template <int EPI>
-__device__ __forceinline__ int first_chunk(int bn, int pi, int pstride) { return EPI == kEpiRowDot ? pi * (bn / 32 / pstride) : pi; }
-
-// Residual / saved pre-activation / second dot operand: 8 columns of a row, or 32 (zeros outside).
-__device__ __forceinline__ uint4 load_aux8(const GemmParams& p, int row, int col)
-{
-    return row < p.M && col < p.N ? *reinterpret_cast<const uint4*>(p.aux_in + static_cast<size_t>(row) * p.ld_aux + col) : make_uint4(0, 0, 0, 0);
-}
-__device__ __forceinline__ void load_aux(uint4 (&aux)[4], const GemmParams& p, int row, int col0)
-{
-#pragma unroll
-    for (int g = 0; g < 4; ++g) aux[g] = load_aux8(p, row, col0 + g * 8);
 }
 
 // fp32 outputs: TMEM -> registers -> swizzled shared slab -> TMA store or reduce-add.
@@ -157,38 +85,105 @@ __device__ __forceinline__ void epilogue_f32(uint32_t taddr, int row0, int n0, i
     }
 }
 
-// Epilogue of one accumulator tile for one warp: TMEM -> registers -> swizzled shared slab -> TMA
-// store (rows >= M and columns >= N are clipped by the tensor map).  `taddr` addresses this warp's
-// lane quarter of the accumulator, row0 is the first of its 32 rows, pi selects which of the pstride
-// warps of the quarter it is.
-// `aux`: the first chunk's pieces, requested by the caller before it waited for the accumulator; a further
-// chunk's are requested as soon as their registers are free, ahead of that chunk's TMEM load, so the reads
-// (row-strided, L2 or DRAM latency) overlap the work.  Measured, requested at the start of their own chunk -> so:
-// 16384 x 4096 x 1024 x GeLU' 126 -> 122 us, 1024 x 4096 x 1024 x GeLU' 14.8 -> 14.1 us, 1024 x 1024 x 4096 + residual
-// 17.9 -> 16.8 us.
-template <int EPI, bool SINGLE_SLAB = false, bool SPLIT = false>
-__device__ __forceinline__ void epilogue_tile(uint4 (&aux)[4], uint32_t taddr, int row0, int n0, int bn, int pi, int pstride, int lane,
-                                              uint8_t* slab, uint32_t slab_u32, uint32_t& nout, const CUtensorMap* tmC,
-                                              const CUtensorMap* tmAux, const GemmParams& p,
-                                              const float* partner = nullptr /* SPLIT: the other K half's partial sums, [chunk][1024] */)
-{
-    const int row = row0 + lane;
-    if constexpr (EPI == kEpiF32) {
-        epilogue_f32(taddr, row0, n0, bn, p.N, pi, pstride, lane, slab, slab_u32, tmC, p.accumulate);
-    } else {
-        // 32 columns per chunk; the slab is two 2 KB halves (32 rows x 64 bytes, 64-byte
-        // swizzle) used alternately, so one store is always in flight behind the math.
-        const int nchunks = bn / 32;
-        const uint32_t sw = (lane >> 1) & 3;
-        constexpr bool kHasAux = EPI == kEpiBiasResid || EPI == kEpiDGelu || EPI == kEpiRowDot;
-        const int ch_first = first_chunk<EPI>(bn, pi, pstride);
-        const int ch_step = EPI == kEpiRowDot ? 1 : pstride;
-        const int ch_end = EPI == kEpiRowDot ? ch_first + nchunks / pstride : nchunks;
+// The epilogues that evaluate GeLU / GeLU' are instruction-bound with 8 warps (two per scheduler), so those instantiations
+// run 16.  A second slab per warp lets one store, or one aux chunk on its way in, travel behind the math.  16 warps
+// get it at the price of a stage: worth it for GeLU' (16384 x 4096 x 1024, six stages and one slab -> five and two: 145 ->
+// 118 us, 8192 x 4096 x 1024 66 -> 62 us), not for GeLU, whose input stream is the longer one (1920 x 3456 x 1280 18.2 -> 19.0).
+constexpr int P_STAGES = 6;
+constexpr int P_STAGE_BYTES = 32768;            // A: 128 x 64 (16 KB) + B half: up to 128 x 64 (16 KB)
+constexpr int P_SLAB_BYTES = 2048;
+constexpr int P_SMEM_BYTES = P_STAGES * P_STAGE_BYTES + 32768 /* slabs */ + 1024 + 512;
+template <int EPI> struct PairCfg {
+    static constexpr int kEpiWarps = (EPI == kEpiBiasGelu || EPI == kEpiDGelu) ? 16 : 8;
+    static constexpr int kStages = EPI == kEpiDGelu ? 5 : P_STAGES;
+    static constexpr int kSlabs = (EPI == kEpiDGelu ? 32 : 16) / kEpiWarps;       // per epilogue warp
+    static constexpr int kThreads = 64 + 32 * kEpiWarps;
+    static constexpr bool kHasAux = EPI == kEpiBiasResid || EPI == kEpiDGelu || EPI == kEpiRowDot;
+    static constexpr bool kHasBias = EPI == kEpiBias || EPI == kEpiBiasResid || EPI == kEpiBiasGelu;
+};
+
+// bf16 epilogue of one warp, in 32 x 32 chunks: TMEM -> registers -> slab (32 rows x 64 bytes, 64-byte swizzle) -> TMA store
+// (rows >= M and columns >= N are clipped by the tensor map).  A chunk of the residual / saved pre-activation / second dot
+// operand comes by TMA into the slab that its result will leave from, requested before the wait for the accumulator
+// (the first of a tile) or before the chunk in front of it is worked on; a lane reads and overwrites only its own row.
+// Against aux read by each lane for its own row, 16 bytes at a time, with row dots bound to 256-wide tiles (us): 8192 x 1024 x
+// 1024 + residual 20.5 -> 17.4, 8192 x 2048 x 2048 + residual 54 -> 52, 1920 x 1280 x 3456 + residual 19.4 -> 18.4, row dots
+// 1920 x 1280 x 1280 14.4 -> 11.5 and 8192 x 1024 x 1024 18.9 -> 17.8, 1024 x 4096 x 1024 x GeLU' 14.2 -> 13.7.  Chunks of 64 columns
+// (128-byte rows) need a stage's worth more slab and were slower: 8192 x 2048 x 8192 175 -> 187, 1920 x 3456 x 1280 GeLU 18.4 -> 21.2.
+template <int EPI>
+struct PairEpilogue {
+    using Cfg = PairCfg<EPI>;
+    static constexpr int kPerQuarter = Cfg::kEpiWarps / 4;   // warps that share the 32 TMEM lanes of a quarter
+    const GemmParams& p;
+    const CUtensorMap *tmC, *tmOut2, *tmIn;
+    uint8_t* slab0;
+    uint32_t slab0_u32, aux_bar;                             // aux_bar: one mbarrier per slab
+    int pi, lane;
+    uint32_t used = 0;           // slabs handed out
+    uint32_t waited = 0;         // aux chunks that have been waited for
+    bool requested = false;      // the next chunk's aux is on its way
+
+    // Chunks of a tile that warp pi of a quarter handles: every kPerQuarter-th; with row dots every kPerQuarter-th head, whose
+    // columns then meet in one thread.
+    __device__ __forceinline__ int run() const { return EPI == kEpiRowDot ? p.head_dim / 32 : 1; }
+    __device__ __forceinline__ int first() const { return pi * run(); }
+    __device__ __forceinline__ int next(int ch) const
+    {
+        if (EPI != kEpiRowDot) return ch + kPerQuarter;
+        return ch + 1 + ((ch + 1) % run() == 0 ? run() * (kPerQuarter - 1) : 0);
+    }
+
+    __device__ __forceinline__ void request(int row0, int col0)
+    {
+        const uint32_t k = used++ % Cfg::kSlabs;
+        if (lane == 0) {
+            bulk_wait_read0();                               // the slab's last store has read it
+            mbar_arrive_expect_tx(aux_bar + 8 * k, P_SLAB_BYTES);
+            tma_load_2d(slab0_u32 + k * P_SLAB_BYTES, tmIn, col0, row0, aux_bar + 8 * k);
+        }
+        requested = true;
+    }
+    __device__ __forceinline__ uint4* piece(uint32_t k, int g) const
+    {
+        return reinterpret_cast<uint4*>(slab0 + k * P_SLAB_BYTES + lane * 64 + ((g ^ ((lane >> 1) & 3)) << 4));
+    }
+    __device__ __forceinline__ uint32_t free_slab()
+    {
+        if (lane == 0) { if (Cfg::kSlabs > 1) bulk_wait_read1(); else bulk_wait_read0(); }
+        __syncwarp();
+        return used++ % Cfg::kSlabs;
+    }
+    __device__ __forceinline__ void store(uint32_t k, const CUtensorMap* map, int row0, int col0) const
+    {
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+            tma_store_2d(map, slab0_u32 + k * P_SLAB_BYTES, col0, row0);
+            bulk_commit();
+        }
+    }
+
+    // Returns false when a wait gave up.  taddr: this warp's lane quarter of the accumulator; row0: its first row;
+    // partner (SPLIT): the other K half's partial sums, [chunk][1024].
+    template <bool SPLIT>
+    __device__ __forceinline__ bool tile(uint32_t taddr, int row0, int n0, int bn, const float* partner, volatile int* abort_flag)
+    {
         float dot = 0.f;
 #pragma unroll 1
-        for (int ch = ch_first; ch < ch_end; ch += ch_step) {
+        for (int ch = first(); ch < bn / 32; ch = next(ch)) {
             const int col0 = n0 + ch * 32;
             if (col0 >= p.N) break;
+            uint32_t k = 0;
+            if constexpr (Cfg::kHasAux) {
+                if (!requested) request(row0, col0);
+                requested = false;
+                k = waited % Cfg::kSlabs;
+                const bool ok = mbar_wait(aux_bar + 8 * k, (waited / Cfg::kSlabs) & 1, abort_flag, p.status, 721);
+                if (!__all_sync(0xffffffffu, ok)) return false;
+                ++waited;
+                const int ahead = next(ch);
+                if (Cfg::kSlabs > 1 && ahead < bn / 32 && n0 + ahead * 32 < p.N) request(row0, n0 + ahead * 32);
+            }
             uint32_t v[32];
             tmem_ld32(taddr + ch * 32, v);
             tc_wait_ld();
@@ -197,46 +192,51 @@ __device__ __forceinline__ void epilogue_tile(uint4 (&aux)[4], uint32_t taddr, i
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
                 float f[8];
-                epilogue_group<EPI>(v + 8 * g, row, col0 + g * 8, p, aux[g], f);
-                o[g] = pack8(f);
-                if constexpr (EPI == kEpiRowDot) {
-                    float r[8];
-                    unpack8(aux[g], r);                      // zeros beyond M and N
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) dot = fmaf(f[j], r[j], dot);
+                for (int j = 0; j < 8; ++j) f[j] = __uint_as_float(v[8 * g + j]);
+                if constexpr (Cfg::kHasBias) {
+                    if (col0 + 8 * g < p.N) {
+                        float b[8];
+                        unpack8(*reinterpret_cast<const uint4*>(p.bias + col0 + 8 * g), b);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) f[j] += b[j];
+                    }
                 }
-                if (kHasAux && ch + ch_step < ch_end) aux[g] = load_aux8(p, row, col0 + 32 * ch_step + g * 8);
+                if constexpr (Cfg::kHasAux) {                // zeros beyond M and N
+                    float r[8];
+                    unpack8(*piece(k, g), r);
+                    if constexpr (EPI == kEpiBiasResid) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) f[j] += r[j];
+                    } else if constexpr (EPI == kEpiDGelu) {
+                        gelu_grad_mul8(f, r, p.act);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) dot = fmaf(f[j], r[j], dot);
+                    }
+                }
+                o[g] = pack8(f);
                 if constexpr (EPI == kEpiBiasGelu) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) v[8 * g + j] = __float_as_uint(f[j]);   // fp32 pre-activation, kept for GeLU
                 }
             }
-            auto store_chunk = [&](const uint4* src, const CUtensorMap* map) {
-                const uint32_t half = SINGLE_SLAB ? 0u : (nout++ & 1u) * 2048u;
-                if (lane == 0) { if (SINGLE_SLAB) bulk_wait_read0(); else bulk_wait_read1(); }
-                __syncwarp();
+            if constexpr (!Cfg::kHasAux) k = free_slab();
 #pragma unroll
-                for (int g = 0; g < 4; ++g)
-                    *reinterpret_cast<uint4*>(slab + half + lane * 64 + ((g ^ sw) << 4)) = src[g];
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) {
-                    tma_store_2d(map, slab_u32 + half, col0, row0);
-                    bulk_commit();
-                }
-            };
-            store_chunk(o, tmC);
+            for (int g = 0; g < 4; ++g) *piece(k, g) = o[g];
+            store(k, tmC, row0, col0);
             if constexpr (EPI == kEpiRowDot) {
                 if ((col0 + 32) % p.head_dim == 0) {         // last chunk of a head: its row sums are complete
+                    const int row = row0 + lane;
                     if (row < p.M) {
-                        const int b = row / p.seq_len, sq = row - b * p.seq_len, h = col0 / p.head_dim;
-                        p.row_dot[(static_cast<size_t>(b) * (p.N / p.head_dim) + h) * p.seq_len + sq] = dot;
+                        const int b = row / p.seq_len, sq = row - b * p.seq_len, hd = col0 / p.head_dim;
+                        p.row_dot[(static_cast<size_t>(b) * (p.N / p.head_dim) + hd) * p.seq_len + sq] = dot;
                     }
                     dot = 0.f;
                 }
             }
             if constexpr (EPI == kEpiBiasGelu) {
-                // GeLU of the fp32 pre-activation, evaluated while the store above drains the slab
+                // evaluated while the store above drains the slab
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
                     float f[8];
@@ -245,172 +245,14 @@ __device__ __forceinline__ void epilogue_tile(uint4 (&aux)[4], uint32_t taddr, i
                     gelu8(f, p.act);
                     o[g] = pack8(f);
                 }
-                store_chunk(o, tmAux);
-            }
-        }
-    }
-}
-
-template <bool A_MN, bool B_MN, int EPI>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
-gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-            const __grid_constant__ CUtensorMap tmBh /* B with a half-width box */,
-            const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmAux, const GemmParams p)
-{
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* slabs = tiles + STAGES * STAGE_BYTES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(slabs + EPI_WARPS * SLAB_BYTES);
-    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
-    const uint32_t accf0 = smem_u32(bars + 2 * STAGES), acce0 = smem_u32(bars + 2 * STAGES + 2);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int num_k = (p.K + BK - 1) / BK;
-    const int total_tiles = p.total_virtual;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 32 * EPI_WARPS); }
-        *abort_flag = 0;
-        fence_barrier_init();
-        fence_proxy_async();
-        prefetch_tmap(&tmA);
-        prefetch_tmap(&tmB);
-        prefetch_tmap(&tmC);
-    }
-    if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    grid_dep_launch();                                  // (after the TMEM allocation: see grid_dep_launch)
-    const uint32_t tmem_base = *tmem_slot;
-    grid_dep_wait();                                    // inputs of this GEMM come from the previous kernel
-
-    if (warp == 0) {
-        if (elect_one()) {
-            uint32_t stage = 0, phase = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-                int m0, n0, bn;
-                tile_info(p, tile, m0, n0, bn);
-                const uint32_t stage_tx = A_TILE_BYTES + bn * BK * 2;
-                const CUtensorMap* mapB = bn == p.bn ? &tmB : &tmBh;
-                for (int kb = 0; kb < num_k; ++kb) {
-                    if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.status, 100)) { ok = false; break; }
-                    const uint32_t fb = full0 + 8 * stage;
-                    mbar_arrive_expect_tx(fb, stage_tx);
-                    const uint32_t a_dst = smem_u32(tiles + stage * STAGE_BYTES), b_dst = a_dst + A_TILE_BYTES;
-                    if constexpr (!A_MN) {
-                        tma_load_2d(a_dst, &tmA, kb * BK, m0, fb);
-                    } else {
+                k = free_slab();
 #pragma unroll
-                        for (int j = 0; j < BM / 64; ++j) tma_load_2d(a_dst + j * 8192, &tmA, m0 + 64 * j, kb * BK, fb);
-                    }
-                    if constexpr (!B_MN) {
-                        tma_load_2d(b_dst, mapB, kb * BK, n0, fb);
-                    } else {
-                        for (int j = 0; j < bn / 64; ++j) tma_load_2d(b_dst + j * 8192, &tmB, n0 + 64 * j, kb * BK, fb);
-                    }
-                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
-                }
+                for (int g = 0; g < 4; ++g) *piece(k, g) = o[g];
+                store(k, tmOut2, row0, col0);
             }
         }
-    } else if (warp == 1) {
-        if (elect_one()) {
-            const uint32_t idesc_full = make_idesc_bf16(BM, p.bn, A_MN, B_MN);
-            const uint32_t idesc_half = make_idesc_bf16(BM, p.bn >> 1, A_MN, B_MN);
-            uint32_t stage = 0, phase = 0, it = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++it) {
-                const uint32_t idesc = tile >= p.split_begin ? idesc_half : idesc_full;
-                const uint32_t buf = it & 1, acc_phase = (it >> 1) & 1;
-                if (!mbar_wait(acce0 + 8 * buf, acc_phase ^ 1, abort_flag, p.status, 200)) break;
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + buf * BN_MAX;
-                for (int kb = 0; kb < num_k; ++kb) {
-                    if (!mbar_wait(full0 + 8 * stage, phase, abort_flag, p.status, 201)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t a_base = smem_u32(tiles + stage * STAGE_BYTES), b_base = a_base + A_TILE_BYTES;
-#pragma unroll
-                    for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-                        // K-major: 16 k = 32 bytes along the swizzled 128-byte row; 8-row groups 1024 B apart.
-                        // MN-major: 16 k = two 8-k groups of 1024 B; 64-row groups 8192 B apart.
-                        const uint64_t adesc = A_MN ? make_smem_desc_sw128(a_base + kk * 2048, 8192, 1024)
-                                                    : make_smem_desc_sw128(a_base + kk * 32, 16, 1024);
-                        const uint64_t bdesc = B_MN ? make_smem_desc_sw128(b_base + kk * 2048, 8192, 1024)
-                                                    : make_smem_desc_sw128(b_base + kk * 32, 16, 1024);
-                        umma_f16(d_tmem, adesc, bdesc, idesc, (kb | kk) != 0 ? 1u : 0u);
-                    }
-                    umma_commit(empty0 + 8 * stage);   // frees the stage once these MMAs have read it
-                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
-                }
-                if (ok) umma_commit(accf0 + 8 * buf);  // accumulator complete
-            }
-        }
-    } else {
-        // Epilogue: warp w may read TMEM lanes 32*(w%4)..+31; the two warps of a lane quarter take
-        // alternate column steps.  Each step goes TMEM -> registers -> swizzled shared slab -> one
-        // TMA store (rows >= M and columns >= N are clipped by the tensor map).
-        const int q = warp & 3, pi = (warp - 2) >> 2;
-        uint8_t* slab = slabs + (warp - 2) * SLAB_BYTES;
-        const uint32_t slab_u32 = smem_u32(slab);
-        uint32_t it = 0, nout = 0;
-        for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
-            int m0, n0, bn;
-            tile_info(p, tile, m0, n0, bn);
-            const uint32_t buf = it & 1, acc_phase = (it >> 1) & 1;
-            uint4 aux[4];
-            if (EPI == kEpiBiasResid || EPI == kEpiDGelu || EPI == kEpiRowDot)
-                load_aux(aux, p, m0 + q * 32 + lane, n0 + 32 * first_chunk<EPI>(bn, pi, 2));
-            bool ok = mbar_wait(accf0 + 8 * buf, acc_phase, abort_flag, p.status, 300);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * BN_MAX;
-            epilogue_tile<EPI>(aux, taddr, m0 + q * 32, n0, bn, pi, 2, lane, slab, slab_u32, nout, &tmC, &tmAux, p);
-            tc_fence_before();
-            mbar_arrive(acce0 + 8 * buf);
-        }
-        if (lane == 0) bulk_wait0();
+        return true;
     }
-
-    __syncwarp();
-    if (*abort_flag) {   // give copies and MMAs still in flight time to land before releasing anything
-        const long long t0 = clock64();
-        while (clock64() - t0 < (1ll << 22)) {}
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc(tmem_base, TMEM_COLS);
-    }
-}
-
-// ------------------------------------------------------------------------------------------------
-// CTA-pair variant (cta_group::2): a cluster of two CTAs computes one 256 x bn tile.  CTA r of the
-// pair loads its own 128 rows of A and its own half (bn/2 rows) of B - with plain per-CTA TMA loads
-// whose bytes are credited to the leader's "full" barrier - and the leader CTA issues one M = 256
-// MMA that reads both CTAs' shared memory and writes each CTA's 128 x bn accumulator into that
-// CTA's own TMEM.  Per FLOP this moves a third less data into shared memory than the one-CTA tile
-// and makes 128-wide tiles affordable, which removes most of the wave-quantisation loss on the
-// N = d_model GEMMs.  Barriers: full[s] (leader, 1 arrival + both CTAs' bytes), empty[s] and
-// acc_full[b] (one in each CTA, signalled by the leader's tcgen05.commit to both), acc_empty[b]
-// (leader, one arrival per epilogue warp of both CTAs).
-// The epilogues that evaluate GeLU / GeLU' are instruction-bound with 8 warps (two per scheduler),
-// so those instantiations run 16 epilogue warps and use one 2 KB output slab per warp instead of two.
-constexpr int P_STAGE_BYTES = 32768;            // A: 128 x 64 (16 KB) + B half: up to 128 x 64 (16 KB)
-template <int EPI> struct PairCfg {
-    static constexpr int kEpiWarps = (EPI == kEpiBiasGelu || EPI == kEpiDGelu) ? 16 : 8;
-    static constexpr int kStages = 6;
-    static constexpr int kSlab = kEpiWarps == 16 ? 2048 : SLAB_BYTES;   // 16 warps: one 2 KB slab each, no ping-pong
-    static constexpr int kThreads = 64 + 32 * kEpiWarps;
-    static constexpr int kSmem = kStages * P_STAGE_BYTES + kEpiWarps * kSlab + 1024 + 256;
 };
 
 // Work unit v of the CTA-pair kernel: a whole tile, or - for the tiles of a thin last round - one
@@ -429,17 +271,20 @@ __device__ __forceinline__ PairUnit pair_unit(const GemmParams& p, int v, int nu
 
 template <bool A_MN, bool B_MN, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<EPI>::kThreads, 1)
-gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                 const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmAux, const GemmParams p)
+gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmC,
+                 const __grid_constant__ CUtensorMap tmOut2 /* kEpiBiasGelu: GeLU */, const __grid_constant__ CUtensorMap tmIn /* aux_in */,
+                 const GemmParams p)
 {
-    constexpr int P_STAGES = PairCfg<EPI>::kStages, NEPI = PairCfg<EPI>::kEpiWarps;
+    constexpr int NEPI = PairCfg<EPI>::kEpiWarps, kStages = PairCfg<EPI>::kStages;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* slabs = tiles + P_STAGES * P_STAGE_BYTES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(slabs + NEPI * PairCfg<EPI>::kSlab);
-    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + P_STAGES);
-    const uint32_t accf0 = smem_u32(bars + 2 * P_STAGES), acce0 = smem_u32(bars + 2 * P_STAGES + 2);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * P_STAGES + 4);
+    uint8_t* slabs = tiles + kStages * P_STAGE_BYTES;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(slabs + NEPI * PairCfg<EPI>::kSlabs * P_SLAB_BYTES);
+    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages);
+    const uint32_t accf0 = smem_u32(bars + 2 * kStages), acce0 = smem_u32(bars + 2 * kStages + 2);
+    const uint32_t aux0 = smem_u32(bars + 2 * kStages + 4);           // one per slab
+    static_assert((2 * kStages + 4 + 32 + 1) * 8 <= 512, "barriers and the words behind them");
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 4 + 32);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -450,8 +295,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int bn = p.bn, half_n = bn >> 1;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < P_STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
+        for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 2 * NEPI); }
+        for (int w = 0; w < 32; ++w) mbar_init(aux0 + 8 * w, 1);
         *abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async();
@@ -506,7 +352,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         tma_load_2d_pair(b_dst, &tmB, n0, kb * BK, fb);
                         if (half_n > 64) tma_load_2d_pair(b_dst + 8192, &tmB, n0 + 64, kb * BK, fb);
                     }
-                    if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+                    if (++stage == kStages) { stage = 0; phase ^= 1; }
                 }
             }
         }
@@ -533,33 +379,34 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         umma_f16_pair(d_tmem, desc_advance(ad, kk * (A_MN ? 2048 : 32)), desc_advance(bd, kk * (B_MN ? 2048 : 32)), idesc,
                                       (kb != un.kb0 || kk != 0) ? 1u : 0u);
                     umma_commit_pair(empty0 + 8 * stage, 3);     // frees the stage in both CTAs
-                    if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
+                    if (++stage == kStages) { stage = 0; phase ^= 1; }
                 }
                 if (ok) umma_commit_pair(accf0 + 8 * buf, 3);     // both CTAs' accumulators complete
             }
         }
     } else {
-        const int q = warp & 3, pi = (warp - 2) >> 2;
-        uint8_t* slab = slabs + (warp - 2) * PairCfg<EPI>::kSlab;
-        const uint32_t slab_u32 = smem_u32(slab);
-        uint32_t it = 0, nout = 0;
+        const int q = warp & 3;
+        constexpr int kSlabs = PairCfg<EPI>::kSlabs;
+        uint8_t* slab0 = slabs + (warp - 2) * kSlabs * P_SLAB_BYTES;
+        PairEpilogue<EPI> epi{p, &tmC, &tmOut2, &tmIn, slab0, smem_u32(slab0), aux0 + 8 * (warp - 2) * kSlabs, (warp - 2) >> 2, lane};
+        uint32_t it = 0;
         for (int unit = pair_id; unit < total_tiles; unit += n_pairs, ++it) {
             const PairUnit un = pair_unit(p, unit, num_k);
             const int tile = un.tile;
             const int mi = p.n_fastest ? tile / p.n_tiles : tile % p.m_tiles;
             const int ni = p.n_fastest ? tile % p.n_tiles : tile / p.m_tiles;
-            const int m0 = mi * 256 + rank * 128, n0 = ni * bn;
+            const int row0 = mi * 256 + rank * 128 + q * 32, n0 = ni * bn;
             const uint32_t buf = it & 1, acc_phase = (it >> 1) & 1;
-            uint4 aux[4];
-            if (EPI == kEpiBiasResid || EPI == kEpiDGelu || EPI == kEpiRowDot)
-                load_aux(aux, p, m0 + q * 32 + lane, n0 + 32 * first_chunk<EPI>(bn, pi, NEPI / 4));
+            // the first chunk's aux travels while the products run (a cut tile may turn out to be finished by its other half)
+            const int col_first = n0 + 32 * epi.first();
+            if (PairCfg<EPI>::kHasAux && un.slot < 0 && epi.first() < bn / 32 && col_first < p.N) epi.request(row0, col_first);
             bool ok = mbar_wait(accf0 + 8 * buf, acc_phase, abort_flag, p.status, 720);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * BN_MAX;
             if (un.slot < 0) {
-                epilogue_tile<EPI, NEPI == 16>(aux, taddr, m0 + q * 32, n0, bn, pi, NEPI / 4, lane, slab, slab_u32, nout, &tmC, &tmAux, p);
+                if (!epi.template tile<false>(taddr, row0, n0, bn, nullptr, abort_flag)) break;
             } else {
                 // Half of a cut tile's K range.  Every epilogue warp leaves its part of the partial sums in
                 // the scratch, then draws a ticket shared with the same warp of the CTA that has the
@@ -571,7 +418,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 float* mine = p.split_ws + ((((static_cast<size_t>(un.slot) * 2 + un.half) * 2 + rank) * 4) + q) * region;
                 const float* other = p.split_ws + ((((static_cast<size_t>(un.slot) * 2 + (un.half ^ 1)) * 2 + rank) * 4) + q) * region;
 #pragma unroll 1
-                for (int ch = pi; ch < nchunks; ch += NEPI / 4) {
+                for (int ch = epi.first(); ch < nchunks; ch = epi.next(ch)) {
                     if (n0 + ch * 32 >= p.N) break;
                     uint32_t v[32];
                     tmem_ld32(taddr + ch * 32, v);
@@ -591,7 +438,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if (before != 0) {
                     if (lane == 0) *ticket = 0;                                  // both halves have drawn: ready for the next launch
                     __threadfence();
-                    epilogue_tile<EPI, NEPI == 16, true>(aux, taddr, m0 + q * 32, n0, bn, pi, NEPI / 4, lane, slab, slab_u32, nout, &tmC, &tmAux, p, other);
+                    if (!epi.template tile<true>(taddr, row0, n0, bn, other, abort_flag)) break;
                 }
             }
             tc_fence_before();
@@ -645,11 +492,11 @@ struct WgradMaps { CUtensorMap a[kWgradMaxJobs], b[kWgradMaxJobs], c[kWgradMaxJo
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<kEpiF32>::kThreads, 1)
 wgrad_group_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant__ WgradParams p)
 {
-    constexpr int P_STAGES = PairCfg<kEpiF32>::kStages, NEPI = PairCfg<kEpiF32>::kEpiWarps;
+    constexpr int NEPI = PairCfg<kEpiF32>::kEpiWarps;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* slabs = tiles + P_STAGES * P_STAGE_BYTES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(slabs + NEPI * PairCfg<kEpiF32>::kSlab);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(slabs + 32768);
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + P_STAGES);
     const uint32_t accf0 = smem_u32(bars + 2 * P_STAGES), acce0 = smem_u32(bars + 2 * P_STAGES + 2);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * P_STAGES + 4);
@@ -733,7 +580,7 @@ wgrad_group_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant
         }
     } else {
         const int q = warp & 3, pi = (warp - 2) >> 2;
-        uint8_t* slab = slabs + (warp - 2) * PairCfg<kEpiF32>::kSlab;
+        uint8_t* slab = slabs + (warp - 2) * 4096;
         const uint32_t slab_u32 = smem_u32(slab);
         uint32_t it = 0;
         for (int t = pair_id; t < p.total; t += n_pairs, ++it) {
@@ -768,37 +615,22 @@ wgrad_group_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant
     if (p.late) grid_dep_wait();
 }
 
-template <bool A_MN, bool B_MN, int EPI>
-const char* launch_inst(Runtime* rt, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmBh,
-                        const CUtensorMap& tmC, const CUtensorMap& tmAux, const GemmParams& p, cudaStream_t stream)
+template <bool B_MN, int EPI>
+const char* launch_pair(Runtime* rt, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmC, const CUtensorMap& tmOut2,
+                        const CUtensorMap& tmIn, const GemmParams& p, cudaStream_t stream)
 {
-    auto kern = gemm_kernel<A_MN, B_MN, EPI>;
-    const int total = p.m_tiles * p.n_tiles;
-    const int grid = total < rt->sm_count ? total : rt->sm_count;
-    return launch_k(kern, dim3(grid), dim3(GEMM_THREADS), SMEM_BYTES, stream, tmA, tmB, tmBh, tmC, tmAux, p) == cudaSuccess
-               ? nullptr : "gemm launch failed";
-}
-
-template <bool A_MN, bool B_MN, int EPI>
-const char* launch_pair(Runtime* rt, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmC,
-                        const CUtensorMap& tmAux, const GemmParams& p, cudaStream_t stream)
-{
-    auto kern = gemm_pair_kernel<A_MN, B_MN, EPI>;
+    auto kern = gemm_pair_kernel<false, B_MN, EPI>;
     const int total = p.total_virtual;
     const int max_pairs = rt->sm_count / 2;
     const int pairs = total < max_pairs ? total : max_pairs;
-    return launch_k(kern, dim3(2 * pairs), dim3(PairCfg<EPI>::kThreads), PairCfg<EPI>::kSmem, stream, tmA, tmB, tmC, tmAux, p) == cudaSuccess
+    return launch_k(kern, dim3(2 * pairs), dim3(PairCfg<EPI>::kThreads), P_SMEM_BYTES, stream, tmA, tmB, tmC, tmOut2, tmIn, p) == cudaSuccess
                ? nullptr : "gemm (CTA pair) launch failed";
 }
 
-template <bool A_MN, bool B_MN, int EPI>
+template <bool B_MN, int EPI>
 bool set_attr()
 {
-    if (cudaFuncSetAttribute(gemm_kernel<A_MN, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess) return false;
-    if constexpr (EPI == kEpiF32)
-        return cudaFuncSetAttribute(wgrad_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<EPI>::kSmem) == cudaSuccess;
-    else
-        return cudaFuncSetAttribute(gemm_pair_kernel<A_MN, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<EPI>::kSmem) == cudaSuccess;
+    return cudaFuncSetAttribute(gemm_pair_kernel<false, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES) == cudaSuccess;
 }
 
 }  // namespace
@@ -807,10 +639,9 @@ bool set_attr()
 // enqueue path, so a stream capture sees launches only).
 const char* configure_gemm()
 {
-    const bool ok = set_attr<false, false, kEpiNone>() && set_attr<false, false, kEpiBias>() &&
-                    set_attr<false, false, kEpiBiasResid>() && set_attr<false, false, kEpiBiasGelu>() &&
-                    set_attr<false, true, kEpiNone>() && set_attr<false, true, kEpiDGelu>() && set_attr<false, true, kEpiRowDot>() &&
-                    set_attr<true, true, kEpiF32>();
+    const bool ok = set_attr<false, kEpiNone>() && set_attr<false, kEpiBias>() && set_attr<false, kEpiBiasResid>() && set_attr<false, kEpiBiasGelu>() &&
+                    set_attr<true, kEpiNone>() && set_attr<true, kEpiDGelu>() && set_attr<true, kEpiRowDot>() &&
+                    cudaFuncSetAttribute(wgrad_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES) == cudaSuccess;
     return ok ? nullptr : "cudaFuncSetAttribute(gemm) failed";
 }
 
@@ -836,31 +667,27 @@ static int pair_tile_width(int m_tiles, int N, int pairs)
 
 static const char* launch_gemm_pair(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cudaStream_t stream)
 {
-    const bool a_mn = false, b_mn = a.layout == kNN;             // (weight gradients: launch_wgrad)
-    const bool f32_out = false;
+    const bool b_mn = a.layout == kNN;                           // (weight gradients: launch_wgrad)
     const int m_tiles = (a.M + 255) / 256, pairs = rt->sm_count / 2;
-    int bn;
-    {
-        const int forced = tuning().gemm_bn;
-        bn = pair_tile_width(m_tiles, a.N, pairs);
-        if (forced == 128 || forced == 192 || forced == 256) bn = forced;
-        if (a.epilogue == kEpiRowDot) bn = 256;              // an epilogue warp must own whole heads (128 columns)
-    }
-    CUtensorMap tmA, tmB, tmC, tmAux;
+    const bool head128 = a.epilogue == kEpiRowDot && a.head_dim == 128;
+    int bn = pair_tile_width(m_tiles, a.N, pairs);
+    const int forced = tuning().gemm_bn;
+    if (forced == 128 || forced == 192 || forced == 256) bn = forced;
+    if (head128 && bn == 192) bn = 256;                          // a tile must hold whole heads
+    const bool has_aux = a.epilogue == kEpiBiasResid || a.epilogue == kEpiDGelu || a.epilogue == kEpiRowDot;
+    CUtensorMap tmA, tmB, tmC, tmOut2, tmIn;
     const char* e;
-    e = a_mn ? encode_2d(rt, &tmA, a.A, a.M, a.K, a.lda, 64, BK) : encode_2d(rt, &tmA, a.A, a.K, a.M, a.lda, BK, BM);
-    if (e) return e;
+    if ((e = encode_2d(rt, &tmA, a.A, a.K, a.M, a.lda, BK, BM))) return e;
     e = b_mn ? encode_2d(rt, &tmB, a.B, a.N, a.K, a.ldb, 64, BK) : encode_2d(rt, &tmB, a.B, a.K, a.N, a.ldb, BK, bn / 2);
     if (e) return e;
-    e = encode_2d(rt, &tmC, a.C, a.N, a.M, a.ldc, 32, 32, f32_out, !f32_out);
-    if (e) return e;
-    e = encode_2d(rt, &tmAux, a.epilogue == kEpiBiasGelu ? a.aux_out : a.C, a.N, a.M, a.ldc, 32, 32, f32_out, !f32_out);
-    if (e) return e;
+    if ((e = encode_2d(rt, &tmC, a.C, a.N, a.M, a.ldc, 32, 32, false, true))) return e;
+    tmOut2 = tmIn = tmC;
+    if (a.epilogue == kEpiBiasGelu && (e = encode_2d(rt, &tmOut2, a.aux_out, a.N, a.M, a.ldc, 32, 32, false, true))) return e;
+    if (has_aux && (e = encode_2d(rt, &tmIn, a.aux_in, a.N, a.M, a.ld_aux, 32, 32, false, true))) return e;
     GemmParams p;
     p.M = a.M; p.N = a.N; p.K = a.K; p.bn = bn;
     p.bias = static_cast<const __nv_bfloat16*>(a.bias);
-    p.aux_in = static_cast<const __nv_bfloat16*>(a.aux_in); p.ld_aux = a.ld_aux;
-    p.accumulate = a.accumulate; p.act = a.act;
+    p.act = a.act;
     p.m_tiles = m_tiles; p.n_tiles = (a.N + bn - 1) / bn;
     p.split_begin = p.m_tiles * p.n_tiles; p.total_virtual = p.split_begin;
     p.split_ws = nullptr;
@@ -873,7 +700,7 @@ static const char* launch_gemm_pair(Runtime* rt, const GemmArgs& a, DeviceStatus
         const int rem = total % pairs;
         const int min_k = tuning().gemm_split_min_k;
         // (short K ranges lose more to the second prologue and epilogue than the idle half round costs)
-        if (a.split_ws && !no_split && !f32_out && a.epilogue != kEpiRowDot && total > pairs && rem > 0 && 2 * rem <= pairs && rem <= kSplitMaxTiles &&
+        if (a.split_ws && !no_split && total > pairs && rem > 0 && 2 * rem <= pairs && rem <= kSplitMaxTiles &&
             num_k >= min_k) {
             p.split_begin = total - rem;
             p.total_virtual = p.split_begin + 2 * rem;
@@ -884,13 +711,13 @@ static const char* launch_gemm_pair(Runtime* rt, const GemmArgs& a, DeviceStatus
     p.status = status;
     const int key = a.layout * 16 + a.epilogue;
     switch (key) {
-        case kTN * 16 + kEpiNone: return launch_pair<false, false, kEpiNone>(rt, tmA, tmB, tmC, tmAux, p, stream);
-        case kTN * 16 + kEpiBias: return launch_pair<false, false, kEpiBias>(rt, tmA, tmB, tmC, tmAux, p, stream);
-        case kTN * 16 + kEpiBiasResid: return launch_pair<false, false, kEpiBiasResid>(rt, tmA, tmB, tmC, tmAux, p, stream);
-        case kTN * 16 + kEpiBiasGelu: return launch_pair<false, false, kEpiBiasGelu>(rt, tmA, tmB, tmC, tmAux, p, stream);
-        case kNN * 16 + kEpiNone: return launch_pair<false, true, kEpiNone>(rt, tmA, tmB, tmC, tmAux, p, stream);
-        case kNN * 16 + kEpiDGelu: return launch_pair<false, true, kEpiDGelu>(rt, tmA, tmB, tmC, tmAux, p, stream);
-        case kNN * 16 + kEpiRowDot: return launch_pair<false, true, kEpiRowDot>(rt, tmA, tmB, tmC, tmAux, p, stream);
+        case kTN * 16 + kEpiNone: return launch_pair<false, kEpiNone>(rt, tmA, tmB, tmC, tmOut2, tmIn, p, stream);
+        case kTN * 16 + kEpiBias: return launch_pair<false, kEpiBias>(rt, tmA, tmB, tmC, tmOut2, tmIn, p, stream);
+        case kTN * 16 + kEpiBiasResid: return launch_pair<false, kEpiBiasResid>(rt, tmA, tmB, tmC, tmOut2, tmIn, p, stream);
+        case kTN * 16 + kEpiBiasGelu: return launch_pair<false, kEpiBiasGelu>(rt, tmA, tmB, tmC, tmOut2, tmIn, p, stream);
+        case kNN * 16 + kEpiNone: return launch_pair<true, kEpiNone>(rt, tmA, tmB, tmC, tmOut2, tmIn, p, stream);
+        case kNN * 16 + kEpiDGelu: return launch_pair<true, kEpiDGelu>(rt, tmA, tmB, tmC, tmOut2, tmIn, p, stream);
+        case kNN * 16 + kEpiRowDot: return launch_pair<true, kEpiRowDot>(rt, tmA, tmB, tmC, tmOut2, tmIn, p, stream);
         default: return "gemm: unsupported layout/epilogue combination";
     }
 }
@@ -970,7 +797,7 @@ const char* launch_wgrad(Runtime* rt, const WgradJob* jobs, int n_jobs, int K, i
     for (int j = n_jobs; j < kWgradMaxJobs; ++j) { p.job[j] = p.job[0]; maps.a[j] = maps.a[0]; maps.b[j] = maps.b[0]; maps.c[j] = maps.c[0]; }
     p.total = first;
     const int used = first < pairs ? first : pairs;
-    return launch_k(wgrad_group_kernel, dim3(2 * used), dim3(PairCfg<kEpiF32>::kThreads), PairCfg<kEpiF32>::kSmem, stream, maps, p) == cudaSuccess
+    return launch_k(wgrad_group_kernel, dim3(2 * used), dim3(PairCfg<kEpiF32>::kThreads), P_SMEM_BYTES, stream, maps, p) == cudaSuccess
                ? nullptr : "weight-gradient launch failed";
 }
 
@@ -990,84 +817,18 @@ const char* launch_gemm(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cu
     if (need_aux_in && (!a.aux_in || misaligned(a.aux_in) || (a.ld_aux % 8))) return "gemm: epilogue needs aux_in";
     if (a.epilogue == kEpiBiasGelu && (!a.aux_out || misaligned(a.aux_out))) return "gemm: epilogue needs aux_out";
 
-    const bool a_mn = a.layout == kNT, b_mn = a.layout == kNN || a.layout == kNT;
     const bool f32_out = a.epilogue == kEpiF32;
-    const int pair_mode = tuning().gemm_pair;
+    if (f32_out != (a.layout == kNT)) return "gemm: unsupported layout/epilogue combination";
+    if (f32_out && (a.ldc % 4)) return "gemm: fp32 ldc must be a multiple of 4";
     GemmClusterPlan plan;
-    if (pair_mode && tuning().gemm_bn == 0 && plan_cluster(a, rt->sm_count, &plan)) {
-        if (f32_out && (a.ldc % 4)) return "gemm: fp32 ldc must be a multiple of 4";
+    if (tuning().gemm_pair == 0) {                                   // no CTA pairs anywhere
+        plan = {0, 128, 1, 6};
         return launch_gemm_cluster(rt, a, plan, status, stream);
     }
-    if (pair_mode && a.M >= 256) {
-        if (!f32_out) return launch_gemm_pair(rt, a, status, stream);
-        const WgradJob w = {a.M, a.N, a.A, a.lda, a.B, a.ldb, a.C, a.ldc};
-        return launch_wgrad(rt, &w, 1, a.K, a.accumulate, false, status, stream);
-    }
-    if (f32_out && (a.ldc % 4)) return "gemm: fp32 ldc must be a multiple of 4";
-    // Tile width: the one that needs the least (rounds x width) on this many SMs; ties go to the
-    // wider tile (less operand traffic per FLOP).
-    const int m_tiles = (a.M + BM - 1) / BM;
-    // Tile width 256 unless that leaves most SMs without a tile (small problems are latency-bound;
-    // a narrower tile spreads them over more SMs).  Narrower tiles cost more operand traffic per
-    // FLOP and were measured slower whenever every SM already has work.
-    int bn = BN_MAX;
-    while (bn > 128 && static_cast<long long>(m_tiles) * ((a.N + bn - 1) / bn) * 2 <= rt->sm_count) bn -= 64;
-    {
-        const int forced = tuning().gemm_bn;
-        if (forced == 128 || forced == 192 || forced == 256) bn = forced;
-        if (a.epilogue == kEpiRowDot) bn = BN_MAX;           // an epilogue warp must own whole heads (128 columns)
-    }
-    CUtensorMap tmA, tmB, tmBh, tmC, tmAux;
-    const char* e;
-    // K-major operand [rows, K]: box 64 k x rows.  MN-major operand stored [K, rows]: box 64 rows x 64 k.
-    e = a_mn ? encode_2d(rt, &tmA, a.A, a.M, a.K, a.lda, 64, BK) : encode_2d(rt, &tmA, a.A, a.K, a.M, a.lda, BK, BM);
-    if (e) return e;
-    e = b_mn ? encode_2d(rt, &tmB, a.B, a.N, a.K, a.ldb, 64, BK) : encode_2d(rt, &tmB, a.B, a.K, a.N, a.ldb, BK, bn);
-    if (e) return e;
-    e = b_mn ? encode_2d(rt, &tmBh, a.B, a.N, a.K, a.ldb, 64, BK) : encode_2d(rt, &tmBh, a.B, a.K, a.N, a.ldb, BK, bn / 2);
-    if (e) return e;
-
-    // Output maps: a store box is 32 rows x 32 columns (fp32: 128-byte rows, 128-byte swizzle;
-    // bf16: 64-byte rows, 64-byte swizzle).
-    e = encode_2d(rt, &tmC, a.C, a.N, a.M, a.ldc, 32, 32, f32_out, !f32_out);
-    if (e) return e;
-    e = encode_2d(rt, &tmAux, a.epilogue == kEpiBiasGelu ? a.aux_out : a.C, a.N, a.M, a.ldc, 32, 32, f32_out, !f32_out);
-    if (e) return e;
-
-    GemmParams p;
-    p.M = a.M; p.N = a.N; p.K = a.K; p.bn = bn;
-    p.bias = static_cast<const __nv_bfloat16*>(a.bias);
-    p.aux_in = static_cast<const __nv_bfloat16*>(a.aux_in); p.ld_aux = a.ld_aux;
-    p.accumulate = a.accumulate; p.act = a.act;
-    p.m_tiles = m_tiles; p.n_tiles = (a.N + bn - 1) / bn;
-    p.n_fastest = p.n_tiles < p.m_tiles ? 1 : 0;
-    p.status = status;
-    p.split_ws = nullptr;
-    p.row_dot = static_cast<float*>(a.row_dot); p.head_dim = a.head_dim; p.seq_len = a.seq_len;
-    {
-        // Tail balancing: when the last round would leave at least half of the SMs idle, its
-        // tiles are issued as two half-width tiles each.
-        const int total = p.m_tiles * p.n_tiles;
-        const int grid = total < rt->sm_count ? total : rt->sm_count;
-        const int rem = total % grid;
-        const bool no_split = tuning().gemm_split == 0;
-        p.split_begin = total;
-        if (bn == BN_MAX && rem > 0 && 2 * rem <= grid && !no_split && a.epilogue != kEpiRowDot) p.split_begin = total - rem;
-        p.total_virtual = p.split_begin + 2 * (total - p.split_begin);
-    }
-
-    const int key = a.layout * 16 + a.epilogue;
-    switch (key) {
-        case kTN * 16 + kEpiNone: return launch_inst<false, false, kEpiNone>(rt, tmA, tmB, tmBh, tmC, tmAux, p, stream);
-        case kTN * 16 + kEpiBias: return launch_inst<false, false, kEpiBias>(rt, tmA, tmB, tmBh, tmC, tmAux, p, stream);
-        case kTN * 16 + kEpiBiasResid: return launch_inst<false, false, kEpiBiasResid>(rt, tmA, tmB, tmBh, tmC, tmAux, p, stream);
-        case kTN * 16 + kEpiBiasGelu: return launch_inst<false, false, kEpiBiasGelu>(rt, tmA, tmB, tmBh, tmC, tmAux, p, stream);
-        case kNN * 16 + kEpiNone: return launch_inst<false, true, kEpiNone>(rt, tmA, tmB, tmBh, tmC, tmAux, p, stream);
-        case kNN * 16 + kEpiDGelu: return launch_inst<false, true, kEpiDGelu>(rt, tmA, tmB, tmBh, tmC, tmAux, p, stream);
-        case kNN * 16 + kEpiRowDot: return launch_inst<false, true, kEpiRowDot>(rt, tmA, tmB, tmBh, tmC, tmAux, p, stream);
-        case kNT * 16 + kEpiF32: return launch_inst<true, true, kEpiF32>(rt, tmA, tmB, tmBh, tmC, tmAux, p, stream);
-        default: return "gemm: unsupported layout/epilogue combination";
-    }
+    if (tuning().gemm_bn == 0 && plan_cluster(a, rt->sm_count, &plan)) return launch_gemm_cluster(rt, a, plan, status, stream);
+    if (!f32_out) return launch_gemm_pair(rt, a, status, stream);
+    const WgradJob w = {a.M, a.N, a.A, a.lda, a.B, a.ldb, a.C, a.ldc};
+    return launch_wgrad(rt, &w, 1, a.K, a.accumulate, false, status, stream);
 }
 
 }  // namespace pw

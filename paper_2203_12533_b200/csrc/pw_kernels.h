@@ -33,7 +33,7 @@ const char* configure_elementwise();
 // Process-wide tuning knobs (pw_set_tuning); the defaults are what every measurement and test uses.
 struct Tuning {
     int pdl = 1;                 // launch with the programmatic-serialization attribute
-    int gemm_pair = 1;           // CTA-pair GEMM kernel whenever M >= 256
+    int gemm_pair = 1;           // 0: no GEMM tile shared by a CTA pair
     int gemm_bn = 0;             // 0 = tile width chosen by the launcher, else 128 / 192 / 256
     int gemm_split = 1;          // cut the tiles of a thin last round along K
     int gemm_split_min_k = 64;   // ... from this many 64-wide K blocks on
