@@ -13,6 +13,8 @@
 //               as packed bf16 over the S columns it came from.  The running maximum is only
 //               advanced when it grows by more than 8 (in log2 units); only then is O rescaled in
 //               TMEM (tcgen05.ld / st) - P stays below 2^8, exact after the final division by l.
+// With too few pairs for the chip (SPLIT) a CTA owns ONE query tile instead: slot A takes its even key tiles, slot B the odd
+// ones, and the epilogue adds the two accumulators under their common maximum.
 // The epilogue divides O by l, stages it as bf16 in the (now idle) Q tile and stores it with TMA.
 // Every mbarrier wait is bounded; on expiry all roles leave, TMEM is released, the status word
 // records PW_ERR_TIMEOUT.
@@ -41,33 +43,49 @@ struct FwdSmem {
 
 struct FwdParams {
     int S, H, B;
-    int pairs_per_seq;          // ceil(S / 256)
-    int n_items;                // B * H * pairs_per_seq
+    int per_seq;                // items of one sequence and head: ceil(S / 256) pairs of query tiles, or S / 128 single ones
+    int n_items;                // B * H * per_seq
     float scale;
     float* lse;
     DeviceStatus* status;
     int* sched;                 // {next ticket, CTAs done}
 };
 
-// Work items (one per sequence, head and pair of query tiles) are numbered heaviest first (latest
+// Work items (one per sequence, head and pair of query tiles, or single one) are numbered heaviest first (latest
 // query tiles first) and handed out in that order: the producer thread draws the next number from
 // a global counter and passes it to the other roles through a two-slot ring in shared memory, so
 // the causal triangle balances itself over the CTAs.  Every CTA draws exactly one number past the
 // end; the last CTA to do so clears the counters for the next launch.
-struct FwdItem { int b, h, q0A, nA, nB; };
+struct FwdItem { int b, h, q0A, nA, nB, n_kv; };             // key tiles: each slot's, and those that are loaded
+template <bool SPLIT>
 __device__ __forceinline__ bool fwd_item(const FwdParams& p, int idx, FwdItem& it)
 {
     if (idx >= p.n_items) return false;
     const int BH = p.B * p.H;
-    const int pair = p.pairs_per_seq - 1 - idx / BH, bh = idx % BH;
+    const int pos = p.per_seq - 1 - idx / BH, bh = idx % BH;
     it.b = bh / p.H; it.h = bh % p.H;
-    it.q0A = pair * 256;
-    it.nA = it.q0A / 128 + 1;                               // key tiles each query tile needs
-    it.nB = it.q0A + 128 < p.S ? it.nA + 1 : 0;
+    if (SPLIT) {
+        it.q0A = pos * 128;
+        it.n_kv = pos + 1;
+        it.nA = (it.n_kv + 1) / 2;
+        it.nB = it.n_kv / 2;
+    } else {
+        it.q0A = pos * 256;
+        it.nA = it.q0A / 128 + 1;
+        it.nB = it.q0A + 128 < p.S ? it.nA + 1 : 0;
+        it.n_kv = it.nB ? it.nB : it.nA;
+    }
     return true;
 }
 
-template <int DH>
+template <int N>
+__device__ __forceinline__ void tmem_ld_n(uint32_t taddr, uint32_t* r)
+{
+    if constexpr (N == 16) tmem_ld16(taddr, r);
+    else tmem_ld32(taddr, r);
+}
+
+template <int DH, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_constant__ CUtensorMap tmO, const FwdParams p)
 {
@@ -106,7 +124,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         mbar_arrive_expect_tx(bar(0 + t), L::kTile);
         for (int kb = 0; kb < L::kBlocks; ++kb)
             tma_load_2d(sbase + L::kQ + t * L::kTile + kb * 16384, &tmQKV, it.h * DH + kb * 64,
-                        it.b * p.S + it.q0A + t * 128, bar(0 + t));
+                        it.b * p.S + it.q0A + (SPLIT ? 0 : t * 128), bar(0 + t));
     };
     auto load_k = [&](const FwdItem& it, int j, int s) {
         mbar_arrive_expect_tx(bar(4 + s), L::kTile);
@@ -125,7 +143,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         for (int i = 0; i < 14; ++i) mbar_init(bar(i), 1);
         mbar_init(bar(14), 256); mbar_init(bar(15), 256);
         mbar_init(bar(16), 1); mbar_init(bar(17), 1);
-        mbar_init(bar(18), 256); mbar_init(bar(19), 256);
+        mbar_init(bar(18), SPLIT ? 512 : 256); mbar_init(bar(19), SPLIT ? 512 : 256);
         mbar_init(bar(20), 1);
         mbar_init(bar(21), 1); mbar_init(bar(22), 1);
         mbar_init(bar(23), 17); mbar_init(bar(24), 17);
@@ -158,9 +176,29 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
             int idx = draw();
             item_slot[0] = idx;
             mbar_arrive(bar(21));
-            for (int k = 0; ok && fwd_item(p, idx, it); ++k) {
-                const int n_kv = it.nB ? it.nB : it.nA;
-                for (int j = 0; j < n_kv && ok; ++j, ++n) {
+            for (int k = 0; ok && fwd_item<SPLIT>(p, idx, it); ++k) {
+                const int n_kv = it.n_kv;
+                if (SPLIT) {
+                    // K_0 Q K_1 V_0 K_2 V_1 ...: the two slots start on their own key tiles.  Q alternates between its two buffers.
+                    auto next_k = [&](int j) {
+                        const uint32_t m = n + j;
+                        if (!mbar_wait(bar(6 + (m & 1)), ((m >> 1) & 1) ^ 1, abort_flag, p.status, 400)) return false;
+                        load_k(it, j, m & 1);
+                        return true;
+                    };
+                    const int t = k & 1;
+                    ok = next_k(0) && mbar_wait(bar(2 + t), ((k >> 1) & 1) ^ 1, abort_flag, p.status, 402);
+                    if (!ok) break;
+                    load_q(it, t);
+                    for (int j = 0; j < n_kv && ok; ++j) {
+                        if (j + 1 < n_kv && !next_k(j + 1)) { ok = false; break; }
+                        const uint32_t m = n + j;
+                        if (!mbar_wait(bar(10 + (m & 1)), ((m >> 1) & 1) ^ 1, abort_flag, p.status, 401)) { ok = false; break; }
+                        load_v(it, j, m & 1);
+                    }
+                    n += n_kv;
+                }
+                for (int j = 0; !SPLIT && j < n_kv && ok; ++j, ++n) {
                     const int s = n & 1;
                     const uint32_t ph = (n >> 1) & 1;
                     if (!mbar_wait(bar(6 + s), ph ^ 1, abort_flag, p.status, 400)) { ok = false; break; }
@@ -193,9 +231,9 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         constexpr uint32_t idesc_pv = make_idesc_bf16(128, DH, false, true);
         const uint32_t tb = tmem_base;
         const uint32_t sb = sbase;
-        // S_t = Q_t K^T from K stage s
-        auto issue_s = [&](int t, int s) {
-            const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + t * L::kTile, 16, 1024);
+        // S_t = Q K^T from a Q buffer and K stage s
+        auto issue_s = [&](int t, int s, int qbuf) {
+            const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + qbuf * L::kTile, 16, 1024);
             const uint64_t dk = make_smem_desc_sw128(sb + L::kK + s * L::kTile, 16, 1024);
             const uint32_t dst = tb + t * 128;
             {
@@ -235,20 +273,48 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
             if (!wait(21 + (k & 1), (k >> 1) & 1, 423)) break;
             const int idx = item_slot[k & 1];
             mbar_arrive(bar(23 + (k & 1)));
-            if (!fwd_item(p, idx, it)) break;
-            const int nA = it.nA, nB = it.nB, n_kv = nB ? nB : nA;
+            if (!fwd_item<SPLIT>(p, idx, it)) break;
+            const int nA = it.nA, nB = it.nB, n_kv = it.n_kv;
+            if (SPLIT) {
+                const int qb = k & 1;
+                auto scores = [&](int j) {                   // S(j) into slot j & 1
+                    const uint32_t m = n + j;
+                    if (!wait(4 + (m & 1), (m >> 1) & 1, 411)) return false;
+                    tc_fence_after();
+                    issue_s(j & 1, m & 1, qb);
+                    commit(6 + (m & 1));
+                    if (j == n_kv - 1) commit(2 + qb);       // Q is not needed again
+                    return true;
+                };
+                ok = wait(qb, (k >> 1) & 1, 410) && scores(0) && (n_kv == 1 || scores(1));
+                for (int j = 0; j < n_kv && ok; ++j) {
+                    const uint32_t m = n + j;
+                    const int t = j & 1;
+                    ok = wait(8 + (m & 1), (m >> 1) & 1, 412) && wait(14 + t, (t ? np[1] : np[0]) & 1, 413) &&
+                         (j > 1 || wait(18 + t, (k & 1) ^ 1, 418));          // the previous item's O_t has been read out
+                    if (!ok) break;
+                    if (t) ++np[1]; else ++np[0];
+                    tc_fence_after();
+                    issue_pv(t, m & 1, j > 1);
+                    commit(10 + (m & 1));
+                    if (j == n_kv - 1) { commit(16); commit(17); }
+                    if (j + 2 < n_kv) ok = scores(j + 2);
+                }
+                n += n_kv;
+                continue;
+            }
             {
                 const int s = n & 1;
                 const uint32_t ph = (n >> 1) & 1;
                 ok = wait(4 + s, ph, 411) && wait(0, qn[0] & 1, 410);
                 if (!ok) break;
                 tc_fence_after();
-                issue_s(0, s);
+                issue_s(0, s, 0);
                 if (nA == 1) commit(2);                     // Q_A is not needed again
                 if (nB) {
                     if (!wait(1, qn[1] & 1, 417)) { ok = false; break; }
                     tc_fence_after();
-                    issue_s(1, s);
+                    issue_s(1, s, 1);
                     if (nB == 1) commit(3);
                 }
                 commit(6 + s);
@@ -272,7 +338,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
                     if (!wait(4 + sn, phn, 414)) { ok = false; break; }
                     k_waited = true;
                     tc_fence_after();
-                    issue_s(0, sn);
+                    issue_s(0, sn, 0);
                     if (j + 2 == nA) commit(2);
                 }
                 if (j < nB) {
@@ -287,7 +353,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
                 if (j + 1 < nB) {
                     if (!k_waited && !wait(4 + sn, phn, 416)) { ok = false; break; }
                     tc_fence_after();
-                    issue_s(1, sn);
+                    issue_s(1, sn, 1);
                     if (j + 2 == nB) commit(3);
                 }
                 if (j + 1 < n_kv) commit(6 + sn);           // K stage free
@@ -325,19 +391,19 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         const int idx = item_slot[k & 1];
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(23 + (k & 1)));
-        if (!fwd_item(p, idx, it)) break;
+        if (!fwd_item<SPLIT>(p, idx, it)) break;
         const int n_t = t == 0 ? it.nA : it.nB;
-        const uint32_t u = u_base + t;                      // staging order: A(k), B(k), A(k+1), ...
+        const uint32_t u = SPLIT ? k : u_base + t;          // staging order: A(k), B(k), A(k+1), ...
         u_base += it.nB ? 2 : 1;
-        if (n_t == 0) continue;
-        const int q0 = it.q0A + t * 128;
+        if (!SPLIT && n_t == 0) continue;
+        const int q0 = it.q0A + (SPLIT ? 0 : t * 128);
         float m_used = -INFINITY, l = 0.f;
         for (int j = 0; j < n_t; ++j, ++ns) {
             ok = mbar_wait(bar(12 + t), ns & 1, abort_flag, p.status, 420);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            const bool diag = j == n_t - 1;
+            const bool diag = SPLIT ? 2 * j + t == it.n_kv - 1 : j == n_t - 1;
             const int lim = diag ? r - hf * 64 : 64;        // columns i > lim of my 64 are masked (diagonal tile)
             // pass 1: row maximum.  Scores 0..31 are read, used and dropped; scores 32..63 stay in
             // registers for the second pass (all 64 would not fit under the 576-thread register limit).
@@ -430,7 +496,8 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
             mbar_arrive(bar(14 + t));
         }
         if (ok) {
-            ok = mbar_wait(bar(16 + t), qn & 1, abort_flag, p.status, 421);
+            if (SPLIT) ok = mbar_wait(bar(16), k & 1, abort_flag, p.status, 421) && mbar_wait(bar(17), k & 1, abort_flag, p.status, 421);
+            else ok = mbar_wait(bar(16 + t), qn & 1, abort_flag, p.status, 421);
             ok = __all_sync(0xffffffffu, ok);
         }
         if (!ok) break;
@@ -440,33 +507,71 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
             xch[hf * 128 + r] = l;
             named_bar_sync(1 + t, 256);
             const float l_row = l + xch[(hf ^ 1) * 128 + r];
-            const float inv_l = 1.0f / l_row;
             uint8_t* stage = sm + L::kO;
             ok = mbar_wait(bar(20), (u & 1) ^ 1, abort_flag, p.status, 422);    // the previous user's store has read it
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
-#pragma unroll 1
-            for (int c = 0; c < DH / 64; ++c) {
-                uint32_t w[32];
-                tmem_ld32(o_addr + c * 32, w);
-                tc_wait_ld();
-                if (c == DH / 64 - 1) {                     // this thread's part of O_t has left TMEM
-                    tc_fence_before();
-                    mbar_arrive(bar(18 + t));
-                }
+            float lse_m = m_used, lse_l = l_row;
+            if constexpr (SPLIT) {
+                // O = (2^(mA - m) O_A + 2^(mB - m) O_B) / (2^(mA - m) lA + 2^(mB - m) lB), m = max(mA, mB): slot and half pick a
+                // quarter of the columns, which the thread reads from both accumulators.  m and l go through the
+                // places whose content this thread has just read.
+                xch[(hf ^ 1) * 128 + r] = hf ? m_used : l_row;
+                named_bar_sync(3, 512);
+                const float* theirs = reinterpret_cast<const float*>(sm + L::kXch) + (t ^ 1) * 256;
+                const float m_o = theirs[r], l_o = theirs[128 + r];
+                lse_m = fmaxf(m_used, m_o);
+                const float mine = ex2_approx((m_used - lse_m) * sl2), other = ex2_approx((m_o - lse_m) * sl2);
+                lse_l = l_row * mine + l_o * other;
+                const float inv_l = 1.0f / lse_l;
+                const float wA = (t == 0 ? mine : other) * inv_l, wB = (t == 0 ? other : mine) * inv_l;
+                constexpr int kCols = DH / 4;
+                const int seg = (t * 2 + hf) * kCols;
+                const uint32_t oa = tmem_base + lane_addr + 256 + seg;
+                uint32_t a[kCols], c[kCols];
+                tmem_ld_n<kCols>(oa, a);
+                if (it.nB) tmem_ld_n<kCols>(oa + 128, c);
+                else {
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
+                    for (int i = 0; i < kCols; ++i) c[i] = 0;
+                }
+                tc_wait_ld();
+                tc_fence_before();
+                mbar_arrive(bar(18)); mbar_arrive(bar(19));
+#pragma unroll
+                for (int g = 0; g < kCols / 8; ++g) {
                     float f[8];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(w[8 * g + i]) * inv_l;
-                    const int col = hf * (DH / 2) + c * 32 + g * 8, blk = col >> 6, chunk = (col & 63) >> 3;
+                    for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(a[8 * g + i]) * wA + __uint_as_float(c[8 * g + i]) * wB;
+                    const int col = seg + g * 8, blk = col >> 6, chunk = (col & 63) >> 3;
                     *reinterpret_cast<uint4*>(stage + blk * 16384 + r * 128 + ((chunk ^ (r & 7)) << 4)) = pack8(f);
                 }
+            } else {
+                const float inv_l = 1.0f / l_row;
+#pragma unroll 1
+                for (int c = 0; c < DH / 64; ++c) {
+                    uint32_t w[32];
+                    tmem_ld32(o_addr + c * 32, w);
+                    tc_wait_ld();
+                    if (c == DH / 64 - 1) {                     // this thread's part of O_t has left TMEM
+                        tc_fence_before();
+                        mbar_arrive(bar(18 + t));
+                    }
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        float f[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(w[8 * g + i]) * inv_l;
+                        const int col = hf * (DH / 2) + c * 32 + g * 8, blk = col >> 6, chunk = (col & 63) >> 3;
+                        *reinterpret_cast<uint4*>(stage + blk * 16384 + r * 128 + ((chunk ^ (r & 7)) << 4)) = pack8(f);
+                    }
+                }
             }
-            if (hf == 0) p.lse[(static_cast<size_t>(it.b) * p.H + it.h) * p.S + q0 + r] = m_used * p.scale + logf(l_row);
+            if (hf == 0 && !(SPLIT && t)) p.lse[(static_cast<size_t>(it.b) * p.H + it.h) * p.S + q0 + r] = lse_m * p.scale + logf(lse_l);
             fence_proxy_async();
-            named_bar_sync(1 + t, 256);
-            if (leader) {
+            if (SPLIT) named_bar_sync(3, 512);
+            else named_bar_sync(1 + t, 256);
+            if (leader && !(SPLIT && t)) {
                 for (int kb = 0; kb < L::kBlocks; ++kb)
                     tma_store_2d(&tmO, sbase + L::kO + kb * 16384, it.h * DH + kb * 64, it.b * p.S + q0);
                 bulk_commit();
@@ -515,10 +620,10 @@ const char* encode_rows(Runtime* rt, CUtensorMap* map, const void* ptr, uint64_t
 
 const char* configure_attention_fwd()
 {
-    if (cudaFuncSetAttribute(attn_fwd_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<64>::kBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(attn_fwd_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<128>::kBytes) != cudaSuccess)
-        return "cudaFuncSetAttribute(attention fwd) failed";
-    return nullptr;
+    auto attr = [](auto kern, int bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; };
+    return attr(attn_fwd_tc_kernel<64, false>, FwdSmem<64>::kBytes) && attr(attn_fwd_tc_kernel<128, false>, FwdSmem<128>::kBytes) &&
+           attr(attn_fwd_tc_kernel<64, true>, FwdSmem<64>::kBytes) && attr(attn_fwd_tc_kernel<128, true>, FwdSmem<128>::kBytes)
+               ? nullptr : "cudaFuncSetAttribute(attention fwd) failed";
 }
 
 const char* launch_attention_fwd(Runtime* rt, const void* qkv, int B, int S, int H, int dh, void* o, void* lse,
@@ -532,15 +637,24 @@ const char* launch_attention_fwd(Runtime* rt, const void* qkv, int B, int S, int
     if ((e = encode_rows(rt, &tmO, o, d, static_cast<uint64_t>(B) * S))) return e;
     FwdParams p;
     p.S = S; p.H = H; p.B = B; p.scale = 1.0f / sqrtf(static_cast<float>(dh));
-    p.pairs_per_seq = (S + 255) / 256;
-    p.n_items = B * H * p.pairs_per_seq;
+    // Pairs of query tiles share what they load and pay one prologue and epilogue for two; their longest item takes S / 128
+    // steps (of a key tile for both).  Where that is more than an even share of all steps, single query tiles whose key
+    // tiles are dealt out to the two slots take half as long.  us, pairs -> singles (B x S x heads x dh): 1 x 2048 x 16 x 128
+    // 34.4 -> 23.3, 2 x 512 x 16 x 64 11.5 -> 8.5, 3 x 640 x 10 x 128 13.3 -> 11.2, 2 x 1024 x 16 x 64 18.5 -> 16.0, 1 x 8192 x 8 x
+    // 64 111 -> 104; on the other side 1 x 4096 x 16 x 64 59.4 -> 59.5, 2 x 2048 x 16 x 64 33.7 -> 37.4, 8 x 1024 x 16 x 64 40.4 -> 45.9,
+    // and 5.4 -> 5.5 with one tile per sequence.
+    const int pairs = (S + 255) / 256, longest = S / 128;
+    const long long steps = static_cast<long long>(B) * H * (S % 256 ? pairs * (pairs - 1) + longest : pairs * (pairs + 1));
+    const bool split = longest > 1 && 10ll * longest * rt->sm_count > 11 * steps;
+    p.per_seq = split ? longest : pairs;
+    p.n_items = B * H * p.per_seq;
     p.lse = static_cast<float*>(lse);
     p.status = status;
     p.sched = status->sched + 0;
     dim3 grid(p.n_items < rt->sm_count ? p.n_items : rt->sm_count);
-    const cudaError_t e2 = dh == 64
-        ? launch_k(attn_fwd_tc_kernel<64>, grid, dim3(kThreads), FwdSmem<64>::kBytes, stream, tmQKV, tmO, p)
-        : launch_k(attn_fwd_tc_kernel<128>, grid, dim3(kThreads), FwdSmem<128>::kBytes, stream, tmQKV, tmO, p);
+    auto launch = [&](auto kern, int bytes) { return launch_k(kern, grid, dim3(kThreads), bytes, stream, tmQKV, tmO, p); };
+    const cudaError_t e2 = dh == 64 ? launch(split ? attn_fwd_tc_kernel<64, true> : attn_fwd_tc_kernel<64, false>, FwdSmem<64>::kBytes)
+                                    : launch(split ? attn_fwd_tc_kernel<128, true> : attn_fwd_tc_kernel<128, false>, FwdSmem<128>::kBytes);
     return e2 == cudaSuccess ? nullptr : "attention fwd launch failed";
 }
 
