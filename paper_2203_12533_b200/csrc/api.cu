@@ -113,7 +113,7 @@ struct LayerPlan {
     float eps;
     size_t ctx_off[PW_CTX_COUNT], ctx_size[PW_CTX_COUNT], ctx_bytes;
     // scratch = [ctx-shaped region used when the caller passes ctx == NULL] [backward temporaries]
-    size_t off_big, off_dqkv, off_td0, off_td1, off_delta, off_partials, off_partials2, off_partials3, off_partials4, scratch_bytes;
+    size_t off_big, off_dqkv, off_td0, off_td1, off_delta, off_partials, off_partials2, off_partials3, scratch_bytes;
     // lean ctx: h1, h2, a (and the statistics the re-derivation writes again) live in scratch
     bool lean;
     size_t off_lean_h1, off_lean_h2, off_lean_a, off_lean_stats;
@@ -227,16 +227,11 @@ static void build_plan(const pw_layer_config_t& c, Runtime* rt, LayerPlan* p)
     p->off_td0 = s; s += align256(T * d * 2);
     p->off_td1 = s; s += align256(T * d * 2);
     p->off_delta = s; s += align256(static_cast<size_t>(p->B) * p->H * p->S * 4);
-    size_t part = layernorm_bwd_scratch_bytes(rt, p->T, p->d);
-    const size_t c1 = colsum_scratch_bytes(rt, p->T, p->F), c2 = colsum_scratch_bytes(rt, p->T, 3 * p->d);
-    if (c1 > part) part = c1;
-    if (c2 > part) part = c2;
-    p->off_partials = s; s += align256(part);
-    // The four sets of partial rows of a backward call (LN2, LN1, the two bias column sums) are
-    // summed by one launch at the end of the call, so each has a region of its own.
-    p->off_partials2 = s; s += align256(c1);                                           // db1 column sums (side stream)
-    p->off_partials3 = s; s += align256(layernorm_bwd_scratch_bytes(rt, p->T, p->d));  // LN1 backward
-    p->off_partials4 = s; s += align256(c2);                                           // dbqkv column sums (side stream)
+    // The partial rows of a backward call (LN2, LN1, the two bias column sums) are
+    // summed by one launch at the end of the call, so each set has a region of its own.
+    p->off_partials = s; s += align256(layernorm_bwd_scratch_bytes(rt, p->T, p->d));
+    p->off_partials2 = s; s += align256(colsum_beside_scratch_bytes(rt, p->T, p->F, 3 * p->d));   // db1 and dbqkv
+    p->off_partials3 = s; s += align256(layernorm_bwd_scratch_bytes(rt, p->T, p->d));             // LN1 backward
     p->off_splitk = s; s += align256(gemm_split_ws_bytes());
     p->off_lean_h1 = p->off_lean_h2 = p->off_lean_a = p->off_lean_stats = 0;
     if (p->lean) {
@@ -345,13 +340,12 @@ static pw_status_t do_ln_bwd(pw_layer_t* L, const void* dh, const void* x, const
                                accumulate, partials, st);
     return e ? fail(PW_ERR_CUDA, e) : PW_OK;
 }
-static pw_status_t do_colsum(pw_layer_t* L, const void* in, int N, void* out, int accumulate, void* partials,
-                             cudaStream_t st, ReduceJob* defer = nullptr)
+static pw_status_t do_colsum(pw_layer_t* L, const void* const in[2], const int n[2], void* const out[2], void* partials, ReduceJob jobs[2], cudaStream_t st)
 {
     const LayerPlan& p = L->plan;
-    LaunchScope sc(L, PW_K_COLSUM, defer ? 1 : 2, 0.0, 2.0 * p.T * N, st);
-    const char* e = defer ? launch_colsum_partial(L->rt, in, p.T, N, N, out, partials, defer, true, st)
-                          : launch_colsum(L->rt, in, p.T, N, N, out, accumulate, partials, st);
+    LaunchScope sc(L, PW_K_COLSUM, 1, 0.0, 2.0 * p.T * (n[0] + n[1]), st);
+    const char* e = launch_colsum_beside(L->rt, in, n, p.T, out, partials, jobs, st);
+    if (e) sc.cancel(1);
     return e ? fail(PW_ERR_CUDA, e) : PW_OK;
 }
 static pw_status_t do_reduce(pw_layer_t* L, const ReduceJob* jobs, int njobs, int accumulate, cudaStream_t st)
@@ -482,8 +476,7 @@ static pw_status_t enqueue_bwd(pw_layer_t* L, const pw_layer_params_t* P, const 
 
     void* part2 = at(scratch, p.off_partials2);
     void* part3 = at(scratch, p.off_partials3);
-    void* part4 = at(scratch, p.off_partials4);
-    ReduceJob jobs[4];                                   // LN2, db1, LN1, dbqkv: summed by one launch at the end
+    ReduceJob jobs[4];                                   // LN2, LN1, db1, dbqkv: summed by one launch at the end
 
     // The four weight gradients hang off the data-gradient chain and nothing waits for them: they run as one pool of tiles
     // at the end of the call.  (On a side stream, each behind the kernel that makes its operand, they finished about as
@@ -544,13 +537,15 @@ static pw_status_t enqueue_bwd(pw_layer_t* L, const pw_layer_params_t* P, const 
                                      nullptr, 0, nullptr, 0, sk), st));
     // LN1 backward + residual: dx = dx1 + LNbwd(dh1)
     PW_DO(do_ln_bwd(L, td0, x, mu1, r1, P->ln1_gamma, dx1, dx, G->ln1_gamma, G->ln1_beta, nullptr,
-                                nullptr, accumulate, part3, st, &jobs[2]));
-    // From here on nothing reads what LN1 backward writes until the reduce launch: the column sums and the weight gradients
-    // start beside it and beside one another.
-    PW_DO(do_colsum(L, du, F, G->b_fc1, accumulate, part2, st, &jobs[1]));
-    PW_DO(do_colsum(L, dqkv, 3 * d, G->b_qkv, accumulate, part4, st, &jobs[3]));
+                                nullptr, accumulate, part3, st, &jobs[1]));
+    // From here on nothing reads what LN1 backward writes until the reduce launch: the weight gradients start beside it, and
+    // the column sums beside the weight gradients.
     if (rederive && !dx_over_dy) PW_DO(order(L->ev[1], ax, st));
     PW_DO(do_wgrad(L, wj, dx_over_dy ? 3 : 4, accumulate, true, st));
+    const void* const cin[2] = {du, dqkv};
+    const int cn[2] = {F, 3 * d};
+    void* const cout[2] = {G->b_fc1, G->b_qkv};
+    PW_DO(do_colsum(L, cin, cn, cout, part2, jobs + 2, st));
     // dgamma1/2, dbeta1/2, db2, dbo, db1, dbqkv: eight vectors, one fixed-order launch
     PW_DO(do_reduce(L, jobs, 4, accumulate, st));
     return PW_OK;

@@ -147,9 +147,11 @@ const char* launch_layernorm_bwd_partial(Runtime* rt, const void* dh, const void
                                          const void* gamma, const void* resid, int T, int d, void* dx, void* dgamma,
                                          void* dbeta, void* db_resid, void* db_dx, void* partials, ReduceJob* job,
                                          cudaStream_t stream);
-// late: as for launch_wgrad.
-const char* launch_colsum_partial(Runtime* rt, const void* in, int T, int N, int ld, void* out, void* partials,
-                                  ReduceJob* job, bool late, cudaStream_t stream);
+// Column sums of two matrices [T, n] to run beside the kernel launched in front, which must be a launch_wgrad(late) that reads
+// the same matrices; jobs go to launch_reduce_jobs.
+size_t colsum_beside_scratch_bytes(Runtime* rt, int T, int N0, int N1);
+const char* launch_colsum_beside(Runtime* rt, const void* const in[2], const int n[2], int T, void* const out[2], void* partials, ReduceJob jobs[2],
+                                 cudaStream_t stream);
 const char* launch_reduce_jobs(const ReduceJob* jobs, int njobs, int accumulate, cudaStream_t stream);
 
 // Column sums with the partial sums in a fixed device array inside the library (no allocation, no Runtime).
