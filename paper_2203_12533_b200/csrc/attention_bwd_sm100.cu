@@ -4,7 +4,7 @@
 // reproducible), after delta = rowsum(dO * O) (attention.cu):
 //
 //   dkdv : CTA = one 128-key tile j of one (sequence, head); streams 64-query sub-tiles u >= 2j.
-//            S^T  = K_j Q_u^T      (128 x 64)   dP^T = V_j dO_u^T   (128 x 64)      -> TMEM, 2 buffers each
+//            S^T  = K_j Q_u^T      (128 x 64)   dP^T = V_j dO_u^T   (128 x 64)      -> TMEM, 2 or 3 buffers each
 //            P^T  = exp2(S^T * scale*log2e - lse*log2e), masked;  dS^T = P^T * (dP^T - delta)
 //            dV_j += P^T dO_u      dK_j += dS^T Q_u                                  -> TMEM accumulators
 //          P^T / dS^T are written back to TMEM as packed bf16 and fed to the MMA from there; the
@@ -13,7 +13,7 @@
 //   dq   : CTA = two adjacent 128-query tiles (ping-pong), streams 64-key sub-tiles.
 //            S = Q K_v^T (128 x 64), dP = dO V_v^T, dS = P * (dP - delta), dQ += dS K_v.
 //
-// Warps: 0 = TMA producer, 1 = MMA issuer (+ TMEM allocation), 2..9 = element-wise warps (a warp
+// Warps: 0 = TMA producer, 1 = MMA issuer (+ TMEM allocation), 2..9 and 10..17 = element-wise warps (a warp
 // may only touch TMEM lanes 32*(warp%4)..+31; the two warps of a lane quarter split the columns).
 // No running maximum is needed: lse from the forward normalises P directly.
 // Every mbarrier wait is bounded (see mbar_wait).
@@ -22,8 +22,7 @@
 namespace pw {
 namespace {
 
-constexpr int kThreads = 320;
-constexpr int kDqThreads = 576;                            // producer warp, MMA warp, 2 x 8 element-wise warps
+constexpr int kThreads = 576;                              // producer warp, MMA warp, 2 x 8 element-wise warps
 constexpr float kLog2e = 1.4426950408889634f;
 
 
@@ -38,6 +37,22 @@ struct BwdParams {
     int* sched;                 // {next ticket, CTAs done} of this kernel
 };
 
+template <int N>
+__device__ __forceinline__ void tmem_ld_n(uint32_t taddr, uint32_t* r)
+{
+    if constexpr (N == 16) tmem_ld16(taddr, r);
+    else tmem_ld32(taddr, r);
+}
+
+// Slot of a ring of N and the parity of its barriers, counted on one by one: the issuing thread, whose every instruction
+// counts, divides nothing.
+template <int N>
+struct Ring {
+    int i = 0;
+    uint32_t parity = 0;
+    __device__ __forceinline__ void next() { if (++i == N) { i = 0; parity ^= 1; } }
+};
+
 // ------------------------------------------------------------------------------------------- dK, dV
 template <int DH>
 struct KvSmem {
@@ -49,7 +64,7 @@ struct KvSmem {
     // TMEM columns: S^T buffer b at 64 b, dP^T buffer b at kDP + 64 b, then dV and dK (DH columns each)
     static constexpr int kDP = 64 * kBufs, kDV = 128 * kBufs, kDK = kDV + (DH == 64 ? 64 : 128);
     // barriers: 0,1 kv_full[buffer] | 2,3 kv_empty[buffer] | kQF+s q_full[stage] | kQE+s q_empty[stage] | kSF+b st_full[b]
-    //   kPF+b p_full[b] (256 arrivals) | kAF acc_full | kAE acc_empty (256 arrivals) | kIF+i item_full | kIE+i item_empty (9 arrivals)
+    //   kPF+b p_full[b] (256 arrivals) | kAF acc_full | kAE acc_empty (512 arrivals) | kIF+i item_full | kIE+i item_empty (17 arrivals)
     static constexpr int kQF = 4, kQE = kQF + kStages, kSF = kQE + kStages, kPF = kSF + kBufs, kAF = kPF + kBufs, kAE = kAF + 1,
                          kIF = kAE + 1, kIE = kIF + 2, kNumBars = kIE + 2;
     static constexpr int kK = 0;                             // item buffer i: K_j at i*2*kKV, V_j right after (two buffers)
@@ -134,9 +149,9 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
         for (int i = 0; i < L::kPF; ++i) mbar_init(bar(i), 1);
         for (int i = 0; i < L::kBufs; ++i) mbar_init(bar(L::kPF + i), 256);
         mbar_init(bar(L::kAF), 1);
-        mbar_init(bar(L::kAE), 256);
+        mbar_init(bar(L::kAE), 512);
         mbar_init(bar(L::kIF), 1); mbar_init(bar(L::kIF + 1), 1);
-        mbar_init(bar(L::kIE), 9); mbar_init(bar(L::kIE + 1), 9);
+        mbar_init(bar(L::kIE), 17); mbar_init(bar(L::kIE + 1), 17);
         *abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async();
@@ -187,11 +202,12 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
         constexpr uint32_t idesc_acc = make_idesc_bf16(128, DH, false, true);
         const uint32_t tb = tmem_base;
         const uint32_t sb = sbase;
-        auto issue_scores = [&](uint32_t g, int buf) {      // S^T and dP^T of stream position g into buffer g % kBufs
-            const int s = g % L::kStages, hb = g % L::kBufs;
-            const uint64_t desc_k = make_smem_desc_sw128(sb + L::kK + buf * 2 * L::kKV, 16, 1024);
+        const uint64_t desc_k0 = make_smem_desc_sw128(sb + L::kK, 16, 1024), desc_q0 = make_smem_desc_sw128(sb + L::kQ, 16, 1024);
+        const uint64_t desc_qt0 = make_smem_desc_sw128(sb + L::kQ, 8192, 1024);
+        auto issue_scores = [&](int s, int hb, int buf) {   // S^T and dP^T from ring stage s into buffer hb
+            const uint64_t desc_k = desc_slot<2 * L::kKV>(desc_k0, buf);
             const uint64_t desc_v = desc_advance(desc_k, L::kKV);
-            const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + s * 2 * L::kSub, 16, 1024), dg = desc_advance(dq, L::kSub);
+            const uint64_t dq = desc_slot<2 * L::kSub>(desc_q0, s), dg = desc_advance(dq, L::kSub);
             const uint32_t st = tb + hb * 64;
             {
                 // the two products are independent accumulation chains: their steps alternate, so that a step
@@ -208,9 +224,8 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
                 umma_commit(bar(L::kSF + hb));
             }
         };
-        auto issue_acc = [&](uint32_t g, bool first) {      // dV += P^T dO_u, dK += dS^T Q_u
-            const int s = g % L::kStages, hb = g % L::kBufs;
-            const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + s * 2 * L::kSub, 8192, 1024), dg = desc_advance(dq, L::kSub);
+        auto issue_acc = [&](int s, int hb, bool first) {   // dV += P^T dO_u, dK += dS^T Q_u
+            const uint64_t dq = desc_slot<2 * L::kSub>(desc_qt0, s), dg = desc_advance(dq, L::kSub);
             const uint32_t pt = tb + hb * 64;
             const uint32_t acc0 = first ? 0u : 1u;
             {
@@ -227,7 +242,8 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
         auto wait = [&](int b, uint32_t parity, int site) {
             return mbar_wait(bar(b), parity, abort_flag, p.status, site);
         };
-        uint32_t g0 = 0;                                    // stream position of this item's first sub-tile
+        Ring<L::kStages> ss, sa;                            // stage of the next sub-tile for the scores / for dV and dK
+        Ring<L::kBufs> bs, ba;                              // and its buffer
         bool ok = true;
         KvItem it;
         for (int k = 0; ok; ++k) {
@@ -238,40 +254,39 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
             const int buf = k & 1, n_u = it.n_u;
             // the scores run kBufs - 1 sub-tiles ahead of the accumulation products
             constexpr int kAhead = L::kBufs - 1;
-            ok = wait(0 + buf, (k >> 1) & 1, 510);
-            for (int a = 0; a < kAhead && a < n_u && ok; ++a) {
-                const uint32_t ga = g0 + a;
-                ok = wait(L::kQF + ga % L::kStages, (ga / L::kStages) & 1, 511);
-                if (!ok) break;
+            auto scores = [&]() {
+                if (!wait(L::kQF + ss.i, ss.parity, 511)) return false;
                 tc_fence_after();
-                issue_scores(ga, buf);
-            }
+                issue_scores(ss.i, bs.i, buf);
+                ss.next(); bs.next();
+                return true;
+            };
+            ok = wait(0 + buf, (k >> 1) & 1, 510);
+            for (int a = 0; a < kAhead && a < n_u && ok; ++a) ok = scores();
             if (!ok) break;
             for (int i = 0; i < n_u && ok; ++i) {
-                const uint32_t g = g0 + i;
-                if (i + kAhead < n_u) {
-                    const uint32_t gn = g + kAhead;
-                    if (!wait(L::kQF + gn % L::kStages, (gn / L::kStages) & 1, 512)) { ok = false; break; }
-                    tc_fence_after();
-                    issue_scores(gn, buf);
-                }
-                if (!wait(L::kPF + g % L::kBufs, (g / L::kBufs) & 1, 513)) { ok = false; break; }
+                if (i + kAhead < n_u && !scores()) { ok = false; break; }
+                if (!wait(L::kPF + ba.i, ba.parity, 513)) { ok = false; break; }
                 // the previous item's dV / dK must have been read out before they are overwritten
                 if (i == 0 && !wait(L::kAE, (k & 1) ^ 1, 515)) { ok = false; break; }
                 tc_fence_after();
-                issue_acc(g, i == 0);
+                issue_acc(sa.i, ba.i, i == 0);
+                sa.next(); ba.next();
             }
             if (!ok) break;
             umma_commit(bar(L::kAF));
-            g0 += n_u;
         }
         }
     } else {
-        const int q = warp & 3, ch = (warp - 2) >> 2;       // lane quarter, column half (32 of the 64 queries)
+        // Two sets of eight warps take the sub-tiles in turn (n_u is even, so the sets alternate across items too).  One set
+        // alone, two warps per scheduler, spent most of its time on the latencies between the arrival of
+        // a sub-tile's scores and its P^T / dS^T (figures: see the dQ kernel's items).
+        const int q = warp & 3, w4 = (warp - 2) >> 2;       // lane quarter
+        const int set = w4 >> 1, ch = w4 & 1;               // sub-tiles set, set + 2, ...; column half (32 of the 64 queries)
         const int r = q * 32 + lane;                        // key row inside the tile
         const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
         const float sl2 = p.scale * kLog2e;
-        uint32_t g = 0;                                     // stream position
+        uint32_t g0 = 0;                                    // stream position of this item's first sub-tile
         bool ok = true;
         KvItem it;
         for (int k = 0; ok; ++k) {
@@ -283,85 +298,93 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
             if (lane == 0) mbar_arrive(bar(L::kIE + (k & 1)));
             if (!kv_item(p, idx, it)) break;
             const int kv0 = it.j * 128, u0 = 2 * it.j;
-            for (int i = 0; i < it.n_u; ++i, ++g) {
+            for (int i = set; i < it.n_u; i += 2) {
+                const uint32_t g = g0 + i;
                 const int hb = g % L::kBufs, qc0 = (u0 + i) * 64 + ch * 32;   // first query column of this thread's slice
                 ok = mbar_wait(bar(L::kSF + hb), (g / L::kBufs) & 1, abort_flag, p.status, 520);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                uint32_t sv[32], dv[32];
-                tmem_ld32(tmem_base + lane_addr + hb * 64 + ch * 32, sv);
-                tmem_ld32(tmem_base + lane_addr + L::kDP + hb * 64 + ch * 32, dv);
-                tc_wait_ld();
+                // The slice is read as an mma.sync accumulator is laid out: a thread owns 8 query columns of 4 key rows, so that
+                // a query's lse and delta are read for 8 threads at once and used four times (with a key row per thread
+                // all 32 pairs went to every thread, and the shared-memory reads alone took 24 of 155 us).
+                const uint32_t s_at = tmem_base + lane_addr + hb * 64 + ch * 32;
+                uint32_t sv[2][16], dv[2][16];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    tmem_ld_16x256_x4(s_at + (h << 20), sv[h]);
+                    tmem_ld_16x256_x4(s_at + L::kDP + (h << 20), dv[h]);
+                }
+                // lse and delta came with Q_u, whose products are complete, and the stage is not released before dV / dK
+                // have used it
+                const float2* lse2 = reinterpret_cast<const float2*>(sm + L::kRow + (g % L::kStages) * 512 + ch * 128) + (lane & 3);
+                const uint64_t nlog2e = pack_f32x2(-kLog2e, -kLog2e), neg1 = pack_f32x2(-1.0f, -1.0f), sl2x2 = pack_f32x2(sl2, sl2);
+                uint64_t nl2[4], ndl[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 l = lse2[4 * j], e = lse2[32 + 4 * j];
+                    nl2[j] = fmul2(pack_f32x2(l.x, l.y), nlog2e);
+                    ndl[j] = fmul2(pack_f32x2(e.x, e.y), neg1);
+                }
                 const bool diag = qc0 < kv0 + 128;           // some (key, query) pairs of this slice are masked
-                // lse and delta of this slice's 32 queries: they came with Q_u, whose products are complete, and the
-                // stage is not released before dV / dK have used it (every lane reads the same address: one broadcast)
-                const float4* lse4 = reinterpret_cast<const float4*>(sm + L::kRow + (g % L::kStages) * 512 + ch * 128);
-                const uint64_t nlog2e = pack_f32x2(-kLog2e, -kLog2e), neg1 = pack_f32x2(-1.0f, -1.0f);
-                uint32_t pp[16], dd[16];
-                const uint64_t sl2x2 = pack_f32x2(sl2, sl2);
+                const int first = kv0 + q * 32 + (lane >> 2) - qc0 - 2 * (lane & 3);     // query columns below this (+ the row's offset) are masked
+                tc_wait_ld();
 #pragma unroll
-                for (int c4 = 0; c4 < 32; c4 += 4) {
-                    const float4 l4 = lse4[c4 >> 2], d4 = lse4[16 + (c4 >> 2)];
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t pp[8], dd[8];
 #pragma unroll
-                    for (int h2 = 0; h2 < 2; ++h2) {
-                        const int c = c4 + 2 * h2;
-                        const uint64_t nl2 = fmul2(h2 ? pack_f32x2(l4.z, l4.w) : pack_f32x2(l4.x, l4.y), nlog2e);
-                        const uint64_t dl = h2 ? pack_f32x2(d4.z, d4.w) : pack_f32x2(d4.x, d4.y);
+                    for (int i = 0; i < 8; ++i) {            // pair i: columns 8 (i / 2) + 2 (lane % 4), + 1 of row 16 h + 8 (i % 2) + lane / 4
                         float a0, a1, d0, d1;
-                        unpack_f32x2(ffma2(pack_f32x2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1])), sl2x2, nl2), a0, a1);
+                        unpack_f32x2(ffma2(pack_f32x2(__uint_as_float(sv[h][2 * i]), __uint_as_float(sv[h][2 * i + 1])), sl2x2, nl2[i >> 1]), a0, a1);
                         float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
                         if (diag) {
-                            if (qc0 + c < kv0 + r) p0 = 0.f;
-                            if (qc0 + c + 1 < kv0 + r) p1 = 0.f;
+                            const int m = first + 16 * h + 8 * (i & 1) - 8 * (i >> 1);
+                            if (0 < m) p0 = 0.f;
+                            if (1 < m) p1 = 0.f;
                         }
-                        const uint64_t pv = pack_f32x2(p0, p1);
-                        unpack_f32x2(fmul2(pv, ffma2(dl, neg1, pack_f32x2(__uint_as_float(dv[c]), __uint_as_float(dv[c + 1])))), d0, d1);
-                        pp[c >> 1] = pack_bf16(p0, p1);
-                        dd[c >> 1] = pack_bf16(d0, d1);
+                        unpack_f32x2(fmul2(pack_f32x2(p0, p1), fadd2(pack_f32x2(__uint_as_float(dv[h][2 * i]), __uint_as_float(dv[h][2 * i + 1])), ndl[i >> 1])), d0, d1);
+                        pp[i] = pack_bf16(p0, p1);
+                        dd[i] = pack_bf16(d0, d1);
                     }
+                    // packed operands go back into this warp's own (loaded) columns: P^T over S^T, dS^T over dP^T
+                    tmem_st_16x128_x4(s_at + (h << 20), pp);
+                    tmem_st_16x128_x4(s_at + L::kDP + (h << 20), dd);
                 }
-                // packed operands go back into this warp's own columns: P^T over S^T, dS^T over dP^T
-                tmem_st16(tmem_base + lane_addr + hb * 64 + ch * 32, pp);
-                tmem_st16(tmem_base + lane_addr + L::kDP + hb * 64 + ch * 32, dd);
                 tc_wait_st();
                 tc_fence_before();
                 mbar_arrive(bar(L::kPF + hb));
             }
+            g0 += it.n_u;
             if (ok) {
                 ok = mbar_wait(bar(L::kAF), k & 1, abort_flag, p.status, 521);
                 ok = __all_sync(0xffffffffu, ok);
             }
             if (!ok) break;
             tc_fence_after();
-            // this warp converts columns [ch*DH/2, +DH/2) of dV and dK and stages them over V_j / K_j
+            // this warp converts columns [w4 * DH/4, + DH/4) of dV and dK and stages them over V_j / K_j
             const int buf = k & 1;
-#pragma unroll 1
+            constexpr int kCols = DH / 4;
+            uint32_t v[2][kCols];
+            tmem_ld_n<kCols>(tmem_base + lane_addr + L::kDV + w4 * kCols, v[0]);
+            tmem_ld_n<kCols>(tmem_base + lane_addr + L::kDK + w4 * kCols, v[1]);
+            tc_wait_ld();
+            tc_fence_before();
+            mbar_arrive(bar(L::kAE));                        // dV and dK have left TMEM: the next item may overwrite them
+#pragma unroll
             for (int which = 0; which < 2; ++which) {
                 uint8_t* stage = sm + L::kK + buf * 2 * L::kKV + (which == 0 ? L::kKV : 0);
                 const float mul = which == 0 ? 1.0f : p.scale;
-#pragma unroll 1
-                for (int c = 0; c < DH / 64; ++c) {
-                    const int col0 = ch * (DH / 2) + c * 32;
-                    uint32_t v[32];
-                    tmem_ld32(tmem_base + lane_addr + (which == 0 ? L::kDV : L::kDK) + col0, v);
-                    tc_wait_ld();
-                    if (which == 1 && c == DH / 64 - 1) {    // dV and dK have left TMEM: the next item may overwrite them
-                        tc_fence_before();
-                        mbar_arrive(bar(L::kAE));
-                    }
 #pragma unroll
-                    for (int gq = 0; gq < 4; ++gq) {
-                        float f[8];
+                for (int gq = 0; gq < kCols / 8; ++gq) {
+                    float f[8];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * gq + e]) * mul;
-                        const int col = col0 + gq * 8, blk = col >> 6, chunk = (col & 63) >> 3;
-                        *reinterpret_cast<uint4*>(stage + blk * 16384 + r * 128 + ((chunk ^ (r & 7)) << 4)) = pack8(f);
-                    }
+                    for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[which][8 * gq + e]) * mul;
+                    const int col = w4 * kCols + gq * 8, blk = col >> 6, chunk = (col & 63) >> 3;
+                    *reinterpret_cast<uint4*>(stage + blk * 16384 + r * 128 + ((chunk ^ (r & 7)) << 4)) = pack8(f);
                 }
             }
             fence_proxy_async();
-            named_bar_sync(1, 256);
+            named_bar_sync(1, 512);
             if (warp == 2 && lane == 0) {
                 const uint32_t ks = sbase + L::kK + buf * 2 * L::kKV, vs = ks + L::kKV;
                 for (int kb = 0; kb < L::kBlocks; ++kb) {
@@ -396,16 +419,36 @@ struct DqSmem {
     static constexpr int kBlocks = DH / 64;
     static constexpr int kTile = 128 * DH * 2;               // Q_t or dO_t
     static constexpr int kSub = 64 * DH * 2;                 // 64-key sub-tile of K or V
+    static constexpr int kStages = DH == 64 ? 5 : 2;         // K_v / V_v ring
+    static constexpr int kBufs = DH == 64 ? 3 : 2;           // S / dP buffers in TMEM: with 64-wide heads dQ leaves room for a third pair
+    static constexpr int kDQ = 128 * kBufs;                  // TMEM columns: S of buffer b at 128 b, dP at 128 b + 64, then dQ_A and dQ_B
     static constexpr int kQ = 0;                             // Q_A, Q_B, dO_A, dO_B
-    static constexpr int kKV = 4 * kTile;                    // 2 stages x (K_v, V_v)
-    static constexpr int kOut = kKV + 4 * kSub;              // dQ staging tile (shared by both query tiles)
+    static constexpr int kKV = 4 * kTile;                    // stage s holds K_v at kKV + s*2*kSub, V_v right after
+    static constexpr int kOut = kKV + kStages * 2 * kSub;    // dQ staging tile (shared by both query tiles)
     static constexpr int kBars = kOut + kTile;
+    // barriers (t = query tile): 0+t q_full | 2+t q_empty | kKF+s kv_full | kKE+s kv_empty | kSF+b s_full | kDF+b ds_full (256 arrivals)
+    //   kAF+t acc_full | kAE+t acc_empty (256 arrivals) | kST staging free | kIF+i item_full | kIE+i item_empty (17 arrivals)
+    static constexpr int kKF = 4, kKE = kKF + kStages, kSF = kKE + kStages, kDF = kSF + kBufs, kAF = kDF + kBufs, kAE = kAF + 2, kST = kAE + 2,
+                         kIF = kST + 1, kIE = kIF + 2, kNumBars = kIE + 2;
     static constexpr int kBytes = kBars + 256 + 1024;
+    static_assert(kNumBars <= 30 && kBytes <= 232448, "barriers and the words behind them share 256 bytes; shared memory of one CTA");
 };
 
 // Work items of the dQ kernel: one per (sequence, head, pair of query tiles), heaviest first, drawn
 // from a global counter by the producer thread (same scheme as the forward kernel).
-struct DqItem { int b, h, q0A, nA, nB; };
+//
+// The score tiles of an item form one sequence, A_0 B_0 A_1 B_1 ... (tile B ends on two more), whose position p, counted on
+// across items, takes buffer p % kBufs; the scores run kBufs - 1 positions ahead of the dQ products.  With a third buffer a
+// tile's next scores are there when its warps have finished with the last ones; with one buffer per
+// tile they waited out two products and their latencies each time.  Behind that lies the issuing thread, at 900 cycles a
+// position: hence the rings that are counted instead of divided.  Both backward kernels, us before -> with the second set of
+// warps and the narrower reads in dK/dV -> with this sequence -> with counted rings: 16 x 1024 x 16 heads x 64 198 -> 193 ->
+// 180 -> 174, 2 x 4096 x 16 x 64 290 -> 275 -> 274 -> 260; 128 wide (two buffers either way) 1 x 2048 x 64 x 128 240 -> 239 -> 238 -> 233.
+struct DqItem {
+    int b, h, q0A, nA, nB;
+    __device__ __forceinline__ int positions() const { return nA + nB; }
+    __device__ __forceinline__ int position(int t, int v) const { return nB == 0 ? v : t == 0 ? 2 * v : v < nA ? 2 * v + 1 : nA + v; }
+};
 __device__ __forceinline__ bool dq_item(const BwdParams& p, int idx, DqItem& it)
 {
     if (idx >= p.n_items) return false;
@@ -419,7 +462,7 @@ __device__ __forceinline__ bool dq_item(const BwdParams& p, int idx, DqItem& it)
 }
 
 template <int DH>
-__global__ void __launch_bounds__(kDqThreads, 1)
+__global__ void __launch_bounds__(kThreads, 1)
 attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64 x 128 rows
                       const __grid_constant__ CUtensorMap tmDO,   // dout, box 64 x 128 rows
                       const __grid_constant__ CUtensorMap tmKV,   // qkv, box 64 x 64 rows
@@ -431,12 +474,10 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(sm);
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::kBars);
-    // barrier map (t = query tile, s = ring stage):
-    //   0+t q_full | 2+t q_empty | 4+s kv_full | 6+s kv_empty | 8+t s_full | 10+t ds_full (256 arrivals)
-    //   12+t acc_full | 14+t acc_empty (256 arrivals) | 16 staging free | 17+i item_full | 19+i item_empty (17 arrivals)
+    // (barrier map: see DqSmem)
     const uint32_t bar0 = smem_u32(bars);
     auto bar = [&](int i) { return bar0 + 8u * i; };
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 22);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 30);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* item_slot = reinterpret_cast<volatile int*>(tmem_slot + 2);   // two entries
     // draws the next item number; past the end, counts this CTA as done and lets the last one clear the counters
@@ -460,22 +501,22 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
         }
     };
     auto load_kv = [&](const DqItem& it, int v, int s) {    // K_v and V_v (64 keys)
-        mbar_arrive_expect_tx(bar(4 + s), 2 * L::kSub);
+        mbar_arrive_expect_tx(bar(L::kKF + s), 2 * L::kSub);
         const uint32_t ks = sbase + L::kKV + s * 2 * L::kSub, vs = ks + L::kSub;
         for (int kb = 0; kb < L::kBlocks; ++kb) {
-            tma_load_2d(ks + kb * 8192, &tmKV, d + it.h * DH + kb * 64, it.b * p.S + v * 64, bar(4 + s));
-            tma_load_2d(vs + kb * 8192, &tmKV, 2 * d + it.h * DH + kb * 64, it.b * p.S + v * 64, bar(4 + s));
+            tma_load_2d(ks + kb * 8192, &tmKV, d + it.h * DH + kb * 64, it.b * p.S + v * 64, bar(L::kKF + s));
+            tma_load_2d(vs + kb * 8192, &tmKV, 2 * d + it.h * DH + kb * 64, it.b * p.S + v * 64, bar(L::kKF + s));
         }
     };
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 10; ++i) mbar_init(bar(i), 1);
-        mbar_init(bar(10), 256); mbar_init(bar(11), 256);
-        mbar_init(bar(12), 1); mbar_init(bar(13), 1);
-        mbar_init(bar(14), 256); mbar_init(bar(15), 256);
-        mbar_init(bar(16), 1);
-        mbar_init(bar(17), 1); mbar_init(bar(18), 1);
-        mbar_init(bar(19), 17); mbar_init(bar(20), 17);
+        for (int i = 0; i < L::kDF; ++i) mbar_init(bar(i), 1);
+        for (int i = 0; i < L::kBufs; ++i) mbar_init(bar(L::kDF + i), 256);
+        mbar_init(bar(L::kAF), 1); mbar_init(bar(L::kAF + 1), 1);
+        mbar_init(bar(L::kAE), 256); mbar_init(bar(L::kAE + 1), 256);
+        mbar_init(bar(L::kST), 1);
+        mbar_init(bar(L::kIF), 1); mbar_init(bar(L::kIF + 1), 1);
+        mbar_init(bar(L::kIE), 17); mbar_init(bar(L::kIE + 1), 17);
         *abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async();
@@ -491,7 +532,6 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
     const uint32_t tmem_base = *tmem_slot;
     grid_dep_wait();                                        // inputs come from the previous kernels
     grid_dep_launch();                                      // in this order: the dK/dV kernel starts without a wait of its own
-    // TMEM columns of tile t: S at t*256, dP at t*256 + 64, dQ at t*256 + 128
     // the producer and the MMA role are each the loop of one elected thread (see the forward kernel)
     if (warp == 0) {
         if (elect_one()) {
@@ -501,13 +541,12 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
             DqItem it;
             int idx = draw();
             item_slot[0] = idx;
-            mbar_arrive(bar(17));
+            mbar_arrive(bar(L::kIF));
             for (int k = 0; ok && dq_item(p, idx, it); ++k) {
                 const int n_kv = it.nB ? it.nB : it.nA;
                 for (int v = 0; v < n_kv && ok; ++v, ++n) {
-                    const int s = n & 1;
-                    const uint32_t ph = (n >> 1) & 1;
-                    if (!mbar_wait(bar(6 + s), ph ^ 1, abort_flag, p.status, 600)) { ok = false; break; }
+                    const int s = n % L::kStages;
+                    if (!mbar_wait(bar(L::kKE + s), ((n / L::kStages) & 1) ^ 1, abort_flag, p.status, 600)) { ok = false; break; }
                     load_kv(it, v, s);
                     if (v == 0) {
                         // Q_t / dO_t follow the first key sub-tile; their buffers are free once the
@@ -521,10 +560,10 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
                 }
                 if (!ok) break;
                 const int kn = k + 1;
-                if (!mbar_wait(bar(19 + (kn & 1)), ((kn >> 1) & 1) ^ 1, abort_flag, p.status, 602)) break;
+                if (!mbar_wait(bar(L::kIE + (kn & 1)), ((kn >> 1) & 1) ^ 1, abort_flag, p.status, 602)) break;
                 idx = draw();
                 item_slot[kn & 1] = idx;
-                mbar_arrive(bar(17 + (kn & 1)));
+                mbar_arrive(bar(L::kIF + (kn & 1)));
             }
         }
     } else if (warp == 1) {
@@ -533,12 +572,13 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
         constexpr uint32_t idesc_dq = make_idesc_bf16(128, DH, false, true);
         const uint32_t tb = tmem_base;
         const uint32_t sb = sbase;
-        auto issue_scores = [&](int t, int s) {             // S_t = Q_t K_v^T, dP_t = dO_t V_v^T
-            const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + t * L::kTile, 16, 1024);
-            const uint64_t dg = desc_advance(dq, 2 * L::kTile);
-            const uint64_t dk = make_smem_desc_sw128(sb + L::kKV + s * 2 * L::kSub, 16, 1024);
+        const uint64_t desc_q0 = make_smem_desc_sw128(sb + L::kQ, 16, 1024), desc_k0 = make_smem_desc_sw128(sb + L::kKV, 16, 1024);
+        const uint64_t desc_kt0 = make_smem_desc_sw128(sb + L::kKV, 8192, 1024);
+        auto issue_scores = [&](int t, int s, int b) {      // S = Q_t K_v^T, dP = dO_t V_v^T into buffer b
+            const uint64_t dq = desc_slot<L::kTile>(desc_q0, t), dg = desc_advance(dq, 2 * L::kTile);
+            const uint64_t dk = desc_slot<2 * L::kSub>(desc_k0, s);
             const uint64_t dv = desc_advance(dk, L::kSub);
-            const uint32_t dst = tb + t * 256;
+            const uint32_t dst = tb + b * 128;
             {
 #pragma unroll
                 for (int kb = 0; kb < L::kBlocks; ++kb)
@@ -552,12 +592,12 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
                     for (int kk = 0; kk < 4; ++kk)
                         umma_f16(dst + 64, desc_advance(dg, kb * 16384 + kk * 32), desc_advance(dv, kb * 8192 + kk * 32),
                                  idesc_sc, (kb | kk) ? 1u : 0u);
-                umma_commit(bar(8 + t));
+                umma_commit(bar(L::kSF + b));
             }
         };
-        auto issue_dq = [&](int t, int s, bool acc) {       // dQ_t += dS_t K_v (dS packed in the S columns)
-            const uint64_t dk = make_smem_desc_sw128(sb + L::kKV + s * 2 * L::kSub, 8192, 1024);
-            const uint32_t dst = tb + t * 256 + 128, src = tb + t * 256;
+        auto issue_dq = [&](int t, int s, int b, bool acc) {     // dQ_t += dS K_v (dS packed in the S columns of buffer b)
+            const uint64_t dk = desc_slot<2 * L::kSub>(desc_kt0, s);
+            const uint32_t dst = tb + L::kDQ + t * DH, src = tb + b * 128;
             {
                 // dS packed bf16: keys 0..31 in columns 0..15 of S_t, keys 32..63 in columns 32..47
                 umma_f16_ta(dst, src, dk, idesc_dq, acc ? 1u : 0u);
@@ -572,70 +612,50 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
         auto wait = [&](int b, uint32_t parity, int site) {
             return mbar_wait(bar(b), parity, abort_flag, p.status, site);
         };
-        uint32_t n = 0;                                     // key sub-tiles consumed before this item
-        uint32_t nd[2] = {0, 0};                            // dS tiles consumed per query tile
-        uint32_t qn[2] = {0, 0};                            // items each query tile took part in
+        Ring<L::kStages> ss, sd;                            // stage of the next score tile / dQ product
+        Ring<L::kBufs> bs, bd;                              // and its buffer
+        uint32_t nb = 0;                                    // items that had a tile B
         bool ok = true;
         DqItem it;
         for (int k = 0; ok; ++k) {
-            if (!wait(17 + (k & 1), (k >> 1) & 1, 616)) break;
+            if (!wait(L::kIF + (k & 1), (k >> 1) & 1, 616)) break;
             const int idx = item_slot[k & 1];
-            mbar_arrive(bar(19 + (k & 1)));
+            mbar_arrive(bar(L::kIE + (k & 1)));
             if (!dq_item(p, idx, it)) break;
-            const int nA = it.nA, nB = it.nB, n_kv = nB ? nB : nA;
-            {
-                const int s = n & 1;
-                const uint32_t ph = (n >> 1) & 1;
-                ok = wait(4 + s, ph, 611) && wait(0, qn[0] & 1, 610);
-                if (!ok) break;
+            const int nA = it.nA, nB = it.nB, n_pos = it.positions();
+            constexpr int kAhead = L::kBufs - 1;
+            // A_0 B_0 A_1 B_1 ...; without a tile B, and past the end of A, one after the other
+            auto step = [&](int& t, int& v, Ring<L::kStages>& st) {
+                if (t == 0 && nB) { t = 1; return; }
+                ++v;
+                st.next();
+                t = v < nA ? 0 : 1;
+            };
+            int ts = 0, vs = 0, td = 0, vd = 0;
+            auto scores = [&]() {
+                if ((ts == 0 || vs >= nA) && !wait(L::kKF + ss.i, ss.parity, 611)) return false;      // first use of the stage
+                if (vs == 0 && !wait(ts, (ts ? nb : static_cast<uint32_t>(k)) & 1, 610)) return false;
                 tc_fence_after();
-                issue_scores(0, s);
-                if (nB) {
-                    if (!wait(1, qn[1] & 1, 617)) { ok = false; break; }
-                    tc_fence_after();
-                    issue_scores(1, s);
-                }
+                issue_scores(ts, ss.i, bs.i);
+                if (vs + 1 == (ts ? nB : nA)) commit(2 + ts);        // Q_t / dO_t are not needed again
+                step(ts, vs, ss);
+                bs.next();
+                return true;
+            };
+            for (int i = 0; i < kAhead && i < n_pos && ok; ++i) ok = scores();
+            for (int i = 0; i < n_pos && ok; ++i) {
+                if (i + kAhead < n_pos && !scores()) { ok = false; break; }
+                if (!wait(L::kDF + bd.i, bd.parity, 612)) { ok = false; break; }
+                // the previous item's dQ_t must have been read out before it is overwritten
+                if (vd == 0 && !wait(L::kAE + td, ((td ? nb : static_cast<uint32_t>(k)) & 1) ^ 1, 618)) { ok = false; break; }
+                tc_fence_after();
+                issue_dq(td, sd.i, bd.i, vd > 0);
+                if (vd + 1 == (td ? nB : nA)) commit(L::kAF + td);
+                if (td == 1 || nB == 0) commit(L::kKE + sd.i);       // K_v / V_v stage free
+                step(td, vd, sd);
+                bd.next();
             }
-            for (int v = 0; v < n_kv && ok; ++v) {
-                const uint32_t nv = n + v, nn = nv + 1;
-                const int s = nv & 1, sn = nn & 1;
-                const uint32_t phn = (nn >> 1) & 1;
-                bool k_waited = false;
-                if (v < nA) {
-                    if (!wait(10, nd[0] & 1, 612)) { ok = false; break; }
-                    ++nd[0];
-                    // the previous item's dQ_A must have been read out before it is overwritten
-                    if (v == 0 && !wait(14, (qn[0] & 1) ^ 1, 618)) { ok = false; break; }
-                    tc_fence_after();
-                    issue_dq(0, s, v > 0);
-                    if (v == nA - 1) commit(12);
-                }
-                if (v + 1 < nA) {
-                    if (!wait(4 + sn, phn, 613)) { ok = false; break; }
-                    k_waited = true;
-                    tc_fence_after();
-                    issue_scores(0, sn);
-                    if (v + 2 == nA) commit(2);             // Q_A / dO_A are not needed again
-                }
-                if (v < nB) {
-                    if (!wait(11, nd[1] & 1, 614)) { ok = false; break; }
-                    ++nd[1];
-                    if (v == 0 && !wait(15, (qn[1] & 1) ^ 1, 619)) { ok = false; break; }
-                    tc_fence_after();
-                    issue_dq(1, s, v > 0);
-                    if (v == nB - 1) commit(13);
-                }
-                commit(6 + s);                              // K_v / V_v stage free
-                if (v + 1 < nB) {
-                    if (!k_waited && !wait(4 + sn, phn, 615)) { ok = false; break; }
-                    tc_fence_after();
-                    issue_scores(1, sn);
-                    if (v + 2 == nB) commit(3);
-                }
-            }
-            n += n_kv;
-            ++qn[0];
-            if (nB) ++qn[1];
+            if (nB) ++nb;
         }
         }
     } else {
@@ -646,34 +666,44 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
         const int r = q * 32 + lane;
         const bool leader = hf == 0 && q == 2 && lane == 0;
         const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
-        const uint32_t s_addr = tmem_base + lane_addr + t * 256 + hf * 32;       // my S columns; dP is 64 further
-        const uint32_t o_addr = tmem_base + lane_addr + t * 256 + 128 + hf * (DH / 2);
+        const uint32_t o_addr = tmem_base + lane_addr + L::kDQ + t * DH + hf * (DH / 2);
         const float sl2 = p.scale * kLog2e;
-        uint32_t ns = 0, qn = 0;                            // score tiles and items this query tile has seen
+        uint32_t p0 = 0, nb = 0;                            // position of this item's first score tile; items that had a tile B
         uint32_t u_base = 0;                                // uses of the staging tile before this item
         bool ok = true;
         DqItem it;
         for (int k = 0; ok; ++k) {
-            ok = mbar_wait(bar(17 + (k & 1)), (k >> 1) & 1, abort_flag, p.status, 622);
+            ok = mbar_wait(bar(L::kIF + (k & 1)), (k >> 1) & 1, abort_flag, p.status, 622);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             const int idx = item_slot[k & 1];
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(19 + (k & 1)));
+            if (lane == 0) mbar_arrive(bar(L::kIE + (k & 1)));
             if (!dq_item(p, idx, it)) break;
             const int n_t = t == 0 ? it.nA : it.nB;
             const uint32_t u = u_base + t;                  // staging order: A(k), B(k), A(k+1), ...
             u_base += it.nB ? 2 : 1;
-            if (n_t == 0) continue;
+            // Before an item's first s_full is waited for, all score tiles in front of it must be complete: a barrier may then be one
+            // phase behind at most.  Tile A's warps see to it at the end of an item, tile B's of one that has no tile B here.
+            if (n_t == 0) {
+                ok = mbar_wait(bar(L::kAF), k & 1, abort_flag, p.status, 624);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                p0 += it.positions();
+                continue;
+            }
             const int q0 = it.q0A + t * 128;
             const size_t row_idx = (static_cast<size_t>(it.b) * p.H + it.h) * p.S + q0 + r;
             const float lse2 = p.lse[row_idx] * kLog2e, dlt = p.delta[row_idx];
             const uint64_t sl2x2 = pack_f32x2(sl2, sl2), nlse2 = pack_f32x2(-lse2, -lse2), ndlt = pack_f32x2(-dlt, -dlt);
-            for (int v = 0; v < n_t; ++v, ++ns) {
-                ok = mbar_wait(bar(8 + t), ns & 1, abort_flag, p.status, 620);
+            for (int v = 0; v < n_t; ++v) {
+                const uint32_t ps = p0 + it.position(t, v);
+                const int b = ps % L::kBufs;
+                ok = mbar_wait(bar(L::kSF + b), (ps / L::kBufs) & 1, abort_flag, p.status, 620);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
+                const uint32_t s_addr = tmem_base + lane_addr + b * 128 + hf * 32;   // my S columns; dP is 64 further
                 const int key0 = v * 64 + hf * 32;            // first key of my slice
                 const bool diag = key0 + 31 > q0;            // some keys of this slice are masked for some rows
 #pragma unroll
@@ -699,14 +729,14 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
                 }
                 tc_wait_st();
                 tc_fence_before();
-                mbar_arrive(bar(10 + t));
+                mbar_arrive(bar(L::kDF + b));
             }
             if (ok) {
-                ok = mbar_wait(bar(12 + t), qn & 1, abort_flag, p.status, 621);
+                ok = mbar_wait(bar(L::kAF + t), (t ? nb : static_cast<uint32_t>(k)) & 1, abort_flag, p.status, 621);
                 ok = __all_sync(0xffffffffu, ok);
             }
             if (ok) {
-                ok = mbar_wait(bar(16), (u & 1) ^ 1, abort_flag, p.status, 623);    // the previous user's store has read the staging tile
+                ok = mbar_wait(bar(L::kST), (u & 1) ^ 1, abort_flag, p.status, 623);    // the previous user's store has read the staging tile
                 ok = __all_sync(0xffffffffu, ok);
             }
             if (!ok) break;
@@ -719,7 +749,7 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
                 tc_wait_ld();
                 if (c == DH / 64 - 1) {                     // this thread's part of dQ_t has left TMEM
                     tc_fence_before();
-                    mbar_arrive(bar(14 + t));
+                    mbar_arrive(bar(L::kAE + t));
                 }
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
@@ -737,9 +767,15 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
                     tma_store_2d(&tmOut, sbase + L::kOut + kb * 16384, it.h * DH + kb * 64, it.b * p.S + q0);
                 bulk_commit();
                 bulk_wait_read0();                          // the staging tile may be written again
-                mbar_arrive(bar(16));
+                mbar_arrive(bar(L::kST));
             }
-            ++qn;
+            if (t == 0 && it.nB) {
+                ok = mbar_wait(bar(L::kAF + 1), nb & 1, abort_flag, p.status, 625);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+            }
+            p0 += it.positions();
+            if (it.nB) ++nb;
         }
         if (leader) bulk_wait0();
     }
@@ -809,8 +845,8 @@ const char* launch_attention_bwd_dq(Runtime* rt, const void* qkv, const void* do
     p.sched = status->sched + 2;
     dim3 grid(p.n_items < rt->sm_count ? p.n_items : rt->sm_count);
     const cudaError_t e2 = dh == 64
-        ? launch_k(attn_bwd_dq_tc_kernel<64>, grid, dim3(kDqThreads), DqSmem<64>::kBytes, stream, tmQ, tmDO, tmKV, tmOut, p)
-        : launch_k(attn_bwd_dq_tc_kernel<128>, grid, dim3(kDqThreads), DqSmem<128>::kBytes, stream, tmQ, tmDO, tmKV, tmOut, p);
+        ? launch_k(attn_bwd_dq_tc_kernel<64>, grid, dim3(kThreads), DqSmem<64>::kBytes, stream, tmQ, tmDO, tmKV, tmOut, p)
+        : launch_k(attn_bwd_dq_tc_kernel<128>, grid, dim3(kThreads), DqSmem<128>::kBytes, stream, tmQ, tmDO, tmKV, tmOut, p);
     return e2 == cudaSuccess ? nullptr : "attention bwd (dq) launch failed";
 }
 

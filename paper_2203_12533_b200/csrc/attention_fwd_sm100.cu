@@ -231,10 +231,11 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         constexpr uint32_t idesc_pv = make_idesc_bf16(128, DH, false, true);
         const uint32_t tb = tmem_base;
         const uint32_t sb = sbase;
+        const uint64_t desc_q0 = make_smem_desc_sw128(sb + L::kQ, 16, 1024), desc_k0 = make_smem_desc_sw128(sb + L::kK, 16, 1024);
+        const uint64_t desc_v0 = make_smem_desc_sw128(sb + L::kV, 16384, 1024);
         // S_t = Q K^T from a Q buffer and K stage s
         auto issue_s = [&](int t, int s, int qbuf) {
-            const uint64_t dq = make_smem_desc_sw128(sb + L::kQ + qbuf * L::kTile, 16, 1024);
-            const uint64_t dk = make_smem_desc_sw128(sb + L::kK + s * L::kTile, 16, 1024);
+            const uint64_t dq = desc_slot<L::kTile>(desc_q0, qbuf), dk = desc_slot<L::kTile>(desc_k0, s);
             const uint32_t dst = tb + t * 128;
             {
 #pragma unroll
@@ -249,7 +250,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         // O_t (+)= P_t V from V stage s; P_t is bf16 packed over the S columns it came from: the 16
         // keys of step ks sit in 8 columns at (ks/4)*64 + ((ks%4)/2)*32 + (ks%2)*8 of S_t
         auto issue_pv = [&](int t, int s, bool acc) {
-            const uint64_t dv = make_smem_desc_sw128(sb + L::kV + s * L::kTile, 16384, 1024);
+            const uint64_t dv = desc_slot<L::kTile>(desc_v0, s);
             const uint32_t dst = tb + 256 + t * 128, src = tb + t * 128;
             {
                 umma_f16_ta(dst, src, dv, idesc_pv, acc ? 1u : 0u);

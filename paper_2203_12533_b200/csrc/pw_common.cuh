@@ -290,6 +290,23 @@ __device__ __forceinline__ void umma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, ui
         : "memory");
 }
 // 32 lanes x 16 consecutive columns.
+// 16 lanes x 32 fp32 columns as an mma.sync accumulator holds them: thread i gets, for every group g of 8 columns, columns
+// 8 g + 2 (i % 4), + 1 of lane i / 4 in r[4 g], r[4 g + 1] and of lane i / 4 + 8 in r[4 g + 2], r[4 g + 3].
+__device__ __forceinline__ void tmem_ld_16x256_x4(uint32_t taddr, uint32_t* r)
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
+// 16 lanes x 16 columns, the packed pairs of the above: column 4 g + i % 4 of lane i / 4 from r[2 g], of lane i / 4 + 8 from r[2 g + 1].
+__device__ __forceinline__ void tmem_st_16x128_x4(uint32_t taddr, const uint32_t* r)
+{
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 :: "r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r)
 {
     asm volatile(
@@ -456,7 +473,17 @@ __device__ __forceinline__ uint64_t make_smem_desc_sw128(uint32_t saddr, uint32_
 // Descriptor of the same operand starting `bytes` further on (bytes a multiple of 16, the new
 // start still inside the 256 KB shared-memory window, so the add never carries out of the
 // address field).  Lets the MMA-issuing thread build a descriptor once and step it with one add.
-__device__ __forceinline__ uint64_t desc_advance(uint64_t d, uint32_t bytes) { return d + (bytes >> 4); }
+__device__ __forceinline__ uint64_t desc_advance(uint64_t d, uint32_t bytes)
+{
+    return (d & 0xffffffff00000000ull) | (static_cast<uint32_t>(d) + (bytes >> 4));     // (one 32-bit add)
+}
+// The same for slot i of an array of BYTES each.
+template <uint32_t BYTES>
+__device__ __forceinline__ uint64_t desc_slot(uint64_t d, uint32_t i)
+{
+    static_assert(BYTES % 16 == 0, "descriptors address 16-byte units");
+    return (d & 0xffffffff00000000ull) | (static_cast<uint32_t>(d) + i * (BYTES >> 4));
+}
 
 // Instruction descriptor for kind::f16 with bf16 A/B and fp32 D.
 //   [4,6) D format (1 = f32)  [7,10) A format (1 = bf16)  [10,13) B format (1 = bf16)

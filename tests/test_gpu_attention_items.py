@@ -1,9 +1,9 @@
-"""Attention forward on both sides of the launcher's choice between pairs of query tiles and single ones (148 SMs)."""
+"""Attention forward and backward with few and many work items; forward on both sides of the launcher's choice between pairs of query tiles and single ones (148 SMs)."""
 import numpy as np
 import pytest
 import torch
 
-from tests.gpu_util import ACT_TOL, ELEM_ACT, bf16_randn, elem_check, guard_alloc, np64, rel_l2
+from tests.gpu_util import ACT_TOL, ELEM_ACT, GRAD_TOL, bf16_randn, elem_check, guard_alloc, np64, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -41,3 +41,37 @@ def test_attention_fwd_items(pw, oracle64, B, S, H, dh):
     elem_check(o, ow, "o", **ELEM_ACT)
     # scores are sums of dh products of exact bf16 values, good to dh * 2^-24 of sum |q k|, below 2^-13 here; 1e-3 as elsewhere
     assert np.abs(lse.double().cpu().numpy() - lw).max() < 1e-3
+
+
+@pytest.mark.parametrize("B,S,H,dh", [
+    (1, 128, 2, 64),                              # one query tile, no second one
+    (4, 640, 20, 64), (5, 640, 10, 128),          # several items to a CTA, the first of them with a single query tile
+    (3, 768, 17, 64)])                            # and with pairs only: buffers and rings of three and five go round
+def test_attention_bwd_items(pw, oracle64, B, S, H, dh):
+    g = torch.Generator().manual_seed(S + H + 1)
+    d = H * dh
+    qkv, dout = bf16_randn((B * S, 3 * d), g), bf16_randn((B * S, d), g)
+    q, do = qkv.cuda(), dout.cuda()
+    o = torch.empty((B * S, d), dtype=torch.bfloat16, device="cuda")
+    lse = torch.empty((B, H, S), device="cuda")
+    delta = torch.empty((B, H, S), device="cuda")
+    pw.op_attention_fwd(q, B, S, H, dh, o, lse)
+    got = []
+    for _ in range(2):
+        dqkv, check = guard_alloc((B * S, 3 * d), torch.bfloat16)
+        pw.op_attention_bwd(q, o, do, lse, B, S, H, dh, dqkv, delta)
+        torch.cuda.synchronize()
+        assert pw.op_status() == (0, 0)
+        check()
+        got.append(dqkv)
+    assert torch.equal(got[0], got[1])
+    dw = oracle64.attn_bwd(np64(qkv), np64(dout), B, S, H, dh)
+    for name, sl in (("dq", slice(0, d)), ("dk", slice(d, 2 * d)), ("dv", slice(2 * d, 3 * d))):
+        assert rel_l2(got[0][:, sl], dw[:, sl]) < GRAD_TOL, name
+        # The errors are bf16 roundings of P, dS and the result, relative and independent, so every 128 x dh tile keeps the
+        # bound of the whole up to the scatter of its 2^13 or more errors; a wrong tile is off by about 1.  (A bound for single
+        # elements fits the 5e4 of the small tests; the worst of these 3e6 lies a few percent further out in the tail.)
+        diff = (got[0][:, sl].double().cpu().numpy() - dw[:, sl]).reshape(B * S // 128, 128, H, dh)
+        want = np.asarray(dw[:, sl]).reshape(diff.shape)
+        tile = np.sqrt((diff ** 2).sum((1, 3)) / (want ** 2).sum((1, 3)))
+        assert tile.max() < 2 * GRAD_TOL, (name, tile.max())
