@@ -44,15 +44,6 @@ __device__ __forceinline__ void tmem_ld_n(uint32_t taddr, uint32_t* r)
     else tmem_ld32(taddr, r);
 }
 
-// Slot of a ring of N and the parity of its barriers, counted on one by one: the issuing thread, whose every instruction
-// counts, divides nothing.
-template <int N>
-struct Ring {
-    int i = 0;
-    uint32_t parity = 0;
-    __device__ __forceinline__ void next() { if (++i == N) { i = 0; parity ^= 1; } }
-};
-
 // ------------------------------------------------------------------------------------------- dK, dV
 template <int DH>
 struct KvSmem {

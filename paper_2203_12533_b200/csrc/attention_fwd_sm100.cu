@@ -1,14 +1,17 @@
 // Causal attention forward on the 5th-generation tensor cores (tcgen05 + TMEM + TMA).
 //
 // One CTA owns two adjacent 128-query tiles (A, B) of one (sequence, head) and streams the
-// 128-key tiles up to the diagonal through a 2-stage K ring and a 2-stage V ring.  10 warps:
+// 128-key tiles up to the diagonal through a K ring and a V ring.  18 warps:
 //   warp 0      TMA producer: Q once, then K_j / V_j.
 //   warp 1      MMA issuer, owns the TMEM allocation (512 columns):
-//                 S_t = Q_t K_j^T   (128x128, fp32)  -> columns t*128
-//                 O_t += P_t V_j    (128xdh,  fp32)  -> columns 256 + t*128, P_t read from TMEM
-//               issued so that the tensor pipe works on one tile while the other is in softmax:
-//               PV_A(j), S_A(j+1), PV_B(j), S_B(j+1), ...
-//   warps 2..5  softmax of tile A, warps 6..9 softmax of tile B (thread = one query row = one TMEM
+//                 S   = Q_t K_j^T   (128x128, fp32)  -> buffer of 128 columns
+//                 O_t += P V_j      (128xdh,  fp32)  -> columns behind the buffers, P read from TMEM
+//               The score tiles form one sequence, A_0 B_0 A_1 B_1 ..., whose position p, counted on
+//               across items, takes buffer p % kBufs, as soon as the P V product of p - kBufs has been issued.  With 64-wide heads O leaves room for a third buffer: a tile's next scores
+//               are there when its warps have finished with the last ones.
+//               With one buffer per tile -> so, us (B x S x heads x dh): 2 x 4096 x 16 x 64 102 -> 93, 16 x 1024 x
+//               16 x 64 71 -> 66, 2 x 1024 x 16 x 64 15.1 -> 13.8; 128 wide, two buffers, 1 x 2048 x 64 x 128 72.4 -> 73.5.
+//   warps 2..9  softmax of tile A, warps 10..17 softmax of tile B (two threads per query row = TMEM
 //               lane): row max, exp2 with the 1/sqrt(dh) scale folded in, row sum, P written back
 //               as packed bf16 over the S columns it came from.  The running maximum is only
 //               advanced when it grows by more than 8 (in log2 units); only then is O rescaled in
@@ -30,12 +33,22 @@ template <int DH>
 struct FwdSmem {
     static constexpr int kBlocks = DH / 64;                 // 64-column (128-byte) blocks per row
     static constexpr int kTile = 128 * DH * 2;              // one 128-row tile of Q, K or V
+    static constexpr int kStages = DH == 64 ? 3 : 2;        // K and V rings
+    static constexpr int kBufs = DH == 64 ? 3 : 2;          // score buffers in TMEM: buffer b at column 128 b, then O_A and O_B
+    static constexpr int kTO = 128 * kBufs;
     static constexpr int kQ = 0;                            // two Q tiles
-    static constexpr int kK = 2 * kTile;                    // two K stages
-    static constexpr int kV = 4 * kTile;                    // two V stages
-    static constexpr int kO = 6 * kTile;                    // output staging tile (shared by both query tiles)
-    static constexpr int kBars = 7 * kTile;
-    static constexpr int kXch = kBars + 256;                // per-row exchange between the two threads of a row: [tile][half][128] fp32
+    static constexpr int kK = 2 * kTile;                    // K stages
+    static constexpr int kV = kK + kStages * kTile;         // V stages
+    static constexpr int kO = kV + kStages * kTile;         // output staging tile (shared by both query tiles)
+    // barriers (t = query tile / slot, s = ring stage, b = score buffer): 0+t q_full | 2+t q_empty | kKF+s, kKE+s k_full, k_empty |
+    //   kVF+s, kVE+s v_full, v_empty | kSF+b s_full | kPF+b p_full (256 arrivals) | kOF+t o_full | kOE+t o_empty (256 arrivals, 512
+    //   with SPLIT) | kST staging free | kIF+i item_full | kIE+i item_empty (17 arrivals: MMA warp + 16 softmax warps)
+    static constexpr int kKF = 4, kKE = kKF + kStages, kVF = kKE + kStages, kVE = kVF + kStages, kSF = kVE + kStages, kPF = kSF + kBufs,
+                         kOF = kPF + kBufs, kOE = kOF + 2, kST = kOE + 2, kIF = kST + 1, kIE = kIF + 2, kNumBars = kIE + 2;
+    static constexpr int kBars = kO + kTile;
+    static constexpr int kBarBytes = DH == 64 ? 288 : 256;
+    static_assert(kNumBars * 8 + 16 <= kBarBytes, "barriers and the words behind them");
+    static constexpr int kXch = kBars + kBarBytes;          // per-row exchange between the two threads of a row: [tile][half][128] fp32
     static constexpr int kEnd = kXch + 2 * 2 * 128 * 4;
     static constexpr int kBytes = kEnd + ((kEnd + 1024 <= 232448) ? 1024 : 232448 - kEnd);   // alignment slack (checked in the kernel)
 };
@@ -57,6 +70,13 @@ struct FwdParams {
 // the causal triangle balances itself over the CTAs.  Every CTA draws exactly one number past the
 // end; the last CTA to do so clears the counters for the next launch.
 struct FwdItem { int b, h, q0A, nA, nB, n_kv; };             // key tiles: each slot's, and those that are loaded
+// place of slot t's j-th score tile in its item's sequence
+template <bool SPLIT>
+__device__ __forceinline__ int fwd_position(const FwdItem& it, int t, int j)
+{
+    if (SPLIT) return 2 * j + t;
+    return it.nB == 0 ? j : t == 0 ? 2 * j : j < it.nA ? 2 * j + 1 : it.nA + j;
+}
 template <bool SPLIT>
 __device__ __forceinline__ bool fwd_item(const FwdParams& p, int idx, FwdItem& it)
 {
@@ -94,13 +114,10 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(sm);
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::kBars);
-    // barrier map (t = query tile, s = ring stage):
-    //   0+t q_full | 2+t q_empty | 4+s k_full | 6+s k_empty | 8+s v_full | 10+s v_empty
-    //   12+t s_full | 14+t p_full (128 arrivals) | 16+t o_full | 18+t o_empty (128 arrivals) | 20 staging free
-    //   21+i item_full | 23+i item_empty (17 arrivals: MMA warp + 16 softmax warps)
+    // (barrier map: see FwdSmem)
     const uint32_t bar0 = smem_u32(bars);
     auto bar = [&](int i) { return bar0 + 8u * i; };
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 26);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kNumBars);
     volatile int* item_slot = reinterpret_cast<volatile int*>(tmem_slot + 2);   // two entries
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     // draws the next item number; past the end, counts this CTA as done and lets the last one clear the counters
@@ -127,26 +144,26 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
                         it.b * p.S + it.q0A + (SPLIT ? 0 : t * 128), bar(0 + t));
     };
     auto load_k = [&](const FwdItem& it, int j, int s) {
-        mbar_arrive_expect_tx(bar(4 + s), L::kTile);
+        mbar_arrive_expect_tx(bar(L::kKF + s), L::kTile);
         for (int kb = 0; kb < L::kBlocks; ++kb)
             tma_load_2d(sbase + L::kK + s * L::kTile + kb * 16384, &tmQKV, d + it.h * DH + kb * 64,
-                        it.b * p.S + j * 128, bar(4 + s));
+                        it.b * p.S + j * 128, bar(L::kKF + s));
     };
     auto load_v = [&](const FwdItem& it, int j, int s) {
-        mbar_arrive_expect_tx(bar(8 + s), L::kTile);
+        mbar_arrive_expect_tx(bar(L::kVF + s), L::kTile);
         for (int kb = 0; kb < L::kBlocks; ++kb)
             tma_load_2d(sbase + L::kV + s * L::kTile + kb * 16384, &tmQKV, 2 * d + it.h * DH + kb * 64,
-                        it.b * p.S + j * 128, bar(8 + s));
+                        it.b * p.S + j * 128, bar(L::kVF + s));
     };
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 14; ++i) mbar_init(bar(i), 1);
-        mbar_init(bar(14), 256); mbar_init(bar(15), 256);
-        mbar_init(bar(16), 1); mbar_init(bar(17), 1);
-        mbar_init(bar(18), SPLIT ? 512 : 256); mbar_init(bar(19), SPLIT ? 512 : 256);
-        mbar_init(bar(20), 1);
-        mbar_init(bar(21), 1); mbar_init(bar(22), 1);
-        mbar_init(bar(23), 17); mbar_init(bar(24), 17);
+        for (int i = 0; i < L::kPF; ++i) mbar_init(bar(i), 1);
+        for (int i = 0; i < L::kBufs; ++i) mbar_init(bar(L::kPF + i), 256);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar(L::kOF + i), 1); mbar_init(bar(L::kOE + i), SPLIT ? 512 : 256);
+            mbar_init(bar(L::kIF + i), 1); mbar_init(bar(L::kIE + i), 17);
+        }
+        mbar_init(bar(L::kST), 1);
         *abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async();
@@ -169,60 +186,41 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
     // `if (lane == 0)` about 300.
     if (warp == 0) {
         if (elect_one()) {
-            uint32_t n = 0;                                 // key/value tiles requested so far
+            Ring<L::kStages> rk, rv;                        // the next K / V tile's stage
             uint32_t qn[2] = {0, 0};                        // items each query tile took part in
             bool ok = true;
             FwdItem it;
             int idx = draw();
             item_slot[0] = idx;
-            mbar_arrive(bar(21));
+            mbar_arrive(bar(L::kIF));
             for (int k = 0; ok && fwd_item<SPLIT>(p, idx, it); ++k) {
-                const int n_kv = it.n_kv;
-                if (SPLIT) {
-                    // K_0 Q K_1 V_0 K_2 V_1 ...: the two slots start on their own key tiles.  Q alternates between its two buffers.
-                    auto next_k = [&](int j) {
-                        const uint32_t m = n + j;
-                        if (!mbar_wait(bar(6 + (m & 1)), ((m >> 1) & 1) ^ 1, abort_flag, p.status, 400)) return false;
-                        load_k(it, j, m & 1);
-                        return true;
-                    };
-                    const int t = k & 1;
-                    ok = next_k(0) && mbar_wait(bar(2 + t), ((k >> 1) & 1) ^ 1, abort_flag, p.status, 402);
-                    if (!ok) break;
+                auto next_k = [&](int j) {
+                    if (!mbar_wait(bar(L::kKE + rk.i), rk.parity ^ 1, abort_flag, p.status, 400)) return false;
+                    load_k(it, j, rk.i);
+                    rk.next();
+                    return true;
+                };
+                auto next_q = [&](int t, uint32_t use) {
+                    if (!mbar_wait(bar(2 + t), (use & 1) ^ 1, abort_flag, p.status, 402)) return false;
                     load_q(it, t);
-                    for (int j = 0; j < n_kv && ok; ++j) {
-                        if (j + 1 < n_kv && !next_k(j + 1)) { ok = false; break; }
-                        const uint32_t m = n + j;
-                        if (!mbar_wait(bar(10 + (m & 1)), ((m >> 1) & 1) ^ 1, abort_flag, p.status, 401)) { ok = false; break; }
-                        load_v(it, j, m & 1);
-                    }
-                    n += n_kv;
-                }
-                for (int j = 0; !SPLIT && j < n_kv && ok; ++j, ++n) {
-                    const int s = n & 1;
-                    const uint32_t ph = (n >> 1) & 1;
-                    if (!mbar_wait(bar(6 + s), ph ^ 1, abort_flag, p.status, 400)) { ok = false; break; }
-                    load_k(it, j, s);
-                    if (j == 0) {
-                        // Q follows the first key tile; its buffer is free once the previous item's
-                        // last S = Q K^T has been computed.
-                        for (int t = 0; t < (it.nB ? 2 : 1) && ok; ++t) {
-                            if (!mbar_wait(bar(2 + t), (qn[t] & 1) ^ 1, abort_flag, p.status, 402)) { ok = false; break; }
-                            load_q(it, t);
-                            ++qn[t];
-                        }
-                        if (!ok) break;
-                    }
-                    if (!mbar_wait(bar(10 + s), ph ^ 1, abort_flag, p.status, 401)) { ok = false; break; }
-                    load_v(it, j, s);
+                    return true;
+                };
+                // K_0 Q K_1 V_0 K_2 V_1 ...: Q's buffer is free once the previous item's last S = Q K^T has been computed
+                // (SPLIT: Q alternates between its two buffers)
+                ok = next_k(0) && (SPLIT ? next_q(k & 1, k >> 1) : next_q(0, qn[0]++) && (it.nB == 0 || next_q(1, qn[1]++)));
+                for (int j = 0; j < it.n_kv && ok; ++j) {
+                    if (j + 1 < it.n_kv && !next_k(j + 1)) { ok = false; break; }
+                    if (!mbar_wait(bar(L::kVE + rv.i), rv.parity ^ 1, abort_flag, p.status, 401)) { ok = false; break; }
+                    load_v(it, j, rv.i);
+                    rv.next();
                 }
                 if (!ok) break;
                 // next item: its number goes into slot (k+1)&1 once every role has read what was there
                 const int kn = k + 1;
-                if (!mbar_wait(bar(23 + (kn & 1)), ((kn >> 1) & 1) ^ 1, abort_flag, p.status, 403)) break;
+                if (!mbar_wait(bar(L::kIE + (kn & 1)), ((kn >> 1) & 1) ^ 1, abort_flag, p.status, 403)) break;
                 idx = draw();
                 item_slot[kn & 1] = idx;
-                mbar_arrive(bar(21 + (kn & 1)));
+                mbar_arrive(bar(L::kIF + (kn & 1)));
             }
         }
     } else if (warp == 1) {
@@ -233,31 +231,27 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         const uint32_t sb = sbase;
         const uint64_t desc_q0 = make_smem_desc_sw128(sb + L::kQ, 16, 1024), desc_k0 = make_smem_desc_sw128(sb + L::kK, 16, 1024);
         const uint64_t desc_v0 = make_smem_desc_sw128(sb + L::kV, 16384, 1024);
-        // S_t = Q K^T from a Q buffer and K stage s
-        auto issue_s = [&](int t, int s, int qbuf) {
+        // S = Q K^T from a Q buffer and K stage s into score buffer b
+        auto issue_s = [&](int s, int b, int qbuf) {
             const uint64_t dq = desc_slot<L::kTile>(desc_q0, qbuf), dk = desc_slot<L::kTile>(desc_k0, s);
-            const uint32_t dst = tb + t * 128;
-            {
+            const uint32_t dst = tb + b * 128;
 #pragma unroll
-                for (int kb = 0; kb < L::kBlocks; ++kb)
+            for (int kb = 0; kb < L::kBlocks; ++kb)
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        umma_f16(dst, desc_advance(dq, kb * 16384 + kk * 32), desc_advance(dk, kb * 16384 + kk * 32),
-                                 idesc_s, (kb | kk) ? 1u : 0u);
-                umma_commit(bar(12 + t));
-            }
+                for (int kk = 0; kk < 4; ++kk)
+                    umma_f16(dst, desc_advance(dq, kb * 16384 + kk * 32), desc_advance(dk, kb * 16384 + kk * 32),
+                             idesc_s, (kb | kk) ? 1u : 0u);
+            umma_commit(bar(L::kSF + b));
         };
-        // O_t (+)= P_t V from V stage s; P_t is bf16 packed over the S columns it came from: the 16
-        // keys of step ks sit in 8 columns at (ks/4)*64 + ((ks%4)/2)*32 + (ks%2)*8 of S_t
-        auto issue_pv = [&](int t, int s, bool acc) {
+        // O_t (+)= P V from V stage s; P is bf16 packed over the S columns it came from: the 16
+        // keys of step ks sit in 8 columns at (ks/4)*64 + ((ks%4)/2)*32 + (ks%2)*8 of its buffer
+        auto issue_pv = [&](int t, int s, int b, bool acc) {
             const uint64_t dv = desc_slot<L::kTile>(desc_v0, s);
-            const uint32_t dst = tb + 256 + t * 128, src = tb + t * 128;
-            {
-                umma_f16_ta(dst, src, dv, idesc_pv, acc ? 1u : 0u);
+            const uint32_t dst = tb + L::kTO + t * DH, src = tb + b * 128;
+            umma_f16_ta(dst, src, dv, idesc_pv, acc ? 1u : 0u);
 #pragma unroll
-                for (int ks = 1; ks < 8; ++ks)
-                    umma_f16_ta(dst, src + (ks >> 2) * 64 + ((ks & 3) >> 1) * 32 + (ks & 1) * 8, desc_advance(dv, ks * 2048), idesc_pv, 1u);
-            }
+            for (int ks = 1; ks < 8; ++ks)
+                umma_f16_ta(dst, src + (ks >> 2) * 64 + ((ks & 3) >> 1) * 32 + (ks & 1) * 8, desc_advance(dv, ks * 2048), idesc_pv, 1u);
         };
         auto commit = [&](int b) {
             umma_commit(bar(b));
@@ -265,103 +259,59 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         auto wait = [&](int b, uint32_t parity, int site) {
             return mbar_wait(bar(b), parity, abort_flag, p.status, site);
         };
-        uint32_t n = 0;                                 // key/value tiles consumed before this item
-        uint32_t np[2] = {0, 0};                        // P tiles consumed per query tile
-        uint32_t qn[2] = {0, 0};                        // items each query tile took part in
+        Ring<L::kStages> rk, rv;                        // stage of the next score tile / P V product
+        Ring<L::kBufs> bs, bp;                          // and its buffer
+        uint32_t nb = 0;                                // items that had a tile B
         bool ok = true;
         FwdItem it;
         for (int k = 0; ok; ++k) {
-            if (!wait(21 + (k & 1), (k >> 1) & 1, 423)) break;
+            if (!wait(L::kIF + (k & 1), (k >> 1) & 1, 423)) break;
             const int idx = item_slot[k & 1];
-            mbar_arrive(bar(23 + (k & 1)));
+            mbar_arrive(bar(L::kIE + (k & 1)));
             if (!fwd_item<SPLIT>(p, idx, it)) break;
-            const int nA = it.nA, nB = it.nB, n_kv = it.n_kv;
-            if (SPLIT) {
-                const int qb = k & 1;
-                auto scores = [&](int j) {                   // S(j) into slot j & 1
-                    const uint32_t m = n + j;
-                    if (!wait(4 + (m & 1), (m >> 1) & 1, 411)) return false;
-                    tc_fence_after();
-                    issue_s(j & 1, m & 1, qb);
-                    commit(6 + (m & 1));
-                    if (j == n_kv - 1) commit(2 + qb);       // Q is not needed again
-                    return true;
-                };
-                ok = wait(qb, (k >> 1) & 1, 410) && scores(0) && (n_kv == 1 || scores(1));
-                for (int j = 0; j < n_kv && ok; ++j) {
-                    const uint32_t m = n + j;
-                    const int t = j & 1;
-                    ok = wait(8 + (m & 1), (m >> 1) & 1, 412) && wait(14 + t, (t ? np[1] : np[0]) & 1, 413) &&
-                         (j > 1 || wait(18 + t, (k & 1) ^ 1, 418));          // the previous item's O_t has been read out
-                    if (!ok) break;
-                    if (t) ++np[1]; else ++np[0];
-                    tc_fence_after();
-                    issue_pv(t, m & 1, j > 1);
-                    commit(10 + (m & 1));
-                    if (j == n_kv - 1) { commit(16); commit(17); }
-                    if (j + 2 < n_kv) ok = scores(j + 2);
-                }
-                n += n_kv;
-                continue;
-            }
-            {
-                const int s = n & 1;
-                const uint32_t ph = (n >> 1) & 1;
-                ok = wait(4 + s, ph, 411) && wait(0, qn[0] & 1, 410);
-                if (!ok) break;
+            const int nA = it.nA, nB = it.nB, n_pos = nA + nB;
+            // A_0 B_0 A_1 B_1 ... on one key tile each (SPLIT: A_0 B_1 A_2 ...); without a tile B, and past the end of A, one after the other
+            auto shared = [&](int t) { return !SPLIT && t == 0 && nB; };       // tile B uses the same K and V after it
+            auto step = [&](int& t, int& j, Ring<L::kStages>& st) {
+                if (shared(t)) { t = 1; return; }
+                ++j;
+                st.next();
+                t = SPLIT ? j & 1 : j < nA ? 0 : 1;
+            };
+            int ts = 0, js = 0, tp = 0, jp = 0;
+            auto scores = [&]() {
+                if ((SPLIT || ts == 0 || js >= nA) && !wait(L::kKF + rk.i, rk.parity, 411)) return false;      // first use of the stage
+                const int qb = SPLIT ? k & 1 : ts;
+                if (js == 0 && !wait(qb, (SPLIT ? k >> 1 : ts ? static_cast<int>(nb) : k) & 1, 410)) return false;
                 tc_fence_after();
-                issue_s(0, s, 0);
-                if (nA == 1) commit(2);                     // Q_A is not needed again
-                if (nB) {
-                    if (!wait(1, qn[1] & 1, 417)) { ok = false; break; }
-                    tc_fence_after();
-                    issue_s(1, s, 1);
-                    if (nB == 1) commit(3);
+                issue_s(rk.i, bs.i, qb);
+                if (js + 1 == (SPLIT ? it.n_kv : ts ? nB : nA)) commit(2 + qb);        // Q is not needed again
+                if (!shared(ts)) commit(L::kKE + rk.i);     // K stage free
+                step(ts, js, rk);
+                bs.next();
+                return true;
+            };
+            for (int i = 0; i < L::kBufs && i < n_pos && ok; ++i) ok = scores();
+            for (int i = 0; i < n_pos && ok; ++i) {
+                if ((SPLIT || tp == 0 || jp >= nA) && !wait(L::kVF + rv.i, rv.parity, 412)) { ok = false; break; }
+                if (!wait(L::kPF + bp.i, bp.parity, 413)) { ok = false; break; }
+                // the previous item's O_t must have been read out before it is overwritten
+                const bool first = SPLIT ? jp < 2 : jp == 0;
+                if (first && !wait(L::kOE + tp, ((!SPLIT && tp ? static_cast<int>(nb) : k) & 1) ^ 1, 418)) { ok = false; break; }
+                tc_fence_after();
+                issue_pv(tp, rv.i, bp.i, !first);
+                if (L::kStages == 2 && !shared(tp)) commit(L::kVE + rv.i);          // V stage free: the sooner the fewer they are
+                if (i + L::kBufs < n_pos && !scores()) { ok = false; break; }       // the scores that take P's place
+                if (SPLIT) {
+                    if (jp + 1 == it.n_kv) { commit(L::kOF); commit(L::kOF + 1); }
+                } else if (jp + 1 == (tp ? nB : nA)) {
+                    commit(L::kOF + tp);
                 }
-                commit(6 + s);
+                if (L::kStages > 2 && !shared(tp)) commit(L::kVE + rv.i);
+                step(tp, jp, rv);
+                bp.next();
             }
-            for (int j = 0; j < n_kv && ok; ++j) {
-                const uint32_t nj = n + j, nn = nj + 1;
-                const int s = nj & 1, sn = nn & 1;
-                const uint32_t ph = (nj >> 1) & 1, phn = (nn >> 1) & 1;
-                if (!wait(8 + s, ph, 412)) { ok = false; break; }
-                bool k_waited = false;
-                if (j < nA) {
-                    if (!wait(14, np[0] & 1, 413)) { ok = false; break; }
-                    ++np[0];
-                    // the previous item's O_A must have been read out before it is overwritten
-                    if (j == 0 && !wait(18, (qn[0] & 1) ^ 1, 418)) { ok = false; break; }
-                    tc_fence_after();
-                    issue_pv(0, s, j > 0);
-                    if (j == nA - 1) commit(16);
-                }
-                if (j + 1 < nA) {
-                    if (!wait(4 + sn, phn, 414)) { ok = false; break; }
-                    k_waited = true;
-                    tc_fence_after();
-                    issue_s(0, sn, 0);
-                    if (j + 2 == nA) commit(2);
-                }
-                if (j < nB) {
-                    if (!wait(15, np[1] & 1, 415)) { ok = false; break; }
-                    ++np[1];
-                    if (j == 0 && !wait(19, (qn[1] & 1) ^ 1, 419)) { ok = false; break; }
-                    tc_fence_after();
-                    issue_pv(1, s, j > 0);
-                    if (j == nB - 1) commit(17);
-                }
-                commit(10 + s);                             // V stage free once these MMAs are done
-                if (j + 1 < nB) {
-                    if (!k_waited && !wait(4 + sn, phn, 416)) { ok = false; break; }
-                    tc_fence_after();
-                    issue_s(1, sn, 1);
-                    if (j + 2 == nB) commit(3);
-                }
-                if (j + 1 < n_kv) commit(6 + sn);           // K stage free
-            }
-            n += n_kv;
-            ++qn[0];
-            if (nB) ++qn[1];
+            if (nB) ++nb;
         }
         }
     } else {
@@ -377,30 +327,40 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         const int r = q * 32 + lane;                        // query row inside the tile
         const bool leader = hf == 0 && q == 2 && lane == 0;
         const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
-        const uint32_t s_addr = tmem_base + lane_addr + t * 128 + hf * 64;       // my 64 scores
-        const uint32_t o_addr = tmem_base + lane_addr + 256 + t * 128 + hf * (DH / 2);
+        const uint32_t o_addr = tmem_base + lane_addr + L::kTO + t * DH + hf * (DH / 2);
         float* xch = reinterpret_cast<float*>(sm + L::kXch) + t * 256;           // [half][row]
         const float sl2 = p.scale * kLog2e;
-        uint32_t ns = 0, qn = 0;                            // S tiles and items this query tile has seen
+        uint32_t p0 = 0, n0 = 0, nb = 0;                    // score tiles, key tiles and items with a tile B in front of this item
         uint32_t u_base = 0;                                // uses of the output staging tile before this item
         bool ok = true;
         FwdItem it;
         for (int k = 0; ok; ++k) {
-        ok = mbar_wait(bar(21 + (k & 1)), (k >> 1) & 1, abort_flag, p.status, 424);
+        ok = mbar_wait(bar(L::kIF + (k & 1)), (k >> 1) & 1, abort_flag, p.status, 424);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         const int idx = item_slot[k & 1];
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar(23 + (k & 1)));
+        if (lane == 0) mbar_arrive(bar(L::kIE + (k & 1)));
         if (!fwd_item<SPLIT>(p, idx, it)) break;
         const int n_t = t == 0 ? it.nA : it.nB;
         const uint32_t u = SPLIT ? k : u_base + t;          // staging order: A(k), B(k), A(k+1), ...
         u_base += it.nB ? 2 : 1;
-        if (!SPLIT && n_t == 0) continue;
+        // Before a score tile is waited for, all in front of it but kBufs - 1 must be complete (its barrier may then be one phase
+        // behind at most).  The tiles' own sequences see to that, except where tile B sits an item out.
+        if (!SPLIT && n_t == 0) {
+            ok = mbar_wait(bar(L::kOF), k & 1, abort_flag, p.status, 425);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            p0 += it.nA; n0 += it.n_kv;
+            continue;
+        }
         const int q0 = it.q0A + (SPLIT ? 0 : t * 128);
         float m_used = -INFINITY, l = 0.f;
-        for (int j = 0; j < n_t; ++j, ++ns) {
-            ok = mbar_wait(bar(12 + t), ns & 1, abort_flag, p.status, 420);
+        for (int j = 0; j < n_t; ++j) {
+            const uint32_t ps = p0 + fwd_position<SPLIT>(it, t, j);
+            const int sb = ps % L::kBufs;
+            const uint32_t s_addr = tmem_base + lane_addr + sb * 128 + hf * 64;      // my 64 scores
+            ok = mbar_wait(bar(L::kSF + sb), (ps / L::kBufs) & 1, abort_flag, p.status, 420);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -440,6 +400,12 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
                 const float alpha = grow ? ex2_approx((m_used - m_new) * sl2) : 1.0f;
                 if (grow) m_used = m_new;
                 l *= alpha;
+                // the product with this tile's previous P, issued behind these scores, must have left O: its V stage is free then
+                const uint32_t nv = n0 + (SPLIT ? 2 * (j - 1) + t : j - 1);
+                ok = mbar_wait(bar(L::kVE + nv % L::kStages), (nv / L::kStages) & 1, abort_flag, p.status, 426);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
 #pragma unroll 1
                 for (int c = 0; c < DH / 64; ++c) {
                     uint32_t w[32];
@@ -494,11 +460,11 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
             }
             tc_wait_st();
             tc_fence_before();
-            mbar_arrive(bar(14 + t));
+            mbar_arrive(bar(L::kPF + sb));
         }
         if (ok) {
-            if (SPLIT) ok = mbar_wait(bar(16), k & 1, abort_flag, p.status, 421) && mbar_wait(bar(17), k & 1, abort_flag, p.status, 421);
-            else ok = mbar_wait(bar(16 + t), qn & 1, abort_flag, p.status, 421);
+            if (SPLIT) ok = mbar_wait(bar(L::kOF), k & 1, abort_flag, p.status, 421) && mbar_wait(bar(L::kOF + 1), k & 1, abort_flag, p.status, 421);
+            else ok = mbar_wait(bar(L::kOF + t), (t ? nb : static_cast<uint32_t>(k)) & 1, abort_flag, p.status, 421);
             ok = __all_sync(0xffffffffu, ok);
         }
         if (!ok) break;
@@ -509,7 +475,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
             named_bar_sync(1 + t, 256);
             const float l_row = l + xch[(hf ^ 1) * 128 + r];
             uint8_t* stage = sm + L::kO;
-            ok = mbar_wait(bar(20), (u & 1) ^ 1, abort_flag, p.status, 422);    // the previous user's store has read it
+            ok = mbar_wait(bar(L::kST), (u & 1) ^ 1, abort_flag, p.status, 422);    // the previous user's store has read it
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             float lse_m = m_used, lse_l = l_row;
@@ -528,17 +494,17 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
                 const float wA = (t == 0 ? mine : other) * inv_l, wB = (t == 0 ? other : mine) * inv_l;
                 constexpr int kCols = DH / 4;
                 const int seg = (t * 2 + hf) * kCols;
-                const uint32_t oa = tmem_base + lane_addr + 256 + seg;
+                const uint32_t oa = tmem_base + lane_addr + L::kTO + seg;
                 uint32_t a[kCols], c[kCols];
                 tmem_ld_n<kCols>(oa, a);
-                if (it.nB) tmem_ld_n<kCols>(oa + 128, c);
+                if (it.nB) tmem_ld_n<kCols>(oa + DH, c);
                 else {
 #pragma unroll
                     for (int i = 0; i < kCols; ++i) c[i] = 0;
                 }
                 tc_wait_ld();
                 tc_fence_before();
-                mbar_arrive(bar(18)); mbar_arrive(bar(19));
+                mbar_arrive(bar(L::kOE)); mbar_arrive(bar(L::kOE + 1));
 #pragma unroll
                 for (int g = 0; g < kCols / 8; ++g) {
                     float f[8];
@@ -556,7 +522,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
                     tc_wait_ld();
                     if (c == DH / 64 - 1) {                     // this thread's part of O_t has left TMEM
                         tc_fence_before();
-                        mbar_arrive(bar(18 + t));
+                        mbar_arrive(bar(L::kOE + t));
                     }
 #pragma unroll
                     for (int g = 0; g < 4; ++g) {
@@ -577,9 +543,10 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
                     tma_store_2d(&tmO, sbase + L::kO + kb * 16384, it.h * DH + kb * 64, it.b * p.S + q0);
                 bulk_commit();
                 bulk_wait_read0();                          // the staging tile may be written again
-                mbar_arrive(bar(20));
+                mbar_arrive(bar(L::kST));
             }
-            ++qn;
+            p0 += it.nA + it.nB; n0 += it.n_kv;
+            if (it.nB) ++nb;
         }
         }
         if (leader) bulk_wait0();
@@ -640,8 +607,8 @@ const char* launch_attention_fwd(Runtime* rt, const void* qkv, int B, int S, int
     p.S = S; p.H = H; p.B = B; p.scale = 1.0f / sqrtf(static_cast<float>(dh));
     // Pairs of query tiles share what they load and pay one prologue and epilogue for two; their longest item takes S / 128
     // steps (of a key tile for both).  Where that is more than an even share of all steps, single query tiles whose key
-    // tiles are dealt out to the two slots take half as long.  us, pairs -> singles (B x S x heads x dh): 1 x 2048 x 16 x 128
-    // 34.4 -> 23.3, 2 x 512 x 16 x 64 11.5 -> 8.5, 3 x 640 x 10 x 128 13.3 -> 11.2, 2 x 1024 x 16 x 64 18.5 -> 16.0, 1 x 8192 x 8 x
+    // tiles are dealt out to the two slots take half as long.  us, pairs -> singles (B x S x heads x dh; one score buffer per slot): 1 x 2048 x 16 x
+    // 128 34.4 -> 23.3, 2 x 512 x 16 x 64 11.5 -> 8.5, 3 x 640 x 10 x 128 13.3 -> 11.2, 2 x 1024 x 16 x 64 18.5 -> 16.0, 1 x 8192 x 8 x
     // 64 111 -> 104; on the other side 1 x 4096 x 16 x 64 59.4 -> 59.5, 2 x 2048 x 16 x 64 33.7 -> 37.4, 8 x 1024 x 16 x 64 40.4 -> 45.9,
     // and 5.4 -> 5.5 with one tile per sequence.
     const int pairs = (S + 255) / 256, longest = S / 128;

@@ -180,6 +180,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return true;
 }
 
+// Slot of a ring of N and the parity of its barriers, counted on one by one: the issuing thread, whose every instruction
+// counts, divides nothing.
+template <int N>
+struct Ring {
+    int i = 0;
+    uint32_t parity = 0;
+    __device__ __forceinline__ void next() { if (++i == N) { i = 0; parity ^= 1; } }
+};
+
 // One lane of the (converged) warp is picked; the rest of the warp's code stays uniform.
 __device__ __forceinline__ bool elect_one()
 {
