@@ -7,8 +7,9 @@
 //                 S   = Q_t K_j^T   (128x128, fp32)  -> buffer of 128 columns
 //                 O_t += P V_j      (128xdh,  fp32)  -> columns behind the buffers, P read from TMEM
 //               The score tiles form one sequence, A_0 B_0 A_1 B_1 ..., whose position p, counted on
-//               across items, takes buffer p % kBufs, as soon as the P V product of p - kBufs has been issued.  With 64-wide heads O leaves room for a third buffer: a tile's next scores
-//               are there when its warps have finished with the last ones.
+//               across items, takes buffer p % kBufs, as soon as the P V product of p - kBufs has been
+//               issued.  With 64-wide heads O leaves room for a third buffer: a tile's next scores are
+//               there when its warps have finished with the last ones.
 //               With one buffer per tile -> so, us (B x S x heads x dh): 2 x 4096 x 16 x 64 102 -> 93, 16 x 1024 x
 //               16 x 64 71 -> 66, 2 x 1024 x 16 x 64 15.1 -> 13.8; 128 wide, two buffers, 1 x 2048 x 64 x 128 72.4 -> 73.5.
 //   warps 2..9  softmax of tile A, warps 10..17 softmax of tile B (two threads per query row = TMEM
