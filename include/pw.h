@@ -212,8 +212,8 @@ pw_status_t pw_layer_profile_begin(pw_layer_t* layer);
 pw_status_t pw_layer_profile_end(pw_layer_t* layer, pw_profile_t* out);
 /* Kernels launched through this handle since it was created (graph replays count their nodes). */
 pw_status_t pw_layer_launch_count(const pw_layer_t* layer, uint64_t* count);
-/* The backward pass runs its weight-gradient GEMMs and bias column sums on a library-owned side
- * stream beside the data-gradient chain (default).  enabled = 0 keeps every kernel on the calling
+/* The backward pass of a lean layer makes again what was not kept on a library-owned side stream, beside the
+ * data-gradient chain (default).  enabled = 0 keeps every kernel on the calling
  * stream, in program order - the same kernels, the same results, one after the other: what a
  * per-kernel time measured alone corresponds to.  Takes effect from the next call. */
 pw_status_t pw_layer_set_side_stream(pw_layer_t* layer, int enabled);

@@ -220,8 +220,8 @@ static void build_plan(const pw_layer_config_t& c, Runtime* rt, LayerPlan* p)
     p->ctx_bytes = off;
     size_t s = p->ctx_bytes;
     const bool whole = (c.flags & PW_FLAG_WHOLE_LAYER) != 0;
-    // du and dqkv have a buffer each, so that attention's backward need not wait for the weight gradient and the column
-    // sum of du on the side stream; the whole-layer kernels, which have no side stream, share one.
+    // du and dqkv have a buffer each, for the weight gradients and the column sums read both at the end of a backward call;
+    // the whole-layer kernels, which use them in turn, share one.
     p->off_big = s; s += align256((whole ? std::max(T * F, T * 3 * d) : T * F) * 2);
     p->off_dqkv = s; s += whole ? 0 : align256(T * 3 * d * 2);
     p->off_td0 = s; s += align256(T * d * 2);
