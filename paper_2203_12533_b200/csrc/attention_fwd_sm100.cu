@@ -49,8 +49,12 @@ struct FwdSmem {
     static constexpr int kBars = kO + kTile;
     static constexpr int kBarBytes = DH == 64 ? 288 : 256;
     static_assert(kNumBars * 8 + 16 <= kBarBytes, "barriers and the words behind them");
-    static constexpr int kXch = kBars + kBarBytes;          // per-row exchange between the two threads of a row: [tile][half][128] fp32
-    static constexpr int kEnd = kXch + 2 * 2 * 128 * 4;
+    // Per-row exchange between the two threads of a row: [tile][half][128] fp32.  With a third score buffer a thread may be a key
+    // tile ahead of one that has yet to read what it left there, so key tiles alternate between two of them; with two
+    // buffers the next scores are issued behind the product with P, to which both threads have contributed.
+    static constexpr int kXchSets = kBufs > 2 ? 2 : 1, kXchBytes = 2 * 2 * 128 * 4;
+    static constexpr int kXch = kBars + kBarBytes;
+    static constexpr int kEnd = kXch + kXchSets * kXchBytes;
     static constexpr int kBytes = kEnd + ((kEnd + 1024 <= 232448) ? 1024 : 232448 - kEnd);   // alignment slack (checked in the kernel)
 };
 
@@ -390,9 +394,10 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
                 }
             }
             const float mine = fmaxf(fmaxf(mxs[0], mxs[1]), fmaxf(mxs[2], mxs[3]));
-            xch[hf * 128 + r] = mine;
+            float* xj = xch + (L::kXchSets > 1 ? (j & 1) * (L::kXchBytes / 4) : 0);
+            xj[hf * 128 + r] = mine;
             named_bar_sync(1 + t, 256);
-            const float mx = fmaxf(mine, xch[(hf ^ 1) * 128 + r]);
+            const float mx = fmaxf(mine, xj[(hf ^ 1) * 128 + r]);
             const float m_new = fmaxf(m_used, mx);
             const bool grow = (m_new - m_used) * sl2 > 8.0f;        // also true on the first tile (m_used = -inf)
             if (j == 0) {
