@@ -11,7 +11,8 @@
 //               issued.  With 64-wide heads O leaves room for a third buffer: a tile's next scores are
 //               there when its warps have finished with the last ones.
 //               With one buffer per tile -> so, us (B x S x heads x dh): 2 x 4096 x 16 x 64 102 -> 93, 16 x 1024 x
-//               16 x 64 71 -> 66, 2 x 1024 x 16 x 64 15.1 -> 13.8; 128 wide, two buffers, 1 x 2048 x 64 x 128 72.4 -> 73.5.
+//               16 x 64 71 -> 66, 2 x 1024 x 16 x 64 15.1 -> 13.8; 128 wide, two buffers, 1 x 2048 x 64 x 128 72.4 -> 73.5,
+//               16 x 640 x 16 x 128 62.4 -> 58.5.
 //   warps 2..9  softmax of tile A, warps 10..17 softmax of tile B (two threads per query row = TMEM
 //               lane): row max, exp2 with the 1/sqrt(dh) scale folded in, row sum, P written back
 //               as packed bf16 over the S columns it came from.  The running maximum is only
@@ -49,9 +50,11 @@ struct FwdSmem {
     static constexpr int kBars = kO + kTile;
     static constexpr int kBarBytes = DH == 64 ? 288 : 256;
     static_assert(kNumBars * 8 + 16 <= kBarBytes, "barriers and the words behind them");
-    // Per-row exchange between the two threads of a row: [tile][half][128] fp32.  With a third score buffer a thread may be a key
-    // tile ahead of one that has yet to read what it left there, so key tiles alternate between two of them; with two
-    // buffers the next scores are issued behind the product with P, to which both threads have contributed.
+    // Per-row exchange between the two threads of a row: [tile][half][128] fp32.  A thread must not leave its next maximum before its
+    // partner has read the last one.  With a third score buffer it may be a key tile ahead, so key tiles alternate between two
+    // sets of words.  A second set does not fit beside 128-wide tiles.  There a tile's next scores follow the product with its last P, to
+    // which both threads have contributed, as long as A and B take turns; where one of them is alone (an item without a
+    // tile B, B's last key tile) they follow the product in front of that, and a barrier behind the read keeps the order.
     static constexpr int kXchSets = kBufs > 2 ? 2 : 1, kXchBytes = 2 * 2 * 128 * 4;
     static constexpr int kXch = kBars + kBarBytes;
     static constexpr int kEnd = kXch + kXchSets * kXchBytes;
@@ -361,6 +364,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
         }
         const int q0 = it.q0A + (SPLIT ? 0 : t * 128);
         float m_used = -INFINITY, l = 0.f;
+        const int alone_from = t == 0 ? (it.nB ? n_t : 0) : it.nA - 1;      // from here on the next scores do not wait for this tile's P
         for (int j = 0; j < n_t; ++j) {
             const uint32_t ps = p0 + fwd_position<SPLIT>(it, t, j);
             const int sb = ps % L::kBufs;
@@ -398,6 +402,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
             xj[hf * 128 + r] = mine;
             named_bar_sync(1 + t, 256);
             const float mx = fmaxf(mine, xj[(hf ^ 1) * 128 + r]);
+            if (L::kXchSets == 1 && !SPLIT && j >= alone_from && j + 1 < n_t) named_bar_sync(1 + t, 256);      // (see kXchSets)
             const float m_new = fmaxf(m_used, mx);
             const bool grow = (m_new - m_used) * sl2 > 8.0f;        // also true on the first tile (m_used = -inf)
             if (j == 0) {

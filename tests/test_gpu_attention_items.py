@@ -21,7 +21,8 @@ def pw():
     (1, 128, 3, 64),                              # one tile: pairs, whose second slot is idle
     (1, 256, 1, 128), (2, 384, 3, 64),            # singles of one, two and three key tiles
     (2, 1024, 16, 64), (3, 896, 9, 128),          # singles, more than one to a CTA: Q buffers, rings and counters go round
-    (4, 640, 20, 64), (8, 512, 16, 128)])         # pairs, the last one incomplete; several to a CTA
+    (4, 640, 20, 64), (8, 512, 16, 128),          # pairs, the last one incomplete; several to a CTA
+    (8, 640, 13, 128)])                           # the same with two score buffers: a tile alone in its item, and tile B's last one
 def test_attention_fwd_items(pw, oracle64, B, S, H, dh):
     g = torch.Generator().manual_seed(S + H)
     d = H * dh
@@ -101,6 +102,30 @@ def test_attention_same_bits_every_time(pw, B, S, H, dh):
         pw.op_attention_bwd(qkv, o, dout, lse, B, S, H, dh, dqkv, delta)
         ref = dqkv if ref is None else ref
         wrong += (dqkv != ref).sum()
+    torch.cuda.synchronize()
+    assert pw.op_status() == (0, 0)
+    assert wrong.item() == 0
+
+
+@pytest.mark.parametrize("B,S,H", [(8, 1024, 16), (16, 640, 16), (9, 384, 33)])
+def test_attention_fwd_same_bits_128_wide_pairs(pw, B, S, H):
+    """Pairs of query tiles, even and odd numbers of key tiles.  The two threads of a row swap their maxima through one set of
+    words, so neither may write its next maximum before the other has read the last one: on every key tile of an item without a
+    tile B, and in front of tile B's diagonal one, the scores that it comes from may already be there.  Scores as large as these make the maximum jump by more than a rescale."""
+    g = torch.Generator(device="cuda").manual_seed(S)
+    d = H * 128
+    qkv = torch.randn((B * S, 3 * d), generator=g, device="cuda").to(torch.bfloat16)
+    qkv[:, :2 * d] *= 3
+    outs = [(torch.empty((B * S, d), dtype=torch.bfloat16, device="cuda"), torch.empty((B, H, S), device="cuda")) for _ in range(4)]
+    ref = None
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(250):
+        for o, lse in outs:
+            pw.op_attention_fwd(qkv, B, S, H, 128, o, lse)
+        if ref is None:
+            ref = [t.clone() for t in outs[0]]
+        for o, lse in outs:
+            wrong += (o != ref[0]).sum() + (lse != ref[1]).sum()
     torch.cuda.synchronize()
     assert pw.op_status() == (0, 0)
     assert wrong.item() == 0
