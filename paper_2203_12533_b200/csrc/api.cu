@@ -70,6 +70,19 @@ static pw_status_t fail_cuda(const char* what, cudaError_t e)
     return fail(PW_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// Zeroes device memory before the call returns, on a stream of its own.  (cudaMemset runs on the legacy stream and does not hold
+// up the host: a first kernel on a non-blocking stream could start before it, or have its counters zeroed under it.)
+static cudaError_t clear_now(void* q, size_t bytes)
+{
+    cudaStream_t s = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(q, 0, bytes, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaStreamDestroy(s);
+    return e;
+}
+
 Runtime* get_runtime(const char** err)
 {
     static std::mutex mu;
@@ -95,7 +108,7 @@ Runtime* get_runtime(const char** err)
     const char* ce;
     if ((ce = configure_gemm()) || (ce = configure_gemm_cluster()) || (ce = configure_attention()) || (ce = configure_attention_fwd()) || (ce = configure_elementwise()) || (ce = configure_whole_layer())) { delete rt; *err = ce; return nullptr; }
     if (cudaMalloc(reinterpret_cast<void**>(&rt->op_status), sizeof(DeviceStatus)) != cudaSuccess ||
-        cudaMemset(rt->op_status, 0, sizeof(DeviceStatus)) != cudaSuccess) {
+        clear_now(rt->op_status, sizeof(DeviceStatus)) != cudaSuccess) {
         delete rt; *err = "could not allocate the status word"; return nullptr;
     }
     // split-K scratch of the single-step GEMM call; without it that call simply never cuts a tile
@@ -579,8 +592,10 @@ static pw_status_t read_status(DeviceStatus* dev, int* code, int* site)
     // A kernel that gave up may have left the work counters of the persistent attention kernels
     // mid-count; the device is idle here, so they are put back to zero (the error stays recorded).
     // (the same goes for the split-K tickets of the GEMM, which follow the counters in the struct)
-    if (h.code != 0)
-        cudaMemset(reinterpret_cast<char*>(dev) + offsetof(DeviceStatus, sched), 0, sizeof(h.sched) + sizeof(h.tickets));
+    if (h.code != 0) {
+        e = clear_now(reinterpret_cast<char*>(dev) + offsetof(DeviceStatus, sched), sizeof(h.sched) + sizeof(h.tickets));
+        if (e != cudaSuccess) return fail_cuda("work counters", e);
+    }
     return PW_OK;
 }
 
@@ -622,11 +637,11 @@ pw_status_t pw_layer_create(const pw_layer_config_t* cfg, pw_layer_t** out)
     L->rt = rt;
     build_plan(*cfg, rt, &L->plan);
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&L->status), sizeof(DeviceStatus));
-    if (e == cudaSuccess) e = cudaMemset(L->status, 0, sizeof(DeviceStatus));
+    if (e == cudaSuccess) e = clear_now(L->status, sizeof(DeviceStatus));
     if (e == cudaSuccess && L->plan.whole) {
         const size_t bytes = 2 * kWholeLayerSyncWords * sizeof(unsigned);
         e = cudaMalloc(reinterpret_cast<void**>(&L->whole_sync), bytes);
-        if (e == cudaSuccess) e = cudaMemset(L->whole_sync, 0, bytes);
+        if (e == cudaSuccess) e = clear_now(L->whole_sync, bytes);
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&L->aux, cudaStreamNonBlocking);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&L->ev[i], cudaEventDisableTiming);
@@ -1495,7 +1510,7 @@ pw_status_t pw_op_selftest_wait_timeout(uint64_t limit_cycles, int* kernel_retur
     if (limit > 2000000000ll) limit = 2000000000ll;            // about a second at most
     int* flag = nullptr;
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&flag), sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(flag, 0, sizeof(int));
+    if (e == cudaSuccess) e = clear_now(flag, sizeof(int));
     if (e != cudaSuccess) { if (flag) cudaFree(flag); return fail_cuda("self-test flag", e); }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const char* err = launch_wait_selftest(rt->op_status, limit, flag, st);
@@ -1552,7 +1567,7 @@ pw_status_t pw_op_status_reset(void)
 {
     PW_RT_OR_FAIL();
     cudaError_t e = cudaDeviceSynchronize();
-    if (e == cudaSuccess) e = cudaMemset(rt->op_status, 0, sizeof(DeviceStatus));   // the device is idle: code, site, counters, tickets
+    if (e == cudaSuccess) e = clear_now(rt->op_status, sizeof(DeviceStatus));   // the device is idle: code, site, counters, tickets
     return e == cudaSuccess ? PW_OK : fail_cuda("status reset", e);
 }
 
