@@ -19,8 +19,8 @@
  *     with the shape of the parameter.  LayerNorm statistics and log-sum-exp are fp32.
  *   - Ownership: the caller owns every device buffer it passes and keeps it alive until the
  *     stream has passed the enqueued work.  The library owns only host-side handles, one
- *     small device status word per handle, and cached CUDA graphs.  No call on the enqueue
- *     path allocates device memory.
+ *     small device status block per handle (a stage has up to four), and cached CUDA graphs.
+ *     No call on the enqueue path allocates device memory.
  *   - Asynchrony: fwd / bwd / run_chain only enqueue work on `stream` (a cudaStream_t passed
  *     as void*; NULL = the legacy default stream) and return without synchronising - stream
  *     order plays the role of the paper's buffer futures.  Argument errors are detected
@@ -232,7 +232,8 @@ enum {
 
 /* Outside OPBYOP the micro-batches of a chain take turns on up to four streams of the stage (forked from and joined to
  * the caller's), where the workspace that this takes is at most 1 GB beyond one stream's and no two micro-batches' buffers
- * overlap.  Same bits as on one stream; pw_stage_set_side_stream(stage, 0) keeps everything on the calling stream. */
+ * overlap.  Same bits as on one stream; pw_stage_set_side_stream(stage, 0) keeps everything on the calling stream.  The streams
+ * and the handles that go with them (a status block each) are made here, with the stage. */
 pw_status_t pw_stage_create(const pw_layer_config_t* cfg, int n_layers, pw_stage_t** out);
 void pw_stage_destroy(pw_stage_t* stage);
 

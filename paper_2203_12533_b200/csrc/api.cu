@@ -168,7 +168,7 @@ struct pw_stage {
     // GPU (see stage_lanes).  Lane 0 is the caller's stream with `layer`; every further one has a handle (status word,
     // side stream, events), a stream and, in the workspace, a scratch of its own.
     struct Lane { pw_layer_t* layer; cudaStream_t stream; cudaEvent_t done; };
-    std::vector<Lane> lanes;                // lanes 1, 2, ... (made by the first chain that uses them)
+    std::vector<Lane> lanes;                // lanes 1, 2, ...
     std::vector<cudaEvent_t> lane_events;   // [l]: layer l's gradients hold every micro-batch enqueued so far; last: fork
     struct Cached { cudaGraphExec_t exec; uint64_t nodes; };
     std::map<std::vector<uint64_t>, Cached> graphs;
@@ -771,38 +771,26 @@ static int stage_lanes(const pw_stage_t* stage)
     return tiles <= (p.whole ? 8 : 64) ? kMaxLanes : 2;
 }
 
-// Creates the handles, streams and events of the lanes, once per stage.  False: the call goes on on one stream (no memory
-// for them, or the stream is being captured, when nothing can be allocated).
-static bool ensure_lanes(pw_stage_t* stage, cudaStream_t st)
+// The handles, streams and events of the lanes, made with the stage: a chain call allocates nothing.
+static pw_status_t create_lanes(pw_stage_t* stage)
 {
     const int n = stage_lanes(stage);
-    if (n <= 1 || stage->lanes.size() + 1 == static_cast<size_t>(n)) return n > 1;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { (void)cudaGetLastError(); return false; }
-    if (cs != cudaStreamCaptureStatusNone) return false;
-    std::vector<pw_stage::Lane> lanes;
-    std::vector<cudaEvent_t> events;
+    if (n <= 1) return PW_OK;
     cudaError_t e = cudaSuccess;
     for (int i = 1; i < n && e == cudaSuccess; ++i) {
-        pw_stage::Lane lane = {nullptr, nullptr, nullptr};
-        if (pw_layer_create(&stage->layer->plan.cfg, &lane.layer) != PW_OK) { e = cudaErrorMemoryAllocation; break; }
+        pw_layer_t* handle = nullptr;
+        PW_DO(pw_layer_create(&stage->layer->plan.cfg, &handle));
+        stage->lanes.push_back({handle, nullptr, nullptr});
+        pw_stage::Lane& lane = stage->lanes.back();
         e = cudaStreamCreateWithFlags(&lane.stream, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&lane.done, cudaEventDisableTiming);
-        lanes.push_back(lane);
     }
     for (int l = 0; l <= stage->n_layers && e == cudaSuccess; ++l) {
         cudaEvent_t ev = nullptr;
         e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-        if (e == cudaSuccess) events.push_back(ev);
+        if (e == cudaSuccess) stage->lane_events.push_back(ev);
     }
-    if (e != cudaSuccess) {
-        (void)cudaGetLastError();
-        destroy_lanes(lanes, events);
-        return false;
-    }
-    stage->lanes = lanes;
-    stage->lane_events = events;
-    return true;
+    return e == cudaSuccess ? PW_OK : fail_cuda("stage lanes (streams, events)", e);
 }
 
 pw_status_t pw_stage_create(const pw_layer_config_t* cfg, int n_layers, pw_stage_t** out)
@@ -816,6 +804,7 @@ pw_status_t pw_stage_create(const pw_layer_config_t* cfg, int n_layers, pw_stage
     if (!st) { pw_layer_destroy(L); return fail(PW_ERR_INTERNAL, "out of host memory"); }
     st->layer = L;
     st->n_layers = n_layers;
+    if ((s = create_lanes(st)) != PW_OK) { pw_stage_destroy(st); return s; }
     *out = st;
     if (log_enabled(PW_LOG_INFO)) log_line(PW_LOG_INFO, "pw_stage_create: " + std::to_string(n_layers) + " layers of the shape above");
     return PW_OK;
@@ -911,7 +900,7 @@ pw_status_t enqueue_chain(pw_stage_t* stage, const pw_layer_params_t* params, co
 {
     const int L = stage->n_layers;
     const bool gpipe = schedule == PW_SCHEDULE_GPIPE;
-    const int lanes = sync_each || stage->layer->profiling || stage->layer->single_stream || stage->lanes.empty() ||
+    const int lanes = sync_each || stage->layer->profiling || stage->layer->single_stream ||
                       (lay.lanes > 1 && microbatches_overlap(x_mb, dy_mb, y_mb, dx_mb, M, static_cast<size_t>(stage->layer->plan.T) * stage->layer->plan.d * 2))
                           ? 1 : lay.lanes;
     auto lane_of = [&](int m) { return m % lanes; };
@@ -1027,7 +1016,6 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
         if (x_mb[m] == y_mb[m] || x_mb[m] == dx_mb[m]) return fail(PW_ERR_INVALID_ARG, "y and dx must not alias x");
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (dispatch_mode != PW_DISPATCH_OPBYOP && lay.lanes > 1) ensure_lanes(stage, st);
 
     if (dispatch_mode != PW_DISPATCH_GRAPH)
         return enqueue_chain(stage, params, grads, x_mb, dy_mb, y_mb, dx_mb, M, schedule, recompute, workspace, lay,

@@ -73,3 +73,51 @@ def test_one_buffer_for_every_output_keeps_the_last_micro_batch(pw):
     stage.run_chain(params, grads, xs, dys, part, dxs, ws, pw.DISPATCH_ASYNC)
     torch.cuda.synchronize()
     assert torch.equal(y, want) and torch.equal(buf[8:], want)
+
+
+@pytest.mark.parametrize("flags", ["", "whole"])
+@pytest.mark.parametrize("dispatch", ["ASYNC", "GRAPH"])
+def test_first_chain_of_a_stage_beside_a_busy_default_stream(pw, dispatch, flags):
+    """The first chain call finds its lanes made: it allocates nothing, makes no handle and waits for nothing that the default
+    stream still holds."""
+    w = inputs.Workload("lanes", 256, 4, 64, 512, 128, 2)
+    M, L = 6, 3
+    flags = pw.FLAG_WHOLE_LAYER if flags else 0
+    params = [[p.cuda() for p in inputs.layer_params(w, 0, l, random_ln=True)] for l in range(L)]
+    xs, dys = zip(*[[t.cuda().view(w.tokens, -1) for t in inputs.microbatch(w, 0, m)] for m in range(M)])
+
+    def buffers():
+        return ([torch.full_like(x, 7.0) for x in xs], [torch.full_like(x, 7.0) for x in xs],
+                [[torch.full(p.shape, 7.0, device="cuda") for p in ps] for ps in params])
+
+    def stage():
+        return pw.Stage(L, w.d_model, w.n_heads, w.head_dim, w.d_ff, w.seq_len, w.batch, flags=flags)
+
+    first = stage()
+    ws = torch.empty(first.workspace_bytes(M, pw.SCHEDULE_GPIPE, True), dtype=torch.uint8, device="cuda")
+    ys, dxs, grads = buffers()
+    first.run_chain(params, grads, xs, dys, ys, dxs, ws, pw.DISPATCH_OPBYOP)
+    ref = ys + dxs + [g for gs in grads for g in gs]
+    ys, dxs, grads = buffers()
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(500_000_000)                           # a few tenths of a second of work on the default stream
+    done = torch.cuda.Event()
+    done.record()
+    st = stage()
+    lines = []
+    pw.set_log(pw.LOG_INFO, lambda level, msg: lines.append(msg))
+    try:
+        free = torch.cuda.mem_get_info()[0]
+        st.run_chain(params, grads, xs, dys, ys, dxs, ws, getattr(pw, "DISPATCH_" + dispatch), stream=stream)
+        if dispatch == "ASYNC":                              # (an instantiated graph is memory of its own)
+            assert torch.cuda.mem_get_info()[0] == free
+    finally:
+        pw.set_log(pw.LOG_OFF)
+    stream.synchronize()
+    # all of it while the default stream was busy (a cooperative launch may wait for what that holds)
+    assert flags == pw.FLAG_WHOLE_LAYER or not done.query()
+    assert lines and not any("_create" in line for line in lines), lines
+    for a, b in zip(ref, ys + dxs + [g for gs in grads for g in gs]):
+        assert torch.equal(a, b)
+    assert st.status() == (0, 0)
