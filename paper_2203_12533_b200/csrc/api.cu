@@ -142,8 +142,8 @@ struct pw_layer {
     pw::LayerPlan plan;
     pw::Runtime* rt;
     pw::DeviceStatus* status;
-    // Grid-barrier and split-K words of the whole-layer kernels, one set for launches on all SMs and one for launches
-    // that share them with the other lanes of a stage (a set is tied to one grid size).
+    // Grid-barrier and split-K words of the whole-layer kernels, a set for every number of lanes that may share the SMs (a set is
+    // tied to one grid size).
     unsigned* whole_sync = nullptr;
     int whole_share = 1;            // lanes that share the SMs in the call being enqueued
     cudaStream_t aux = nullptr;     // side stream: what a lean save set makes again runs beside the dgrad chain
@@ -414,7 +414,7 @@ static pw_status_t do_whole_layer(pw_layer_t* L, const pw_layer_params_t* P, con
         a.g_w_fc2 = G->w_fc2; a.g_b_fc2 = G->b_fc2;
     }
     a.splitk = at(scratch, p.off_whole_splitk);
-    a.sync = L->whole_sync + (L->whole_share > 1 ? kWholeLayerSyncWords : 0);
+    a.sync = L->whole_sync + (L->whole_share - 1) * kWholeLayerSyncWords;
     a.status = L->status;
     const double T = p.T, d = p.d, F = p.F;
     const double fwd_flops = 2.0 * T * d * (4.0 * d + 2.0 * F) + 2.0 * T * (p.S + 1.0) * d;
@@ -639,7 +639,7 @@ pw_status_t pw_layer_create(const pw_layer_config_t* cfg, pw_layer_t** out)
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&L->status), sizeof(DeviceStatus));
     if (e == cudaSuccess) e = clear_now(L->status, sizeof(DeviceStatus));
     if (e == cudaSuccess && L->plan.whole) {
-        const size_t bytes = 2 * kWholeLayerSyncWords * sizeof(unsigned);
+        const size_t bytes = kMaxLanes * kWholeLayerSyncWords * sizeof(unsigned);
         e = cudaMalloc(reinterpret_cast<void**>(&L->whole_sync), bytes);
         if (e == cudaSuccess) e = clear_now(L->whole_sync, bytes);
     }
@@ -763,6 +763,7 @@ pw_status_t pw_layer_launch_count(const pw_layer_t* layer, uint64_t* count)
 // 5209 / 3620 / 3339 / 3283, 1024 x 1024 7511 / 6126 / 5878 / 5860; 4 micro-batches of 2048 x 1024 (saved) 4544 / 3824 / 3814,
 // of 8192 x 2048 47224 / 44959.  Whole-layer kernels share the SMs by lanes, so they stop gaining earlier: 256 x 256
 // 3252 / 2031 / 1782 / 2514, 1024 x 256 4791 / 3706 / 3748.
+// (Fewer micro-batches than lanes: 2 of 256 x 256 through 4 layers 795 with the SMs shared by four, 545 by two; 3 of them 916, 760 by three.)
 static int stage_lanes(const pw_stage_t* stage)
 {
     const LayerPlan& p = stage->layer->plan;
@@ -982,7 +983,7 @@ pw_status_t enqueue_chain(pw_stage_t* stage, const pw_layer_params_t* params, co
         for (auto& lane : stage->lanes) lane.layer->whole_share = n;
     };
     PW_DO(fork());
-    if (lanes > 1) share(static_cast<int>(stage->lanes.size()) + 1);
+    share(lanes);
     const pw_status_t s = run();
     share(1);
     const pw_status_t j = join();                // also after a failure: a stream capture must find its forks joined

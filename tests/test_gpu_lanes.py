@@ -121,3 +121,24 @@ def test_first_chain_of_a_stage_beside_a_busy_default_stream(pw, dispatch, flags
     for a, b in zip(ref, ys + dxs + [g for gs in grads for g in gs]):
         assert torch.equal(a, b)
     assert st.status() == (0, 0)
+
+
+def test_whole_layer_launches_share_the_sms_by_the_lanes_in_use(pw):
+    """One stage, chains of one to six micro-batches in turn: each number of lanes has grids of its own size, whose barrier words must not mix."""
+    w = inputs.Workload("lanes", 256, 4, 64, 512, 128, 2)
+    L = 2
+    params = [[p.cuda() for p in inputs.layer_params(w, 0, l, random_ln=True)] for l in range(L)]
+    xs, dys = zip(*[[t.cuda().view(w.tokens, -1) for t in inputs.microbatch(w, 0, m)] for m in range(6)])
+    stage = pw.Stage(L, w.d_model, w.n_heads, w.head_dim, w.d_ff, w.seq_len, w.batch, flags=pw.FLAG_WHOLE_LAYER)
+    ws = torch.empty(stage.workspace_bytes(6), dtype=torch.uint8, device="cuda")
+    for M in (2, 4, 3, 1, 2, 6, 3):
+        out = []
+        for dispatch in (pw.DISPATCH_OPBYOP, pw.DISPATCH_ASYNC):
+            ys, dxs = [torch.empty_like(x) for x in xs[:M]], [torch.empty_like(x) for x in xs[:M]]
+            grads = [[torch.empty(p.shape, device="cuda") for p in ps] for ps in params]
+            stage.run_chain(params, grads, xs[:M], dys[:M], ys, dxs, ws, dispatch)
+            torch.cuda.synchronize()
+            assert stage.status() == (0, 0)
+            out.append(ys + dxs + [g for gs in grads for g in gs])
+        for a, b in zip(*out):
+            assert torch.equal(a, b), M
