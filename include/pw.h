@@ -237,7 +237,9 @@ enum {
 pw_status_t pw_stage_create(const pw_layer_config_t* cfg, int n_layers, pw_stage_t** out);
 void pw_stage_destroy(pw_stage_t* stage);
 
-/* Workspace (device, 256-byte aligned) needed by pw_stage_run_chain for these settings. */
+/* Workspace (device, 256-byte aligned) of pw_stage_run_chain for these settings, with all its streams.  A smaller one is taken
+ * too and means fewer of them, down to what one stream needs: the size reported after pw_stage_set_side_stream(stage, 0),
+ * which is also all that OPBYOP uses. */
 pw_status_t pw_stage_workspace_bytes(const pw_stage_t* stage, int n_microbatches, int schedule, int recompute,
                                      size_t* bytes);
 
@@ -253,7 +255,7 @@ pw_status_t pw_stage_workspace_bytes(const pw_stage_t* stage, int n_microbatches
  *                   contexts in the workspace)
  * GRAPH mode caches an instantiated graph keyed by every pointer and setting of the call and
  * replays it when they repeat.  Returns PW_ERR_WORKSPACE_TOO_SMALL before enqueuing anything
- * if workspace_bytes is insufficient.  Enqueue only (OPBYOP synchronises by definition). */
+ * if workspace_bytes is insufficient for one stream.  Enqueue only (OPBYOP synchronises by definition). */
 pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* params, const pw_layer_grads_t* grads,
                                const void* const* x_mb, const void* const* dy_mb, void* const* y_mb,
                                void* const* dx_mb, int n_microbatches, int dispatch_mode, int schedule,

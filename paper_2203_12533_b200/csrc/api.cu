@@ -828,32 +828,32 @@ struct StageLayout {
     int lanes;                    // streams in use; each has its own gradient buffers and scratch
     size_t lane_bytes;            // pitch of those
 };
-pw_status_t stage_layout(const pw_stage_t* stage, int M, int schedule, int recompute, StageLayout* lay)
+// one_stream: a call that will keep to the calling stream.  available: bytes that the caller has; as many lanes as they and the rules allow.
+pw_status_t stage_layout(const pw_stage_t* stage, int M, int schedule, int recompute, bool one_stream, size_t available, StageLayout* lay)
 {
     if (M <= 0 || M > 65536) return fail(PW_ERR_INVALID_ARG, "n_microbatches out of range");
     if (schedule != PW_SCHEDULE_GPIPE && schedule != PW_SCHEDULE_PER_MICROBATCH) return fail(PW_ERR_INVALID_ARG, "unknown schedule");
     if (recompute != 0 && recompute != 1) return fail(PW_ERR_INVALID_ARG, "recompute must be 0 or 1");
     const LayerPlan& p = stage->layer->plan;
     const size_t L = stage->n_layers;
+    const bool gpipe = schedule == PW_SCHEDULE_GPIPE;
     lay->act_bytes = align256(static_cast<size_t>(p.T) * p.d * 2);
     lay->ctx_bytes = p.ctx_bytes;
-    const size_t lane_bytes = 2 * lay->act_bytes + align256(p.scratch_bytes);
-    // what a lane takes beside its gradient buffers and scratch: with one micro-batch alive at a time, that one's activations
-    const size_t lane_live = schedule == PW_SCHEDULE_GPIPE ? 0 : (L - 1) * lay->act_bytes + (recompute ? 0 : L * lay->ctx_bytes);
-    lay->lanes = stage_lanes(stage);
-    if (lay->lanes > M) lay->lanes = M;
-    while (lay->lanes > 1 && (lay->lanes - 1) * (lane_bytes + lane_live) > kMaxLaneExtra) --lay->lanes;
-    const size_t live = (schedule == PW_SCHEDULE_GPIPE) ? M : lay->lanes;
+    lay->lane_bytes = 2 * lay->act_bytes + align256(p.scratch_bytes);
+    // a micro-batch's activations: all of GPipe's are alive at once, otherwise one a lane
+    const size_t live_bytes = (L - 1) * lay->act_bytes + (recompute ? 0 : L * lay->ctx_bytes);
+    const size_t per_lane = lay->lane_bytes + (gpipe ? 0 : live_bytes), fixed = gpipe ? M * live_bytes : 0;
+    lay->lanes = one_stream ? 1 : std::min(stage_lanes(stage), M);
+    while (lay->lanes > 1 && ((lay->lanes - 1) * per_lane > kMaxLaneExtra || fixed + lay->lanes * per_lane > available)) --lay->lanes;
+    const size_t live = gpipe ? M : lay->lanes;
     lay->n_act = (L - 1) * live;
     lay->n_ctx = recompute ? 0 : L * live;
-    size_t s = 0;
-    lay->off_act = s; s += lay->act_bytes * lay->n_act;
-    lay->off_ctx = s; s += lay->ctx_bytes * lay->n_ctx;
-    lay->off_g0 = s;
+    lay->off_act = 0;
+    lay->off_ctx = lay->act_bytes * lay->n_act;
+    lay->off_g0 = lay->off_ctx + lay->ctx_bytes * lay->n_ctx;
     lay->off_g1 = lay->off_g0 + lay->act_bytes;
     lay->off_scratch = lay->off_g1 + lay->act_bytes;
-    lay->lane_bytes = lane_bytes;
-    lay->total = s + lay->lanes * lane_bytes;
+    lay->total = fixed + lay->lanes * per_lane;
     return PW_OK;
 }
 }  // namespace
@@ -863,7 +863,7 @@ pw_status_t pw_stage_workspace_bytes(const pw_stage_t* stage, int n_microbatches
 {
     if (!stage || !bytes) return fail(PW_ERR_INVALID_ARG, "stage or bytes is NULL");
     StageLayout lay;
-    pw_status_t s = stage_layout(stage, n_microbatches, schedule, recompute, &lay);
+    pw_status_t s = stage_layout(stage, n_microbatches, schedule, recompute, stage->layer->single_stream, SIZE_MAX, &lay);
     if (s != PW_OK) return s;
     *bytes = lay.total;
     return PW_OK;
@@ -901,8 +901,7 @@ pw_status_t enqueue_chain(pw_stage_t* stage, const pw_layer_params_t* params, co
 {
     const int L = stage->n_layers;
     const bool gpipe = schedule == PW_SCHEDULE_GPIPE;
-    const int lanes = sync_each || stage->layer->profiling || stage->layer->single_stream ||
-                      (lay.lanes > 1 && microbatches_overlap(x_mb, dy_mb, y_mb, dx_mb, M, static_cast<size_t>(stage->layer->plan.T) * stage->layer->plan.d * 2))
+    const int lanes = (lay.lanes > 1 && microbatches_overlap(x_mb, dy_mb, y_mb, dx_mb, M, static_cast<size_t>(stage->layer->plan.T) * stage->layer->plan.d * 2))
                           ? 1 : lay.lanes;
     auto lane_of = [&](int m) { return m % lanes; };
     auto handle = [&](int m) { return lane_of(m) == 0 ? stage->layer : stage->lanes[lane_of(m) - 1].layer; };
@@ -1001,13 +1000,14 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
         return fail(PW_ERR_INVALID_ARG, "a required pointer is NULL");
     if (dispatch_mode < PW_DISPATCH_OPBYOP || dispatch_mode > PW_DISPATCH_GRAPH) return fail(PW_ERR_INVALID_ARG, "unknown dispatch mode");
     StageLayout lay;
-    pw_status_t s = stage_layout(stage, n_microbatches, schedule, recompute, &lay);
+    const bool one_stream = dispatch_mode == PW_DISPATCH_OPBYOP || stage->layer->single_stream || stage->layer->profiling;
+    pw_status_t s = stage_layout(stage, n_microbatches, schedule, recompute, one_stream, workspace_bytes, &lay);
     if (s == PW_OK && log_enabled(PW_LOG_INFO))
         log_line(PW_LOG_INFO, std::string("pw_stage_run_chain: ") + (dispatch_mode == PW_DISPATCH_OPBYOP ? "OPBYOP" : dispatch_mode == PW_DISPATCH_ASYNC ? "ASYNC" : "GRAPH") +
                                   ", " + std::to_string(stage->n_layers) + " layers x " + std::to_string(n_microbatches) + " micro-batches" + (recompute ? ", recompute" : ""));
     if (s != PW_OK) return s;
     if (!aligned(workspace, 256)) return fail(PW_ERR_INVALID_ARG, "workspace is NULL or not 256-byte aligned");
-    if (workspace_bytes < lay.total) return fail(PW_ERR_WORKSPACE_TOO_SMALL, "workspace smaller than pw_stage_workspace_bytes reports");
+    if (workspace_bytes < lay.total) return fail(PW_ERR_WORKSPACE_TOO_SMALL, "workspace smaller than pw_stage_workspace_bytes reports for one stream");
     const int L = stage->n_layers, M = n_microbatches;
     for (int l = 0; l < L; ++l)
         if (!params_ok(&params[l]) || !grads_ok(&grads[l])) return fail(PW_ERR_INVALID_ARG, "a parameter or gradient pointer is NULL or misaligned");
@@ -1024,9 +1024,9 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
 
     // GRAPH: key = every pointer and setting that the captured launches bake in.
     std::vector<uint64_t> key;
-    key.reserve(8 + 24 * L + 4 * M);
+    key.reserve(7 + 24 * L + 4 * M);
     key.push_back(M); key.push_back(schedule); key.push_back(recompute); key.push_back(stage->layer->single_stream ? 1 : 0);
-    key.push_back(tuning().epoch);
+    key.push_back(tuning().epoch); key.push_back(lay.lanes);
     key.push_back(reinterpret_cast<uint64_t>(workspace));
     for (int l = 0; l < L; ++l) {
         const void* const* pp = reinterpret_cast<const void* const*>(&params[l]);

@@ -142,3 +142,40 @@ def test_whole_layer_launches_share_the_sms_by_the_lanes_in_use(pw):
             out.append(ys + dxs + [g for gs in grads for g in gs])
         for a, b in zip(*out):
             assert torch.equal(a, b), M
+
+
+@pytest.mark.parametrize("gpipe,recompute", [(True, True), (False, False)])
+def test_a_workspace_for_fewer_streams_is_enough(pw, gpipe, recompute):
+    """From one stream's size on every workspace is taken, nothing is written behind it, and no bit changes."""
+    w = inputs.Workload("lanes", 256, 4, 64, 512, 128, 2)
+    M, L = 6, 3
+    schedule = pw.SCHEDULE_GPIPE if gpipe else pw.SCHEDULE_PER_MICROBATCH
+    params = [[p.cuda() for p in inputs.layer_params(w, 0, l, random_ln=True)] for l in range(L)]
+    xs, dys = zip(*[[t.cuda().view(w.tokens, -1) for t in inputs.microbatch(w, 0, m)] for m in range(M)])
+    stage = pw.Stage(L, w.d_model, w.n_heads, w.head_dim, w.d_ff, w.seq_len, w.batch)
+    full = stage.workspace_bytes(M, schedule, recompute)
+    stage.set_side_stream(False)
+    one = stage.workspace_bytes(M, schedule, recompute)
+    stage.set_side_stream(True)
+    assert one < full == stage.workspace_bytes(M, schedule, recompute)
+    ws = torch.empty(full + 1024, dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.Stream()
+    ref = None
+    for dispatch, nbytes in [(pw.DISPATCH_OPBYOP, one), (pw.DISPATCH_ASYNC, full)] + [
+            (d, n) for n in (one, one + (full - one) // 3 - 1, one + (full - one) // 3, one + (full - one) // 3 * 2, full - 1)
+            for d in (pw.DISPATCH_ASYNC, pw.DISPATCH_GRAPH)]:
+        ws.fill_(255)
+        ys, dxs = [torch.empty_like(x) for x in xs], [torch.empty_like(x) for x in xs]
+        grads = [[torch.empty(p.shape, device="cuda") for p in ps] for ps in params]
+        torch.cuda.synchronize()
+        stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, schedule, recompute, stream=stream, workspace_bytes=nbytes)
+        torch.cuda.synchronize()
+        assert stage.status() == (0, 0) and (ws[nbytes:] == 255).all()
+        out = ys + dxs + [g for gs in grads for g in gs]
+        ref = out if ref is None else ref
+        for a, b in zip(ref, out):
+            assert torch.equal(a, b)
+    for dispatch in (pw.DISPATCH_OPBYOP, pw.DISPATCH_ASYNC):
+        with pytest.raises(pw.PwError) as e:
+            stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, schedule, recompute, workspace_bytes=one - 1)
+        assert e.value.status == 3
