@@ -463,7 +463,8 @@ pw_status_t pw_shared_close(void* dev_ptr);
  * has cached (Section 5.1's Fused mode re-captures on its next call).  Values out of range and
  * unknown knobs return PW_ERR_INVALID_ARG and change nothing.
  *   PW_TUNE_PDL               1 (default) / 0: launch kernels with programmatic dependent launch
- *   PW_TUNE_GEMM_PAIR         1 (default) / 0: no GEMM tile is shared by a CTA pair (every 128 x 128 tile a CTA of its own)
+ *   PW_TUNE_GEMM_PAIR         1 (default) / 0: no GEMM tile is shared by a CTA pair (every 128 x 128 tile a CTA of its own;
+ *                             a layer's weight gradients are then four launches instead of one)
  *   PW_TUNE_GEMM_BN           0 (default: chosen per shape) / 128 / 192 / 256: forced GEMM tile width
  *   PW_TUNE_GEMM_SPLIT        1 (default) / 0: cut the tiles of a thin last round along K
  *   PW_TUNE_GEMM_SPLIT_MIN_K  64 (default): ... only from this many 64-wide K blocks on

@@ -325,9 +325,10 @@ static pw_status_t do_wgrad(pw_layer_t* L, const WgradJob* jobs, int n, int accu
 {
     double flops = 0.0;
     for (int j = 0; j < n; ++j) flops += 2.0 * jobs[j].M * jobs[j].N * L->plan.T;
-    LaunchScope sc(L, PW_K_GEMM_NT, 1, flops, 0.0, st);
+    const int launches = wgrad_launches(n);
+    LaunchScope sc(L, PW_K_GEMM_NT, launches, flops, 0.0, st);
     const char* e = launch_wgrad(L->rt, jobs, n, L->plan.T, accumulate, late, L->status, st);
-    if (e) sc.cancel(1);
+    if (e) sc.cancel(launches);
     return e ? fail(PW_ERR_CUDA, e) : PW_OK;
 }
 static pw_status_t do_ln_fwd(pw_layer_t* L, const void* x, const void* gamma, const void* beta, void* h, void* mu,

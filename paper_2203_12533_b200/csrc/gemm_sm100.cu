@@ -759,6 +759,9 @@ static bool plan_cluster(const GemmArgs& a, int sms, GemmClusterPlan* plan)
 // Scratch for the K halves of cut tiles: (cut tile, half, CTA of the pair) x 128 rows x 256 columns, fp32.
 size_t gemm_split_ws_bytes() { return static_cast<size_t>(kSplitMaxTiles) * 2 * 2 * 128 * BN_MAX * sizeof(float); }
 
+static constexpr GemmClusterPlan kSingleCtaPlan = {0, 128, 1, 6};        // PW_TUNE_GEMM_PAIR 0: no CTA pairs anywhere
+int wgrad_launches(int n_jobs) { return tuning().gemm_pair == 0 ? n_jobs : 1; }
+
 const char* launch_wgrad(Runtime* rt, const WgradJob* jobs, int n_jobs, int K, int accumulate, bool late, DeviceStatus* status,
                          cudaStream_t stream)
 {
@@ -768,6 +771,19 @@ const char* launch_wgrad(Runtime* rt, const WgradJob* jobs, int n_jobs, int K, i
         const WgradJob& w = jobs[j];
         if (w.M <= 0 || w.N <= 0 || (w.M % 8) || (w.N % 8) || (w.lda % 8) || (w.ldb % 8) || (w.ldc % 4)) return "weight gradients: bad dimension";
         if (misaligned(w.A) || misaligned(w.B) || misaligned(w.C)) return "weight gradients: null or misaligned operand";
+    }
+    if (tuning().gemm_pair == 0) {
+        // One after the other, each with a wait of its own: what may follow a late launch may follow these too, for they started
+        // only after the kernel in front had let them, and the last of them ends after all of it.
+        for (int j = 0; j < n_jobs; ++j) {
+            const WgradJob& w = jobs[j];
+            GemmArgs g = {};
+            g.layout = kNT; g.epilogue = kEpiF32; g.M = w.M; g.N = w.N; g.K = K; g.accumulate = accumulate;
+            g.A = w.A; g.lda = w.lda; g.B = w.B; g.ldb = w.ldb; g.C = w.C; g.ldc = w.ldc;
+            const char* e = launch_gemm_cluster(rt, g, kSingleCtaPlan, status, stream);
+            if (e) return e;
+        }
+        return nullptr;
     }
     const int pairs = rt->sm_count / 2;
     auto cost = [&](int bn) {
@@ -821,10 +837,7 @@ const char* launch_gemm(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cu
     if (f32_out != (a.layout == kNT)) return "gemm: unsupported layout/epilogue combination";
     if (f32_out && (a.ldc % 4)) return "gemm: fp32 ldc must be a multiple of 4";
     GemmClusterPlan plan;
-    if (tuning().gemm_pair == 0) {                                   // no CTA pairs anywhere
-        plan = {0, 128, 1, 6};
-        return launch_gemm_cluster(rt, a, plan, status, stream);
-    }
+    if (tuning().gemm_pair == 0) return launch_gemm_cluster(rt, a, kSingleCtaPlan, status, stream);
     if (tuning().gemm_bn == 0 && plan_cluster(a, rt->sm_count, &plan)) return launch_gemm_cluster(rt, a, plan, status, stream);
     if (!f32_out) return launch_gemm_pair(rt, a, status, stream);
     const WgradJob w = {a.M, a.N, a.A, a.lda, a.B, a.ldb, a.C, a.ldc};

@@ -118,6 +118,7 @@ const char* launch_gemm_cluster(Runtime* rt, const GemmArgs& a, const GemmCluste
 constexpr int kWgradMaxJobs = 4;
 struct WgradJob { int M, N; const void* A; int lda; const void* B; int ldb; void* C; int ldc; };
 const char* launch_wgrad(Runtime* rt, const WgradJob* jobs, int n_jobs, int K, int accumulate, bool late, DeviceStatus* status, cudaStream_t stream);
+int wgrad_launches(int n_jobs);     // kernels that takes
 
 // Encodes the two tensor maps and launches.  Returns nullptr on success, else a static message.
 const char* launch_gemm(Runtime* rt, const GemmArgs& a, DeviceStatus* status, cudaStream_t stream);

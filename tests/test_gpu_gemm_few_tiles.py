@@ -89,7 +89,7 @@ def test_few_tiles(pw, M, N, K, kind):
 
 
 @pytest.mark.parametrize("knob,value", [("TUNE_GEMM_BN", 128), ("TUNE_GEMM_BN", 192), ("TUNE_GEMM_BN", 256), ("TUNE_GEMM_PAIR", 0)])
-@pytest.mark.parametrize("kind", ["bias", "resid", "gelu", "dgrad", "dgelu", "rowdot"])
+@pytest.mark.parametrize("kind", ["bias", "resid", "gelu", "dgrad", "dgelu", "rowdot", "wgrad"])
 @pytest.mark.parametrize("M,N,K", [(200, 5056, 264), (1000, 5184, 2056)])     # less than one pair's rows; tiles cut in two, ragged K
 def test_tile_widths(pw, M, N, K, kind, knob, value):
     before = pw.get_tuning(getattr(pw, knob))

@@ -61,3 +61,31 @@ def test_pool_of_a_layer(pw, d, H, F, S, B, alias, lean):
         assert torch.equal(g0, g1), name
     # fp32 sums of T products of bf16 values; lean: a's bf16 roundings of two GeLU forms differ by a tie here and there
     assert rel_l2(grads[10], dy.double().T @ a.double()) < (1e-3 if lean else 1e-5)
+
+
+@pytest.mark.parametrize("alias", [False, True], ids=["dx", "dx_over_dy"])
+def test_pool_without_cta_pairs(pw, alias):
+    """PW_TUNE_GEMM_PAIR = 0 reaches the weight gradients of a layer: four launches of single-CTA tiles, the same fp32 sums."""
+    w = inputs.Workload("pool", 512, 4, 128, 2048, 256, 4)
+    params = [p.cuda() for p in inputs.layer_params(w, 0, 0, random_ln=True)]
+    x, dy = (t.cuda().view(w.tokens, -1) for t in inputs.microbatch(w, 0, 0))
+    layer = make_layer(pw, w)
+    y, ctx = torch.empty_like(x), torch.empty(layer.ctx_bytes, dtype=torch.uint8, device="cuda")
+    scratch = torch.empty(layer.scratch_bytes, dtype=torch.uint8, device="cuda")
+    launches = {}
+    for value in (1, 0):
+        grads = [torch.full(p.shape, float("nan"), device="cuda") for p in params]
+        g = dy.clone()
+        pw.set_tuning(pw.TUNE_GEMM_PAIR, value)
+        try:
+            layer.fwd(params, x, y, ctx, scratch)
+            before = layer.launch_count()
+            layer.bwd(params, x, g, g if alias else torch.empty_like(x), grads, False, ctx, scratch)
+            launches[value] = layer.launch_count() - before
+        finally:
+            pw.set_tuning(pw.TUNE_GEMM_PAIR, 1)
+        torch.cuda.synchronize()
+        assert layer.status() == (0, 0) and all(torch.isfinite(t).all() for t in grads)
+        # fp32 sums of T products of bf16 values, as above
+        assert rel_l2(grads[10], dy.double().T @ layer.ctx_view(ctx, "a").double()) < 1e-5
+    assert launches[0] == launches[1] + (2 if alias else 3)
