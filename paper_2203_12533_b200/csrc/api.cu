@@ -1333,7 +1333,7 @@ pw_status_t pw_op_attention_bwd(const void* qkv, const void* o, const void* dout
                                 int dh, void* dqkv, void* delta, void* stream)
 {
     PW_RT_OR_FAIL();
-    if (!aligned(qkv, 16) || (o && !aligned(o, 16)) || !aligned(dout, 16) || !aligned(lse, 16) || !aligned(dqkv, 16) || !aligned(delta, 16))
+    if (!aligned(qkv, 16) || (o && !aligned(o, 16)) || !aligned(dout, 16) || !aligned(lse, 4) || !aligned(dqkv, 16) || !aligned(delta, 4))
         return fail(PW_ERR_INVALID_ARG, "attention bwd: NULL or misaligned pointer");
     PW_OP(launch_attention_bwd(rt, qkv, o, dout, lse, B, S, H, dh, dqkv, delta, rt->op_status, static_cast<cudaStream_t>(stream)));
     return PW_OK;

@@ -83,7 +83,8 @@ __device__ __forceinline__ bool kv_item(const BwdParams& p, int idx, KvItem& it)
 // Persistent: K_j / V_j are double-buffered across items (the finished item's buffer doubles as the
 // staging area of its dK / dV store while the next item's tiles are already in the other one); the
 // Q_u / dO_u ring, the S^T / dP^T buffers and every barrier phase run on across item boundaries.
-template <int DH>
+// ROWS: lse and delta come with the query tiles (16-byte aligned pointers).  Otherwise each thread reads its own from global memory.
+template <int DH, bool ROWS>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 64 x 128 rows
                         const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64 x 64 rows
@@ -124,10 +125,12 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
         }
     };
     auto load_q = [&](const KvItem& it, int i, int s) {     // Q_u and dO_u, u = 2j + i, and their rows' lse and delta
-        mbar_arrive_expect_tx(bar(L::kQF + s), 2 * L::kSub + 512);
-        const size_t row = (static_cast<size_t>(it.b) * p.H + it.h) * p.S + (2 * it.j + i) * 64;
-        bulk_load(sbase + L::kRow + s * 512, p.lse + row, 256, bar(L::kQF + s));
-        bulk_load(sbase + L::kRow + s * 512 + 256, p.delta + row, 256, bar(L::kQF + s));
+        mbar_arrive_expect_tx(bar(L::kQF + s), 2 * L::kSub + (ROWS ? 512 : 0));
+        if constexpr (ROWS) {
+            const size_t row = (static_cast<size_t>(it.b) * p.H + it.h) * p.S + (2 * it.j + i) * 64;
+            bulk_load(sbase + L::kRow + s * 512, p.lse + row, 256, bar(L::kQF + s));
+            bulk_load(sbase + L::kRow + s * 512 + 256, p.delta + row, 256, bar(L::kQF + s));
+        }
         const uint32_t qs = sbase + L::kQ + s * 2 * L::kSub, gs = qs + L::kSub;
         const int qrow = it.b * p.S + (2 * it.j + i) * 64;
         for (int kb = 0; kb < L::kBlocks; ++kb) {
@@ -313,7 +316,14 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
                 uint64_t nl2[4], ndl[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float2 l = lse2[4 * j], e = lse2[32 + 4 * j];
+                    float2 l, e;
+                    if constexpr (ROWS) {
+                        l = lse2[4 * j]; e = lse2[32 + 4 * j];
+                    } else {                                 // (past the L1, which may hold what was there before they were written)
+                        const size_t row = (static_cast<size_t>(it.b) * p.H + it.h) * p.S + qc0 + 2 * (lane & 3) + 8 * j;
+                        l = make_float2(__ldcg(p.lse + row), __ldcg(p.lse + row + 1));
+                        e = make_float2(__ldcg(p.delta + row), __ldcg(p.delta + row + 1));
+                    }
                     nl2[j] = fmul2(pack_f32x2(l.x, l.y), nlog2e);
                     ndl[j] = fmul2(pack_f32x2(e.x, e.y), neg1);
                 }
@@ -807,8 +817,9 @@ const char* encode_rows(Runtime* rt, CUtensorMap* map, const void* ptr, uint64_t
 
 const char* configure_attention_bwd_tc()
 {
-    if (cudaFuncSetAttribute(attn_bwd_dkdv_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, KvSmem<64>::kBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(attn_bwd_dkdv_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, KvSmem<128>::kBytes) != cudaSuccess)
+    auto attr = [](auto kern, int bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; };
+    if (!attr(attn_bwd_dkdv_tc_kernel<64, true>, KvSmem<64>::kBytes) || !attr(attn_bwd_dkdv_tc_kernel<128, true>, KvSmem<128>::kBytes) ||
+        !attr(attn_bwd_dkdv_tc_kernel<64, false>, KvSmem<64>::kBytes) || !attr(attn_bwd_dkdv_tc_kernel<128, false>, KvSmem<128>::kBytes))
         return "cudaFuncSetAttribute(attention bwd) failed";
     if (cudaFuncSetAttribute(attn_bwd_dq_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqSmem<64>::kBytes) != cudaSuccess ||
         cudaFuncSetAttribute(attn_bwd_dq_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqSmem<128>::kBytes) != cudaSuccess)
@@ -860,9 +871,10 @@ const char* launch_attention_bwd_dkdv(Runtime* rt, const void* qkv, const void* 
     p.B = B; p.tiles_per_seq = S / 128; p.n_items = B * H * p.tiles_per_seq;
     p.sched = status->sched + 4;
     dim3 grid(p.n_items < rt->sm_count ? p.n_items : rt->sm_count);
-    const cudaError_t e2 = dh == 64
-        ? launch_k(attn_bwd_dkdv_tc_kernel<64>, grid, dim3(kThreads), KvSmem<64>::kBytes, stream, tmKV, tmQ, tmDO, tmOut, p)
-        : launch_k(attn_bwd_dkdv_tc_kernel<128>, grid, dim3(kThreads), KvSmem<128>::kBytes, stream, tmKV, tmQ, tmDO, tmOut, p);
+    const bool rows = ((reinterpret_cast<uintptr_t>(lse) | reinterpret_cast<uintptr_t>(delta)) & 15) == 0;      // what a bulk copy takes
+    auto launch = [&](auto kern, int bytes) { return launch_k(kern, grid, dim3(kThreads), bytes, stream, tmKV, tmQ, tmDO, tmOut, p); };
+    const cudaError_t e2 = dh == 64 ? launch(rows ? attn_bwd_dkdv_tc_kernel<64, true> : attn_bwd_dkdv_tc_kernel<64, false>, KvSmem<64>::kBytes)
+                                    : launch(rows ? attn_bwd_dkdv_tc_kernel<128, true> : attn_bwd_dkdv_tc_kernel<128, false>, KvSmem<128>::kBytes);
     return e2 == cudaSuccess ? nullptr : "attention bwd (dk, dv) launch failed";
 }
 

@@ -78,6 +78,29 @@ def test_attention_bwd_items(pw, oracle64, B, S, H, dh):
         assert tile.max() < 2 * GRAD_TOL, (name, tile.max())
 
 
+@pytest.mark.parametrize("shift", [1, 2, 3])
+@pytest.mark.parametrize("B,S,H,dh", [(1, 128, 2, 64), (2, 384, 3, 128), (3, 640, 17, 64)])
+def test_attention_bwd_takes_any_float_pointers(pw, B, S, H, dh, shift):
+    """lse and delta at any multiple of four bytes give the bits of 16-byte aligned ones."""
+    g = torch.Generator().manual_seed(S + shift)
+    d, n = H * dh, B * H * S
+    q, do = bf16_randn((B * S, 3 * d), g).cuda(), bf16_randn((B * S, d), g).cuda()
+    o = torch.empty((B * S, d), dtype=torch.bfloat16, device="cuda")
+    got = []
+    for at in [(0, 0), (shift, 0), (0, shift), (shift, (shift + 1) % 4)]:
+        lse, delta = (torch.full((n + 4,), float("nan"), device="cuda")[k:k + n].view(B, H, S) for k in at)
+        dqkv, check = guard_alloc((B * S, 3 * d), torch.bfloat16)
+        pw.op_attention_fwd(q, B, S, H, dh, o, lse)
+        pw.op_attention_bwd(q, o, do, lse, B, S, H, dh, dqkv, delta)
+        torch.cuda.synchronize()
+        assert pw.op_status() == (0, 0)
+        check()
+        got.append(dqkv)
+    assert torch.isfinite(got[0]).all()
+    for t in got[1:]:
+        assert torch.equal(t, got[0])
+
+
 @pytest.mark.parametrize("B,S,H,dh", [(2, 4096, 16, 64), (2, 1024, 16, 64), (4, 1024, 16, 64), (1, 2048, 16, 128)])
 def test_attention_same_bits_every_time(pw, B, S, H, dh):
     """Thousands of launches back to back: warps of a tile that drift apart must not change a bit."""
