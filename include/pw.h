@@ -231,8 +231,8 @@ enum {
 };
 
 /* Outside OPBYOP the micro-batches of a chain take turns on up to four streams of the stage (forked from and joined to
- * the caller's), where the workspace that this takes is at most 1 GB beyond one stream's and no two micro-batches' buffers
- * overlap.  Same bits as on one stream; pw_stage_set_side_stream(stage, 0) keeps everything on the calling stream.  The streams
+ * the caller's), where the workspace that this takes is at most 1 GB beyond one stream's and neither two micro-batches' buffers nor
+ * two layers' gradients overlap.  Same bits as on one stream; pw_stage_set_side_stream(stage, 0) keeps everything on the calling stream.  The streams
  * and the handles that go with them (a status block each) are made here, with the stage. */
 pw_status_t pw_stage_create(const pw_layer_config_t* cfg, int n_layers, pw_stage_t** out);
 void pw_stage_destroy(pw_stage_t* stage);

@@ -13,7 +13,6 @@
 #include <mutex>
 #include <new>
 #include <string>
-#include <utility>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -871,24 +870,45 @@ pw_status_t pw_stage_workspace_bytes(const pw_stage_t* stage, int n_microbatches
 }
 
 namespace {
-// Do buffers of different micro-batches overlap (a caller that does not need every y may pass one for all)?  Then their
-// order matters and the chain keeps to one stream.
-bool microbatches_overlap(const void* const* x, const void* const* dy, void* const* y, void* const* dx, int M, size_t bytes)
+struct Span { uintptr_t begin, end; int owner; };
+// Do two spans of different owners overlap?
+bool owners_overlap(std::vector<Span>& spans)
 {
-    std::vector<std::pair<uintptr_t, int>> b;
-    b.reserve(4 * static_cast<size_t>(M));
-    for (int m = 0; m < M; ++m)
-        for (const void* q : {x[m], dy[m], static_cast<const void*>(y[m]), static_cast<const void*>(dx[m])})
-            b.emplace_back(reinterpret_cast<uintptr_t>(q), m);
-    std::sort(b.begin(), b.end());
-    uintptr_t end = 0, other_end = 0;            // furthest end so far, and the furthest of another micro-batch than that one's
+    std::sort(spans.begin(), spans.end(), [](const Span& a, const Span& b) { return a.begin < b.begin; });
+    uintptr_t end = 0, other_end = 0;            // furthest end so far, and the furthest of another owner than that one's
     int owner = -1;
-    for (const auto& [start, m] : b) {
-        if (start < (m == owner ? other_end : end)) return true;
-        if (m != owner) { other_end = end; owner = m; }
-        end = start + bytes;                     // starts ascend and all lengths are equal
+    for (const Span& s : spans) {
+        if (s.begin < (s.owner == owner ? other_end : end)) return true;
+        // (no overlap: begin >= the ends it was compared with, so a span of another owner ends furthest)
+        if (s.owner != owner) { other_end = end; owner = s.owner; end = s.end; }
+        else end = std::max(end, s.end);
     }
     return false;
+}
+
+// May the micro-batches run on several streams?  Not where their buffers overlap (a caller that does not need every y may pass
+// one for all), nor where two layers' gradients do (tied layers, or one buffer for what nobody reads): their order then matters.
+bool lanes_are_independent(const pw_stage_t* stage, const pw_layer_grads_t* grads, const void* const* x, const void* const* dy, void* const* y,
+                           void* const* dx, int M)
+{
+    const LayerPlan& p = stage->layer->plan;
+    std::vector<Span> spans;
+    spans.reserve(std::max<size_t>(4 * static_cast<size_t>(M), 12 * static_cast<size_t>(stage->n_layers)));
+    auto add = [&](const void* q, size_t bytes, int owner) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(q);
+        spans.push_back({a, a + bytes, owner});
+    };
+    const size_t act = static_cast<size_t>(p.T) * p.d * 2, d = p.d, F = p.F;
+    for (int m = 0; m < M; ++m)
+        for (const void* q : {x[m], dy[m], static_cast<const void*>(y[m]), static_cast<const void*>(dx[m])}) add(q, act, m);
+    if (owners_overlap(spans)) return false;
+    spans.clear();
+    const size_t n[12] = {d, d, 3 * d * d, 3 * d, d * d, d, d, d, F * d, F, d * F, d};      // as the members of pw_layer_grads_t
+    for (int l = 0; l < stage->n_layers; ++l) {
+        void* const* g = reinterpret_cast<void* const*>(&grads[l]);
+        for (int i = 0; i < 12; ++i) add(g[i], 4 * n[i], l);
+    }
+    return !owners_overlap(spans);
 }
 
 // Enqueues the whole chain on `st`.  sync_each = OPBYOP.
@@ -902,8 +922,7 @@ pw_status_t enqueue_chain(pw_stage_t* stage, const pw_layer_params_t* params, co
 {
     const int L = stage->n_layers;
     const bool gpipe = schedule == PW_SCHEDULE_GPIPE;
-    const int lanes = (lay.lanes > 1 && microbatches_overlap(x_mb, dy_mb, y_mb, dx_mb, M, static_cast<size_t>(stage->layer->plan.T) * stage->layer->plan.d * 2))
-                          ? 1 : lay.lanes;
+    const int lanes = lay.lanes > 1 && lanes_are_independent(stage, grads, x_mb, dy_mb, y_mb, dx_mb, M) ? lay.lanes : 1;
     auto lane_of = [&](int m) { return m % lanes; };
     auto handle = [&](int m) { return lane_of(m) == 0 ? stage->layer : stage->lanes[lane_of(m) - 1].layer; };
     auto stream = [&](int m) { return lane_of(m) == 0 ? st : stage->lanes[lane_of(m) - 1].stream; };

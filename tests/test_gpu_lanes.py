@@ -179,3 +179,34 @@ def test_a_workspace_for_fewer_streams_is_enough(pw, gpipe, recompute):
         with pytest.raises(pw.PwError) as e:
             stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, schedule, recompute, workspace_bytes=one - 1)
         assert e.value.status == 3
+
+
+@pytest.mark.parametrize("tied", ["layers", "one_vector", "partly"])
+def test_layers_that_share_gradient_buffers_keep_their_order(pw, tied):
+    """Two layers that write one gradient buffer: who writes when decides what stays, so the chain keeps to one stream."""
+    w = inputs.Workload("lanes", 256, 4, 64, 512, 128, 2)
+    M, L = 6, 4
+    params = [[p.cuda() for p in inputs.layer_params(w, 0, l, random_ln=True)] for l in range(L)]
+    xs, dys = zip(*[[t.cuda().view(w.tokens, -1) for t in inputs.microbatch(w, 0, m)] for m in range(M)])
+    stage = pw.Stage(L, w.d_model, w.n_heads, w.head_dim, w.d_ff, w.seq_len, w.batch)
+    ws = torch.empty(stage.workspace_bytes(M), dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.Stream()
+    ref = None
+    for dispatch in [pw.DISPATCH_OPBYOP] + [pw.DISPATCH_ASYNC, pw.DISPATCH_GRAPH] * 3:
+        ys, dxs = [torch.empty_like(x) for x in xs], [torch.empty_like(x) for x in xs]
+        grads = [[torch.empty(p.shape, device="cuda") for p in ps] for ps in params]
+        if tied == "layers":
+            grads[2] = grads[0]
+        elif tied == "one_vector":
+            grads[3][3] = grads[1][3]                        # b_qkv
+        else:
+            both = torch.empty(w.d_model + 64, device="cuda")
+            grads[0][0], grads[1][7] = both[:w.d_model], both[64:]           # ln1_gamma of one over ln2_beta of the other
+        torch.cuda.synchronize()
+        stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, stream=stream)
+        torch.cuda.synchronize()
+        assert stage.status() == (0, 0)
+        out = ys + dxs + [g for gs in grads for g in gs]
+        ref = out if ref is None else ref
+        for a, b in zip(ref, out):
+            assert torch.equal(a, b)
