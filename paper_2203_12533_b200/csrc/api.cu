@@ -1097,9 +1097,14 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
 pw_status_t pw_stage_status(pw_stage_t* stage, int* device_status, int* site)
 {
     if (!stage) return fail(PW_ERR_INVALID_ARG, "stage is NULL");
+    // every handle is read: one that gave up gets its work counters back even where another is the one reported
     int code = 0, where = 0;
     PW_DO(read_status(stage->layer->status, &code, &where));
-    for (size_t i = 0; i < stage->lanes.size() && code == 0; ++i) PW_DO(read_status(stage->lanes[i].layer->status, &code, &where));
+    for (const auto& lane : stage->lanes) {
+        int c = 0, w = 0;
+        PW_DO(read_status(lane.layer->status, &c, &w));
+        if (code == 0) { code = c; where = w; }
+    }
     if (device_status) *device_status = code;
     if (site) *site = where;
     return PW_OK;
