@@ -3,6 +3,7 @@
 // preprocess of the attention backward.  All use 16-byte accesses (8 bf16 per thread per
 // access), fp32 arithmetic, warp shuffles plus one shared-memory hop for row reductions, and
 // fixed-order two-stage reductions for anything summed over tokens (bitwise reproducible).
+#include <algorithm>
 #include <map>
 #include <mutex>
 
@@ -324,7 +325,9 @@ ln_bwd_kernel(const __nv_bfloat16* dh, const __nv_bfloat16* x,
     }
     constexpr int NQ = BIAS_SUMS ? 4 : 2;
     float* prow = partials + static_cast<size_t>(blockIdx.x) * NQ * d;
-    if (rows_per_cta > 1) {                             // narrow rows (one piece per thread): the CTA's row slots add up first
+    // Narrow rows (one piece per thread): the CTA's row slots add up first.  (Wider instances have one slot; with this code in them all the
+    // same, 4096 tokens x 8192 took 95.1 us instead of 91.5.)
+    if (CHUNKS == 1 && rows_per_cta > 1) {
         float* sums = reinterpret_cast<float*>(ln_bwd_ring);             // [slot][NQ][d], at most 8 K floats; the ring is idle
         cp_async_wait<0>();
         __syncthreads();
@@ -530,14 +533,17 @@ int colsum_splits(int sm_count, int T, int N)
     return r;
 }
 
-// A row slot takes at least four rows: on few tokens the partial rows, one per CTA, then stay a small part of the input.
-// (With one partial row per slot and a CTA for every group of rows, 1024 tokens x 512 left as many partial rows as there are
-// tokens: 11.8 us with the reduce launch, 5.5 now; 1024 x 1024 10.9 -> 7.5, 16384 x 1024 35.3 -> 32.1.)
+// A row slot takes at least four rows, unless that leaves fewer CTAs than keep the loads in flight: 64, or 128 for rows of
+// more than 4096, where a CTA has one slot and a row takes longer.  On few tokens the partial rows, one per CTA, then stay a small part
+// of the input.  us with the reduce launch, one row / four rows a slot / this: 128 tokens x 512 5.2 / 5.4 / 4.3, 1024 x 512 11.9 / 5.6 / 5.6,
+// 128 x 1024 4.7 / 5.6 / 4.5, 1024 x 1024 10.8 / 7.5 / 7.5, 256 x 2048 8.4 / 6.4 / 6.3, 128 x 6144 11.4 / 12.9 / 11.4, 128 x 8192 14.0 / 16.7 / 13.8,
+// 256 x 8192 16.9 / 18.6 / 16.1, 512 x 4096 10.0 / 10.5 / 10.6.
 int ln_bwd_grid(Runtime* rt, int T, const RowPlan& rp)
 {
     const int row_groups = (T + rp.rows_per_cta - 1) / rp.rows_per_cta;
-    const int cap = (rp.chunks == 1 ? 2 : 1) * rt->sm_count, want = (row_groups + 3) / 4;
-    return want < cap ? want : cap;
+    const int cap = (rp.chunks == 1 ? 2 : 1) * rt->sm_count;
+    const int least = rp.chunks == 4 ? std::min(row_groups, 128) : std::min((row_groups + 1) / 2, 64);
+    return std::min(std::max((row_groups + 3) / 4, least), cap);
 }
 
 }  // namespace

@@ -167,7 +167,8 @@ def test_gemm_rejects_bad_arguments(pw):
 
 
 # ------------------------------------------------------------------------------------------ LayerNorm / column sums
-@pytest.mark.parametrize("T,d", [(77, 256), (130, 1024), (515, 2048), (70, 4096), (33, 8192), (64, 1536)])
+@pytest.mark.parametrize("T,d", [(77, 256), (130, 1024), (515, 2048), (70, 4096), (33, 8192), (64, 1536),
+                                 (255, 1024), (261, 2048), (129, 6144), (530, 8192)])      # rows per CTA: two, four, one, four
 def test_layernorm_fwd_bwd(pw, oracle64, T, d):
     g = torch.Generator().manual_seed(6)
     x = bf16_randn((T, d), g, 2.0) + 0.5
