@@ -911,6 +911,12 @@ bool lanes_are_independent(const pw_stage_t* stage, const pw_layer_grads_t* grad
     return !owners_overlap(spans);
 }
 
+int chain_lanes(const pw_stage_t* stage, const StageLayout& lay, const pw_layer_grads_t* grads, const void* const* x, const void* const* dy,
+                void* const* y, void* const* dx, int M)
+{
+    return lay.lanes > 1 && lanes_are_independent(stage, grads, x, dy, y, dx, M) ? lay.lanes : 1;
+}
+
 // Enqueues the whole chain on `st`.  sync_each = OPBYOP.
 // With lanes, micro-batch m runs on lane m % lanes.  A lane keeps its own micro-batches in order; across lanes
 // the only ties are the parameter gradients: layer l of micro-batch m adds to what layer l of micro-batch m - 1 left, so its
@@ -922,7 +928,7 @@ pw_status_t enqueue_chain(pw_stage_t* stage, const pw_layer_params_t* params, co
 {
     const int L = stage->n_layers;
     const bool gpipe = schedule == PW_SCHEDULE_GPIPE;
-    const int lanes = lay.lanes > 1 && lanes_are_independent(stage, grads, x_mb, dy_mb, y_mb, dx_mb, M) ? lay.lanes : 1;
+    const int lanes = chain_lanes(stage, lay, grads, x_mb, dy_mb, y_mb, dx_mb, M);
     auto lane_of = [&](int m) { return m % lanes; };
     auto handle = [&](int m) { return lane_of(m) == 0 ? stage->layer : stage->lanes[lane_of(m) - 1].layer; };
     auto stream = [&](int m) { return lane_of(m) == 0 ? st : stage->lanes[lane_of(m) - 1].stream; };
@@ -1022,9 +1028,6 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
     StageLayout lay;
     const bool one_stream = dispatch_mode == PW_DISPATCH_OPBYOP || stage->layer->single_stream || stage->layer->profiling;
     pw_status_t s = stage_layout(stage, n_microbatches, schedule, recompute, one_stream, workspace_bytes, &lay);
-    if (s == PW_OK && log_enabled(PW_LOG_INFO))
-        log_line(PW_LOG_INFO, std::string("pw_stage_run_chain: ") + (dispatch_mode == PW_DISPATCH_OPBYOP ? "OPBYOP" : dispatch_mode == PW_DISPATCH_ASYNC ? "ASYNC" : "GRAPH") +
-                                  ", " + std::to_string(stage->n_layers) + " layers x " + std::to_string(n_microbatches) + " micro-batches" + (recompute ? ", recompute" : ""));
     if (s != PW_OK) return s;
     if (!aligned(workspace, 256)) return fail(PW_ERR_INVALID_ARG, "workspace is NULL or not 256-byte aligned");
     if (workspace_bytes < lay.total) return fail(PW_ERR_WORKSPACE_TOO_SMALL, "workspace smaller than pw_stage_workspace_bytes reports for one stream");
@@ -1035,6 +1038,12 @@ pw_status_t pw_stage_run_chain(pw_stage_t* stage, const pw_layer_params_t* param
         if (!aligned(x_mb[m], 16) || !aligned(dy_mb[m], 16) || !aligned(y_mb[m], 16) || !aligned(dx_mb[m], 16))
             return fail(PW_ERR_INVALID_ARG, "a micro-batch pointer is NULL or misaligned");
         if (x_mb[m] == y_mb[m] || x_mb[m] == dx_mb[m]) return fail(PW_ERR_INVALID_ARG, "y and dx must not alias x");
+    }
+    if (log_enabled(PW_LOG_INFO)) {
+        const int lanes = chain_lanes(stage, lay, grads, x_mb, dy_mb, y_mb, dx_mb, M);
+        log_line(PW_LOG_INFO, std::string("pw_stage_run_chain: ") + (dispatch_mode == PW_DISPATCH_OPBYOP ? "OPBYOP" : dispatch_mode == PW_DISPATCH_ASYNC ? "ASYNC" : "GRAPH") +
+                                  ", " + std::to_string(L) + " layers x " + std::to_string(M) + " micro-batches" + (recompute ? ", recompute" : "") + ", " +
+                                  std::to_string(lanes) + (lanes == 1 ? " stream" : " streams"));
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 

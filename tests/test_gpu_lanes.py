@@ -19,6 +19,19 @@ def pw():
     return binding
 
 
+def streams_of(pw, call):
+    """How many streams a chain call says that it uses."""
+    lines = []
+    pw.set_log(pw.LOG_INFO, lambda level, msg: lines.append(msg))
+    try:
+        call()
+    finally:
+        pw.set_log(pw.LOG_OFF)
+    chains = [line for line in lines if line.startswith("pw_stage_run_chain:")]
+    assert len(chains) == 1, lines
+    return int(chains[0].split(", ")[-1].split()[0])
+
+
 @pytest.mark.parametrize("width,heads,seq,batch,layers,M,flags", [
     (256, 4, 128, 2, 3, 1, 0), (256, 4, 128, 2, 3, 2, 0), (256, 4, 128, 1, 2, 5, 0), (256, 4, 128, 2, 3, 9, 0),     # four lanes
     (256, 4, 128, 2, 2, 6, "lean"), (256, 4, 128, 2, 3, 6, "whole"), (512, 8, 256, 2, 2, 3, "whole"),
@@ -40,7 +53,8 @@ def test_lanes_change_no_bit(pw, width, heads, seq, batch, layers, M, flags, gpi
         grads = [[torch.full(p.shape, 7.0, device="cuda") for p in ps] for ps in params]
         torch.cuda.synchronize()
         with torch.cuda.stream(stream):
-            stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, schedule, recompute, stream=stream)
+            n = streams_of(pw, lambda: stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, schedule, recompute, stream=stream))
+        assert n == (1 if dispatch == pw.DISPATCH_OPBYOP else min(M, 4 if w.tokens * width <= 256 * 256 else 2))
         torch.cuda.synchronize()
         assert stage.status() == (0, 0)
         return ys + dxs + [g for gs in grads for g in gs]
@@ -64,13 +78,17 @@ def test_one_buffer_for_every_output_keeps_the_last_micro_batch(pw):
     stage = pw.Stage(L, w.d_model, w.n_heads, w.head_dim, w.d_ff, w.seq_len, w.batch)
     ws = torch.empty(stage.workspace_bytes(M, pw.SCHEDULE_GPIPE, True), dtype=torch.uint8, device="cuda")
     ys, dxs = [torch.empty_like(x) for x in xs], [torch.empty_like(x) for x in xs]
-    stage.run_chain(params, grads, xs, dys, ys, dxs, ws, pw.DISPATCH_ASYNC)
+    chain = lambda ys: streams_of(pw, lambda: stage.run_chain(params, grads, xs, dys, ys, dxs, ws, pw.DISPATCH_ASYNC))
+    assert chain(ys) == 4
+    stage.set_side_stream(False)
+    assert chain(ys) == 1
+    stage.set_side_stream(True)
     y = torch.empty_like(xs[0])
     buf = torch.empty((w.tokens + 8, 256), dtype=torch.bfloat16, device="cuda")
-    stage.run_chain(params, grads, xs, dys, [y] * M, dxs, ws, pw.DISPATCH_ASYNC)
+    assert chain([y] * M) == 1
     part = [buf[:w.tokens]] + ys[1:-1] + [buf[8:]]           # the first and the last overlap by all but eight rows
     want = ys[-1].clone()
-    stage.run_chain(params, grads, xs, dys, part, dxs, ws, pw.DISPATCH_ASYNC)
+    assert chain(part) == 1
     torch.cuda.synchronize()
     assert torch.equal(y, want) and torch.equal(buf[8:], want)
 
@@ -136,7 +154,8 @@ def test_whole_layer_launches_share_the_sms_by_the_lanes_in_use(pw):
         for dispatch in (pw.DISPATCH_OPBYOP, pw.DISPATCH_ASYNC):
             ys, dxs = [torch.empty_like(x) for x in xs[:M]], [torch.empty_like(x) for x in xs[:M]]
             grads = [[torch.empty(p.shape, device="cuda") for p in ps] for ps in params]
-            stage.run_chain(params, grads, xs[:M], dys[:M], ys, dxs, ws, dispatch)
+            n = streams_of(pw, lambda: stage.run_chain(params, grads, xs[:M], dys[:M], ys, dxs, ws, dispatch))
+            assert n == (1 if dispatch == pw.DISPATCH_OPBYOP else min(M, 4))
             torch.cuda.synchronize()
             assert stage.status() == (0, 0)
             out.append(ys + dxs + [g for gs in grads for g in gs])
@@ -168,7 +187,9 @@ def test_a_workspace_for_fewer_streams_is_enough(pw, gpipe, recompute):
         ys, dxs = [torch.empty_like(x) for x in xs], [torch.empty_like(x) for x in xs]
         grads = [[torch.empty(p.shape, device="cuda") for p in ps] for ps in params]
         torch.cuda.synchronize()
-        stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, schedule, recompute, stream=stream, workspace_bytes=nbytes)
+        n = streams_of(pw, lambda: stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, schedule, recompute, stream=stream,
+                                                   workspace_bytes=nbytes))
+        assert n == (1 if dispatch == pw.DISPATCH_OPBYOP else 1 + (nbytes - one) * 3 // (full - one))
         torch.cuda.synchronize()
         assert stage.status() == (0, 0) and (ws[nbytes:] == 255).all()
         out = ys + dxs + [g for gs in grads for g in gs]
@@ -203,10 +224,37 @@ def test_layers_that_share_gradient_buffers_keep_their_order(pw, tied):
             both = torch.empty(w.d_model + 64, device="cuda")
             grads[0][0], grads[1][7] = both[:w.d_model], both[64:]           # ln1_gamma of one over ln2_beta of the other
         torch.cuda.synchronize()
-        stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, stream=stream)
+        assert streams_of(pw, lambda: stage.run_chain(params, grads, xs, dys, ys, dxs, ws, dispatch, stream=stream)) == 1
         torch.cuda.synchronize()
         assert stage.status() == (0, 0)
         out = ys + dxs + [g for gs in grads for g in gs]
         ref = out if ref is None else ref
         for a, b in zip(ref, out):
             assert torch.equal(a, b)
+
+
+def test_a_chain_first_called_inside_a_capture_uses_its_lanes(pw):
+    w = inputs.Workload("lanes", 256, 4, 64, 512, 128, 2)
+    M, L = 5, 2
+    params = [[p.cuda() for p in inputs.layer_params(w, 0, l, random_ln=True)] for l in range(L)]
+    xs, dys = zip(*[[t.cuda().view(w.tokens, -1) for t in inputs.microbatch(w, 0, m)] for m in range(M)])
+    out = []
+    for captured in (False, True):
+        stage = pw.Stage(L, w.d_model, w.n_heads, w.head_dim, w.d_ff, w.seq_len, w.batch)
+        ws = torch.empty(stage.workspace_bytes(M), dtype=torch.uint8, device="cuda")
+        ys, dxs = [torch.full_like(x, 7.0) for x in xs], [torch.full_like(x, 7.0) for x in xs]
+        grads = [[torch.full(p.shape, 7.0, device="cuda") for p in ps] for ps in params]
+        torch.cuda.synchronize()
+        call = lambda: stage.run_chain(params, grads, xs, dys, ys, dxs, ws, pw.DISPATCH_ASYNC)
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                assert streams_of(pw, call) == 4
+            graph.replay()
+        else:
+            call()
+        torch.cuda.synchronize()
+        assert stage.status() == (0, 0)
+        out.append(ys + dxs + [g for gs in grads for g in gs])
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
