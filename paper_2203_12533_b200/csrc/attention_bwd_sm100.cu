@@ -203,35 +203,31 @@ attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tmKV,   // qkv, box 
             const uint64_t desc_v = desc_advance(desc_k, L::kKV);
             const uint64_t dq = desc_slot<2 * L::kSub>(desc_q0, s), dg = desc_advance(dq, L::kSub);
             const uint32_t st = tb + hb * 64;
-            {
-                // the two products are independent accumulation chains: their steps alternate, so that a step
-                // never has to wait for the one before it to leave the pipe
+            // the two products are independent accumulation chains: their steps alternate, so that a step
+            // never has to wait for the one before it to leave the pipe
 #pragma unroll
-                for (int kb = 0; kb < L::kBlocks; ++kb)
+            for (int kb = 0; kb < L::kBlocks; ++kb)
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        umma_f16(st, desc_advance(desc_k, kb * 16384 + kk * 32), desc_advance(dq, kb * 8192 + kk * 32),
-                                 idesc_st, (kb | kk) ? 1u : 0u);
-                        umma_f16(st + L::kDP, desc_advance(desc_v, kb * 16384 + kk * 32), desc_advance(dg, kb * 8192 + kk * 32),
-                                 idesc_st, (kb | kk) ? 1u : 0u);
-                    }
-                umma_commit(bar(L::kSF + hb));
-            }
+                for (int kk = 0; kk < 4; ++kk) {
+                    umma_f16(st, desc_advance(desc_k, kb * 16384 + kk * 32), desc_advance(dq, kb * 8192 + kk * 32),
+                             idesc_st, (kb | kk) ? 1u : 0u);
+                    umma_f16(st + L::kDP, desc_advance(desc_v, kb * 16384 + kk * 32), desc_advance(dg, kb * 8192 + kk * 32),
+                             idesc_st, (kb | kk) ? 1u : 0u);
+                }
+            umma_commit(bar(L::kSF + hb));
         };
         auto issue_acc = [&](int s, int hb, bool first) {   // dV += P^T dO_u, dK += dS^T Q_u
             const uint64_t dq = desc_slot<2 * L::kSub>(desc_qt0, s), dg = desc_advance(dq, L::kSub);
             const uint32_t pt = tb + hb * 64;
             const uint32_t acc0 = first ? 0u : 1u;
-            {
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks) {             // dV and dK alternate (independent accumulators)
-                    umma_f16_ta(tb + L::kDV, pt + (ks >> 1) * 32 + (ks & 1) * 8, desc_advance(dg, ks * 2048), idesc_acc,
-                                ks ? 1u : acc0);
-                    umma_f16_ta(tb + L::kDK, pt + L::kDP + (ks >> 1) * 32 + (ks & 1) * 8, desc_advance(dq, ks * 2048), idesc_acc,
-                                ks ? 1u : acc0);
-                }
-                umma_commit(bar(L::kQE + s));               // Q_u / dO_u stage free
+            for (int ks = 0; ks < 4; ++ks) {             // dV and dK alternate (independent accumulators)
+                umma_f16_ta(tb + L::kDV, pt + (ks >> 1) * 32 + (ks & 1) * 8, desc_advance(dg, ks * 2048), idesc_acc,
+                            ks ? 1u : acc0);
+                umma_f16_ta(tb + L::kDK, pt + L::kDP + (ks >> 1) * 32 + (ks & 1) * 8, desc_advance(dq, ks * 2048), idesc_acc,
+                            ks ? 1u : acc0);
             }
+            umma_commit(bar(L::kQE + s));               // Q_u / dO_u stage free
         };
         auto wait = [&](int b, uint32_t parity, int site) {
             return mbar_wait(bar(b), parity, abort_flag, p.status, site);
@@ -580,32 +576,28 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
             const uint64_t dk = desc_slot<2 * L::kSub>(desc_k0, s);
             const uint64_t dv = desc_advance(dk, L::kSub);
             const uint32_t dst = tb + b * 128;
-            {
 #pragma unroll
-                for (int kb = 0; kb < L::kBlocks; ++kb)
+            for (int kb = 0; kb < L::kBlocks; ++kb)
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        umma_f16(dst, desc_advance(dq, kb * 16384 + kk * 32), desc_advance(dk, kb * 8192 + kk * 32),
-                                 idesc_sc, (kb | kk) ? 1u : 0u);
+                for (int kk = 0; kk < 4; ++kk)
+                    umma_f16(dst, desc_advance(dq, kb * 16384 + kk * 32), desc_advance(dk, kb * 8192 + kk * 32),
+                             idesc_sc, (kb | kk) ? 1u : 0u);
 #pragma unroll
-                for (int kb = 0; kb < L::kBlocks; ++kb)
+            for (int kb = 0; kb < L::kBlocks; ++kb)
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        umma_f16(dst + 64, desc_advance(dg, kb * 16384 + kk * 32), desc_advance(dv, kb * 8192 + kk * 32),
-                                 idesc_sc, (kb | kk) ? 1u : 0u);
-                umma_commit(bar(L::kSF + b));
-            }
+                for (int kk = 0; kk < 4; ++kk)
+                    umma_f16(dst + 64, desc_advance(dg, kb * 16384 + kk * 32), desc_advance(dv, kb * 8192 + kk * 32),
+                             idesc_sc, (kb | kk) ? 1u : 0u);
+            umma_commit(bar(L::kSF + b));
         };
         auto issue_dq = [&](int t, int s, int b, bool acc) {     // dQ_t += dS K_v (dS packed in the S columns of buffer b)
             const uint64_t dk = desc_slot<2 * L::kSub>(desc_kt0, s);
             const uint32_t dst = tb + L::kDQ + t * DH, src = tb + b * 128;
-            {
-                // dS packed bf16: keys 0..31 in columns 0..15 of S_t, keys 32..63 in columns 32..47
-                umma_f16_ta(dst, src, dk, idesc_dq, acc ? 1u : 0u);
+            // dS packed bf16: keys 0..31 in columns 0..15 of S_t, keys 32..63 in columns 32..47
+            umma_f16_ta(dst, src, dk, idesc_dq, acc ? 1u : 0u);
 #pragma unroll
-                for (int kq = 1; kq < 4; ++kq)
-                    umma_f16_ta(dst, src + (kq >> 1) * 32 + (kq & 1) * 8, desc_advance(dk, kq * 2048), idesc_dq, 1u);
-            }
+            for (int kq = 1; kq < 4; ++kq)
+                umma_f16_ta(dst, src + (kq >> 1) * 32 + (kq & 1) * 8, desc_advance(dk, kq * 2048), idesc_dq, 1u);
         };
         auto commit = [&](int b) {
             umma_commit(bar(b));
@@ -794,24 +786,6 @@ attn_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ,    // qkv, box 64
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// bf16 [rows, cols] row-major, box 64 columns x box_rows rows, 128-byte swizzle.
-const char* encode_rows(Runtime* rt, CUtensorMap* map, const void* ptr, uint64_t cols, uint64_t rows, uint32_t box_rows)
-{
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {cols * 2};
-    cuuint32_t box[2] = {64, box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = reinterpret_cast<EncodeTiledFn>(rt->encode_tiled)(
-        map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? nullptr : "cuTensorMapEncodeTiled failed";
-}
-
 }  // namespace
 
 
@@ -835,10 +809,10 @@ const char* launch_attention_bwd_dq(Runtime* rt, const void* qkv, const void* do
     const uint64_t T = static_cast<uint64_t>(B) * S;
     CUtensorMap tmQ, tmDO, tmKV, tmOut;
     const char* e;
-    if ((e = encode_rows(rt, &tmQ, qkv, 3ull * d, T, 128))) return e;
-    if ((e = encode_rows(rt, &tmDO, dout, d, T, 128))) return e;
-    if ((e = encode_rows(rt, &tmKV, qkv, 3ull * d, T, 64))) return e;
-    if ((e = encode_rows(rt, &tmOut, dqkv, 3ull * d, T, 128))) return e;
+    if ((e = encode_2d(rt, &tmQ, qkv, 3ull * d, T, 3ull * d, 64, 128))) return e;
+    if ((e = encode_2d(rt, &tmDO, dout, d, T, d, 64, 128))) return e;
+    if ((e = encode_2d(rt, &tmKV, qkv, 3ull * d, T, 3ull * d, 64, 64))) return e;
+    if ((e = encode_2d(rt, &tmOut, dqkv, 3ull * d, T, 3ull * d, 64, 128))) return e;
     BwdParams p;
     p.S = S; p.H = H; p.scale = 1.0f / sqrtf(static_cast<float>(dh));
     p.lse = static_cast<const float*>(lse); p.delta = static_cast<const float*>(delta);
@@ -860,10 +834,10 @@ const char* launch_attention_bwd_dkdv(Runtime* rt, const void* qkv, const void* 
     const uint64_t T = static_cast<uint64_t>(B) * S;
     CUtensorMap tmKV, tmQ, tmDO, tmOut;
     const char* e;
-    if ((e = encode_rows(rt, &tmKV, qkv, 3ull * d, T, 128))) return e;
-    if ((e = encode_rows(rt, &tmQ, qkv, 3ull * d, T, 64))) return e;
-    if ((e = encode_rows(rt, &tmDO, dout, d, T, 64))) return e;
-    if ((e = encode_rows(rt, &tmOut, dqkv, 3ull * d, T, 128))) return e;
+    if ((e = encode_2d(rt, &tmKV, qkv, 3ull * d, T, 3ull * d, 64, 128))) return e;
+    if ((e = encode_2d(rt, &tmQ, qkv, 3ull * d, T, 3ull * d, 64, 64))) return e;
+    if ((e = encode_2d(rt, &tmDO, dout, d, T, d, 64, 64))) return e;
+    if ((e = encode_2d(rt, &tmOut, dqkv, 3ull * d, T, 3ull * d, 64, 128))) return e;
     BwdParams p;
     p.S = S; p.H = H; p.scale = 1.0f / sqrtf(static_cast<float>(dh));
     p.lse = static_cast<const float*>(lse); p.delta = static_cast<const float*>(delta);

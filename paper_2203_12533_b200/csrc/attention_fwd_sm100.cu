@@ -576,24 +576,6 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_const
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// bf16 [rows, cols] row-major, box 64 columns x 128 rows, 128-byte swizzle.
-const char* encode_rows(Runtime* rt, CUtensorMap* map, const void* ptr, uint64_t cols, uint64_t rows)
-{
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {cols * 2};
-    cuuint32_t box[2] = {64, 128};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = reinterpret_cast<EncodeTiledFn>(rt->encode_tiled)(
-        map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? nullptr : "cuTensorMapEncodeTiled failed";
-}
-
 }  // namespace
 
 
@@ -612,8 +594,8 @@ const char* launch_attention_fwd(Runtime* rt, const void* qkv, int B, int S, int
     const int d = H * dh;
     CUtensorMap tmQKV, tmO;
     const char* e;
-    if ((e = encode_rows(rt, &tmQKV, qkv, 3ull * d, static_cast<uint64_t>(B) * S))) return e;
-    if ((e = encode_rows(rt, &tmO, o, d, static_cast<uint64_t>(B) * S))) return e;
+    if ((e = encode_2d(rt, &tmQKV, qkv, 3ull * d, static_cast<uint64_t>(B) * S, 3ull * d, 64, 128))) return e;
+    if ((e = encode_2d(rt, &tmO, o, d, static_cast<uint64_t>(B) * S, d, 64, 128))) return e;
     FwdParams p;
     p.S = S; p.H = H; p.B = B; p.scale = 1.0f / sqrtf(static_cast<float>(dh));
     // Pairs of query tiles share what they load and pay one prologue and epilogue for two; their longest item takes S / 128

@@ -349,8 +349,8 @@ const char* launch_gemm_cluster(Runtime* rt, const GemmArgs& a, const GemmCluste
     p.e.aux_out = a.aux_out; p.e.accumulate = a.accumulate; p.e.act = a.act;
     p.e.row_dot = static_cast<float*>(a.row_dot); p.e.head_dim = a.head_dim; p.e.seq_len = a.seq_len;
     p.K = a.K; p.bn = plan.bn; p.slices = plan.slices; p.stages = plan.stages;
-    p.tmem_cols = plan.bn;                               // 64, 128 or 256: what an allocation may be
-    p.log_groups = plan.bn == 256 ? 5 : plan.bn == 128 ? 4 : 3;
+    p.tmem_cols = plan.bn;                               // 64 or 128: what an allocation may be
+    p.log_groups = plan.bn == 128 ? 4 : 3;
     p.m_tiles = (a.M + tile_m - 1) / tile_m;
     p.status = status;
     const int n_tiles = (a.N + plan.bn - 1) / plan.bn;

@@ -269,7 +269,7 @@ __device__ __forceinline__ PairUnit pair_unit(const GemmParams& p, int v, int nu
     return u;
 }
 
-template <bool A_MN, bool B_MN, int EPI>
+template <bool B_MN, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<EPI>::kThreads, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmC,
                  const __grid_constant__ CUtensorMap tmOut2 /* kEpiBiasGelu: GeLU */, const __grid_constant__ CUtensorMap tmIn /* aux_in */,
@@ -340,12 +340,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     const uint32_t a_dst = ring0 + stage * P_STAGE_BYTES, b_dst = a_dst + A_TILE_BYTES;
                     const uint32_t fb = full_lead + 8 * stage;
                     if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * stage, pair_tx);
-                    if constexpr (!A_MN) {
-                        tma_load_2d_pair(a_dst, &tmA, kb * BK, m0, fb);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) tma_load_2d_pair(a_dst + j * 8192, &tmA, m0 + 64 * j, kb * BK, fb);
-                    }
+                    tma_load_2d_pair(a_dst, &tmA, kb * BK, m0, fb);
                     if constexpr (!B_MN) {
                         tma_load_2d_pair(b_dst, &tmB, kb * BK, n0, fb);
                     } else {
@@ -358,8 +353,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
     } else if (warp == 1) {
         if (rank == 0 && elect_one()) {
-            const uint32_t idesc = make_idesc_bf16(256, bn, A_MN, B_MN);
-            const uint64_t adesc0 = make_smem_desc_sw128(smem_u32(tiles), A_MN ? 8192 : 16, 1024);
+            const uint32_t idesc = make_idesc_bf16(256, bn, false, B_MN);
+            const uint64_t adesc0 = make_smem_desc_sw128(smem_u32(tiles), 16, 1024);
             const uint64_t bdesc0 = make_smem_desc_sw128(smem_u32(tiles) + A_TILE_BYTES, B_MN ? 8192 : 16, 1024);
             uint32_t stage = 0, phase = 0, it = 0;
             bool ok = true;
@@ -376,7 +371,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     // K-major: 16 k = 32 bytes along the swizzled 128-byte row; MN-major: two 8-k groups of 1024 B
 #pragma unroll
                     for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                        umma_f16_pair(d_tmem, desc_advance(ad, kk * (A_MN ? 2048 : 32)), desc_advance(bd, kk * (B_MN ? 2048 : 32)), idesc,
+                        umma_f16_pair(d_tmem, desc_advance(ad, kk * 32), desc_advance(bd, kk * (B_MN ? 2048 : 32)), idesc,
                                       (kb != un.kb0 || kk != 0) ? 1u : 0u);
                     umma_commit_pair(empty0 + 8 * stage, 3);     // frees the stage in both CTAs
                     if (++stage == kStages) { stage = 0; phase ^= 1; }
@@ -619,7 +614,7 @@ template <bool B_MN, int EPI>
 const char* launch_pair(Runtime* rt, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmC, const CUtensorMap& tmOut2,
                         const CUtensorMap& tmIn, const GemmParams& p, cudaStream_t stream)
 {
-    auto kern = gemm_pair_kernel<false, B_MN, EPI>;
+    auto kern = gemm_pair_kernel<B_MN, EPI>;
     const int total = p.total_virtual;
     const int max_pairs = rt->sm_count / 2;
     const int pairs = total < max_pairs ? total : max_pairs;
@@ -630,7 +625,7 @@ const char* launch_pair(Runtime* rt, const CUtensorMap& tmA, const CUtensorMap& 
 template <bool B_MN, int EPI>
 bool set_attr()
 {
-    return cudaFuncSetAttribute(gemm_pair_kernel<false, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES) == cudaSuccess;
+    return cudaFuncSetAttribute(gemm_pair_kernel<B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES) == cudaSuccess;
 }
 
 }  // namespace

@@ -304,7 +304,6 @@ __device__ __forceinline__ void umma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, ui
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// 32 lanes x 16 consecutive columns.
 // 16 lanes x 32 fp32 columns as an mma.sync accumulator holds them: thread i gets, for every group g of 8 columns, columns
 // 8 g + 2 (i % 4), + 1 of lane i / 4 in r[4 g], r[4 g + 1] and of lane i / 4 + 8 in r[4 g + 2], r[4 g + 3].
 __device__ __forceinline__ void tmem_ld_16x256_x4(uint32_t taddr, uint32_t* r)
@@ -322,6 +321,7 @@ __device__ __forceinline__ void tmem_st_16x128_x4(uint32_t taddr, const uint32_t
     asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                  :: "r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
 }
+// 32 lanes x 16 consecutive columns.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r)
 {
     asm volatile(

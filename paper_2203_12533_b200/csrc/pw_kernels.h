@@ -76,6 +76,26 @@ inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_
     return launch_cluster_k(kern, grid, block, smem, 1, st, static_cast<Args&&>(args)...);
 }
 
+// 2-D tensor map (bf16, or fp32 when f32 is set): `inner` contiguous elements per row, `outer`
+// rows, row pitch ld elements; 128-byte swizzle, so box_inner * element size must be 128 bytes
+// (64 bytes with swizzle64).
+inline const char* encode_2d(Runtime* rt, CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer, uint64_t ld,
+                             uint32_t box_inner, uint32_t box_outer, bool f32 = false, bool swizzle64 = false)
+{
+    typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                      const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                      CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    cuuint64_t dims[2] = {inner, outer};
+    cuuint64_t strides[1] = {ld * (f32 ? 4 : 2)};
+    cuuint32_t box[2] = {box_inner, box_outer};
+    cuuint32_t estr[2] = {1, 1};
+    CUresult r = reinterpret_cast<EncodeTiledFn>(rt->encode_tiled)(
+        map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? nullptr : "cuTensorMapEncodeTiled failed";
+}
+
 enum GemmLayout { kTN = 0, kNN = 1, kNT = 2 };
 enum GemmEpi { kEpiNone = 0, kEpiBias = 1, kEpiBiasResid = 2, kEpiBiasGelu = 3, kEpiDGelu = 4, kEpiF32 = 5,
                kEpiRowDot = 6 /* C bf16 = acc, and rowdot[b][h][s] = sum over the columns of head h of acc * aux_in */ };
@@ -102,8 +122,8 @@ size_t gemm_split_ws_bytes();
 // One cluster per output tile, the K range cut into slices (gemm_cluster_sm100.cu).
 struct GemmClusterPlan {
     int pair;                   // 1: 256-row tiles on CTA pairs, 0: 128-row tiles on single CTAs
-    int bn;                     // tile width: 64 (single CTAs only), 128 or 256
-    int slices;                 // K slices: 1, 2, 4 or 8; at most eight CTAs in a cluster
+    int bn;                     // tile width: 64 (single CTAs only) or 128
+    int slices;                 // K slices: 1, 2 or 4; at most eight CTAs in a cluster
     int stages;                 // ring depth, at most 8
 };
 // At least a third of an SM's shared memory per CTA: never more than two of them on an SM, whose TMEM two
