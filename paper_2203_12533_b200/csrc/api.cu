@@ -69,17 +69,12 @@ static pw_status_t fail_cuda(const char* what, cudaError_t e)
     return fail(PW_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-// Zeroes device memory before the call returns, on a stream of its own.  (cudaMemset runs on the legacy stream and does not hold
-// up the host: a first kernel on a non-blocking stream could start before it, or have its counters zeroed under it.)
-static cudaError_t clear_now(void* q, size_t bytes)
+// Zeroes device memory before the call returns, on a stream that nothing else uses.  (cudaMemset runs on the legacy stream and does
+// not hold up the host: a first kernel on a non-blocking stream could start before it, or have its counters zeroed under it.)
+static cudaError_t clear_now(Runtime* rt, void* q, size_t bytes)
 {
-    cudaStream_t s = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(q, 0, bytes, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaStreamDestroy(s);
-    return e;
+    const cudaError_t e = cudaMemsetAsync(q, 0, bytes, rt->clear_stream);
+    return e == cudaSuccess ? cudaStreamSynchronize(rt->clear_stream) : e;
 }
 
 Runtime* get_runtime(const char** err)
@@ -106,8 +101,9 @@ Runtime* get_runtime(const char** err)
     }
     const char* ce;
     if ((ce = configure_gemm()) || (ce = configure_gemm_cluster()) || (ce = configure_attention()) || (ce = configure_attention_fwd()) || (ce = configure_elementwise()) || (ce = configure_whole_layer())) { delete rt; *err = ce; return nullptr; }
-    if (cudaMalloc(reinterpret_cast<void**>(&rt->op_status), sizeof(DeviceStatus)) != cudaSuccess ||
-        clear_now(rt->op_status, sizeof(DeviceStatus)) != cudaSuccess) {
+    if (cudaStreamCreateWithFlags(&rt->clear_stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaMalloc(reinterpret_cast<void**>(&rt->op_status), sizeof(DeviceStatus)) != cudaSuccess ||
+        clear_now(rt, rt->op_status, sizeof(DeviceStatus)) != cudaSuccess) {
         delete rt; *err = "could not allocate the status word"; return nullptr;
     }
     // split-K scratch of the single-step GEMM call; without it that call simply never cuts a tile
@@ -145,7 +141,7 @@ struct pw_layer {
     // tied to one grid size).
     unsigned* whole_sync = nullptr;
     int whole_share = 1;            // lanes that share the SMs in the call being enqueued
-    cudaStream_t aux = nullptr;     // side stream: what a lean save set makes again runs beside the dgrad chain
+    cudaStream_t aux = nullptr;     // side stream (lean save set only): what it makes again runs beside the dgrad chain
     cudaEvent_t ev[2] = {nullptr, nullptr};
     uint64_t launches = 0;          // kernels launched (or replayed) through this handle
     bool single_stream = false;     // pw_layer_set_side_stream(layer, 0): everything on the calling stream
@@ -580,7 +576,7 @@ static bool grads_ok(const pw_layer_grads_t* G)
 }
 static bool aligned(const void* q, size_t a) { return q != nullptr && (reinterpret_cast<uintptr_t>(q) & (a - 1)) == 0; }
 
-static pw_status_t read_status(DeviceStatus* dev, int* code, int* site)
+static pw_status_t read_status(Runtime* rt, DeviceStatus* dev, int* code, int* site)
 {
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return fail_cuda("cudaDeviceSynchronize", e);
@@ -593,7 +589,7 @@ static pw_status_t read_status(DeviceStatus* dev, int* code, int* site)
     // mid-count; the device is idle here, so they are put back to zero (the error stays recorded).
     // (the same goes for the split-K tickets of the GEMM, which follow the counters in the struct)
     if (h.code != 0) {
-        e = clear_now(reinterpret_cast<char*>(dev) + offsetof(DeviceStatus, sched), sizeof(h.sched) + sizeof(h.tickets));
+        e = clear_now(rt, reinterpret_cast<char*>(dev) + offsetof(DeviceStatus, sched), sizeof(h.sched) + sizeof(h.tickets));
         if (e != cudaSuccess) return fail_cuda("work counters", e);
     }
     return PW_OK;
@@ -637,14 +633,16 @@ pw_status_t pw_layer_create(const pw_layer_config_t* cfg, pw_layer_t** out)
     L->rt = rt;
     build_plan(*cfg, rt, &L->plan);
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&L->status), sizeof(DeviceStatus));
-    if (e == cudaSuccess) e = clear_now(L->status, sizeof(DeviceStatus));
+    if (e == cudaSuccess) e = clear_now(rt, L->status, sizeof(DeviceStatus));
     if (e == cudaSuccess && L->plan.whole) {
         const size_t bytes = kMaxLanes * kWholeLayerSyncWords * sizeof(unsigned);
         e = cudaMalloc(reinterpret_cast<void**>(&L->whole_sync), bytes);
-        if (e == cudaSuccess) e = clear_now(L->whole_sync, bytes);
+        if (e == cudaSuccess) e = clear_now(rt, L->whole_sync, bytes);
     }
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&L->aux, cudaStreamNonBlocking);
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&L->ev[i], cudaEventDisableTiming);
+    if (L->plan.lean) {
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&L->aux, cudaStreamNonBlocking);
+        for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&L->ev[i], cudaEventDisableTiming);
+    }
     if (e != cudaSuccess) { pw_layer_destroy(L); return fail_cuda("handle resources (status word, side stream, events)", e); }
     if (log_enabled(PW_LOG_INFO)) {
         const LayerPlan& p = L->plan;
@@ -718,7 +716,7 @@ pw_status_t pw_layer_bwd(pw_layer_t* layer, const pw_layer_params_t* params, con
 pw_status_t pw_layer_status(pw_layer_t* layer, int* device_status, int* site)
 {
     if (!layer) return fail(PW_ERR_INVALID_ARG, "layer is NULL");
-    return read_status(layer->status, device_status, site);
+    return read_status(layer->rt, layer->status, device_status, site);
 }
 
 pw_status_t pw_layer_profile_begin(pw_layer_t* layer)
@@ -1108,10 +1106,10 @@ pw_status_t pw_stage_status(pw_stage_t* stage, int* device_status, int* site)
     if (!stage) return fail(PW_ERR_INVALID_ARG, "stage is NULL");
     // every handle is read: one that gave up gets its work counters back even where another is the one reported
     int code = 0, where = 0;
-    PW_DO(read_status(stage->layer->status, &code, &where));
+    PW_DO(read_status(stage->layer->rt, stage->layer->status, &code, &where));
     for (const auto& lane : stage->lanes) {
         int c = 0, w = 0;
-        PW_DO(read_status(lane.layer->status, &c, &w));
+        PW_DO(read_status(lane.layer->rt, lane.layer->status, &c, &w));
         if (code == 0) { code = c; where = w; }
     }
     if (device_status) *device_status = code;
@@ -1533,7 +1531,7 @@ pw_status_t pw_op_selftest_wait_timeout(uint64_t limit_cycles, int* kernel_retur
     if (limit > 2000000000ll) limit = 2000000000ll;            // about a second at most
     int* flag = nullptr;
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&flag), sizeof(int));
-    if (e == cudaSuccess) e = clear_now(flag, sizeof(int));
+    if (e == cudaSuccess) e = clear_now(rt, flag, sizeof(int));
     if (e != cudaSuccess) { if (flag) cudaFree(flag); return fail_cuda("self-test flag", e); }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const char* err = launch_wait_selftest(rt->op_status, limit, flag, st);
@@ -1590,14 +1588,14 @@ pw_status_t pw_op_status_reset(void)
 {
     PW_RT_OR_FAIL();
     cudaError_t e = cudaDeviceSynchronize();
-    if (e == cudaSuccess) e = clear_now(rt->op_status, sizeof(DeviceStatus));   // the device is idle: code, site, counters, tickets
+    if (e == cudaSuccess) e = clear_now(rt, rt->op_status, sizeof(DeviceStatus));   // the device is idle: code, site, counters, tickets
     return e == cudaSuccess ? PW_OK : fail_cuda("status reset", e);
 }
 
 pw_status_t pw_op_status(int* device_status, int* site)
 {
     PW_RT_OR_FAIL();
-    return read_status(rt->op_status, device_status, site);
+    return read_status(rt, rt->op_status, device_status, site);
 }
 
 }  // extern "C"
