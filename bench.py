@@ -31,10 +31,10 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
-# dram bytes read+written per GEMM launch (average over the 12 GEMM launches of a workload-2 step),
+# dram bytes read+written per GEMM launch (average over the nine GEMM launches of a workload-2 step),
 # from one ncu pass (dram__bytes_read.sum + dram__bytes_write.sum) over those launches; None for
 # workloads without a capture.
-GEMM_DRAM_TRAFFIC_PER_LAUNCH = {"cfg2_d2048_s1024_b8": 220.7e6}
+GEMM_DRAM_TRAFFIC_PER_LAUNCH = {"cfg2_d2048_s1024_b8": 311.4e6}
 
 
 def load_peaks():
@@ -484,7 +484,7 @@ def run_ours(args, w, brief=False):
         g = [prof[n] for n in ("gemm_tn", "gemm_nn", "gemm_nt")]
         g_flops, g_ms, g_n = sum(v["flops"] for v in g), sum(v["ms"] for v in g), sum(v["launches"] for v in g)
         line["roofline"] = gemm_roofline(g_flops, g_ms, g_n, tot_ms, ms_one_stream, args.steps, peaks,
-                                         "gemm_pair_kernel (tcgen05 bf16 GEMM: forward, dgrad and wgrad instantiations)",
+                                         "gemm_pair_kernel, wgrad_group_kernel, gemm_cluster_kernel (tcgen05 bf16 GEMMs)",
                                          GEMM_DRAM_TRAFFIC_PER_LAUNCH.get(w.name))
         line["ms_per_step_one_stream"] = ms_one_stream
 

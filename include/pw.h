@@ -73,7 +73,7 @@ enum { PW_ACT_GELU_ERF = 0, PW_ACT_GELU_TANH = 1 };
  * size 0 for the three tensors; pw_layer_fwd then needs `scratch` even when ctx is given. */
 enum { PW_FLAG_LEAN_CTX = 1u, PW_FLAG_WHOLE_LAYER = 2u };
 /* PW_FLAG_WHOLE_LAYER: pw_layer_fwd and pw_layer_bwd are ONE cooperative kernel launch each instead of
- * 7 and 15 - for calls so small that launches and hand-offs between kernels, not arithmetic, set the
+ * 7 and 11 - for calls so small that launches and hand-offs between kernels, not arithmetic, set the
  * time (Section 5.1, Figures 5 and 6: computations shorter than the cost of issuing them).  Same
  * tensors, same saved context, same bf16 hand-off points as the default path; results agree with
  * it within rounding (different tile shapes and summation orders), bit-reproducibly.  Supported:
@@ -230,7 +230,7 @@ enum {
     PW_SCHEDULE_PER_MICROBATCH = 1 /* forward and backward of micro-batch m before m+1              */
 };
 
-/* Outside OPBYOP the micro-batches of a chain take turns on up to four streams of the stage (forked from and joined to
+/* Outside OPBYOP the micro-batches of a chain of 2 to 64 layers take turns on up to four streams of the stage (forked from and joined to
  * the caller's), where the workspace that this takes is at most 1 GB beyond one stream's and neither two micro-batches' buffers nor
  * two layers' gradients overlap.  Same bits as on one stream; pw_stage_set_side_stream(stage, 0) keeps everything on the calling stream.  The streams
  * and the handles that go with them (a status block each) are made here, with the stage. */

@@ -762,6 +762,8 @@ pw_status_t pw_layer_launch_count(const pw_layer_t* layer, uint64_t* count)
 // of 8192 x 2048 47224 / 44959.  Whole-layer kernels share the SMs by lanes, so they stop gaining earlier: 256 x 256
 // 3252 / 2031 / 1782 / 2514, 1024 x 256 4791 / 3706 / 3748.
 // (Fewer micro-batches than lanes: 2 of 256 x 256 through 4 layers 795 with the SMs shared by four, 545 by two; 3 of them 916, 760 by three.)
+// One layer: no lanes, for only its forwards could overlap (the next micro-batch's backward adds to its gradients).  More than 64: an
+// event each is no longer a few.
 static int stage_lanes(const pw_stage_t* stage)
 {
     const LayerPlan& p = stage->layer->plan;
