@@ -20,9 +20,9 @@ def pw():
 
 
 def busy_default_stream():
-    """A few tenths of a second of work on the default stream, and an event behind it."""
+    """Most of a second of work on the default stream, and an event behind it."""
     torch.cuda.synchronize()
-    torch.cuda._sleep(500_000_000)
+    torch.cuda._sleep(1_500_000_000)
     done = torch.cuda.Event()
     done.record()
     return done

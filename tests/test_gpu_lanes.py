@@ -119,7 +119,7 @@ def test_first_chain_of_a_stage_beside_a_busy_default_stream(pw, dispatch, flags
     ys, dxs, grads = buffers()
     stream = torch.cuda.Stream()
     torch.cuda.synchronize()
-    torch.cuda._sleep(500_000_000)                           # a few tenths of a second of work on the default stream
+    torch.cuda._sleep(1_500_000_000)                         # most of a second of work on the default stream
     done = torch.cuda.Event()
     done.record()
     st = stage()
