@@ -474,16 +474,18 @@ __device__ __forceinline__ uint64_t exp2_poly2(uint64_t a)
 }
 
 // GeLU and GeLU' of two values at once, in two-wide fp32 instructions.  With x = |u| and the lower tail L(x) of the distribution function,
-//   GeLU(u) = max(u, 0) - x L(x),   GeLU'(u) = 1/2 + sign(u) (1/2 - D(x)),   D(x) = GeLU'(-x).
+//   GeLU(u) = max(u, 0) - x L(x),   GeLU'(u) = D(x) for u < 0, 1 - D(x) for u > 0,   D(x) = GeLU'(-x).
 // Erf form, one MUFU op a value: both have a smooth logarithm, L(x) = 2^P(x) and D(x) = (x0 - x) 2^Q(x) (x0: D's zero), so a
-// polynomial in the exponent gives them to fp32: P of degree 10 on [0, 7], Q of degree 9 on [0, 6.5], fitted here by iteratively
-// reweighted least squares for the smallest largest error of x L and of D (2.2e-9 and 1.0e-8; where these are below 3e-5, for the smallest
-// relative error).  The leading coefficients are negative, so that beyond the fit the tails go to zero.
+// polynomial in the exponent gives them: P of degree 10 on [0, 7], Q of degree 9 on [0, 9.5].  P was fitted by iteratively
+// reweighted least squares, Q as a linear program with its coefficients rounded one after the other, both for the smallest largest
+// error.  With the constants as they stand, in 64 bits: x L is off by at most 8.5e-9 and by 7.6e-5 of its value on [0, 7], D by at most
+// 1.7e-8 and from 5.5 on by at most 1 / x^2 of its value.  Beyond the fits (x L is 1e-11 at 7, D 1e-19 at 9.5) the leading coefficients,
+// which are negative, take the tails to zero sooner than they should go there: they lie between 0 and the value.
 // Tanh form, two: L(x) = 1 / (1 + e) with e = exp(2 z(x)), 1 - L = e L; for the derivative x is bounded so that e stays finite.
 // Errors against 64 bits, a Hastings-type erfc (reciprocal, exponential, six terms) and 1 - 2 / (exp(2 z) + 1) / these: normally distributed
-// u, root mean square, GeLU erf 2.64e-8 / 1.88e-8, tanh 3.38e-8 / 1.83e-8, derivative 3.63e-8 / 2.79e-8, 5.14e-8 / 2.96e-8; largest, |u| <= 6, GeLU
-// 4.47e-7 / 2.40e-7, 4.33e-7 / 2.38e-7, derivative 1.89e-7 / 1.16e-7, 1.97e-6 / 1.39e-7.  Cycles a value and scheduler (sixteen warps an SM): GeLU erf
-// 17.3 -> 13.8, tanh 25.6 -> 16.5, derivative times a factor 18.9 -> 16.5, 29.5 -> 19.3.
+// u, root mean square, GeLU erf 2.64e-8 / 1.88e-8, tanh 3.38e-8 / 1.83e-8, derivative 3.63e-8 / 2.22e-8, 5.23e-8 / 2.50e-8; largest, |u| <= 6, GeLU
+// 4.47e-7 / 2.40e-7, 4.33e-7 / 2.38e-7, derivative 1.94e-7 / 9.5e-8, 1.97e-6 / 1.20e-7; mean over -5 < u < -4, derivative 7.5e-9 / 3.5e-9,
+// 8.1e-7 / 3e-11, over -10 < u < -9 1.2e-20 / 2e-21, 1e-28 / 3e-34.
 template <int N>
 __device__ __forceinline__ uint64_t poly2(const float (&c)[N], uint64_t x)
 {
@@ -520,14 +522,11 @@ __device__ __forceinline__ void gelu_from_tail(float& u0, float& u1, uint64_t ta
     u0 = fmaf(-fabsf(u0), t0, fmaxf(u0, 0.f));
     u1 = fmaf(-fabsf(u1), t1, fmaxf(u1, 0.f));
 }
-// g *= 1/2 + sign(u) (1/2 - D): the sign of u is OR-ed into 1/2 - D (>= 0), no compare / select
-__device__ __forceinline__ void mul_by_grad(float& g0, float& g1, float u0, float u1, uint64_t D)
+// -sign(u) (of -0: +1) and the step function that goes with it: D then stays a small number of its own for u < 0.
+__device__ __forceinline__ void sign_and_step(float u0, float u1, uint64_t& minus_sign, uint64_t& step)
 {
-    float s0, s1;
-    unpack_f32x2(ffma2(D, pack_f32x2(-1.0f, -1.0f), pack_f32x2(0.5f, 0.5f)), s0, s1);
-    s0 = __uint_as_float(__float_as_uint(s0) | (__float_as_uint(u0) & 0x80000000u));
-    s1 = __uint_as_float(__float_as_uint(s1) | (__float_as_uint(u1) & 0x80000000u));
-    unpack_f32x2(fmul2(pack_f32x2(g0, g1), fadd2(pack_f32x2(s0, s1), pack_f32x2(0.5f, 0.5f))), g0, g1);
+    minus_sign = pack_f32x2(copysignf(1.0f, -u0), copysignf(1.0f, -u1));
+    step = ffma2(minus_sign, pack_f32x2(-0.5f, -0.5f), pack_f32x2(0.5f, 0.5f));
 }
 __device__ __forceinline__ void gelu2_erf(float& u0, float& u1)
 {
@@ -559,22 +558,27 @@ __device__ __forceinline__ void gelu2(float& u0, float& u1, int act)
 // g0, g1 *= GeLU'(u0), GeLU'(u1)
 __device__ __forceinline__ void gelu_grad_mul2_erf(float& g0, float& g1, float u0, float u1)
 {
-    constexpr float kQ[10] = {-0.588404536f, -0.383201301f, -0.560572028f, -0.0551539063f, 0.0152386362f, -0.0032621522f,
-                              0.00050939736f, -5.32459781e-05f, 3.2489877e-06f, -8.53910507e-08f};
+    constexpr float kQ[10] = {-0.588404536f, -0.383201122f, -0.560573637f, -0.0551479943f, 0.0152288247f, -0.00325373653f,
+                              0.000505461416f, -5.22578848e-05f, 3.12947805e-06f, -8.04726952e-08f};
     constexpr float kZero = 0.75179153f;
-    const uint64_t x = pack_f32x2(fabsf(u0), fabsf(u1));
-    mul_by_grad(g0, g1, u0, u1, fmul2(ex2_2(poly2(kQ, x)), ffma2(x, pack_f32x2(-1.0f, -1.0f), pack_f32x2(kZero, kZero))));
+    uint64_t ms, step;
+    sign_and_step(u0, u1, ms, step);
+    // step - sign D = step + 2^Q (u - sign x0)
+    const uint64_t grad = ffma2(ex2_2(poly2(kQ, pack_f32x2(fabsf(u0), fabsf(u1)))), ffma2(ms, pack_f32x2(kZero, kZero), pack_f32x2(u0, u1)), step);
+    unpack_f32x2(fmul2(pack_f32x2(g0, g1), grad), g0, g1);
 }
 __device__ __forceinline__ void gelu_grad_mul2_tanh(float& g0, float& g1, float u0, float u1)
 {
     constexpr float kC0 = 1.5957692f, kC1 = 0.21406445f;     // 2 z'(x) = c0 + c1 x^2
-    constexpr float kFar = 9.5f;                             // D is below 1e-30 there, e below 2^112
+    constexpr float kFar = 10.05f;                           // e is 2^127.6 there, finite, and its reciprocal flushed to zero: D = 0
     const uint64_t x = pack_f32x2(min_or_nan(fabsf(u0), kFar), min_or_nan(fabsf(u1), kFar)), x2 = fmul2(x, x);
-    uint64_t e, tail;
+    uint64_t e, tail, ms, step;
     tanh_tail(x, x2, e, tail);
+    sign_and_step(u0, u1, ms, step);
     // D = L (1 - (1 - L) x 2 z')
     const uint64_t q = fmul2(x, ffma2(x2, pack_f32x2(-kC1, -kC1), pack_f32x2(-kC0, -kC0)));
-    mul_by_grad(g0, g1, u0, u1, fmul2(tail, ffma2(fmul2(e, tail), q, pack_f32x2(1.0f, 1.0f))));
+    const uint64_t D = fmul2(tail, ffma2(fmul2(e, tail), q, pack_f32x2(1.0f, 1.0f)));
+    unpack_f32x2(fmul2(pack_f32x2(g0, g1), ffma2(ms, D, step)), g0, g1);
 }
 __device__ __forceinline__ void gelu_grad_mul2(float& g0, float& g1, float u0, float u1, int act)
 {

@@ -45,10 +45,25 @@ def gelu_grad(pw, u, f, act):
     return got
 
 
+def allowance(act, x, want, grad):
+    """What the fp32 evaluation may be off by, before its rounding to bf16.  Body: a few roundings of 2^-24 and the fits' error, of |u| for GeLU
+    and of 1 for the derivative.  Lower tail: the fits' error relative to the value (7.6e-5 for L; 1.7e-8, but at most 1 / x^2 of the value, for D; the
+    tanh form has only roundings, 2^-24 of an exponent of up to 2^7), and beyond the fits, or where fp32 ends, no more than the value itself."""
+    ax, aw = x.abs(), want.abs()
+    body = (1.5e-7 if grad else 2e-7 * ax) + 0 * ax
+    if act == 1:
+        tail, end = 2e-5 * aw, 9.9
+    elif grad:
+        tail, end = torch.minimum(2e-8 + 0 * ax, aw / (x * x)), 9.5
+    else:
+        tail, end = 1.5e-4 * aw, 7.0
+    return torch.where((x < -3), torch.where(ax <= end, tail, aw), body) + 1e-35
+
+
 @pytest.mark.parametrize("act", [0, 1])
 def test_every_exponent(pw, act):
-    """All bf16 values from 2^-20 to the largest, both signs: bf16 of the exact value to half a spacing and 1e-6, and the limits
-    far out: u and 0 for GeLU, 1 and 0 for the derivative."""
+    """All bf16 values from 2^-20 to the largest, both signs: bf16 of the exact value to half a spacing and what the evaluation may be off by, and the
+    limits far out: u and 0 for GeLU, 1 and 0 for the derivative."""
     bits = torch.arange((127 - 20) << 7, 0x7f80, dtype=torch.int32, device="cuda")
     v = torch.cat([bits, bits + 0x8000]).to(torch.int16).view(torch.bfloat16)
     v = torch.cat([v, torch.zeros(-len(v) % 128, dtype=torch.bfloat16, device="cuda")])
@@ -60,13 +75,14 @@ def test_every_exponent(pw, act):
     d = gelu_grad(pw, u, one, act)
     x = v.double()
     far = x.abs() > 40
-    for got, want, limit in ((a, exact(x, act)[0], torch.where(x > 0, x, 0.0)), (d, exact(x, act)[1], (x > 0).double())):
+    for got, want, limit, grad in ((a, exact(x, act)[0], torch.where(x > 0, x, 0.0), False), (d, exact(x, act)[1], (x > 0).double(), True)):
         assert torch.equal(got[:, 0], got[:, 127])
         g = got[:, 5].double()
         assert ((g - limit).abs()[far] <= 1e-30 * limit.abs()[far] + 1e-30).all()
         near = ~far
-        err, spacing = (g - want).abs()[near], torch.exp2(torch.floor(torch.log2(want.abs().clamp_min(2.0 ** -100))) - 7)[near]
-        assert (err <= 0.51 * spacing + 1e-6).all(), err.max()
+        err, spacing = (g - want).abs(), torch.exp2(torch.floor(torch.log2(want.abs().clamp_min(2.0 ** -126))) - 7)
+        bad = (err > 0.51 * spacing + allowance(act, x, want, grad)) & near
+        assert not bad.any(), (x[bad][:8].tolist(), g[bad][:8].tolist(), want[bad][:8].tolist())
 
 
 # 1 - 2 / (exp(2 z) + 1) gives 3.4e-8 and 5.1e-8 root mean square before rounding; what is in use 1.8e-8 and 3.0e-8 (the mean of the
