@@ -5,6 +5,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <float.h>
 #include <stdint.h>
 
 namespace pw {
@@ -514,13 +515,15 @@ __device__ __forceinline__ float min_or_nan(float a, float b)
     asm("min.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
     return y;
 }
-// u, x = |u| -> max(u, 0) - x L
+// u -> max(u, 0) - |u| L.  At u = infinity L is 0: the factor is bounded, so that the product is 0 too (at minus infinity it is no number, as
+// u times the distribution function is none).
+__device__ __forceinline__ float gelu_from_tail(float u, float tail) { return fmaf(-fabsf(fminf(u, FLT_MAX)), tail, fmaxf(u, 0.f)); }
 __device__ __forceinline__ void gelu_from_tail(float& u0, float& u1, uint64_t tail)
 {
     float t0, t1;
     unpack_f32x2(tail, t0, t1);
-    u0 = fmaf(-fabsf(u0), t0, fmaxf(u0, 0.f));
-    u1 = fmaf(-fabsf(u1), t1, fmaxf(u1, 0.f));
+    u0 = gelu_from_tail(u0, t0);
+    u1 = gelu_from_tail(u1, t1);
 }
 // -sign(u) (of -0: +1) and the step function that goes with it: D then stays a small number of its own for u < 0.
 __device__ __forceinline__ void sign_and_step(float u0, float u1, uint64_t& minus_sign, uint64_t& step)

@@ -85,6 +85,22 @@ def test_every_exponent(pw, act):
         assert not bad.any(), (x[bad][:8].tolist(), g[bad][:8].tolist(), want[bad][:8].tolist())
 
 
+# a tile of its own, and CTA pairs
+@pytest.mark.parametrize("m,n", [(128, 128), (4096, 4096)])
+@pytest.mark.parametrize("act", [0, 1])
+def test_infinities(pw, act, m, n):
+    """What u times the distribution function gives: infinity at infinity, no number at minus infinity and for none."""
+    A, B = torch.zeros((m, 8), dtype=torch.bfloat16, device="cuda"), torch.zeros((n, 8), dtype=torch.bfloat16, device="cuda")
+    A[:, 0], B[:, 0] = 1.0, 1.0
+    A[5, 0], A[70, 0], A[99, 0] = math.inf, -math.inf, math.nan
+    u, a = gelu(pw, A, B, act, n)
+    assert (u[5] == math.inf).all() and (u[70] == -math.inf).all() and torch.isnan(u[99]).all()
+    assert (a[5] == math.inf).all() and torch.isnan(a[70]).all() and torch.isnan(a[99]).all()
+    rest = torch.ones(m, dtype=torch.bool, device="cuda")
+    rest[[5, 70, 99]] = False
+    assert (a[rest] == torch.nn.functional.gelu(torch.ones((), device="cuda"), approximate="tanh" if act else "none").to(torch.bfloat16)).all()
+
+
 # 1 - 2 / (exp(2 z) + 1) gives 3.4e-8 and 5.1e-8 root mean square before rounding; what is in use 1.8e-8 and 3.0e-8 (the mean of the
 # magnitudes, which is measured here, is lower).
 def test_tanh_form(pw):
