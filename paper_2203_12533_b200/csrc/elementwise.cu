@@ -460,7 +460,7 @@ ln_bwd_rows_kernel(const __nv_bfloat16* dh, const __nv_bfloat16* x, const float*
         }
         const uint4 out = make_uint4(w[0], w[1], w[2], w[3]);
         if (live) *reinterpret_cast<uint4*>(dx + off + 256 * j) = out;
-        if (BIAS_SUMS) mine[3 * kTensor + 32 * j] = out;
+        if (BIAS_SUMS) mine[3 * kTensor + 32 * j] = live ? out : make_uint4(0, 0, 0, 0);    // (0 times an infinite gamma is no zero)
     }
     __syncthreads();
     // columns 4 c .. + 3 of the eight rows

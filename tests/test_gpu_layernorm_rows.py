@@ -63,3 +63,24 @@ def test_forward_against_64_bits(pw, T, d):
     assert ((h.double() - want).abs() <= 2.0 ** -8 * want.abs() + 1e-5).all()
     assert (mu.double() - m).abs().max() < 1e-6 and ((rstd.double() - r) / r).abs().max() < 1e-6
     assert torch.isnan(buf[0].float()).all() and torch.isnan(buf[-1].float()).all()
+
+
+# one row of eight, a started eighth, and the persistent form
+@pytest.mark.parametrize("T,d", [(1, 256), (9, 512), (17, 1280), (3, 4096)])
+def test_infinite_gamma(pw, T, d):
+    """An infinity in gamma takes whole rows of dx to infinities (and to no numbers): their column sums are those of the rows that are there."""
+    g = torch.Generator(device="cuda").manual_seed(T * 5 + d)
+    n = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    row, gamma = n(1, d), n(d)
+    x, dh, resid = (t.expand(T, d).contiguous() for t in (row, n(1, d), n(1, d)))
+    gamma[7] = float("inf")
+    mu, rstd = x.double().mean(1).float(), (x.double().var(1, unbiased=False) + 1e-5).rsqrt().float()
+    dx = torch.empty_like(x)
+    vec = [torch.zeros(d, device="cuda") for _ in range(4)]
+    part = torch.empty(pw.op_layernorm_bwd_scratch_bytes(T, d), dtype=torch.uint8, device="cuda")
+    pw.op_layernorm_bwd(dh, x, mu, rstd, gamma, resid, dx, *vec, False, part)
+    torch.cuda.synchronize()
+    want = dx.float().sum(0)
+    assert torch.isinf(want).sum() > d // 8                    # (equal rows: no infinities of both signs in a column)
+    assert torch.equal(torch.isnan(vec[3]), torch.isnan(want)) and torch.equal(vec[3][torch.isinf(want)], want[torch.isinf(want)])
+    assert all(torch.isfinite(v).all() for v in vec[:3])
