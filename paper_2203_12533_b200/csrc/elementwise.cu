@@ -392,14 +392,14 @@ ln_bwd_kernel(const __nv_bfloat16* dh, const __nv_bfloat16* x,
 // CTA's one barrier a thread owns columns and adds up the eight rows.  What bounds it is one trip to memory and the two
 // hand-overs, where the persistent kernel above makes a trip, a barrier and two exchanges for every row of a slot.  Figures: ln_bwd_by_rows.
 constexpr int kLnRows = 8;
-constexpr int ln_rows_smem_bytes(int ch) { return 4 * kLnRows * 512 * ch; }
+constexpr int ln_rows_smem_bytes(int ch, bool sums) { return (sums ? 4 : 3) * kLnRows * 512 * ch; }      // dx stays there for its sums only
 template <int CH, bool BIAS_SUMS>
 __global__ void __launch_bounds__(32 * kLnRows)
 ln_bwd_rows_kernel(const __nv_bfloat16* dh, const __nv_bfloat16* x, const float* mu, const float* rstd, const __nv_bfloat16* gamma,
                    const __nv_bfloat16* resid, int T, __nv_bfloat16* dx, float* partials)
 {
     constexpr int d = 256 * CH, kPieces = d / 8;            // 16-byte pieces of a row
-    extern __shared__ uint4 ln_rows_smem[];                 // [dh, x, resid, dx][row][piece]
+    extern __shared__ uint4 ln_rows_smem[];                 // [dh, x, resid, with BIAS_SUMS dx][row][piece]
     __shared__ float stats[kLnRows][2];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = blockIdx.x * kLnRows + warp;
@@ -668,7 +668,8 @@ int colsum_splits(int sm_count, int T, int N)
 // 3.9 -> 3.0, 2048 x 256 4.8 -> 4.5, 3072 x 256 5.3 -> 5.7; 1024 x 512 5.6 -> 3.8, 4096 x 512 8.4 -> 8.4, 8192 x 512 13.5 -> 14.3; 512 x 1024
 // 5.8 -> 4.2, 1024 x 1024 7.5 -> 4.7, 2368 x 1024 9.8 -> 8.7, 4096 x 1024 13.6 -> 12.2, 8192 x 1024 19.7 -> 20.1; 2048 x 1280 12.6 -> 7.6, 4096 x 1280
 // 18.6 -> 14.2, 4096 x 1792 19.6 -> 18.3, 6144 x 1792 25.6 -> 26.1; a row of 2048 leaves one CTA an SM: 512 x 2048 8.6 -> 6.0, 2048 x 2048 15.0 -> 14.0,
-// 3072 x 2048 17.9 -> 19.5, and 128 x 2048 5.2 -> 5.7.
+// 3072 x 2048 17.9 -> 19.5, and 128 x 2048 5.2 -> 5.7.  Without the two bias sums the lines lie where they do with them: 256 x 2048 5.05 -> 5.15, 512 x 2048
+// 6.4 -> 5.7, 2048 x 2048 12.7 -> 12.5, 4096 x 1792 17.3 -> 15.8, 4096 x 1024 12.3 -> 11.3.
 bool ln_bwd_by_rows(int T, int d)
 {
     return d < 2048 ? T <= (d == 256 ? 2048 : 4096) : d == 2048 && T > 128 && T <= 2048;
@@ -720,8 +721,8 @@ const char* configure_elementwise()
 #define PW_LN_ATTR(C, B) if (e == cudaSuccess) e = cudaFuncSetAttribute(ln_bwd_kernel<C, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, ln_bwd_depth(C) * 3 * C * kRowThreadsMax * 16)
     PW_LN_ATTR(1, true); PW_LN_ATTR(1, false); PW_LN_ATTR(2, true); PW_LN_ATTR(2, false); PW_LN_ATTR(4, true); PW_LN_ATTR(4, false);
 #undef PW_LN_ATTR
-#define PW_LN_ATTR(N) if (e == cudaSuccess) e = cudaFuncSetAttribute(ln_bwd_rows_kernel<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ln_rows_smem_bytes(N)); \
-                      if (e == cudaSuccess) e = cudaFuncSetAttribute(ln_bwd_rows_kernel<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ln_rows_smem_bytes(N))
+#define PW_LN_ATTR(N) if (e == cudaSuccess) e = cudaFuncSetAttribute(ln_bwd_rows_kernel<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ln_rows_smem_bytes(N, true)); \
+                      if (e == cudaSuccess) e = cudaFuncSetAttribute(ln_bwd_rows_kernel<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ln_rows_smem_bytes(N, false))
     PW_LN_ATTR(1); PW_LN_ATTR(2); PW_LN_ATTR(3); PW_LN_ATTR(4); PW_LN_ATTR(5); PW_LN_ATTR(6); PW_LN_ATTR(7); PW_LN_ATTR(8);
 #undef PW_LN_ATTR
     return e == cudaSuccess ? nullptr : "could not raise the shared-memory limit of the layernorm kernels";
@@ -756,8 +757,8 @@ const char* launch_layernorm_bwd_partial(Runtime* rt, const void* dh, const void
     const size_t ring_bytes = static_cast<size_t>(ln_bwd_depth(rp.chunks)) * 3 * rp.chunks * rp.threads * 16;
     const bool sums = db_resid != nullptr || db_dx != nullptr;
 #define PW_LN_BWD(C, B) le = launch_k(ln_bwd_kernel<C, B>, dim3(grid), dim3(rp.threads), ring_bytes, stream, DH, X, Mu, Rs, G, R, T, d, DX, P, rp.tpr, rp.rows_per_cta)
-#define PW_LN_ROWS(N) case N: le = sums ? launch_k(ln_bwd_rows_kernel<N, true>, dim3(grid), dim3(32 * kLnRows), ln_rows_smem_bytes(N), stream, DH, X, Mu, Rs, G, R, T, DX, P) \
-                                        : launch_k(ln_bwd_rows_kernel<N, false>, dim3(grid), dim3(32 * kLnRows), ln_rows_smem_bytes(N), stream, DH, X, Mu, Rs, G, R, T, DX, P); break
+#define PW_LN_ROWS(N) case N: le = sums ? launch_k(ln_bwd_rows_kernel<N, true>, dim3(grid), dim3(32 * kLnRows), ln_rows_smem_bytes(N, true), stream, DH, X, Mu, Rs, G, R, T, DX, P) \
+                                        : launch_k(ln_bwd_rows_kernel<N, false>, dim3(grid), dim3(32 * kLnRows), ln_rows_smem_bytes(N, false), stream, DH, X, Mu, Rs, G, R, T, DX, P); break
     if (by_rows) {
         switch (d / 256) { PW_LN_ROWS(1); PW_LN_ROWS(2); PW_LN_ROWS(3); PW_LN_ROWS(4); PW_LN_ROWS(5); PW_LN_ROWS(6); PW_LN_ROWS(7); PW_LN_ROWS(8); default: return "layernorm: unsupported row width"; }
     } else switch (rp.chunks) {
