@@ -1199,9 +1199,10 @@ const char* launch_whole_layer(Runtime* rt, WholeLayerArgs a, bool backward, int
     // Where three or four lanes share the SMs, a lane's CTAs take several units one after the other in every phase, each a chain of latencies: two CTAs
     // an SM, of half the registers, then run two such chains side by side.  Chains of 4 layers x 8 micro-batches, us one -> two: 256 tokens
     // 1720 -> 1532, 512 tokens 2395 -> 2181, 4 micro-batches 1032 -> 895 and 1441 -> 1258; 8 layers x 8 of 256 tokens 3119 -> 2840.  Not for wider rows (their
-    // panel does not fit twice) and not from 1024 tokens on, where attention's longer loops feel the spilled registers (4031 -> 4541), nor for one or
-    // two lanes (2 of 512 tokens 726 -> 784).  The same for every call of a handle that shares the SMs alike, for the grid barrier counts on it.
-    const bool two = a.d == 256 && share > 2 && a.T <= 512;
+    // panel does not fit twice), nor for one or two lanes (2 of 512 tokens 726 -> 784).  That more than two lanes end at 512 tokens (stage_lanes) suits
+    // it: at 1024, with four lanes all the same, attention's longer loops feel the spilled registers (4031 -> 4541).  The same for every call of a
+    // handle that shares the SMs alike, for the grid barrier counts on it.
+    const bool two = a.d == 256 && share > 2;
     const cudaError_t e = two ? launch_coop(backward ? whole_layer_bwd_kernel<2> : whole_layer_fwd_kernel<2>, 2 * grid / share, Lay<2>::kBytes, stream, a)
                               : launch_coop(backward ? whole_layer_bwd_kernel<1> : whole_layer_fwd_kernel<1>, grid / share, Lay<1>::kBytes, stream, a);
     return e == cudaSuccess ? nullptr : cudaGetErrorString(e);

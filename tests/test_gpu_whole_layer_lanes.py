@@ -1,4 +1,4 @@
-"""Whole-layer chains on three and four lanes, where two CTAs share an SM: the same bits as one call after the other."""
+"""Whole-layer chains on two, three and four lanes (on three and four two CTAs share an SM): the same bits as one call after the other."""
 import pytest
 import torch
 
@@ -17,7 +17,7 @@ def pw():
     return binding
 
 
-# the fewest tokens, K ranges of two to sixteen blocks, several key blocks, the most tokens with two CTAs an SM and the first without
+# the fewest tokens, K ranges of two to sixteen blocks, several key blocks, the most tokens with two CTAs an SM, and so many that the chain takes two lanes
 @pytest.mark.parametrize("F,S,B,M", [(128, 128, 1, 4), (1024, 128, 2, 3), (1024, 128, 2, 5), (640, 384, 1, 4), (1408, 128, 3, 4), (1024, 512, 1, 4), (1024, 128, 4, 3), (1024, 640, 1, 4)])
 def test_same_bits(pw, F, S, B, M):
     w = inputs.Workload("lanes", 256, 4, 64, F, S, B, sigma_w=0.05)
