@@ -52,8 +52,15 @@ __device__ __forceinline__ uint4 pack8(const float* f)
 // A kernel launched with the programmatic-serialization attribute may start while the previous
 // kernel of its stream is still running.  grid_dep_launch() lets the next kernel be scheduled as
 // early as possible; grid_dep_wait() blocks until the previous kernel has completed and its
-// memory is visible - every kernel calls it before its first global-memory access, so only the
-// launch latency and the on-chip set-up overlap.  Both are no-ops for a plain launch.
+// memory is visible.  Both are no-ops for a plain launch.  A kernel calls grid_dep_wait() before its first
+// global-memory access, so only the launch latency and the on-chip set-up overlap, with these exceptions:
+//   GEMMs of kOrderWeightsReady (see GemmOrder) read B and the bias before it.  Safe because LN1, or the first GEMM of a backward, waits BEFORE it
+//     lets its successor start: whoever runs behind it runs after all that was written in front of the call.
+//   The dK/dV kernel waits at its end only: the dQ kernel in front of it waits before it lets it start, reads the same inputs and
+//     writes other columns.
+//   The weight gradients of a layer with `late` set, and the column sums behind them, likewise: LN1 backward in front of them waits before it lets them
+//     start, and nothing that they read is written by it (see launch_wgrad).
+// Each of them still waits before it ends, so that its own end means the end of all in front of it.
 // A kernel that uses TMEM allocates it (and passes a CTA-wide barrier) BEFORE grid_dep_launch(): the next
 // kernel's CTAs may then share an SM with it, and one that got its TMEM first would wait for a predecessor
 // that waits for its TMEM.

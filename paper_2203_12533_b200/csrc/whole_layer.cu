@@ -4,8 +4,9 @@
 // Section 5.1 (Figures 5 and 6), where a computation is shorter than the cost of issuing it.
 //
 // The 7 forward / 11 backward launches of the multi-kernel path become 5 / 7 phases of one persistent grid
-// (one 256-thread CTA per SM); a phase is a list of independent units (a 64 x 64 output tile of a
-// GEMM, a slice of its K range, 64 query or key rows of one head, four LayerNorm rows, 16 columns of
+// (one 256-thread CTA per SM; two where a chain of 256-wide rows shares the SMs among three or four lanes, see
+// Lay and launch_whole_layer); a phase is a list of independent units (a 64 x 64 output tile of a
+// GEMM, a slice of its K range, 64 query or key rows of one head, eight LayerNorm rows, 32 columns of
 // a bias sum) that the CTAs take round-robin, and phases are separated by a bounded grid barrier.
 // Steps that do not depend on one another share a phase (a data-gradient GEMM, the weight-gradient
 // GEMM and the bias sum that hang off the same tensor), LayerNorm is applied while a GEMM stages its
