@@ -17,8 +17,9 @@ def pw():
     return binding
 
 
-# Hastings' five terms give 1.08e-7 and 5.4e-8 here with a correctly rounded reciprocal, 1.06e-7 and 5.7e-8 with one to an ulp; the six
-# terms in use 2.5e-8 and 2.8e-8, of which the roundings of the last products are most.  The bounds lie between.
+# Hastings' five terms give 1.08e-7 and 5.4e-8 here with a correctly rounded reciprocal, 1.06e-7 and 5.7e-8 with one to an ulp, six fitted
+# terms 2.5e-8 and 2.8e-8; the polynomials in the exponent that are in use 6.4e-9 and 1.8e-8, of which the roundings of the last products are most.
+# The bounds lie between.
 M, N = 4096, 16384
 
 
